@@ -106,3 +106,25 @@ def test_frame_bits_i_frame_and_refined_ranges(gs):
     oc, _, _ = Q.quantize(p, q.bits, refine=True)
     ref = B.code_entropy_bits(oc, q.bits).sum() + 64 * sum(b > 0 for b in q.bits)
     assert got == pytest.approx(ref, rel=1e-12)
+
+
+@pytest.mark.parametrize("n", [3000, 65535, 65536])
+def test_code_entropy_symbol_widths_and_counts(gs, n):
+    """Both sides of the column count up to which rows are counted in shared
+    memory, every layout of its counters (up to 10 bits, wider), counts on
+    both sides of the tally's 2048, and rows of one symbol."""
+    from paper_2505_09324_gb300.quant import code_bits
+    rng = np.random.default_rng(n)
+    bits = [Q.HALF, 16, 15, 11, 10, 9, 1, 10, 12]
+    c = np.zeros((9, n), np.uint16)
+    c[0] = rng.integers(0, 1 << 16, n)
+    c[1] = 65535  # one symbol, the last counter
+    for r in (2, 3, 4, 5, 6):
+        c[r] = rng.integers(0, 1 << bits[r], n)
+    c[7] = np.where(rng.random(n) < 0.9, 1023, rng.integers(0, 1024, n))
+    c[8] = np.minimum(rng.geometric(0.3, n) - 1, 4095)
+    sel = (rng.random(n) < 0.5).astype(np.uint8)
+    for s in (None, sel):
+        got = code_bits(dev_codes(c), bits,
+                        None if s is None else torch.from_numpy(s).cuda()).cpu().numpy()
+        np.testing.assert_allclose(got, B.code_entropy_bits(c, bits, s), rtol=1e-12, atol=1e-8)
