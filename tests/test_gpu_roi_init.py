@@ -173,3 +173,17 @@ def test_roi_init_equals_its_trace(gs):
     b, nb, _, _ = gs.roi_init_trace(f, m, 600, 0.7, bg)
     assert na == nb
     assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("w,h,n,frac", [
+    (1, 1, 2, 0.5), (31, 15, 300, 1.0), (33, 17, 561, 1.0), (97, 49, 40, 0.9),
+    (200, 130, 26, 1.0), (200, 130, 25, 1.0)])
+def test_tile_edges_and_both_sum_paths(gs, w, h, n, frac):
+    """Sizes around the assignment's 32 x 16 tiles, a step of one pixel (the
+    most cells a tile can see), and steps of 31.6 and 32.2 pixels, either side
+    of the line between gathered and atomic segment sums."""
+    frame, mask = conferencing_frame(max(w, 8), max(h, 8), seed=w)
+    frame, mask = np.ascontiguousarray(frame[:, :h, :w]), np.ones((h, w), bool)
+    if w == 97:
+        mask[:, ::3] = False
+    check_step_by_step(gs, frame, mask, n, frac, seed=5)
