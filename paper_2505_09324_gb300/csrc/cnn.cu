@@ -731,84 +731,6 @@ __global__ void k_head_decode_bwd(const float* __restrict__ out, int ldo, int B,
   }
 }
 
-// Nearest neighbour of every point of P among Q (per frame): points are rows
-// 0, 1 of [9][count] parameter blocks.
-__global__ void __launch_bounds__(256)
-k_nearest(const float* __restrict__ P, int np, int ldp, const float* __restrict__ Q, int nq,
-          int ldq, int* __restrict__ nn, float* __restrict__ dist) {
-  __shared__ float2 s_q[1024];
-  const int b = blockIdx.y;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const float* pb = P + (size_t)b * np;
-  const float* qb = Q + (size_t)b * nq;
-  const float px = i < np ? pb[i] : 0.0f, py = i < np ? pb[ldp + i] : 0.0f;
-  float best = INFINITY;
-  int arg = 0;
-  for (int j0 = 0; j0 < nq; j0 += 1024) {
-    const int cnt = min(1024, nq - j0);
-    __syncthreads();
-    for (int k = threadIdx.x; k < cnt; k += blockDim.x)
-      s_q[k] = make_float2(qb[j0 + k], qb[(size_t)ldq + j0 + k]);
-    __syncthreads();
-    for (int k = 0; k < cnt; k++) {
-      const float dx = px - s_q[k].x, dy = py - s_q[k].y;
-      const float d = fmaf(dx, dx, dy * dy);
-      if (d < best) {
-        best = d;
-        arg = j0 + k;
-      }
-    }
-  }
-  if (i < np) {
-    nn[(size_t)b * np + i] = arg;
-    dist[(size_t)b * np + i] = best;
-  }
-}
-
-// Gradient of the Chamfer term with respect to the predicted means: each
-// predicted point towards its nearest target, each target pulling its
-// nearest predicted point (accumulated with atomics).  Also the per-frame
-// loss (a fixed-order sum).
-__global__ void __launch_bounds__(256)
-k_chamfer_grad(const float* __restrict__ P, int np, int ldp, const float* __restrict__ Q, int nq,
-               int ldq, const int* __restrict__ nn1, const int* __restrict__ nn2, float lambda,
-               float* __restrict__ dP) {
-  const int b = blockIdx.y;
-  const float* pb = P + (size_t)b * np;
-  const float* qb = Q + (size_t)b * nq;
-  float* db = dP + (size_t)b * np;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < np) {
-    const int j = nn1[(size_t)b * np + i];
-    atomicAdd(&db[i], lambda * 2.0f * (pb[i] - qb[j]) / (float)np);
-    atomicAdd(&db[ldp + i], lambda * 2.0f * (pb[ldp + i] - qb[ldq + j]) / (float)np);
-  }
-  if (i < nq) {
-    const int k = nn2[(size_t)b * nq + i];
-    atomicAdd(&db[k], lambda * 2.0f * (pb[k] - qb[i]) / (float)nq);
-    atomicAdd(&db[ldp + k], lambda * 2.0f * (pb[ldp + k] - qb[ldq + i]) / (float)nq);
-  }
-}
-
-__global__ void __launch_bounds__(1024)
-k_chamfer_loss(const float* __restrict__ d1, int np, const float* __restrict__ d2, int nq,
-               float* __restrict__ loss) {
-  __shared__ double s[32];
-  const int b = blockIdx.x;
-  double a = 0.0, c = 0.0;
-  for (int i = threadIdx.x; i < np; i += blockDim.x) a += d1[(size_t)b * np + i];
-  for (int i = threadIdx.x; i < nq; i += blockDim.x) c += d2[(size_t)b * nq + i];
-  double v = a / np + c / nq;
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = v;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double tot = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); w++) tot += s[w];
-    loss[b] = (float)tot;
-  }
-}
-
 }  // namespace
 
 extern "C" uint64_t gs2d_head_smem_bytes(int32_t gh, int32_t gw, int32_t slots) {
@@ -856,29 +778,4 @@ extern "C" gs2d_status gs2d_head_decode_bwd(const float* out, int32_t ldo, int32
                                                          scale, n, sel, dparams, ldp,
                                                          static_cast<bf16*>(dout));
   return launched("gs2d_head_decode_bwd");
-}
-
-extern "C" uint64_t gs2d_chamfer_scratch_bytes(int32_t n, int32_t m, int32_t B) {
-  return (uint64_t)B * ((uint64_t)n + m) * (sizeof(int) + sizeof(float)) + 64;
-}
-
-extern "C" gs2d_status gs2d_chamfer(const float* params, int32_t n, int32_t ldp,
-                                    const float* targets, int32_t m, int32_t ldq, int32_t B,
-                                    float lambda, float* dparams, float* loss, void* scratch,
-                                    void* stream) {
-  if (n < 1 || m < 1 || B < 1 || !params || !targets || !scratch ||
-      (int64_t)ldp < (int64_t)B * n || (int64_t)ldq < (int64_t)B * m)
-    return set_error(GS2D_ERR_INVALID_ARG, "gs2d_chamfer: arguments");
-  cudaStream_t s = (cudaStream_t)stream;
-  int* nn1 = static_cast<int*>(scratch);
-  int* nn2 = nn1 + (size_t)B * n;
-  float* d1 = reinterpret_cast<float*>(nn2 + (size_t)B * m);
-  float* d2 = d1 + (size_t)B * n;
-  k_nearest<<<dim3((n + 255) / 256, B), 256, 0, s>>>(params, n, ldp, targets, m, ldq, nn1, d1);
-  k_nearest<<<dim3((m + 255) / 256, B), 256, 0, s>>>(targets, m, ldq, params, n, ldp, nn2, d2);
-  if (dparams)
-    k_chamfer_grad<<<dim3((std::max(n, m) + 255) / 256, B), 256, 0, s>>>(
-        params, n, ldp, targets, m, ldq, nn1, nn2, lambda, dparams);
-  if (loss) k_chamfer_loss<<<B, 1024, 0, s>>>(d1, n, d2, m, loss);
-  return launched("gs2d_chamfer");
 }

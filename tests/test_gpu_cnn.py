@@ -446,3 +446,55 @@ def test_implicit_conv_bad_arguments(nat):
     with pytest.raises(nat.Gs2dError):   # no room for the bias column
         nat.call("gs2d_conv_bf16", d.data_ptr(), 1, 4, 4, 8, 3, 2, 1, d.data_ptr(), 72, 8, 1, 0,
                  d.data_ptr(), 8, 0, 0)
+
+
+def _chamfer_sets():
+    g = np.random.Generator(np.random.PCG64(77))
+    lattice = np.stack(np.meshgrid(np.arange(20.0), np.arange(20.0)), -1).reshape(-1, 2)
+    spread = g.uniform(0, 1000, (3000, 2))
+    far = np.concatenate([g.normal(500, 3, (2500, 2)), [[1e6, -1e6], [-3e5, 2e4]]])
+    line = np.stack([np.full(700, 3.0), np.arange(700.0)], 1)
+    broken = g.uniform(0, 50, (90, 2))
+    broken[[3, 40], 0], broken[7, 1] = np.nan, np.inf
+    return {"spread": (spread, g.uniform(-100, 1100, (2000, 2))), "far": (far, spread[:50]),
+            "ties": (lattice, np.concatenate([lattice + 0.5, lattice + 0.5])),
+            "same": (np.ones((300, 2)), np.full((500, 2), 4.0)), "line": (line, line[::-1] + 0.25),
+            "one": (np.zeros((1, 2)), spread), "broken": (spread[:64], broken)}
+
+
+@pytest.mark.parametrize("name", list(_chamfer_sets()))
+def test_chamfer_nearest_neighbours(nat, name):
+    """The grid search against a scan of all pairs: spread and clustered sets,
+    far outliers, exact ties (lowest index), identical points, a line, one
+    point, non-finite targets.  lambda is chosen so that the gradient shows
+    which neighbour was taken."""
+    P, Q = (np.ascontiguousarray(s, np.float32) for s in _chamfer_sets()[name])
+    n, m = len(P), len(Q)
+    D = ((P[:, None].astype(np.float64) - Q[None]) ** 2).sum(-1)
+    D = np.where(np.isfinite(D), D, np.inf)
+    j1, j2 = D.argmin(1), D.argmin(0)  # the first of equal ones; 0 if none is finite
+    with np.errstate(invalid="ignore"):
+        grad = 2 * (P - Q[j1]).astype(np.float64) / n
+        np.add.at(grad, j2, 2 * (P[j2] - Q).astype(np.float64) / m)
+    loss = D.min(1).mean() + D.min(0).mean()
+    dP, dQ = dev_f32(np.concatenate([P.T, np.zeros((7, n))])), dev_f32(
+        np.concatenate([Q.T, np.zeros((7, m))]))
+    dg, dl = torch.zeros((9, n), device="cuda"), torch.zeros(1, device="cuda")
+    scratch = torch.empty(nat.load().gs2d_chamfer_scratch_bytes(n, m, 1), dtype=torch.uint8,
+                          device="cuda")
+    nat.call("gs2d_chamfer", dP.data_ptr(), n, n, dQ.data_ptr(), m, m, 1, 1.0, dg.data_ptr(),
+             dl.data_ptr(), scratch.data_ptr(), 0)
+    got = dg.cpu().numpy().astype(np.float64)
+    # FP32 atomic sums of up to m terms of size |P - Q| / min(n, m)
+    with np.errstate(invalid="ignore"):
+        size = 2 * np.abs(P - Q[j1]) / n
+        np.add.at(size, j2, 2 * np.abs(P[j2] - Q) / m)
+    tol = 1e-5 * size.T + 1e-9
+    bad = np.isnan(grad.T)
+    np.testing.assert_array_equal(np.isnan(got[:2]) | np.isinf(got[:2]),
+                                  bad | np.isinf(grad.T))
+    ok = np.isfinite(grad.T)
+    assert np.all(np.abs(got[:2] - grad.T)[ok] <= tol[ok])
+    assert not got[2:].any()
+    if np.isfinite(loss):
+        assert abs(float(dl[0]) - loss) <= 1e-5 * loss
