@@ -262,14 +262,59 @@ __global__ void k_cnn_input(int B, int H, int W, const float* __restrict__ frame
   }
 }
 
-// One thread per (output pixel, 8-wide chunk of k).
-// One thread per 16-byte chunk of col (consecutive threads, consecutive
-// chunks of a row: coalesced stores).  I is the index type: 32-bit whenever
-// the chunk count fits, since 64-bit divisions are long emulated sequences
-// and this kernel is a few divisions per 16 bytes moved.
-template <typename I>
-__global__ void k_im2col(int B, int Hi, int Wi, int C, int Ho, int Wo, int ks, int stride,
+// Output pixels of one row per block of k_im2col: about kColChunks 16-byte
+// chunks of col.
+constexpr int kColChunks = 2048;
+
+// A block writes the col rows of `run` consecutive output pixels of one output
+// row, consecutive threads consecutive 16-byte chunks.  Memory-bound by what
+// it writes (1.8 GB per training step at 1080p, batch 8), provided the index
+// work stays small: the tap of a chunk is looked up in a table that the block
+// builds once, and the row is the block's, so a chunk costs one division by a
+// multiplication: 461 us a step (599 with three or four divisions each).
+__global__ void __launch_bounds__(256)
+k_im2col(int Hi, int Wi, int C, int Ho, int Wo, int ks, int stride, int pad, int ldk, int run,
+         int segs, const bf16* __restrict__ x, bf16* __restrict__ col) {
+  extern __shared__ int2 s_tap[];  // per chunk: (ky << 16 | kx, element offset) or (-1, one?)
+  const int chunks = ldk / 8, kk = ks * ks * C;
+  for (int c = threadIdx.x; c < chunks; c += blockDim.x) {
+    const int k0 = 8 * c;
+    int2 e = make_int2(-1, k0 == kk ? 1 : 0);
+    if (k0 < kk) {
+      const int tap = k0 / C, ky = tap / ks, kx = tap - ky * ks;
+      e = make_int2((ky << 16) | kx, (ky * Wi + kx) * C + k0 - tap * C);
+    }
+    s_tap[c] = e;
+  }
+  __syncthreads();
+  const int row = blockIdx.x / segs, ox0 = (blockIdx.x - row * segs) * run;  // row = b Ho + oy
+  const int b = row / Ho, oy = row - b * Ho;
+  const int count = min(run, Wo - ox0) * chunks;
+  const int iy0 = oy * stride - pad;
+  const bf16* xr = x + ((size_t)b * Hi + iy0) * Wi * C;
+  uint4* out = reinterpret_cast<uint4*>(col + ((size_t)row * Wo + ox0) * ldk);
+  const float inv = 1.0f / (float)chunks;
+  for (int t = threadIdx.x; t < count; t += blockDim.x) {
+    // t / chunks: t < 2 kColChunks + chunks, exact after the half offset
+    const int p = (int)(((float)t + 0.5f) * inv), c = t - p * chunks;
+    const int2 e = s_tap[c];
+    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+    if (e.x >= 0) {
+      const int iy = iy0 + (e.x >> 16), ix0 = (ox0 + p) * stride - pad, ix = ix0 + (e.x & 0xffff);
+      if (iy >= 0 && iy < Hi && ix >= 0 && ix < Wi)
+        v = *reinterpret_cast<const uint4*>(xr + (ptrdiff_t)ix0 * C + e.y);
+    } else if (e.y) {
+      v.x = 0x3F80u;  // bf16 1.0 in the low half: the bias column
+    }
+    out[t] = v;
+  }
+}
+
+// The same for shapes beyond the block kernel's table or index range, one
+// thread per chunk.
+__global__ void k_im2col_any(int B, int Hi, int Wi, int C, int Ho, int Wo, int ks, int stride,
                          int pad, int ldk, const bf16* __restrict__ x, bf16* __restrict__ col) {
+  using I = size_t;
   const I chunks = (I)(ldk / 8), hw = (I)Ho * (I)Wo;
   const int kk = ks * ks * C;
   const I total = (I)B * hw * chunks;
@@ -294,8 +339,67 @@ __global__ void k_im2col(int B, int Hi, int Wi, int C, int Ho, int Wo, int ks, i
   }
 }
 
-// One thread per (input pixel, channel): the taps that read it.
-// I: the index type, 32-bit whenever the element count fits (as k_im2col).
+// Gradient of im2col, one thread per (input pixel, 8 channels): the taps that
+// read it, FP32 sums in the order of the taps, 16-byte loads and one 16-byte
+// store.  KS and ST fixed at compile time for the network's 3 x 3 stride-2
+// layers (0: runtime), where a pixel is read by one, two or four taps.
+// Memory-bound by dcol (2.3 GB per training step at 1080p, batch 8); with a
+// thread per channel the index arithmetic bounded it at a tenth of that rate
+// (3.74 ms a step, 0.69 now).
+template <int KS, int ST>
+__global__ void __launch_bounds__(256)
+k_col2im8(const float* __restrict__ dcol, int ldk, unsigned total, int Hi, int Wi, int C8, int Ho,
+          int Wo, int ks_, int stride_, int pad, const bf16* __restrict__ act,
+          bf16* __restrict__ dx) {
+  const int ks = KS ? KS : ks_, stride = ST ? ST : stride_;
+  for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < total;
+       t += gridDim.x * blockDim.x) {
+    const unsigned pin = t / (unsigned)C8;
+    const int ci = 8 * (int)(t - pin * (unsigned)C8);
+    const unsigned row = pin / (unsigned)Wi;  // b Hi + iy
+    const int ix = (int)(pin - row * (unsigned)Wi);
+    const int b = (int)(row / (unsigned)Hi), iy = (int)(row - (unsigned)b * (unsigned)Hi);
+    float s[8];
+#pragma unroll
+    for (int k = 0; k < 8; k++) s[k] = 0.0f;
+#pragma unroll
+    for (int ky = 0; ky < (KS ? KS : ks); ky++) {
+      const int ny = iy + pad - ky, oy = ny / stride;
+      if (ny < 0 || ny != oy * stride || oy >= Ho) continue;
+#pragma unroll
+      for (int kx = 0; kx < (KS ? KS : ks); kx++) {
+        const int nx = ix + pad - kx, ox = nx / stride;
+        if (nx < 0 || nx != ox * stride || ox >= Wo) continue;
+        const float4* src = reinterpret_cast<const float4*>(
+            dcol + (((size_t)b * Ho + oy) * Wo + ox) * ldk + (ky * ks + kx) * 8 * C8 + ci);
+        const float4 u = __ldcs(src), v = __ldcs(src + 1);
+        s[0] += u.x;
+        s[1] += u.y;
+        s[2] += u.z;
+        s[3] += u.w;
+        s[4] += v.x;
+        s[5] += v.y;
+        s[6] += v.z;
+        s[7] += v.w;
+      }
+    }
+    if (act) {
+      const uint4 av = reinterpret_cast<const uint4*>(act)[t];
+      const bf16* ab = reinterpret_cast<const bf16*>(&av);
+#pragma unroll
+      for (int k = 0; k < 8; k++)
+        if (!(__bfloat162float(ab[k]) > 0.0f)) s[k] = 0.0f;
+    }
+    __align__(16) bf16 d[8];
+#pragma unroll
+    for (int k = 0; k < 8; k++) d[k] = __float2bfloat16_rn(s[k]);
+    reinterpret_cast<uint4*>(dx)[t] = *reinterpret_cast<const uint4*>(d);
+  }
+}
+
+// The same, one thread per (input pixel, channel): channel counts that are no
+// multiple of 8, unaligned rows.  I: the index type, 32-bit whenever the
+// element count fits.
 template <typename I>
 __global__ void k_col2im(const float* __restrict__ dcol, int ldk, int B, int Hi, int Wi, int C,
                          int Ho, int Wo, int ks, int stride, int pad,
@@ -407,14 +511,19 @@ extern "C" gs2d_status gs2d_im2col(const void* x, int32_t B, int32_t Hi, int32_t
     return set_error(GS2D_ERR_INVALID_ARG, "gs2d_im2col: arguments");
   const int Ho = (Hi + 2 * pad - ks) / stride + 1, Wo = (Wi + 2 * pad - ks) / stride + 1;
   if (Ho < 1 || Wo < 1) return set_error(GS2D_ERR_INVALID_ARG, "gs2d_im2col: empty output");
-  const size_t total = (size_t)B * Ho * Wo * (ldk / 8);
-  if (total == 0) return set_error(GS2D_OK, "");
-  if (total < (size_t)INT32_MAX)
-    k_im2col<uint32_t><<<grid_for(total, 256), 256, 0, (cudaStream_t)stream>>>(
-        B, Hi, Wi, C, Ho, Wo, ks, stride, pad, ldk, static_cast<const bf16*>(x),
+  const int64_t rows = (int64_t)B * Ho;
+  if (rows == 0) return set_error(GS2D_OK, "");
+  const int chunks = ldk / 8;
+  const int run = std::max(1, std::min(Wo, kColChunks / chunks));
+  const int segs = (Wo + run - 1) / run;
+  // 48 KB of table, 32-bit offsets inside a tap window, one block per segment
+  if (ks <= 0x7fff && chunks <= (48 << 10) / 8 && (int64_t)ks * Wi * C <= INT32_MAX &&
+      rows * segs <= INT32_MAX)
+    k_im2col<<<(unsigned)(rows * segs), 256, chunks * sizeof(int2), (cudaStream_t)stream>>>(
+        Hi, Wi, C, Ho, Wo, ks, stride, pad, ldk, run, segs, static_cast<const bf16*>(x),
         static_cast<bf16*>(col));
   else
-    k_im2col<size_t><<<grid_for(total, 256), 256, 0, (cudaStream_t)stream>>>(
+    k_im2col_any<<<grid_for((size_t)rows * Wo * chunks, 256), 256, 0, (cudaStream_t)stream>>>(
         B, Hi, Wi, C, Ho, Wo, ks, stride, pad, ldk, static_cast<const bf16*>(x),
         static_cast<bf16*>(col));
   return launched("gs2d_im2col");
@@ -429,6 +538,15 @@ extern "C" gs2d_status gs2d_col2im(const float* dcol, int32_t ldk, int32_t B, in
   const int Ho = (Hi + 2 * pad - ks) / stride + 1, Wo = (Wi + 2 * pad - ks) / stride + 1;
   const size_t total = (size_t)B * Hi * Wi * C;
   if (total == 0) return set_error(GS2D_OK, "");
+  if (C % 8 == 0 && ldk % 4 == 0 && total / 8 < (size_t)INT32_MAX && aligned16(dcol) &&
+      aligned16(dx) && aligned16(act)) {
+    const unsigned t8 = (unsigned)(total / 8);
+    const auto kernel = ks == 3 && stride == 2 ? k_col2im8<3, 2> : k_col2im8<0, 0>;
+    kernel<<<grid_for(t8, 256), 256, 0, (cudaStream_t)stream>>>(
+        dcol, ldk, t8, Hi, Wi, C / 8, Ho, Wo, ks, stride, pad, static_cast<const bf16*>(act),
+        static_cast<bf16*>(dx));
+    return launched("gs2d_col2im");
+  }
   if (total < (size_t)INT32_MAX)
     k_col2im<uint32_t><<<grid_for(total, 256), 256, 0, (cudaStream_t)stream>>>(
         dcol, ldk, B, Hi, Wi, C, Ho, Wo, ks, stride, pad, static_cast<const bf16*>(act),

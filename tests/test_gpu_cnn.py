@@ -448,6 +448,32 @@ def test_implicit_conv_bad_arguments(nat):
                  d.data_ptr(), 8, 0, 0)
 
 
+@pytest.mark.parametrize("C,ks,st,pad,H,W", [(8, 3, 2, 1, 5, 301), (24, 3, 2, 1, 3, 40),
+                                             (16, 5, 3, 2, 11, 9), (256, 3, 2, 1, 4, 7)])
+def test_im2col_and_col2im_by_definition(nat, C, ks, st, pad, H, W):
+    """Row segments and chunk tables of the block kernels: im2col exact, col2im
+    (8 channels a thread) with and without the ReLU mask within one BF16 unit."""
+    B, ldk = 2, -(-(ks * ks * C + 1) // 8) * 8
+    g = np.random.Generator(np.random.PCG64(C + W))
+    x = cnn.bf16_round(g.normal(size=(B, H, W, C)))
+    ref = cnn.im2col(x, ks, st, pad, ldk)
+    col = torch.full(ref.shape, 9.0, dtype=torch.bfloat16, device="cuda")
+    dx = bf16_dev(x)
+    nat.call("gs2d_im2col", dx.data_ptr(), B, H, W, C, ks, st, pad, col.data_ptr(), ldk, 0)
+    np.testing.assert_array_equal(to_np_bf16(col), ref)
+    dcol = g.normal(size=ref.shape).astype(np.float32)
+    back = cnn.col2im(dcol, x.shape, ks, st, pad)
+    d_dcol = dev_f32(dcol)
+    out = torch.empty(x.shape, dtype=torch.bfloat16, device="cuda")
+    for act in (None, dx):
+        nat.call("gs2d_col2im", d_dcol.data_ptr(), ldk, B, H, W, C, ks, st, pad,
+                 0 if act is None else act.data_ptr(), out.data_ptr(), 0)
+        want = back if act is None else back * (x > 0)
+        # FP32 sums of up to ks^2 terms, then one BF16 rounding
+        tol = np.abs(want) * 2.0 ** -8 + 1e-6 * cnn.col2im(np.abs(dcol), x.shape, ks, st, pad)
+        assert np.all(np.abs(to_np_bf16(out) - want) <= tol + 1e-30)
+
+
 def _chamfer_sets():
     g = np.random.Generator(np.random.PCG64(77))
     lattice = np.stack(np.meshgrid(np.arange(20.0), np.arange(20.0)), -1).reshape(-1, 2)
