@@ -604,6 +604,20 @@ gs2d_status gs2d_gemm_bf16(const void* A, int32_t lda, const void* B, int32_t ld
                            int32_t* status, void* stream);
 uint64_t gs2d_gemm_partial_bytes(int32_t M, int32_t N, int32_t ldc, int32_t K, int32_t splits);
 
+/* C[M][N] = sum over K rows p of A[p][m] B[p][n], i.e. A^T B, with BF16 A and
+ * B (device, row-major [K][lda] and [K][ldb], leading dimensions in elements,
+ * multiples of 8; 16-byte aligned), FP32 accumulation and FP32 output (device
+ * [M][ldc]): the weight gradient of a convolution from dZ and the im2col
+ * operand, without transposing either.  K is split over at least min_splits
+ * groups of thread blocks, as far as it goes (FP32 sums lose precision with
+ * their length); partial (device, gs2d_gemm_tn_partial_bytes bytes) then holds FP32 partial sums that a second kernel adds in a fixed order
+ * (deterministic).  status as gs2d_gemm_bf16. */
+gs2d_status gs2d_gemm_tn_bf16(const void* A, int32_t lda, const void* B, int32_t ldb, int32_t M,
+                              int32_t N, int32_t K, float* out, int32_t ldc, int32_t min_splits,
+                              float* partial, int32_t* status, void* stream);
+uint64_t gs2d_gemm_tn_partial_bytes(int32_t M, int32_t N, int32_t ldc, int32_t K,
+                                    int32_t min_splits);
+
 /* Failure-detection check of the GEMM's bounded waits (not part of the
  * paper's method).  Launches the gs2d_gemm_bf16 kernel on one 128 x 32 x 64
  * tile (A: device bf16 [128][64], B: device bf16 [32][64], 16-byte aligned;

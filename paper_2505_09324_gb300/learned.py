@@ -9,12 +9,13 @@ into cell-anchored Gaussians; each frame keeps the n with the largest |w|.
 About 1.3 M parameters; BF16 weights and activations, FP32 accumulation and
 FP32 master weights.
 
-In training every convolution is im2col + one BF16 tensor-core GEMM
-(gs2d_gemm_bf16, the bias a weight column against a column of ones); at
-inference the convolutions run as implicit GEMMs that read their operands
-straight from the activations (gs2d_conv_bf16, gs2d_conv_frame_bf16), with
-the same sums in the same order.  The backward pass is one
-weight-gradient GEMM (dZ^T . col, split over pixels) and one input-gradient
+Every convolution is a BF16 tensor-core GEMM over its im2col operand (the
+bias a weight column against a column of ones), run as an implicit GEMM that
+reads its operands straight from the activations (gs2d_conv_bf16,
+gs2d_conv_frame_bf16; the same sums in the same order as gs2d_gemm_bf16 on
+the operand); training also writes the operand out for the backward pass.  The backward pass is one
+weight-gradient GEMM (dZ^T . col, both read as they lie, split over pixels;
+gs2d_gemm_tn_bf16) and one input-gradient
 GEMM (dZ . W) + col2im with the ReLU mask per layer.  The optimiser is the
 library's Adam on the FP32 master weights.  Training minimises the L2 render
 loss of the decoded Gaussians through the rasterizer (the colour and shape
@@ -100,14 +101,12 @@ class LearnedInitializer:
     def _alloc(self):
         B, dev, bf = self.B, self.dev, torch.bfloat16
         self.x = [torch.empty((B * self.H * self.W, 8), dtype=bf, device=dev)]
-        self.col, self.colT, self.dz, self.dzT, self.dcol = [], [], [], [], []
+        self.col, self.dz, self.dcol = [], [], []
         for li, (ci, co, ks, ldk) in enumerate(self.layers):
             h, w = self.sizes[li + 1] if li < self.L else self.sizes[-1]
             P = B * h * w
             self.col.append(torch.empty((P, ldk), dtype=bf, device=dev))
-            self.colT.append(torch.empty((ldk, _ceil8(P)), dtype=bf, device=dev))
             self.dz.append(torch.empty((P, co), dtype=bf, device=dev))
-            self.dzT.append(torch.empty((co, _ceil8(P)), dtype=bf, device=dev))
             self.dcol.append(torch.empty((P, ldk), device=dev) if li > 0 else None)
             if li < self.L:
                 self.x.append(torch.empty((P, co), dtype=bf, device=dev))
@@ -119,8 +118,8 @@ class LearnedInitializer:
         for li, (ci, co, ks, ldk) in enumerate(self.layers):
             h, w = self.sizes[li + 1] if li < self.L else self.sizes[-1]
             P = B * h * w
-            most = max(most, nat.load().gs2d_gemm_partial_bytes(co, ldk, ldk, P,
-                                                                 self._splits(P)))
+            most = max(most, nat.load().gs2d_gemm_tn_partial_bytes(co, ldk, ldk, P,
+                                                                    self._splits(P)))
         self.partial = torch.empty(max(most // 4, 1), device=dev)
 
     def _splits(self, pixels: int) -> int:
@@ -160,41 +159,41 @@ class LearnedInitializer:
             mptr = masks.data_ptr()
         st = self.status.data_ptr()
         ci0, co0, ks0, ldk0 = self.layers[0]
-        first = 0
-        if not keep_col and self.W % 16 == 0 and ks0 == 3 and co0 <= 128 and self.L > 0:
-            # the first convolution straight from the frames and masks (the
-            # 8-channel input never written; the same result bit for bit)
-            nat.call("gs2d_conv_frame_bf16", frames.data_ptr(), mptr, B, self.H, self.W, 3, 2,
-                     1, self.wb[0].data_ptr(), ldk0, co0, 1, 0, self.x[1].data_ptr(), co0, st, s)
-            first = 1
-        else:
+        # the first convolution straight from the frames and masks (the
+        # 8-channel input never read; the same result bit for bit); its loads
+        # need 16-byte aligned inputs, which training does not ask for
+        from_frames = self.W % 16 == 0 and ks0 == 3 and co0 <= 128 and self.L > 0 and \
+            (not keep_col or (frames.data_ptr() | mptr) % 16 == 0)
+        if keep_col or not from_frames:
             nat.call("gs2d_cnn_input", frames.data_ptr(), mptr, B, self.H, self.W,
                      self.x[0].data_ptr(), s)
         for li, (ci, co, ks, ldk) in enumerate(self.layers):
-            if li < first:
-                continue
             src = self.x[li]
             hi, wi = self.sizes[li] if li < self.L else self.sizes[-1]
             stride, pad = (2, 1) if ks == 3 else (1, 0)
+            last = li == self.L
+            out32 = self.out.data_ptr() if last else 0
+            out16 = 0 if last else self.x[li + 1].data_ptr()
             # implicit GEMM unless K is very deep (the last 3 x 3 layer: 37
             # k-tiles over 32 tiles, where the TMA-fed GEMM over an im2col
-            # operand is faster); the results are identical either way
-            if not keep_col and (ldk + 63) // 64 <= 32:
-                last = li == self.L
+            # operand is faster); the results are identical either way, so
+            # training too only writes the operand (for backward) and does
+            # not read it back here
+            implicit = (ldk + 63) // 64 <= 32
+            if keep_col or not implicit:
+                nat.call("gs2d_im2col", src.data_ptr(), B, hi, wi, ci, ks, stride, pad,
+                         self.col[li].data_ptr(), ldk, s)
+            if li == 0 and from_frames:
+                nat.call("gs2d_conv_frame_bf16", frames.data_ptr(), mptr, B, self.H, self.W, 3, 2,
+                         1, self.wb[0].data_ptr(), ldk, co, 1, 0, out16, co, st, s)
+            elif implicit:
                 nat.call("gs2d_conv_bf16", src.data_ptr(), B, hi, wi, ci, ks, stride, pad,
-                         self.wb[li].data_ptr(), ldk, co, 0 if last else 1,
-                         self.out.data_ptr() if last else 0,
-                         0 if last else self.x[li + 1].data_ptr(), co, st, s)
-                continue
-            nat.call("gs2d_im2col", src.data_ptr(), B, hi, wi, ci, ks, stride, pad,
-                     self.col[li].data_ptr(), ldk, s)
-            P = self.col[li].shape[0]
-            if li < self.L:
-                nat.gemm_bf16(self.col[li].data_ptr(), ldk, self.wb[li].data_ptr(), ldk, P, co,
-                              ldk, 0, True, 0, self.x[li + 1].data_ptr(), co, 1, 0, st, s)
+                         self.wb[li].data_ptr(), ldk, co, 0 if last else 1, out32, out16, co, st,
+                         s)
             else:
-                nat.gemm_bf16(self.col[li].data_ptr(), ldk, self.wb[li].data_ptr(), ldk, P, co,
-                              ldk, 0, False, self.out.data_ptr(), 0, co, 1, 0, st, s)
+                nat.gemm_bf16(self.col[li].data_ptr(), ldk, self.wb[li].data_ptr(), ldk,
+                              self.col[li].shape[0], co, ldk, 0, not last, out32, out16, co, 1, 0,
+                              st, s)
         c = self.cfg
         nat.call("gs2d_head_decode", self.out.data_ptr(), self.ldo, B, self.gh, self.gw, c.slots,
                  self.cell, c.scale, self.n, self.params.data_ptr(), B * self.n,
@@ -236,15 +235,10 @@ class LearnedInitializer:
         for li in range(self.L, -1, -1):
             ci, co, ks, ldk = self.layers[li]
             P = self.col[li].shape[0]
-            ldp = self.dzT[li].shape[1]
             # weight gradient: dW[co][k] = sum_p dZ[p][co] col[p][k]
-            nat.call("gs2d_transpose_bf16", self.dz[li].data_ptr(), P, co, co,
-                     self.dzT[li].data_ptr(), ldp, s)
-            nat.call("gs2d_transpose_bf16", self.col[li].data_ptr(), P, ldk, ldk,
-                     self.colT[li].data_ptr(), ldp, s)
-            nat.gemm_bf16(self.dzT[li].data_ptr(), ldp, self.colT[li].data_ptr(), ldp, co, ldk, P,
-                          0, False, self.dw[li].data_ptr(), 0, ldk, self._splits(P),
-                          self.partial.data_ptr(), st, s)
+            nat.call("gs2d_gemm_tn_bf16", self.dz[li].data_ptr(), co, self.col[li].data_ptr(),
+                     ldk, co, ldk, P, self.dw[li].data_ptr(), ldk, self._splits(P),
+                     self.partial.data_ptr(), st, s)
             if li == 0:
                 break
             # input gradient: dcol[p][k] = sum_co dZ[p][co] W[co][k], then the

@@ -448,6 +448,34 @@ def test_implicit_conv_bad_arguments(nat):
                  d.data_ptr(), 8, 0, 0)
 
 
+@pytest.mark.parametrize("M,N,K,splits", [
+    (32, 80, 1000, 512), (64, 296, 700, 3), (64, 320, 257, 2), (128, 584, 130, 1),
+    (256, 1160, 300, 4), (384, 2312, 129, 2), (96, 392, 64, 1), (8, 16, 5, 8), (130, 65, 1, 1)])
+def test_gemm_over_rows_matches_oracle(nat, M, N, K, splits):
+    """gs2d_gemm_tn_bf16 (both operands summed over their rows): one and two
+    row chunks, one to five column chunks, ragged tiles and row counts around
+    a stage of 128, split and not; within the GEMM bar."""
+    g = np.random.Generator(np.random.PCG64(M + 3 * N + K))
+    a, b = (cnn.bf16_round(g.normal(size=(K, n))) for n in (M, N))
+    ld = [-(-n // 8) * 8 for n in (M, N)]
+    A, Bm = np.full((K, ld[0]), 7.0, np.float32), np.full((K, ld[1]), 7.0, np.float32)
+    A[:, :M], Bm[:, :N] = a, b
+    dA, dB = bf16_dev(A), bf16_dev(Bm)
+    ldc = N + 3
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    pb = nat.load().gs2d_gemm_tn_partial_bytes(M, N, ldc, K, splits)
+    part = torch.empty(max(pb // 4, 1), device="cuda")
+    C = torch.full((M, ldc), float("nan"), device="cuda")
+    nat.call("gs2d_gemm_tn_bf16", dA.data_ptr(), ld[0], dB.data_ptr(), ld[1], M, N, K, C.data_ptr(),
+             ldc, splits, part.data_ptr(), status.data_ptr(), 0)
+    got = C.cpu().numpy().astype(np.float64)
+    assert int(status.item()) == 0
+    ref, scale = cnn.gemm(a.T, b.T), cnn.gemm_abs(a.T, b.T)
+    assert np.all(np.abs(got[:, :N] - ref) <= REL * scale + 1e-30)
+    if pb == 0:
+        assert np.all(np.isnan(got[:, N:]))
+
+
 @pytest.mark.parametrize("C,ks,st,pad,H,W", [(8, 3, 2, 1, 5, 301), (24, 3, 2, 1, 3, 40),
                                              (16, 5, 3, 2, 11, 9), (256, 3, 2, 1, 4, 7)])
 def test_im2col_and_col2im_by_definition(nat, C, ks, st, pad, H, W):
