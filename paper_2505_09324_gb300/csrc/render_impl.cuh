@@ -54,12 +54,16 @@
 
 namespace gs2d {
 
+// Rows per thread of the usual kernels: 2, 4, 4.
 template <int T>
+constexpr int kRows = T == 8 ? 2 : 4;
+
+template <int T, int R_>
 struct TileGeom {
-  static constexpr int R = T == 8 ? 2 : 4;  // rows per thread
-  static constexpr int NT = T * T / R;      // threads per block: 32, 64, 256
-  static constexpr int NW = NT / 32;        // warps: 1, 2, 8
-  static constexpr int RW = 32 / T * R;     // rows per warp band: 8, 8, 4
+  static constexpr int R = R_;              // rows per thread: kRows<T>, or 1 (few tiles)
+  static constexpr int NT = T * T / R;      // threads per block: 32, 64, 256 (R = 1: 256, 1024)
+  static constexpr int NW = NT / 32;        // warps: 1, 2, 8 (R = 1: 8, 32)
+  static constexpr int RW = 32 / T * R;     // rows per warp band: 8, 8, 4 (R = 1: 2, 1)
   static constexpr int GPW = 32 / T;        // Gaussians per warp in the backward pass
   static constexpr int Q = T / 8;           // lanes per reduced value
 };
@@ -104,10 +108,10 @@ __device__ __forceinline__ TileFrame tile_frame(const RenderArgs& a, int tile) {
 }
 
 // Stage entries [b, b + cnt) of the tile's list (cnt <= S).
-template <int T, int S>
+template <int T, int S, int R>
 __device__ __forceinline__ void stage_batch(TileSmem<S>& sm, const RenderArgs& a,
                                             const TileFrame& f, int b, int cnt) {
-  using G = TileGeom<T>;
+  using G = TileGeom<T, R>;
   if (threadIdx.x == 0) sm.next = 0;
   for (int k = threadIdx.x; k < cnt; k += G::NT) {
     const int g = (int)a.list[b + k];
@@ -163,8 +167,8 @@ struct WarpEntry {
 template <int T, int S>
 __device__ __forceinline__ void fwd_batch(const TileSmem<S>& sm, const WarpEntry* __restrict__ wl,
                                           int wn, float pxl, float drow,
-                                          float (&acc)[TileGeom<T>::R][3]) {
-  constexpr int R = TileGeom<T>::R;
+                                          float (&acc)[kRows<T>][3]) {
+  constexpr int R = kRows<T>;
   const char* fa_base = reinterpret_cast<const char*>(sm.fa);
   const char* fb_base = reinterpret_cast<const char*>(sm.fb);
   for (int i = 0; i < wn; i++) {
@@ -226,7 +230,7 @@ __device__ __forceinline__ float group_transpose_sum(const float (&v)[8], int j)
 template <int T, int S>
 __device__ __forceinline__ void bwd_batch(TileSmem<S>& sm, const float4* __restrict__ s_g,
                                           int cnt, const RenderArgs& a, int b) {
-  using G = TileGeom<T>;
+  using G = TileGeom<T, kRows<T>>;  // (the rows per thread play no part here)
   float* __restrict__ partial = a.partial;
   const int lane = threadIdx.x & 31;
   const int h = lane / T, j = lane % T;
@@ -302,13 +306,15 @@ __device__ __forceinline__ void bwd_batch(TileSmem<S>& sm, const float4* __restr
 }
 
 // Per-mode shared memory beyond the staged batch.
-template <int T, int S, int MODE>
+template <int T, int S, int MODE, int R>
 struct ModeSmem {
   static constexpr int kGrad = (MODE == kModeBwd || MODE == kModeL2) ? T * T : 1;
-  static constexpr int kList = (MODE == kModeFwd || MODE == kModeL2) ? S : 1;
-  float4 g[kGrad];                       // dL/dC of the tile
-  WarpEntry wl[TileGeom<T>::NW][kList];  // per-warp lists of the staged batch
-  float2 red[TileGeom<T>::NW];         // loss partials per warp
+  static constexpr int kList = (MODE == kModeFwd || MODE == kModeL2) && R > 1 ? S : 1;
+  static constexpr int kSse = MODE == kModeL2 && R == 1 ? T * T : 1;
+  float4 g[kGrad];                          // dL/dC of the tile
+  WarpEntry wl[TileGeom<T, R>::NW][kList];  // per-warp lists of the staged batch
+  float2 red[TileGeom<T, kRows<T>>::NW];    // loss partials per warp
+  float2 sse[kSse];                         // R = 1: squared errors per pixel
   unsigned hits;                       // kModeCount
 };
 
@@ -335,11 +341,44 @@ __device__ __forceinline__ int warp_list(const TileSmem<S>& sm, int cnt, int wid
   return m;
 }
 
-template <int T, int S, int MODE>
+// The forward pass of the kernels with one row per thread (few tiles): the
+// warp walks the staged Gaussians that touch its rows by ballot (ascending
+// index, as warp_list leaves them) and every lane evaluates its pixel with
+// the roundings of the usual kernels: the row term at the first row of their
+// band (t0), one FMA to the thread's strip (drow), then one addition per row
+// down the strip (steps of them).  So the image is theirs bit for bit.
+template <int T, int S>
+__device__ __forceinline__ void fwd_batch_rows(const TileSmem<S>& sm, int cnt, int wid, int lane,
+                                               float pxl, float pyw, float drow, int steps,
+                                               float (&acc)[3]) {
+  for (int base = 0; base < cnt; base += 32) {
+    const int k = base + lane;
+    const bool on = k < cnt && ((sm.wmask[k] >> wid) & 1u);
+    for (unsigned m = __ballot_sync(0xffffffffu, on); m; m &= m - 1) {
+      const int j = base + __ffs(m) - 1;
+      const float4 fa = sm.fa[j], fb = sm.fb[j];
+      const float dx = pxl - fa.x;
+      const float u1 = fa.y * dx;
+      const float u1sq = u1 * u1;
+      float u2 = fmaf(fa.z, dx, fa.w * (pyw - sm.my[j]));
+      if constexpr (T != 32) u2 = fmaf(fa.w, drow, u2);
+#pragma unroll
+      for (int r = 1; r < kRows<T>; r++) u2 = r <= steps ? u2 + fa.w : u2;
+      const float q = fmaf(u2, u2, u1sq);
+      if (q <= fb.x) {
+        const float e = ex2_approx(-q);
+        acc[0] = fmaf(fb.y, e, acc[0]);
+        acc[1] = fmaf(fb.z, e, acc[1]);
+        acc[2] = fmaf(fb.w, e, acc[2]);
+      }
+    }
+  }
+}
+
+template <int T, int S, int MODE, int R>
 __device__ __forceinline__ void process_tile(const RenderArgs& a, const TileFrame& f,
-                                             TileSmem<S>& sm, ModeSmem<T, S, MODE>& ms) {
-  using G = TileGeom<T>;
-  constexpr int R = G::R;
+                                             TileSmem<S>& sm, ModeSmem<T, S, MODE, R>& ms) {
+  using G = TileGeom<T, R>;
   const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
   const int x = f.ox + t % T, y0 = f.oy + R * (t / T);
   // tile-local pixel centres of this thread's column and first row
@@ -360,7 +399,7 @@ __device__ __forceinline__ void process_tile(const RenderArgs& a, const TileFram
     for (int b = rg.x; b < rg.y; b += S) {
       const int cnt = min(S, rg.y - b);
       __syncthreads();
-      stage_batch<T, S>(sm, a, f, b, cnt);
+      stage_batch<T, S, R>(sm, a, f, b, cnt);
       __syncthreads();
       bwd_batch<T, S>(sm, ms.g, cnt, a, b);
     }
@@ -388,7 +427,7 @@ __device__ __forceinline__ void process_tile(const RenderArgs& a, const TileFram
     for (int b = rg.x; b < rg.y; b += S) {
       const int cnt = min(S, rg.y - b);
       __syncthreads();
-      stage_batch<T, S>(sm, a, f, b, cnt);
+      stage_batch<T, S, R>(sm, a, f, b, cnt);
       __syncthreads();
       if (!any) continue;
       for (int j = 0; j < cnt; j++) {
@@ -413,7 +452,7 @@ __device__ __forceinline__ void process_tile(const RenderArgs& a, const TileFram
     for (int b = rg.x; b < rg.y; b += S) {
       const int cnt = min(S, rg.y - b);
       __syncthreads();
-      stage_batch<T, S>(sm, a, f, b, cnt);
+      stage_batch<T, S, R>(sm, a, f, b, cnt);
       __syncthreads();
       for (int j = 0; j < cnt && x < f.W; j++) {
         const float4 fa = sm.fa[j];
@@ -445,11 +484,19 @@ __device__ __forceinline__ void process_tile(const RenderArgs& a, const TileFram
     for (int b = rg.x; b < rg.y; b += S) {
       const int cnt = min(S, rg.y - b);
       __syncthreads();
-      stage_batch<T, S>(sm, a, f, b, cnt);
+      stage_batch<T, S, R>(sm, a, f, b, cnt);
       __syncthreads();
-      const int wn = warp_list<T, S>(sm, cnt, wid, lane, (float)(G::RW * wid) + 0.5f,
-                                     ms.wl[wid]);
-      fwd_batch<T, S>(sm, ms.wl[wid], wn, pxl, (float)(R * (lane / T)), acc);
+      if constexpr (R == 1) {
+        // this pixel's row in the usual kernels: band, strip and row of the strip
+        constexpr int kBand = 32 / T * kRows<T>;
+        const int row = t / T, in = row % kBand;
+        fwd_batch_rows<T, S>(sm, cnt, wid, lane, pxl, (float)(row - in) + 0.5f,
+                             (float)(in - in % kRows<T>), in % kRows<T>, acc[0]);
+      } else {
+        const int wn = warp_list<T, S>(sm, cnt, wid, lane, (float)(G::RW * wid) + 0.5f,
+                                       ms.wl[wid]);
+        fwd_batch<T, S>(sm, ms.wl[wid], wn, pxl, (float)(R * (lane / T)), acc);
+      }
       staged = b;
     }
     if constexpr (MODE == kModeFwd) {
@@ -480,8 +527,14 @@ __device__ __forceinline__ void process_tile(const RenderArgs& a, const TileFram
         const float d0 = acc[r][0] - t0, d1 = acc[r][1] - t1, d2 = acc[r][2] - t2;
         const float e0 = __saturatef(acc[r][0]) - t0, e1 = __saturatef(acc[r][1]) - t1,
                     e2 = __saturatef(acc[r][2]) - t2;
-        l.x += fmaf(d0, d0, fmaf(d1, d1, d2 * d2));
-        l.y += fmaf(e0, e0, fmaf(e1, e1, e2 * e2));
+        const float2 p = make_float2(fmaf(d0, d0, fmaf(d1, d1, d2 * d2)),
+                                     fmaf(e0, e0, fmaf(e1, e1, e2 * e2)));
+        if constexpr (R == 1) {
+          l = p;
+        } else {
+          l.x += p.x;
+          l.y += p.y;
+        }
         g = make_float4(gscale * d0, gscale * d1, gscale * d2, 0.f);
         if (a.img) {
           a.img[o] = acc[r][0];
@@ -491,17 +544,32 @@ __device__ __forceinline__ void process_tile(const RenderArgs& a, const TileFram
       }
       ms.g[(R * (t / T) + r) * T + t % T] = g;
     }
+    // the tile's loss: the usual kernels' sums (strips of rows, the warp's
+    // lanes, the warps), whatever R is
+    using GO = TileGeom<T, kRows<T>>;
+    if constexpr (R == 1) {
+      ms.sse[t] = l;  // t = row T + column
+      __syncthreads();
+      l = make_float2(0.f, 0.f);
+      if (t < GO::NT)
+#pragma unroll
+        for (int r = 0; r < GO::R; r++) {
+          const float2 p = ms.sse[(GO::R * (t / T) + r) * T + t % T];
+          l.x += p.x;
+          l.y += p.y;
+        }
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       l.x += __shfl_xor_sync(0xffffffffu, l.x, o);
       l.y += __shfl_xor_sync(0xffffffffu, l.y, o);
     }
-    if (lane == 0) ms.red[wid] = l;
+    if (lane == 0 && wid < GO::NW) ms.red[wid] = l;
     __syncthreads();
     if (t == 0) {
       float2 s = make_float2(0.f, 0.f);
 #pragma unroll
-      for (int w = 0; w < G::NW; w++) {
+      for (int w = 0; w < GO::NW; w++) {
         s.x += ms.red[w].x;
         s.y += ms.red[w].y;
       }
@@ -512,7 +580,7 @@ __device__ __forceinline__ void process_tile(const RenderArgs& a, const TileFram
       const int cnt = min(S, rg.y - b);
       if (b != staged) {
         __syncthreads();
-        stage_batch<T, S>(sm, a, f, b, cnt);
+        stage_batch<T, S, R>(sm, a, f, b, cnt);
         __syncthreads();
         staged = b;
       }
@@ -522,16 +590,17 @@ __device__ __forceinline__ void process_tile(const RenderArgs& a, const TileFram
 }
 
 // Blocks per SM the register budget must allow (about 50 registers per
-// thread of the 64 K per SM; 32 blocks at most): 32, 20, 5 for T = 8, 16, 32.
-template <int T>
-constexpr int kMinBlocks = 65536 / (TileGeom<T>::NT * 50) < 32 ? 65536 / (TileGeom<T>::NT * 50)
-                                                                 : 32;
+// thread of the 64 K per SM; 32 blocks at most): 32, 20, 5 for T = 8, 16, 32,
+// and with one row per thread 5 and 1 for T = 16, 32.
+template <int NT>
+constexpr int kMinBlocks = 65536 / (NT * 50) < 32 ? 65536 / (NT * 50) : 32;
 
-template <int T, int S, int MODE, int LAUNCH>
-__global__ void __launch_bounds__(TileGeom<T>::NT, kMinBlocks<T>) k_render(RenderArgs a) {
+template <int T, int S, int MODE, int LAUNCH, int R>
+__global__ void __launch_bounds__(TileGeom<T, R>::NT, kMinBlocks<TileGeom<T, R>::NT>)
+k_render(RenderArgs a) {
   pdl_begin();
   __shared__ TileSmem<S> sm;
-  __shared__ ModeSmem<T, S, MODE> ms;
+  __shared__ ModeSmem<T, S, MODE, R> ms;
   if constexpr (LAUNCH == GS2D_LAUNCH_GRID) {
     if (a.active && (int)blockIdx.x >= *a.active) return;  // a P-frame's subset
     const int tile = a.order[blockIdx.x];
@@ -539,7 +608,7 @@ __global__ void __launch_bounds__(TileGeom<T>::NT, kMinBlocks<T>) k_render(Rende
       if (threadIdx.x == 0) set_status(a.hdr, GS2D_ERR_BOUNDS);
       return;
     }
-    process_tile<T, S, MODE>(a, tile_frame<T>(a, tile), sm, ms);
+    process_tile<T, S, MODE, R>(a, tile_frame<T>(a, tile), sm, ms);
   } else {
     __shared__ int s_next[2];
     if (threadIdx.x == 0) s_next[0] = atomicAdd(&a.hdr->queue, 1);
@@ -553,7 +622,7 @@ __global__ void __launch_bounds__(TileGeom<T>::NT, kMinBlocks<T>) k_render(Rende
       if (threadIdx.x == 0) next = atomicAdd(&a.hdr->queue, 1);
       const int tile = a.order[q];
       if ((unsigned)tile < (unsigned)a.num_tiles)
-        process_tile<T, S, MODE>(a, tile_frame<T>(a, tile), sm, ms);
+        process_tile<T, S, MODE, R>(a, tile_frame<T>(a, tile), sm, ms);
       else if (threadIdx.x == 0)
         set_status(a.hdr, GS2D_ERR_BOUNDS);  // a stale queue: report, skip
       if (threadIdx.x == 0) s_next[k ^ 1] = next;
@@ -567,15 +636,42 @@ __global__ void __launch_bounds__(TileGeom<T>::NT, kMinBlocks<T>) k_render(Rende
   }
 }
 
+// Warps of the usual kernels (kRows<T> rows per thread) up to which a launch
+// takes the kernels with one row per thread (four times the warps).  With few
+// tiles the usual ones leave the chip's 608 schedulers a warp or two each, and
+// both passes are chains of dependent instructions.  The backward gains, since
+// the warps share a tile's Gaussians; the forward does not (a pixel's chain
+// is as long as before and a warp's setup per Gaussian serves a quarter of
+// the pixels: 4.5 -> 5.3 us at 256 x 256), so it never does alone and the
+// fused call does only while the backward's gain is the larger.  Measured with
+// 104 pixels per Gaussian, usual kernels against these, us: fused, tile 16:
+// 22.3 / 15.3 at 256 x 256 (512 warps), 27.4 / 25.9 at 640 x 360 (1840), 36.2 /
+// 39.7 at 960 x 540 (4080); tile 32: 20.2 / 19.5 (512 warps), 24.5 / 31.5
+// (1920); backward alone, tile 16: 18.2 / 11.3, 38.4 / 36.5 at 1280 x 720
+// (7200); tile 32: 17.7 / 16.5 (1920), 19.1 / 21.3 (3000).
+template <int T, int MODE>
+constexpr int kFewWarps = MODE == kModeL2    ? (T == 16 ? 2400 : 1200)
+                          : MODE == kModeBwd ? (T == 16 ? 7200 : 1920)
+                                             : 0;
+
+template <int T, int S, int MODE, int LAUNCH, int R>
+cudaError_t launch_rows(const RenderArgs& a, cudaStream_t s) {
+  constexpr int NT = TileGeom<T, R>::NT;
+  int grid = a.num_tiles;
+  if (LAUNCH == GS2D_LAUNCH_PERSISTENT)
+    grid = persistent_grid((const void*)k_render<T, S, MODE, LAUNCH, R>, NT, a.num_tiles);
+  if (grid <= 0) return cudaErrorInvalidConfiguration;
+  return launch_pdl(k_render<T, S, MODE, LAUNCH, R>, grid, NT, 0, s, a);
+}
+
 template <int T, int S, int MODE, int LAUNCH>
 cudaError_t launch_mode(const RenderArgs& a, cudaStream_t s) {
   if (a.num_tiles <= 0) return cudaSuccess;
-  int grid = a.num_tiles;
-  if (LAUNCH == GS2D_LAUNCH_PERSISTENT)
-    grid = persistent_grid((const void*)k_render<T, S, MODE, LAUNCH>, TileGeom<T>::NT,
-                           a.num_tiles);
-  if (grid <= 0) return cudaErrorInvalidConfiguration;
-  return launch_pdl(k_render<T, S, MODE, LAUNCH>, grid, TileGeom<T>::NT, 0, s, a);
+  if constexpr (T > 8 && LAUNCH == GS2D_LAUNCH_GRID && kFewWarps<T, MODE> > 0) {
+    if (a.num_tiles <= kFewWarps<T, MODE> / TileGeom<T, kRows<T>>::NW)
+      return launch_rows<T, S, MODE, LAUNCH, 1>(a, s);
+  }
+  return launch_rows<T, S, MODE, LAUNCH, kRows<T>>(a, s);
 }
 
 template <int T, int S, int LAUNCH>
@@ -613,13 +709,13 @@ cudaError_t launch_tile(int stage, int launch, RenderMode mode, const RenderArgs
 template <int T>
 cudaError_t prime_tile(int stage, int launch) {
   if (launch == GS2D_LAUNCH_GRID) return cudaSuccess;
-  constexpr int NT = TileGeom<T>::NT, P = GS2D_LAUNCH_PERSISTENT;
+  constexpr int R = kRows<T>, NT = TileGeom<T, R>::NT, P = GS2D_LAUNCH_PERSISTENT;
   int g = 0;
   switch (stage) {
-    case 32: g = persistent_grid((const void*)k_render<T, 32, kModeL2, P>, NT, 1); break;
-    case 64: g = persistent_grid((const void*)k_render<T, 64, kModeL2, P>, NT, 1); break;
-    case 128: g = persistent_grid((const void*)k_render<T, 128, kModeL2, P>, NT, 1); break;
-    case 256: g = persistent_grid((const void*)k_render<T, 256, kModeL2, P>, NT, 1); break;
+    case 32: g = persistent_grid((const void*)k_render<T, 32, kModeL2, P, R>, NT, 1); break;
+    case 64: g = persistent_grid((const void*)k_render<T, 64, kModeL2, P, R>, NT, 1); break;
+    case 128: g = persistent_grid((const void*)k_render<T, 128, kModeL2, P, R>, NT, 1); break;
+    case 256: g = persistent_grid((const void*)k_render<T, 256, kModeL2, P, R>, NT, 1); break;
     default: return cudaErrorInvalidValue;
   }
   return g > 0 ? cudaSuccess : cudaErrorInvalidConfiguration;

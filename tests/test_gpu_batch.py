@@ -274,3 +274,33 @@ def test_one_clip_batch_is_the_single_frame_plan(gs):
     g2, l2, i2 = b.render_l2(p, t.reshape(-1), want_image=True)
     assert r.read_bins()["n_entries"] == b.read_bins()["n_entries"] > 0
     assert torch.equal(g1, g2) and torch.equal(l1, l2) and torch.equal(i1.reshape(-1), i2)
+
+
+@pytest.mark.parametrize("tile", [16, 32])
+def test_few_tiles_equal_many_bit_for_bit(gs, tile):
+    """Single small frames take the render kernels with one row per thread, a
+    batch of them (more tiles) the usual ones: image, gradients and losses of
+    every clip are the same bit for bit, in every mode."""
+    cfg = gs.RasterConfig(tile=tile, stage=64)
+    sizes = [(301, 211, 700 + 31 * k) for k in range(12)]
+    batch = gs.BatchRasterizer(sizes, config=cfg)
+    ps = [torch.from_numpy(random_gaussians(n, w, h, seed=k)).cuda()
+          for k, (w, h, n) in enumerate(sizes)]
+    ts = [torch.from_numpy(smooth_noise_target(w, h, seed=50 + k)).cuda()
+          for k, (w, h, _) in enumerate(sizes)]
+    P, T = batch.pack_params(ps), batch.pack_images(ts)
+    batch.prepare(P)
+    img, dimg = batch.render_fwd(), T - 0.5
+    grad = batch.render_bwd(P, dimg)
+    g2, _, i2 = batch.render_l2(P, T, want_image=True)
+    losses = batch.clip_losses()
+    for c, (w, h, n) in enumerate(sizes):
+        one = gs.GaussianRasterizer(w, h, n, config=cfg)
+        one.prepare(ps[c])
+        cols = slice(batch.offsets[c], batch.offsets[c] + n)
+        assert torch.equal(one.render_fwd(), batch.clip_view(img, c))
+        assert torch.equal(one.render_bwd(ps[c], batch.clip_view(dimg, c).contiguous()),
+                           grad[:, cols])
+        sg, loss, si = one.render_l2(ps[c], ts[c], want_image=True)
+        assert torch.equal(sg, g2[:, cols]) and torch.equal(si, batch.clip_view(i2, c))
+        assert (float(loss[0]), float(loss[1])) == losses[c]
