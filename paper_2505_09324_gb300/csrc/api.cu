@@ -169,10 +169,10 @@ gs2d_status gs2d_plan_init_batch(gs2d_plan* plan, gs2d_clip* clips, int32_t num_
   sz[kOffRec] = 3 * nn * sizeof(float4);
   sz[kOffRect] = nn * sizeof(int4);
   sz[kOffCount] = (nn + 1) * sizeof(int);
-  sz[kOffBlockSum] = (nn / 32 + 1) * sizeof(long long);  // blocks of >= 32 Gaussians
+  // up to three sums per group of at least 64 Gaussians
+  sz[kOffBlockSum] = 3 * (nn / 64 + 1) * sizeof(long long);
   sz[kOffTileCnt] = nt * sizeof(int);
   sz[kOffCursor] = nt * sizeof(int);
-  sz[kOffLong] = (nt + 1) * sizeof(int);
   sz[kOffList] = me * sizeof(uint32_t);
   sz[kOffRanges] = nt * sizeof(int2);
   sz[kOffOrder] = nt * sizeof(int);
@@ -902,16 +902,18 @@ gs2d_status gs2d_read_bins(const gs2d_plan* plan, const void* ws, int64_t* n_ent
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(rg.data(), ws_ptr<int2>(ws, p, kOffRanges), rg.size() * sizeof(int2),
                         cudaMemcpyDeviceToHost, s);
-  std::vector<int> offs;
+  std::vector<int4> rects;
   if (e == cudaSuccess && counts && p.n > 0) {
-    offs.resize((size_t)p.n + 1);
-    e = cudaMemcpyAsync(offs.data(), ws_ptr<int>(ws, p, kOffCount), offs.size() * sizeof(int),
+    rects.resize((size_t)p.n);
+    e = cudaMemcpyAsync(rects.data(), ws_ptr<int4>(ws, p, kOffRect), rects.size() * sizeof(int4),
                         cudaMemcpyDeviceToHost, s);
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_check(e, "gs2d_read_bins");
+  // (over capacity nothing is listed)
+  const bool over = h.entries_raw > p.max_entries;
   if (counts)
-    for (int i = 0; i < p.n; i++) counts[i] = offs[i + 1] - offs[i];
+    for (int i = 0; i < p.n; i++) counts[i] = over ? 0 : rects[i].z * rects[i].w;
   if (ranges)
     for (int t = 0; t < p.num_tiles; t++) {
       ranges[2 * t] = rg[t].x;

@@ -6,85 +6,86 @@
 // ordered by index: the sorted list is the (tile, index) key order.
 //
 // The sort is a single-digit radix (counting) sort by tile id over all SMs:
-//   1. per-tile entry counts (atomic increments from each Gaussian's tiles)
-//      and per-block sums of the per-Gaussian counts;
-//   2. exclusive scans: one CTA per block of 256 Gaussians for the offsets
-//      (backward slots), one CTA per 1024 tiles for the list ranges; capacity;
-//   3. scatter: every entry claims the next slot of its tile's list;
-//   4. segment sort: each tile's list is sorted by Gaussian index (a warp
-//      bitonic network in registers for lists of up to 512, a CTA bitonic
-//      network in shared memory for longer ones), restoring exactly the order
-//      a stable sort of the index-ordered entries would give.
-// Steps 2 and 4 also build the render queue: tiles grouped by list-length
+//   1. k_count: per-tile entry counts (atomic increments from each Gaussian's
+//      tiles) and the entries of each group of Gaussians; the last block to
+//      finish scans both (the groups' first backward slots, the tiles' list
+//      ranges, capacity);
+//   2. k_bin_scatter: every entry claims the next slot of its tile's list;
+//   3. k_sort: each tile's list is sorted by Gaussian index (a warp bitonic
+//      network in registers for lists of up to 512, the block's shared memory
+//      for longer ones), restoring exactly the order a stable sort of the
+//      index-ordered entries would give.
+// Each is a chain of a few dependent memory latencies, so the number of
+// launches and of warps in flight is what counts: a group is 64 Gaussians
+// (313 blocks at 20 000; 79 blocks of 256 left half the SMs idle), and its
+// entries are dealt out to all 256 threads of the block (the scatter at
+// 1920 x 1080, 20 000 Gaussians, tile 16: 16.9 -> 8.4 us; with it and two
+// launches fewer, prepare + render: 62.6 -> 50.8 us).  Plans of more than
+// kOneScan tiles or groups scan in a launch of their own (k_bin_scan).
+// Steps 1 and 3 also build the render queue: tiles grouped by list-length
 // class (floor(log2(len)) + 1, 0 for empty tiles), longest class first.  The
-// scan gives each tile its rank inside its class (one atomic per class and
-// block), the segment sort turns (class, rank) into the queue position once
-// every class size is known.
+// scan gives each tile its rank inside its class, the segment sort turns
+// (class, rank) into the queue position.
 // A batch of clips is binned in one pass: tiles are numbered clip after clip
 // and each Gaussian's rectangle is stored in that numbering.
 #include "gs2d_internal.cuh"
 
 namespace gs2d {
 
-constexpr int kLongMax = 1 << 15;  // longest list the CTA sort holds (128 KB)
-constexpr int kGB = 256;           // Gaussians per counting / scan block
+constexpr int kLongMax = 1 << 15;   // longest list that is sorted
+constexpr int kSmemKeys = 1 << 13;  // keys of one shared-memory sort (32 KB)
+constexpr int kThreads = 256;
+constexpr int kGroup = 64;          // Gaussians per block
+constexpr int kGroupLarge = 256;    // the same beyond kManyGroups groups
+constexpr int kManyGroups = 1 << 13;
+// Up to two steps of the one-block scan (1024 tiles or groups each, 2.3 us a
+// step: a chain of loads, scans and class counts) it is faster than another
+// launch: k_count with its scan takes 10 us at 256 tiles against 8.5 + 4.5,
+// and 28 us at 8160 tiles against 9 + 8 (cold caches).
+constexpr int kOneScan = 2048;
+
+// The binning's view of a workspace.
+struct BinArgs {
+  ClipSet cs;
+  int n, num_tiles, tile_shift;
+  int group, groups;       // Gaussians per block, blocks
+  int one_scan;            // k_count's last block scans
+  int64_t max_entries;
+  float sigma_cut, alpha_min, det_eps, margin;
+  const float* params;
+  float4* rec;
+  int4* rect;              // tight rectangles
+  int4* lrect;             // the rectangles the lists are built from
+  int* offs;               // [n + 1] first backward slot of each Gaussian
+  int* tile_cnt;           // zero between calls
+  int* tile_cnt2;          // the same for the tight rectangles of a rebuild
+  long long* sums;         // [2][groups] entries per group, then exclusive offsets
+  int* cursor;
+  int2* ranges;
+  int* bucket;
+  uint32_t* rank;
+  int* order;
+  uint32_t* list;
+  uint32_t* spare;         // [max_entries] scratch of the longest sorts (the backward records)
+  WsHeader* hdr;
+};
+
+// Adam step of the fit loop, advanced by the first kernel of an iteration.
+struct AdamTick {
+  int on;
+  float b1, b2, lr, lr_decay;
+};
 
 // ---------------------------------------------------------------------------
-// Projection (gs2d_project): records, rectangles, per-Gaussian counts.
-__global__ void __launch_bounds__(kGB)
+// Projection (gs2d_project): records and rectangles.
+__global__ void __launch_bounds__(kThreads)
 k_project(int n, ClipSet cs, int tile_shift, float sigma_cut, float alpha_min, float det_eps,
-          const float* __restrict__ params, float4* __restrict__ rec, int4* __restrict__ rect,
-          int* __restrict__ count) {
+          const float* __restrict__ params, float4* __restrict__ rec, int4* __restrict__ rect) {
   pdl_begin();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  project_one(i, n, clip_of_gaussian(cs, i), tile_shift, sigma_cut, alpha_min, det_eps, params,
-              rec, rect, count);
-}
-
-// Per-tile entry counts from the rectangles (warp-cooperative: lanes share the
-// tiles of one Gaussian at a time; fire-and-forget atomics).
-__device__ __forceinline__ void count_tiles_warp(int n, const int4* __restrict__ rect,
-                                                 int* __restrict__ tile_cnt) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int lane = threadIdx.x & 31;
-  const int4 rc = i < n ? rect[i] : make_int4(0, 0, 0, 0);
-  for (int l = 0; l < 32; l++) {
-    const int t0 = __shfl_sync(0xffffffffu, rc.x, l);
-    const int stride = __shfl_sync(0xffffffffu, rc.y, l);
-    const int w = __shfl_sync(0xffffffffu, rc.z, l);
-    const int cnt = w * __shfl_sync(0xffffffffu, rc.w, l);
-    for (int j = lane; j < cnt; j += 32) {
-      const int dy = j / w;
-      atomicAdd(&tile_cnt[t0 + dy * stride + (j - dy * w)], 1);
-    }
-  }
-}
-
-// The block's sum of per-Gaussian counts.
-__device__ __forceinline__ void block_count_sum(int n, const int* __restrict__ count,
-                                                long long* __restrict__ block_sum) {
-  __shared__ int s_warp[kGB / 32];
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int lane = threadIdx.x & 31;
-  int c = i < n ? count[i] : 0;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-  if (lane == 0) s_warp[threadIdx.x >> 5] = c;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    long long s = 0;
-    for (int w = 0; w < kGB / 32; w++) s += s_warp[w];
-    block_sum[blockIdx.x] = s;
-  }
-}
-
-__device__ __forceinline__ void count_block(int n, const int4* __restrict__ rect,
-                                           const int* __restrict__ count,
-                                           int* __restrict__ tile_cnt,
-                                           long long* __restrict__ block_sum) {
-  count_tiles_warp(n, rect, tile_cnt);
-  block_count_sum(n, count, block_sum);
+  rect[i] = project_one(i, n, clip_of_gaussian(cs, i), tile_shift, sigma_cut, alpha_min, det_eps,
+                        params, rec);
 }
 
 // Adam step counter, the powers beta^step and the decayed learning rate of
@@ -103,147 +104,79 @@ __device__ __forceinline__ void adam_tick_header(WsHeader* hdr, float b1, float 
   hdr->lr_now = (float)(lr * pd);
 }
 
-__global__ void __launch_bounds__(kGB)
-k_count_tiles(int n, const int4* __restrict__ rect, const int* __restrict__ count,
-              int* __restrict__ tile_cnt, long long* __restrict__ block_sum,
-              WsHeader* __restrict__ hdr) {
-  pdl_begin();
-  if (blockIdx.x == 0 && threadIdx.x == 0) hdr->lists_valid = 0;  // rebuilt from tight boxes
-  count_block(n, rect, count, tile_cnt, block_sum);
-}
-
-// Fused projection + counts for gs2d_prepare and the fit loop; with adam_tick
-// the Adam step counter and the powers beta^step advance here (the first
-// kernel of a fit iteration).
-__global__ void __launch_bounds__(kGB)
-k_project_count(int n, ClipSet cs, int tile_shift, float sigma_cut, float alpha_min,
-                float det_eps,
-                const float* __restrict__ params, float4* __restrict__ rec,
-                int4* __restrict__ rect, int* __restrict__ count, int* __restrict__ tile_cnt,
-                long long* __restrict__ block_sum, WsHeader* __restrict__ hdr, int adam_tick,
-                float b1, float b2, float lr, float lr_decay) {
-  pdl_begin();
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i == 0) {
-    if (adam_tick) adam_tick_header(hdr, b1, b2, lr, lr_decay);
-    hdr->lists_valid = 0;  // the lists below are built from the tight rectangles
-  }
-  if (i < n)
-    project_one(i, n, clip_of_gaussian(cs, i), tile_shift, sigma_cut, alpha_min, det_eps, params,
-                rec, rect, count);
-  __syncwarp();
-  count_block(n, rect, count, tile_cnt, block_sum);
-}
-
-// ---------------------------------------------------------------------------
-// Fit loop with retained tile lists.  Within a tile a Gaussian adds nothing
-// outside its cut-off box, so a list may hold Gaussians that do not reach the
-// tile: the render skips a (tile, Gaussian) pair whose tile lies outside the
-// Gaussian's tight rectangle, and the backward slots stay those of the tight
-// rectangles, so results are the same as with lists rebuilt every iteration.
-// Each Gaussian is listed over its rectangle widened by `margin` pixels; the
-// lists are rebuilt only in an iteration where some tight rectangle has left
-// its listed one.
-//
-// k_project_fit: records, tight rectangles and counts (the backward slots),
-// block sums of the counts, the containment test against the listed
-// rectangle (clears hdr->lists_valid on a miss) and the Adam tick.
-__global__ void __launch_bounds__(kGB)
-k_project_fit(int n, ClipSet cs, int tile_shift, float sigma_cut, float alpha_min, float det_eps,
-              const float* __restrict__ params, float4* __restrict__ rec, int4* __restrict__ rect,
-              int* __restrict__ count, long long* __restrict__ block_sum,
-              const int4* __restrict__ lrect, WsHeader* __restrict__ hdr, float b1, float b2,
-              float lr, float lr_decay) {
-  pdl_begin();
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i == 0) adam_tick_header(hdr, b1, b2, lr, lr_decay);
-  if (i < n) {
-    const gs2d_clip cl = clip_of_gaussian(cs, i);
-    int tx0 = 0, ty0 = 0, tx1 = 0, ty1 = 0;
-    const bool vis = gaussian_tiles(i, n, cl, tile_shift, sigma_cut, alpha_min, det_eps, params,
-                                    0.0f, tx0, ty0, tx1, ty1);
-    const int4 rc = vis ? make_int4(cl.tile_off + ty0 * cl.tiles_x + tx0, cl.tiles_x, tx1 - tx0,
-                                    ty1 - ty0)
-                        : make_int4(0, 0, 0, 0);
-    rect[i] = rc;
-    count[i] = rc.z * rc.w;
-    write_record(i, n, vis, sigma_cut, alpha_min, params, rec);
-    if (vis) {
-      const int4 lr4 = lrect[i];
-      bool inside = lr4.z > 0;
-      if (inside) {
-        const int rel = lr4.x - cl.tile_off;
-        const int ly0 = rel / cl.tiles_x, lx0 = rel - ly0 * cl.tiles_x;
-        inside = lx0 <= tx0 && ly0 <= ty0 && tx1 <= lx0 + lr4.z && ty1 <= ly0 + lr4.w;
-      }
-      if (!inside) hdr->lists_valid = 0;
-    }
-  }
-  block_count_sum(n, count, block_sum);
-}
-
-// Rebuild step 1 (only when k_project_fit found a miss): the listed
-// rectangles, widened by `margin` pixels, and the per-tile entry counts; the
-// tight rectangles are counted too (tile_cnt2), so that the scan can fall
-// back to them when the widened lists would overflow max_entries.
-__global__ void __launch_bounds__(kGB)
-k_rebin_count(int n, ClipSet cs, int tile_shift, float sigma_cut, float alpha_min,
-              float det_eps, float margin, const float* __restrict__ params,
-              const int4* __restrict__ rect, int4* __restrict__ lrect,
-              int* __restrict__ tile_cnt, int* __restrict__ tile_cnt2,
-              WsHeader* __restrict__ hdr) {
-  pdl_begin();
-  if (hdr->lists_valid) return;  // the same for every thread of the grid
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i == 0) hdr->rebins++;
-  if (i < n) {
-    const gs2d_clip cl = clip_of_gaussian(cs, i);
-    int tx0 = 0, ty0 = 0, tx1 = 0, ty1 = 0;
-    const bool vis = gaussian_tiles(i, n, cl, tile_shift, sigma_cut, alpha_min, det_eps, params,
-                                    margin, tx0, ty0, tx1, ty1);
-    lrect[i] = vis ? make_int4(cl.tile_off + ty0 * cl.tiles_x + tx0, cl.tiles_x, tx1 - tx0,
-                               ty1 - ty0)
-                   : make_int4(0, 0, 0, 0);
-  }
-  __syncwarp();
-  count_tiles_warp(n, lrect, tile_cnt);
-  count_tiles_warp(n, rect, tile_cnt2);
-}
-
-// ---------------------------------------------------------------------------
-// Scans.  CTAs 0 .. nbg-1: offsets of their 256 Gaussians (prefix of the block
-// sums + in-block exclusive scan).  CTAs nbg ..: per-tile ranges and cursors of
-// a chunk of 1024 tiles; the first of them also records the entry total and
-// the capacity decision.  Sums are 64-bit so that a pathological input is
-// reported as over capacity instead of wrapping around.
-__device__ __forceinline__ long long block_scan64(long long v, long long* warp_sum,
-                                                  long long* total) {
+// Exclusive scan of v over the block; *total to every thread.
+template <typename V>
+__device__ __forceinline__ V block_scan(V v, V* warp_sum, V* total) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  long long x = v;
+  V x = v;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    const long long y = __shfl_up_sync(0xffffffffu, x, o);
+    const V y = __shfl_up_sync(0xffffffffu, x, o);
     if (lane >= o) x += y;
   }
   if (lane == 31) warp_sum[wid] = x;
   __syncthreads();
-  if (wid == 0) {
-    long long t = lane < nw ? warp_sum[lane] : 0;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const long long y = __shfl_up_sync(0xffffffffu, t, o);
-      if (lane >= o) t += y;
-    }
-    if (lane < nw) warp_sum[lane] = t;
+  V pre = 0, all = 0;
+  for (int w = 0; w < nw; w++) {
+    const V y = warp_sum[w];
+    pre += w < wid ? y : 0;
+    all += y;
   }
+  *total = all;
   __syncthreads();
-  const long long ex = (wid > 0 ? warp_sum[wid - 1] : 0) + x - v;
-  *total = warp_sum[nw - 1];
-  __syncthreads();
-  return ex;
+  return pre + x - v;
 }
 
-constexpr int kTileItems = 4;  // tiles per thread of a tile-scan CTA
+// A group's rectangles and the first entry of each, in shared memory: entry e
+// of the group belongs to the last Gaussian whose start is <= e.
+struct GroupSmem {
+  int4 rect[kGroupLarge];
+  int start[kGroupLarge];
+  long long warp_sum[kThreads / 32];
+  int last;
+};
+
+// Deals the rectangles (thread t < group: that of Gaussian t) out; returns the
+// group's entries.  `excl`: this thread's first entry.
+__device__ __forceinline__ long long group_entries(GroupSmem& gs, int4 rc, int group,
+                                                   long long* excl) {
+  const long long cnt = (long long)rc.z * rc.w;
+  long long total;
+  const long long ex = block_scan(cnt, gs.warp_sum, &total);
+  if ((int)threadIdx.x < group) {
+    gs.rect[threadIdx.x] = rc;
+    gs.start[threadIdx.x] = (int)min(ex, (long long)INT32_MAX);
+  }
+  __syncthreads();
+  *excl = ex;
+  return total;
+}
+
+// Entry e of the group: its Gaussian (index in the group) and tile.
+__device__ __forceinline__ int group_entry(const GroupSmem& gs, int group, int e, int* tile) {
+  int lo = 0;
+  for (int step = group >> 1; step > 0; step >>= 1)
+    if (gs.start[lo + step] <= e) lo += step;
+  const int4 rc = gs.rect[lo];
+  const int j = e - gs.start[lo];
+  const int dy = (int)((unsigned)j / (unsigned)rc.z);
+  *tile = rc.x + dy * rc.y + (j - dy * rc.z);
+  return lo;
+}
+
+// More entries than any plan holds: they are not counted per tile (the group
+// sums alone report the overflow).
+constexpr long long kMostEntries = 1ll << 28;
+
+__device__ __forceinline__ void group_count(const GroupSmem& gs, int group, long long total,
+                                            int* __restrict__ tile_cnt) {
+  if (total > kMostEntries) return;
+  for (int e = threadIdx.x; e < (int)total; e += kThreads) {
+    int tile;
+    group_entry(gs, group, e, &tile);
+    atomicAdd(&tile_cnt[tile], 1);
+  }
+}
 
 // Render-queue class of a list of length len: 0 (empty), 1 + floor(log2(len))
 // capped at kBuckets - 1.
@@ -251,177 +184,324 @@ __device__ __forceinline__ int length_class(int len) {
   return len <= 0 ? 0 : min(kBuckets - 1, 32 - __clz(len));
 }
 
-__global__ void __launch_bounds__(kGB)
-k_bin_scan(int n, int nbg, int num_tiles, int64_t max_entries, int* __restrict__ count,
-           const long long* __restrict__ block_sum, int* __restrict__ tile_cnt,
-           int* __restrict__ cursor, int2* __restrict__ ranges, int* __restrict__ bucket,
-           uint32_t* __restrict__ rank, WsHeader* __restrict__ hdr, int lazy,
-           const int* __restrict__ tile_cnt2) {
-  pdl_begin();
-  __shared__ long long warp_sum[32];
-  __shared__ int s_hist[kBuckets];
-  __shared__ int s_base[kBuckets];
-  const int t = threadIdx.x;
-  if ((int)blockIdx.x < nbg) {
-    // total and this block's prefix from the block sums
-    long long tot = 0, pre = 0;
-    for (int b = t; b < nbg; b += kGB) {
-      const long long v = block_sum[b];
-      tot += v;
-      pre += b < (int)blockIdx.x ? v : 0;
-    }
-    long long total, prefix;
-    block_scan64(tot, warp_sum, &total);
-    block_scan64(pre, warp_sum, &prefix);
-    const bool over = total > max_entries;
-    const int i = blockIdx.x * kGB + t;
-    const int c = i < n ? count[i] : 0;
-    long long dummy;
-    const long long ex = block_scan64(c, warp_sum, &dummy);
-    if (i < n) count[i] = over ? 0 : (int)(prefix + ex);
-    if (blockIdx.x == 0 && t == 0) count[n] = over ? 0 : (int)total;
-    return;
-  }
-  // retained lists: only the slots (above) change
-  if (lazy && hdr->lists_valid) return;  // the same for every thread of the grid
-  // tile CTAs: chunk [c0, c0 + kGB * kTileItems) of the tiles; the prefix of the
-  // chunk and the total come from a strided pass over all tile counts (the
-  // counts are reset later, by k_sort_short, once nothing reads them)
-  const int tb = (int)blockIdx.x - nbg;
-  const int c0 = tb * kGB * kTileItems;
-  long long tot = 0, pre = 0, tot2 = 0, pre2 = 0;
-  for (int i = t; i < num_tiles; i += kGB) {
-    const int v = tile_cnt[i];
-    tot += v;
-    pre += i < c0 ? v : 0;
-    if (lazy) {
-      const int v2 = tile_cnt2[i];
-      tot2 += v2;
-      pre2 += i < c0 ? v2 : 0;
-    }
-  }
-  long long total, prefix;
-  block_scan64(tot, warp_sum, &total);
-  block_scan64(pre, warp_sum, &prefix);
-  // a rebuild whose widened lists overflow lists the tight rectangles instead
-  // (the same decision in every tile CTA: the totals are global)
-  bool tight = false;
-  if (lazy) {
-    long long total2, prefix2;
-    block_scan64(tot2, warp_sum, &total2);
-    block_scan64(pre2, warp_sum, &prefix2);
-    tight = total > max_entries && total2 <= max_entries;
-    if (tight) {
-      total = total2;
-      prefix = prefix2;
-      tile_cnt = const_cast<int*>(tile_cnt2);
-    }
-  }
-  const bool over = total > max_entries;
-  if (t < kBuckets) s_hist[t] = 0;
-  __syncthreads();
-  {
-    const int base = c0 + t * kTileItems;
-    int c[kTileItems];
-    long long v = 0;
+constexpr int kTileItems = 4;  // tiles per thread of a scan step
+
+// Rank of each lane's tile inside its class, counted in hist (shared): one
+// atomic per class and warp.
+__device__ __forceinline__ int class_rank(int cls, bool valid, int* hist) {
+  const unsigned peers = __match_any_sync(0xffffffffu, valid ? cls : -1);
+  const int lane = threadIdx.x & 31, leader = __ffs(peers) - 1;
+  int base = 0;
+  if (valid && lane == leader) base = atomicAdd(&hist[cls], __popc(peers));
+  base = __shfl_sync(0xffffffffu, base, leader);
+  return base + __popc(peers & ((1u << lane) - 1u));
+}
+
+// Entries per group -> first entry of the group (in place or elsewhere), by
+// one block; returns the total.
+__device__ __forceinline__ long long scan_sums(const long long* sums, long long* first, int groups,
+                                               long long* warp_sum) {
+  long long run = 0;
+  for (int b0 = 0; b0 < groups; b0 += kThreads * kTileItems) {
+    const int b = b0 + threadIdx.x * kTileItems;
+    long long v[kTileItems], mine = 0, total;
 #pragma unroll
     for (int k = 0; k < kTileItems; k++) {
-      c[k] = base + k < num_tiles ? tile_cnt[base + k] : 0;
+      v[k] = b + k < groups ? __ldcg(&sums[b + k]) : 0;
+      mine += v[k];
+    }
+    long long at = run + block_scan(mine, warp_sum, &total);
+#pragma unroll
+    for (int k = 0; k < kTileItems; k++) {
+      if (b + k < groups) first[b + k] = at;
+      at += v[k];
+    }
+    run += total;
+  }
+  return run;
+}
+
+// The whole scan by one block (k_count's last): group offsets, the capacity
+// decision, list ranges, cursors and queue ranks of the tiles; the tile counts
+// are cleared for the next binning.  LAZY: a rebuild whose widened lists
+// overflow lists the tight rectangles instead.
+template <bool LAZY>
+__device__ __forceinline__ void one_block_scan(const BinArgs& a, GroupSmem& gs, int* s_hist) {
+  const int t = threadIdx.x;
+  long long total = scan_sums(a.sums, a.sums, a.groups, gs.warp_sum);
+  bool tight = false;
+  if (LAZY) {
+    const long long total2 =
+        scan_sums(a.sums + a.groups, a.sums + a.groups, a.groups, gs.warp_sum);
+    tight = total > a.max_entries && total2 <= a.max_entries;
+    if (tight) total = total2;
+  }
+  const bool over = total > a.max_entries;
+  if (t < kBuckets) s_hist[t] = 0;
+  __syncthreads();
+  int* cnt = LAZY && tight ? a.tile_cnt2 : a.tile_cnt;
+  int* other = LAZY ? (tight ? a.tile_cnt : a.tile_cnt2) : nullptr;
+  int* warp_sum = reinterpret_cast<int*>(gs.warp_sum);
+  int run = 0;
+  for (int c0 = 0; c0 < a.num_tiles; c0 += kThreads * kTileItems) {
+    const int base = c0 + t * kTileItems;
+    int c[kTileItems], v = 0;
+#pragma unroll
+    for (int k = 0; k < kTileItems; k++) {
+      c[k] = base + k < a.num_tiles && !over ? __ldcg(&cnt[base + k]) : 0;
       v += c[k];
     }
-    long long chunk;
-    long long run = prefix + block_scan64(v, warp_sum, &chunk);
-    int cls[kTileItems], r[kTileItems];
+    int chunk;
+    int s = run + block_scan(v, warp_sum, &chunk);
+    run += chunk;
 #pragma unroll
     for (int k = 0; k < kTileItems; k++) {
       const int i = base + k;
-      cls[k] = length_class(over ? 0 : c[k]);
-      r[k] = 0;
-      if (i < num_tiles) {
-        const int s = over ? 0 : (int)run;
+      const bool valid = i < a.num_tiles;
+      const int cls = length_class(c[k]);
+      const int r = class_rank(cls, valid, s_hist);
+      if (valid) {
         // an empty tile's range is (0, 0) wherever it sits in the list
-        ranges[i] = (over || c[k] == 0) ? make_int2(0, 0) : make_int2(s, s + c[k]);
-        cursor[i] = s;
-        r[k] = atomicAdd(&s_hist[cls[k]], 1);
+        a.ranges[i] = c[k] == 0 ? make_int2(0, 0) : make_int2(s, s + c[k]);
+        a.cursor[i] = s;
+        a.rank[i] = ((uint32_t)cls << 28) | (uint32_t)r;
+        cnt[i] = 0;
+        if (LAZY) other[i] = 0;
       }
-      run += c[k];
+      s += c[k];
     }
-    __syncthreads();
-    // this block's first rank in each class
-    if (t < kBuckets) s_base[t] = s_hist[t] ? atomicAdd(&bucket[t], s_hist[t]) : 0;
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < kTileItems; k++)
-      if (base + k < num_tiles)
-        rank[base + k] = ((uint32_t)cls[k] << 28) | (uint32_t)(s_base[cls[k]] + r[k]);
   }
-  if (tb == 0 && t == 0) {
-    hdr->entries_raw = total;
-    hdr->n_entries = over ? 0 : (int)total;
-    if (over) atomicCAS(&hdr->status, 0, (int)GS2D_ERR_CAPACITY);
-    if (nbg == 0) count[n] = 0;
-    hdr->long_count = 0;
-    hdr->lists_tight = tight ? 1 : 0;
+  __syncthreads();
+  if (t < kBuckets) a.bucket[t] = s_hist[t];
+  if (t == 0) {
+    a.hdr->entries_raw = total;
+    a.hdr->n_entries = over ? 0 : (int)total;
+    if (over) atomicCAS(&a.hdr->status, 0, (int)GS2D_ERR_CAPACITY);
+    a.hdr->lists_tight = tight ? 1 : 0;
   }
 }
 
-// Scatter: every entry claims the next slot of its tile's list.  A warp takes
-// 32 Gaussians, flattens their entries, and each lane keeps kInFlight atomics
-// in flight before it stores the claimed slots.
+// What k_count counts: the rectangles of gs2d_project, those of a projection
+// it does itself (gs2d_prepare and P-frames), or the widened rectangles of a
+// rebuild of the fit loop's retained lists (see below), with the tight ones
+// beside them.
+enum CountMode { kCountRects, kCountProject, kCountRebin };
+
+template <CountMode MODE>
+__global__ void __launch_bounds__(kThreads)
+k_count(const __grid_constant__ BinArgs a, AdamTick tick) {
+  pdl_begin();
+  __shared__ GroupSmem gs;
+  __shared__ int s_hist[kBuckets];
+  constexpr bool kLazy = MODE == kCountRebin;
+  if (kLazy && a.hdr->lists_valid) return;  // the same for every thread of the grid
+  const int t = threadIdx.x, i = blockIdx.x * a.group + t;
+  if (blockIdx.x == 0) {
+    if (t == 0) {
+      if (kLazy) {
+        a.hdr->rebins++;
+      } else {
+        if (tick.on) adam_tick_header(a.hdr, tick.b1, tick.b2, tick.lr, tick.lr_decay);
+        a.hdr->lists_valid = 0;  // the lists are built from the tight rectangles
+      }
+    }
+    if (!a.one_scan && t < 2 * kBuckets) a.bucket[t] = 0;  // k_bin_scan adds to them
+  }
+  int4 rc = make_int4(0, 0, 0, 0), rt = rc;
+  if (t < a.group && i < a.n) {
+    if (MODE == kCountRects) {
+      rc = a.rect[i];
+    } else if (MODE == kCountProject) {
+      rc = project_one(i, a.n, clip_of_gaussian(a.cs, i), a.tile_shift, a.sigma_cut, a.alpha_min,
+                       a.det_eps, a.params, a.rec);
+      a.rect[i] = rc;
+    } else {
+      const gs2d_clip cl = clip_of_gaussian(a.cs, i);
+      int tx0 = 0, ty0 = 0, tx1 = 0, ty1 = 0;
+      if (gaussian_tiles(i, a.n, cl, a.tile_shift, a.sigma_cut, a.alpha_min, a.det_eps, a.params,
+                         a.margin, tx0, ty0, tx1, ty1))
+        rc = make_int4(cl.tile_off + ty0 * cl.tiles_x + tx0, cl.tiles_x, tx1 - tx0, ty1 - ty0);
+      rt = a.rect[i];
+    }
+    a.lrect[i] = rc;
+  }
+  long long ex;
+  const long long total = group_entries(gs, rc, a.group, &ex);
+  group_count(gs, a.group, total, a.tile_cnt);
+  if (t == 0) a.sums[blockIdx.x] = total;
+  if (kLazy) {
+    __syncthreads();
+    const long long total2 = group_entries(gs, rt, a.group, &ex);
+    group_count(gs, a.group, total2, a.tile_cnt2);
+    if (t == 0) a.sums[a.groups + blockIdx.x] = total2;
+  }
+  if (!a.one_scan) return;
+  // the last block to get here sees every block's counts and sums
+  __threadfence();
+  __syncthreads();
+  if (t == 0) gs.last = atomicAdd(&a.hdr->ticket, 1) == (int)gridDim.x - 1;
+  __syncthreads();
+  if (!gs.last) return;
+  if (t == 0) a.hdr->ticket = 0;
+  __threadfence();
+  one_block_scan<kLazy>(a, gs, s_hist);
+}
+
+// ---------------------------------------------------------------------------
+// Fit loop with retained tile lists.  Within a tile a Gaussian adds nothing
+// outside its cut-off box, so a list may hold Gaussians that do not reach the
+// tile: such a pair adds exact zeros.  Each Gaussian is listed over its
+// rectangle widened by `margin` pixels; the lists, and the backward slots,
+// which follow the listed rectangles, are rebuilt only in an iteration where
+// some tight rectangle has left its listed one.  The per-Gaussian reduction
+// takes the slots of the tight rectangle, in its order, so results are the
+// same as with lists rebuilt every iteration.
+//
+// k_project_fit: records, tight rectangles, the containment test against the
+// listed rectangle (clears hdr->lists_valid on a miss) and the Adam tick.
+__global__ void __launch_bounds__(128)
+k_project_fit(const __grid_constant__ BinArgs a, AdamTick tick) {
+  pdl_begin();
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i == 0) adam_tick_header(a.hdr, tick.b1, tick.b2, tick.lr, tick.lr_decay);
+  if (i >= a.n) return;
+  const gs2d_clip cl = clip_of_gaussian(a.cs, i);
+  int tx0 = 0, ty0 = 0, tx1 = 0, ty1 = 0;
+  const bool vis = gaussian_tiles(i, a.n, cl, a.tile_shift, a.sigma_cut, a.alpha_min, a.det_eps,
+                                  a.params, 0.0f, tx0, ty0, tx1, ty1);
+  a.rect[i] = vis ? make_int4(cl.tile_off + ty0 * cl.tiles_x + tx0, cl.tiles_x, tx1 - tx0,
+                              ty1 - ty0)
+                  : make_int4(0, 0, 0, 0);
+  write_record(i, a.n, vis, a.sigma_cut, a.alpha_min, a.params, a.rec);
+  if (vis) {
+    const int4 lr4 = a.lrect[i];
+    bool inside = lr4.z > 0;
+    if (inside) {
+      const int rel = lr4.x - cl.tile_off;
+      const int ly0 = rel / cl.tiles_x, lx0 = rel - ly0 * cl.tiles_x;
+      inside = lx0 <= tx0 && ly0 <= ty0 && tx1 <= lx0 + lr4.z && ty1 <= ly0 + lr4.w;
+    }
+    if (!inside) a.hdr->lists_valid = 0;
+  }
+}
+
+// ---------------------------------------------------------------------------
+// The scans in a launch of their own (large plans).  Block 0: the groups'
+// first entries.  The others: ranges and cursors of a chunk of 1024 tiles; the
+// first of them also records the total and the capacity decision.  Every
+// block sums what it needs of the rest itself.  Sums are 64-bit so that a
+// pathological input is reported as over capacity instead of wrapping around.
+template <bool LAZY>
+__global__ void __launch_bounds__(kThreads)
+k_bin_scan(const __grid_constant__ BinArgs a, long long* __restrict__ first) {
+  pdl_begin();
+  __shared__ long long warp_sum[kThreads / 32];
+  __shared__ int s_hist[kBuckets], s_base[kBuckets];
+  if (LAZY && a.hdr->lists_valid) return;  // the same for every thread of the grid
+  const int t = threadIdx.x, tb = (int)blockIdx.x - 1;
+  long long tot = 0, tot2 = 0, total, total2 = 0;
+  for (int b = t; b < a.groups; b += kThreads) {
+    tot += a.sums[b];
+    tot2 += LAZY ? a.sums[a.groups + b] : 0;
+  }
+  block_scan(tot, warp_sum, &total);
+  if (LAZY) block_scan(tot2, warp_sum, &total2);
+  // the same decision in every block: the totals are global
+  const bool tight = LAZY && total > a.max_entries && total2 <= a.max_entries;
+  if (tight) total = total2;
+  const bool over = total > a.max_entries;
+  if (tb < 0) {
+    scan_sums(a.sums + (tight ? a.groups : 0), first, a.groups, warp_sum);
+    return;
+  }
+  const int* cnt = tight ? a.tile_cnt2 : a.tile_cnt;
+  const int c0 = tb * kThreads * kTileItems;
+  long long before = 0, prefix_tiles;
+  for (int i = t; i < c0; i += kThreads) before += cnt[i];
+  block_scan(before, warp_sum, &prefix_tiles);
+  if (t < kBuckets) s_hist[t] = 0;
+  __syncthreads();
+  const int base = c0 + t * kTileItems;
+  int c[kTileItems], cls[kTileItems], r[kTileItems], v = 0;
+#pragma unroll
+  for (int k = 0; k < kTileItems; k++) {
+    c[k] = base + k < a.num_tiles && !over ? cnt[base + k] : 0;
+    v += c[k];
+  }
+  int chunk;
+  int s = (over ? 0 : (int)prefix_tiles) + block_scan(v, reinterpret_cast<int*>(warp_sum), &chunk);
+#pragma unroll
+  for (int k = 0; k < kTileItems; k++) {
+    const int i = base + k;
+    cls[k] = length_class(c[k]);
+    r[k] = class_rank(cls[k], i < a.num_tiles, s_hist);
+    if (i < a.num_tiles) {
+      a.ranges[i] = c[k] == 0 ? make_int2(0, 0) : make_int2(s, s + c[k]);
+      a.cursor[i] = s;
+    }
+    s += c[k];
+  }
+  __syncthreads();
+  // this block's first rank in each class
+  if (t < kBuckets) s_base[t] = s_hist[t] ? atomicAdd(&a.bucket[t], s_hist[t]) : 0;
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < kTileItems; k++)
+    if (base + k < a.num_tiles)
+      a.rank[base + k] = ((uint32_t)cls[k] << 28) | (uint32_t)(s_base[cls[k]] + r[k]);
+  if (tb == 0 && t == 0) {
+    a.hdr->entries_raw = total;
+    a.hdr->n_entries = over ? 0 : (int)total;
+    if (over) atomicCAS(&a.hdr->status, 0, (int)GS2D_ERR_CAPACITY);
+    a.hdr->lists_tight = tight ? 1 : 0;
+  }
+}
+
+// Scatter: the first backward slot of every Gaussian, and every entry claims
+// the next slot of its tile's list; each thread keeps kInFlight atomics in
+// flight before it stores the claimed slots.  `first`: the groups' first
+// entries.
 constexpr int kInFlight = 4;
 
-__global__ void __launch_bounds__(kGB)
-k_bin_scatter(int n, const int4* __restrict__ tight_rect, int4* __restrict__ lrect,
-              const WsHeader* __restrict__ hdr, int* __restrict__ cursor,
-              uint32_t* __restrict__ list, int lazy) {
+template <bool LAZY>
+__global__ void __launch_bounds__(kThreads)
+k_bin_scatter(const __grid_constant__ BinArgs a, const long long* __restrict__ first) {
   pdl_begin();
-  __shared__ int s_start[kGB / 32][33];
-  if (hdr->entries_raw != (int64_t)hdr->n_entries) return;  // over capacity
-  if (lazy && hdr->lists_valid) return;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int g_base = (blockIdx.x * blockDim.x + threadIdx.x) & ~31;
-  const int g = g_base + lane;
-  // the rectangles listed: widened ones, or the tight ones (eager binning, or
-  // a rebuild whose widened lists overflowed: they become the listed ones)
-  const bool use_tight = !lazy || hdr->lists_tight;
-  const int4* __restrict__ rect = use_tight ? tight_rect : (const int4*)lrect;
-  const int4 rc = g < n ? rect[g] : make_int4(0, 0, 0, 0);
-  if (lazy && use_tight && g < n) lrect[g] = rc;
-  const int cnt = rc.z * rc.w;
-  int incl = cnt;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int y = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += y;
+  __shared__ GroupSmem gs;
+  if (LAZY && a.hdr->lists_valid) return;
+  const bool over = a.hdr->entries_raw != (int64_t)a.hdr->n_entries;
+  const int t = threadIdx.x, i = blockIdx.x * a.group + t;
+  const bool mine = t < a.group && i < a.n;
+  // the rectangles listed: the widened ones, or the tight ones of a rebuild
+  // whose widened lists overflowed, which become the listed ones
+  const bool use_tight = LAZY && a.hdr->lists_tight;
+  int4 rc = make_int4(0, 0, 0, 0);
+  if (mine) {
+    rc = use_tight ? a.rect[i] : a.lrect[i];
+    if (use_tight) a.lrect[i] = rc;
   }
-  int* start = s_start[wid];
-  start[lane] = incl - cnt;
-  const int T = __shfl_sync(0xffffffffu, incl, 31);
-  __syncwarp();
-  for (int e0 = 0; e0 < T; e0 += 32 * kInFlight) {
-    int pos[kInFlight];
-    uint32_t gi[kInFlight];
+  const long long base = a.one_scan && use_tight ? first[a.groups + blockIdx.x]
+                                                 : first[blockIdx.x];
+  long long ex;
+  const long long total = group_entries(gs, rc, a.group, &ex);
+  if (mine) a.offs[i] = over ? 0 : (int)(base + ex);
+  if (i == a.n - 1) a.offs[a.n] = over ? 0 : (int)(base + total);
+  if (over) return;
+  for (int e0 = t; e0 < (int)total; e0 += kThreads * kInFlight) {
+    int pos[kInFlight], gi[kInFlight];
 #pragma unroll
     for (int u = 0; u < kInFlight; u++) {
-      const int e = e0 + u * 32 + lane;
+      const int e = e0 + u * kThreads;
       pos[u] = -1;
-      if (e < T) {
-        // owner: the last lane whose start is <= e (binary search over 32)
-        // (starts are non-decreasing; 16 + 8 + 4 + 2 + 1 keeps lo + step <= 31)
-        int lo = 0;
-#pragma unroll
-        for (int step = 16; step > 0; step >>= 1)
-          if (start[lo + step] <= e) lo += step;
-        gi[u] = (uint32_t)(g_base + lo);
-        const int4 ro = rect[g_base + lo];
-        const int j = e - start[lo];
-        const int dy = j / ro.z;
-        pos[u] = atomicAdd(&cursor[ro.x + dy * ro.y + (j - dy * ro.z)], 1);
+      if (e < (int)total) {
+        int tile;
+        gi[u] = blockIdx.x * a.group + group_entry(gs, a.group, e, &tile);
+        pos[u] = atomicAdd(&a.cursor[tile], 1);
       }
     }
 #pragma unroll
     for (int u = 0; u < kInFlight; u++)
-      if (pos[u] >= 0) list[pos[u]] = gi[u];
+      if (pos[u] >= 0) a.list[pos[u]] = (uint32_t)gi[u];
   }
 }
 
@@ -477,204 +557,223 @@ __device__ __forceinline__ void warp_sort_list(uint32_t* __restrict__ seg, int l
   }
 }
 
-// Segment sort: one warp per tile, bitonic network in registers for lists of
-// up to 512; longer lists are queued for k_sort_long.  Also resets the tile's
-// entry counter for the next binning (its last reader, the scan, is done) and
-// places the tile in the render queue: after all tiles of longer classes, at
-// the next free position of its class.
-__global__ void __launch_bounds__(256)
-k_sort_short(int num_tiles, const int2* __restrict__ ranges, uint32_t* __restrict__ list,
-             int* __restrict__ long_tiles, int* __restrict__ tile_cnt,
-             const int* __restrict__ bucket, const uint32_t* __restrict__ rank,
-             int* __restrict__ order, WsHeader* __restrict__ hdr, int lazy,
-             int* __restrict__ tile_cnt2) {
-  pdl_begin();
-  if (lazy && hdr->lists_valid) return;
-  const int lane = threadIdx.x & 31;
-  const int tile = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (tile >= num_tiles) return;
-  const int2 rg = ranges[tile];
-  const int len = rg.y - rg.x;
-  {
-    // queue position: the tiles of all longer classes, then the rank in its own
-    const uint32_t rk = rank[tile];
-    const int cls = (int)(rk >> 28);
-    int x = lane < kBuckets && lane > cls ? bucket[lane] : 0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    if (lane == 0) {
-      tile_cnt[tile] = 0;
-      if (lazy) tile_cnt2[tile] = 0;
-      const int q = x + (int)(rk & 0x0fffffffu);
-      if (q < num_tiles)
-        order[q] = tile;
-      else
-        set_status(hdr, GS2D_ERR_BOUNDS);  // class sizes out of step with the ranks
+// Bitonic sort of `len` keys (at most kSmemKeys) at seg, by the block, in
+// shared memory padded to a power of two.
+__device__ __forceinline__ void block_sort(uint32_t* __restrict__ seg, int len,
+                                           uint32_t* s_keys) {
+  const int t = threadIdx.x;
+  int P = 64;
+  while (P < len) P <<= 1;
+  __syncthreads();
+  for (int i = t; i < P; i += kThreads) s_keys[i] = i < len ? seg[i] : 0xffffffffu;
+  __syncthreads();
+  for (int k = 2; k <= P; k <<= 1) {
+    for (int j = k >> 1; j > 0; j >>= 1) {
+      for (int x = t; x < P / 2; x += kThreads) {
+        // the x-th pair (i, i + j) of this distance
+        const int i = ((x & ~(j - 1)) << 1) | (x & (j - 1)), p = i | j;
+        const uint32_t u = s_keys[i], v = s_keys[p];
+        if ((u > v) == ((i & k) == 0)) {
+          s_keys[i] = v;
+          s_keys[p] = u;
+        }
+      }
+      __syncthreads();
     }
   }
-  uint32_t* seg = list + rg.x;
-  if (len <= 1) return;
-  if (len <= 32)
-    warp_sort_list<1>(seg, len, lane);
-  else if (len <= 64)
-    warp_sort_list<2>(seg, len, lane);
-  else if (len <= 128)
-    warp_sort_list<4>(seg, len, lane);
-  else if (len <= 256)
-    warp_sort_list<8>(seg, len, lane);
-  else if (len <= 512)
-    warp_sort_list<16>(seg, len, lane);
-  else if (lane == 0)
-    long_tiles[atomicAdd(&hdr->long_count, 1)] = tile;
+  for (int i = t; i < len; i += kThreads) seg[i] = s_keys[i];
+  __syncthreads();
 }
 
-// Segment sort, long lists: one CTA per queued tile, bitonic network in shared
-// memory over the list padded to a power of two.  A list longer than kLongMax
-// is reported as over capacity: its tile is emptied and the entry count is
-// zeroed so that no gradient is reduced from this binning.
-__global__ void __launch_bounds__(1024)
-k_sort_long(int2* __restrict__ ranges, uint32_t* __restrict__ list,
-            const int* __restrict__ long_tiles, int* __restrict__ bucket,
-            WsHeader* __restrict__ hdr, int lazy) {
+// Keys below v among the `len` ascending keys at seg.
+__device__ __forceinline__ int lower_count(const uint32_t* seg, int len, uint32_t v) {
+  int lo = 0, hi = len;
+  while (lo < hi) {
+    const int mid = (lo + hi) >> 1;
+    if (seg[mid] < v) lo = mid + 1; else hi = mid;
+  }
+  return lo;
+}
+
+// Sort of a list of up to kLongMax keys by the block: runs of kSmemKeys in
+// shared memory, then each key's place among the other runs by binary search
+// (the keys are distinct), through `spare`.
+__device__ __forceinline__ void block_sort_long(uint32_t* seg, int len, uint32_t* spare,
+                                                uint32_t* s_keys) {
+  for (int r = 0; r < len; r += kSmemKeys)
+    block_sort(seg + r, min(kSmemKeys, len - r), s_keys);
+  if (len <= kSmemKeys) return;
+  for (int i = threadIdx.x; i < len; i += kThreads) {
+    const uint32_t v = seg[i];
+    int at = i % kSmemKeys;
+    for (int r = 0; r < len; r += kSmemKeys)
+      if (r != i - i % kSmemKeys) at += lower_count(seg + r, min(kSmemKeys, len - r), v);
+    spare[at] = v;
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < len; i += kThreads) seg[i] = spare[i];
+  __syncthreads();
+}
+
+// Segment sort: one warp per tile for lists of up to 512 (bitonic network in
+// registers), the block for its longer ones, one after another; TPB tiles per
+// block (8, or 1 with few tiles, whose lists may all be long).  Also places
+// the tile in the render queue: after all tiles of longer classes, at the
+// next free position of its class.  A list longer than kLongMax is reported as
+// over capacity: its tile is emptied and the entry count is zeroed so that no
+// gradient is reduced from this binning.
+template <bool LAZY, int TPB>
+__global__ void __launch_bounds__(kThreads) k_sort(const __grid_constant__ BinArgs a) {
   pdl_begin();
-  extern __shared__ uint32_t s_keys[];
-  if (lazy && hdr->lists_valid) return;
-  const int t = threadIdx.x;
-  // the queue classes were last read by k_sort_short: clear them for the next binning
-  if (blockIdx.x == 0 && t < 2 * kBuckets) bucket[t] = 0;
-  const int count = hdr->long_count;
-  for (int q = blockIdx.x; q < count; q += gridDim.x) {
-    const int tile = long_tiles[q];
-    const int2 rg = ranges[tile];
-    const int len = rg.y - rg.x;
+  __shared__ uint32_t s_keys[kSmemKeys];
+  __shared__ int s_len[TPB];
+  if (LAZY && a.hdr->lists_valid) return;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int tile = blockIdx.x * TPB + wid;
+  if (wid < TPB) {
+    int len = 0;
+    if (tile < a.num_tiles) {
+      const int2 rg = a.ranges[tile];
+      len = rg.y - rg.x;
+      // queue position: the tiles of all longer classes, then the rank in its own
+      const uint32_t rk = a.rank[tile];
+      const int cls = (int)(rk >> 28);
+      int x = lane < kBuckets && lane > cls ? a.bucket[lane] : 0;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+      if (lane == 0) {
+        if (!a.one_scan) {  // (a one-block scan has cleared them)
+          a.tile_cnt[tile] = 0;
+          if (LAZY) a.tile_cnt2[tile] = 0;
+        }
+        const int q = x + (int)(rk & 0x0fffffffu);
+        if (q < a.num_tiles)
+          a.order[q] = tile;
+        else
+          set_status(a.hdr, GS2D_ERR_BOUNDS);  // class sizes out of step with the ranks
+      }
+      uint32_t* seg = a.list + rg.x;
+      if (len <= 1) {
+      } else if (len <= 32) {
+        warp_sort_list<1>(seg, len, lane);
+      } else if (len <= 64) {
+        warp_sort_list<2>(seg, len, lane);
+      } else if (len <= 128) {
+        warp_sort_list<4>(seg, len, lane);
+      } else if (len <= 256) {
+        warp_sort_list<8>(seg, len, lane);
+      } else if (len <= 512) {
+        warp_sort_list<16>(seg, len, lane);
+      }
+    }
+    if (lane == 0) s_len[wid] = len;
+  }
+  __syncthreads();
+#pragma unroll 1
+  for (int w = 0; w < TPB; w++) {
+    const int len = s_len[w], tl = blockIdx.x * TPB + w;
+    if (len <= 512) continue;
+    const int x = a.ranges[tl].x;
     if (len > kLongMax) {
-      if (t == 0) {
-        atomicCAS(&hdr->status, 0, (int)GS2D_ERR_CAPACITY);
-        hdr->n_entries = 0;
-        ranges[tile] = make_int2(rg.x, rg.x);
+      __syncthreads();  // every thread has read the range
+      if (threadIdx.x == 0) {
+        atomicCAS(&a.hdr->status, 0, (int)GS2D_ERR_CAPACITY);
+        a.hdr->n_entries = 0;
+        a.ranges[tl] = make_int2(x, x);
       }
       continue;
     }
-    int P = 64;
-    while (P < len) P <<= 1;
-    __syncthreads();
-    for (int i = t; i < P; i += blockDim.x) s_keys[i] = i < len ? list[rg.x + i] : 0xffffffffu;
-    __syncthreads();
-    for (int k = 2; k <= P; k <<= 1) {
-      for (int j = k >> 1; j > 0; j >>= 1) {
-        for (int i = t; i < P; i += blockDim.x) {
-          const int p = i ^ j;
-          if (p > i) {
-            const uint32_t a = s_keys[i], b = s_keys[p];
-            const bool asc = (i & k) == 0;
-            if ((a > b) == asc) {
-              s_keys[i] = b;
-              s_keys[p] = a;
-            }
-          }
-        }
-        __syncthreads();
-      }
-    }
-    for (int i = t; i < len; i += blockDim.x) list[rg.x + i] = s_keys[i];
+    block_sort_long(a.list + x, len, a.spare + x, s_keys);
   }
 }
 
 // ---------------------------------------------------------------------------
 // Every kernel of the chain starts with pdl_begin() and is launched with
 // launch_pdl: each one's blocks become resident while its predecessor drains.
+static BinArgs bin_args(const gs2d_plan& p, void* ws, const float* params) {
+  BinArgs a;
+  a.cs = clip_set(p, ws);
+  a.n = p.n;
+  a.num_tiles = p.num_tiles;
+  a.tile_shift = tile_shift_of(p.tile);
+  a.group = (p.n + kGroup - 1) / kGroup <= kManyGroups ? kGroup : kGroupLarge;
+  a.groups = (p.n + a.group - 1) / a.group;
+  a.one_scan = p.num_tiles <= kOneScan && a.groups <= kOneScan;
+  a.max_entries = p.max_entries;
+  a.sigma_cut = p.cfg.sigma_cut;
+  a.alpha_min = p.cfg.alpha_min;
+  a.det_eps = p.cfg.det_eps;
+  a.margin = p.cfg.bin_margin;
+  a.params = params;
+  a.rec = ws_ptr<float4>(ws, p, kOffRec);
+  a.rect = ws_ptr<int4>(ws, p, kOffRect);
+  a.lrect = ws_ptr<int4>(ws, p, kOffLRect);
+  a.offs = ws_ptr<int>(ws, p, kOffCount);
+  a.tile_cnt = ws_ptr<int>(ws, p, kOffTileCnt);
+  a.tile_cnt2 = ws_ptr<int>(ws, p, kOffTileCnt2);
+  a.sums = ws_ptr<long long>(ws, p, kOffBlockSum);
+  a.cursor = ws_ptr<int>(ws, p, kOffCursor);
+  a.ranges = ws_ptr<int2>(ws, p, kOffRanges);
+  a.bucket = ws_ptr<int>(ws, p, kOffBucket);
+  a.rank = ws_ptr<uint32_t>(ws, p, kOffRank);
+  a.order = ws_ptr<int>(ws, p, kOffOrder);
+  a.list = ws_ptr<uint32_t>(ws, p, kOffList);
+  a.spare = ws_ptr<uint32_t>(ws, p, kOffPartial);
+  a.hdr = ws_ptr<WsHeader>(ws, p, kOffHeader);
+  return a;
+}
+
+static AdamTick adam_tick(const gs2d_plan& p, bool on) {
+  return AdamTick{on ? 1 : 0, p.cfg.beta1, p.cfg.beta2, p.cfg.lr, p.cfg.lr_decay};
+}
+
 cudaError_t launch_project(const gs2d_plan& p, void* ws, const float* params, cudaStream_t s) {
   if (p.n == 0) return cudaSuccess;
-  return launch_pdl(k_project, (p.n + kGB - 1) / kGB, kGB, 0, s, p.n, clip_set(p, ws),
-                    tile_shift_of(p.tile), p.cfg.sigma_cut, p.cfg.alpha_min, p.cfg.det_eps,
-                    params, ws_ptr<float4>(ws, p, kOffRec), ws_ptr<int4>(ws, p, kOffRect),
-                    ws_ptr<int>(ws, p, kOffCount));
+  return launch_pdl(k_project, (p.n + kThreads - 1) / kThreads, kThreads, 0, s, p.n,
+                    clip_set(p, ws), tile_shift_of(p.tile), p.cfg.sigma_cut, p.cfg.alpha_min,
+                    p.cfg.det_eps, params, ws_ptr<float4>(ws, p, kOffRec),
+                    ws_ptr<int4>(ws, p, kOffRect));
 }
 
-cudaError_t prime_binning() {
-  return opt_in_smem((const void*)k_sort_long, kLongMax * (int)sizeof(uint32_t));
-}
-
-// Scans, scatter and segment sorts (everything after the counts); `lists`:
-// the rectangles the lists are built from; with `lazy` the tile part returns
-// at once while hdr->lists_valid is set.
-static cudaError_t launch_bin_rest(const gs2d_plan& p, void* ws, cudaStream_t s, int lazy) {
-  WsHeader* hdr = ws_ptr<WsHeader>(ws, p, kOffHeader);
-  int* count = ws_ptr<int>(ws, p, kOffCount);
-  int* tile_cnt = ws_ptr<int>(ws, p, kOffTileCnt);
-  int* cursor = ws_ptr<int>(ws, p, kOffCursor);
-  int* long_tiles = ws_ptr<int>(ws, p, kOffLong);
-  uint32_t* list = ws_ptr<uint32_t>(ws, p, kOffList);
-  int2* ranges = ws_ptr<int2>(ws, p, kOffRanges);
-  int* bucket = ws_ptr<int>(ws, p, kOffBucket);
-  int* order = ws_ptr<int>(ws, p, kOffOrder);
-  uint32_t* rank = ws_ptr<uint32_t>(ws, p, kOffRank);
-  int* tile_cnt2 = ws_ptr<int>(ws, p, kOffTileCnt2);
-  const int nbg = (p.n + kGB - 1) / kGB;
-  const int nbt = (p.num_tiles + kGB * kTileItems - 1) / (kGB * kTileItems);
-  cudaError_t e = prime_binning();
-  if (e == cudaSuccess)
-    e = launch_pdl(k_bin_scan, nbg + nbt, kGB, 0, s, p.n, nbg, p.num_tiles, p.max_entries, count,
-                   ws_ptr<long long>(ws, p, kOffBlockSum), tile_cnt, cursor, ranges, bucket,
-                   rank, hdr, lazy, (const int*)tile_cnt2);
-  if (e == cudaSuccess && p.n > 0)
-    e = launch_pdl(k_bin_scatter, nbg, kGB, 0, s, p.n, (const int4*)ws_ptr<int4>(ws, p, kOffRect),
-                   ws_ptr<int4>(ws, p, kOffLRect), hdr, cursor, list, lazy);
-  if (e == cudaSuccess)
-    e = launch_pdl(k_sort_short, (p.num_tiles + 7) / 8, 256, 0, s, p.num_tiles, ranges, list,
-                   long_tiles, tile_cnt, bucket, rank, order, hdr, lazy, tile_cnt2);
-  if (e == cudaSuccess)
-    e = launch_pdl(k_sort_long, 152, 1024, kLongMax * sizeof(uint32_t), s, ranges, list,
-                   long_tiles, bucket, hdr, lazy);
-  return e;
+// Counts, scans, scatter and segment sorts.  LAZY modes return at once while
+// hdr->lists_valid is set.
+template <CountMode MODE>
+static cudaError_t launch_bin(const BinArgs& a, AdamTick tick, cudaStream_t s) {
+  constexpr bool kLazy = MODE == kCountRebin;
+  const int blocks = std::max(1, a.groups);
+  // where the scan leaves the groups' first entries: in place, or behind the sums
+  long long* first = a.one_scan ? a.sums : a.sums + 2 * (size_t)a.groups;
+  cudaError_t e = launch_pdl(k_count<MODE>, blocks, kThreads, 0, s, a, tick);
+  if (e == cudaSuccess && !a.one_scan)
+    e = launch_pdl(k_bin_scan<kLazy>,
+                   1 + (a.num_tiles + kThreads * kTileItems - 1) / (kThreads * kTileItems),
+                   kThreads, 0, s, a, first);
+  if (e == cudaSuccess && a.n > 0)
+    e = launch_pdl(k_bin_scatter<kLazy>, blocks, kThreads, 0, s, a, (const long long*)first);
+  if (e != cudaSuccess) return e;
+  // few tiles: a block each (eight per block would leave most SMs idle)
+  if (a.num_tiles <= 152 * 4) return launch_pdl(k_sort<kLazy, 1>, a.num_tiles, kThreads, 0, s, a);
+  return launch_pdl(k_sort<kLazy, 8>, (a.num_tiles + 7) / 8, kThreads, 0, s, a);
 }
 
 cudaError_t launch_bin_sort(const gs2d_plan& p, void* ws, cudaStream_t s) {
-  cudaError_t e = cudaSuccess;
-  if (p.n > 0)
-    e = launch_pdl(k_count_tiles, (p.n + kGB - 1) / kGB, kGB, 0, s, p.n,
-                   ws_ptr<int4>(ws, p, kOffRect), ws_ptr<int>(ws, p, kOffCount),
-                   ws_ptr<int>(ws, p, kOffTileCnt), ws_ptr<long long>(ws, p, kOffBlockSum),
-                   ws_ptr<WsHeader>(ws, p, kOffHeader));
-  if (e != cudaSuccess) return e;
-  return launch_bin_rest(p, ws, s, 0);
+  return launch_bin<kCountRects>(bin_args(p, ws, nullptr), adam_tick(p, false), s);
 }
 
-cudaError_t launch_prepare(const gs2d_plan& p, void* ws, const float* params, bool adam_tick,
+cudaError_t launch_prepare(const gs2d_plan& p, void* ws, const float* params, bool tick,
                            cudaStream_t s) {
-  const int blocks = (p.n + kGB - 1) / kGB;
-  const cudaError_t e = launch_pdl(
-      k_project_count, blocks > 0 ? blocks : 1, kGB, 0, s, p.n, clip_set(p, ws),
-      tile_shift_of(p.tile), p.cfg.sigma_cut, p.cfg.alpha_min, p.cfg.det_eps, params,
-      ws_ptr<float4>(ws, p, kOffRec), ws_ptr<int4>(ws, p, kOffRect), ws_ptr<int>(ws, p, kOffCount),
-      ws_ptr<int>(ws, p, kOffTileCnt), ws_ptr<long long>(ws, p, kOffBlockSum),
-      ws_ptr<WsHeader>(ws, p, kOffHeader), adam_tick ? 1 : 0, p.cfg.beta1, p.cfg.beta2, p.cfg.lr,
-      p.cfg.lr_decay);
-  if (e != cudaSuccess) return e;
-  return launch_bin_rest(p, ws, s, 0);
+  return launch_bin<kCountProject>(bin_args(p, ws, params), adam_tick(p, tick), s);
 }
 
 cudaError_t launch_prepare_fit(const gs2d_plan& p, void* ws, const float* params,
                                cudaStream_t s) {
   if (!fit_lists_retained(p.cfg)) return launch_prepare(p, ws, params, true, s);
-  const int blocks = (p.n + kGB - 1) / kGB;
-  WsHeader* hdr = ws_ptr<WsHeader>(ws, p, kOffHeader);
-  int4* lrect = ws_ptr<int4>(ws, p, kOffLRect);
-  const ClipSet cs = clip_set(p, ws);
-  const int shift = tile_shift_of(p.tile);
-  cudaError_t e = launch_pdl(
-      k_project_fit, blocks > 0 ? blocks : 1, kGB, 0, s, p.n, cs, shift, p.cfg.sigma_cut,
-      p.cfg.alpha_min, p.cfg.det_eps, params, ws_ptr<float4>(ws, p, kOffRec),
-      ws_ptr<int4>(ws, p, kOffRect), ws_ptr<int>(ws, p, kOffCount),
-      ws_ptr<long long>(ws, p, kOffBlockSum), (const int4*)lrect, hdr, p.cfg.beta1, p.cfg.beta2,
-      p.cfg.lr, p.cfg.lr_decay);
-  if (e == cudaSuccess)
-    e = launch_pdl(k_rebin_count, blocks > 0 ? blocks : 1, kGB, 0, s, p.n, cs, shift,
-                   p.cfg.sigma_cut, p.cfg.alpha_min, p.cfg.det_eps, p.cfg.bin_margin, params,
-                   (const int4*)ws_ptr<int4>(ws, p, kOffRect), lrect,
-                   ws_ptr<int>(ws, p, kOffTileCnt), ws_ptr<int>(ws, p, kOffTileCnt2), hdr);
+  const BinArgs a = bin_args(p, ws, params);
+  const AdamTick tick = adam_tick(p, true);
+  const cudaError_t e = launch_pdl(k_project_fit, std::max(1, (p.n + 127) / 128), 128, 0, s, a,
+                                   tick);
   if (e != cudaSuccess) return e;
-  return launch_bin_rest(p, ws, s, 1);
+  return launch_bin<kCountRebin>(a, tick, s);
 }
 
 }  // namespace gs2d

@@ -24,16 +24,15 @@ enum WsSection {
   kOffClips,        // gs2d_clip[num_clips] (batch plans)
   kOffRec,          // float4[3][n]  render records (SoA of float4 rows)
   kOffRect,         // int4[n]       tile rectangle (first tile, row stride, w, h)
-  kOffCount,        // int32[n + 1]  per-Gaussian tile counts, then exclusive offsets
-  kOffBlockSum,     // int64[n / 32 + 1]  entry counts per block of Gaussians
+  kOffCount,        // int32[n + 1]  first backward slot of each Gaussian (listed rectangles)
+  kOffBlockSum,     // int64[3][n / 64 + 1]  entries per group of Gaussians, their offsets
   kOffTileCnt,      // int32[num_tiles]  entries per tile (zero between calls)
   kOffCursor,       // int32[num_tiles]  next free slot of each tile's list
-  kOffLong,         // int32[num_tiles + 1]  tiles whose list needs the CTA sort
   kOffList,         // uint32[max_entries]  Gaussian indices, tile-major
   kOffRanges,       // int2[num_tiles]
   kOffOrder,        // int32[num_tiles]  render queue: tiles, longest list first
   kOffRank,         // uint32[num_tiles]  (class << 28 | rank in class) of each tile
-  kOffBucket,       // int32[2][kBuckets]  queue class sizes (zero between calls)
+  kOffBucket,       // int32[2][kBuckets]  queue class sizes
   kOffPartial,      // float[max_entries][kPartials] backward sums per (tile, Gaussian)
   kOffLossPart,     // float2[num_tiles]  per-tile (sse, clamped sse) / (3 W H of the clip)
   kOffClipLoss,     // float2[num_clips]
@@ -41,7 +40,7 @@ enum WsSection {
   kOffActOrder,     // int32[num_tiles + 1] P-frame: active tiles (count last)
   kOffQuant,        // float[9 n] quantisation-aware fitting: the fake-quantised parameters
   kOffGrad,         // float[9 n] gradient scratch
-  kOffLRect,        // int4[n]  fit loop: the (widened) rectangle each Gaussian is listed in
+  kOffLRect,        // int4[n]  the rectangle each Gaussian is listed in (fit loop: widened)
   kOffTileCnt2,     // int32[num_tiles]  fit loop: tight-rectangle entries per tile (zero
                     //                   between calls; the fallback of a list rebuild)
   kOffAcc,          // float[n][kPartials]  GS2D_REDUCE_ATOMIC: per-Gaussian backward sums
@@ -56,7 +55,7 @@ struct WsHeader {
   int64_t entries_raw;  // total entries requested by the tile counts
   int32_t step;         // Adam step counter of the fit loop
   float bc1, bc2;       // Adam bias corrections for that step
-  int32_t long_count;   // tiles queued for the long-list sort
+  int32_t ticket;       // binning: blocks that have counted (zero between calls)
   float loss[2];        // last reduced {loss, clamped mse}
   unsigned long long pairs, hits;  // gs2d_count_pairs results
   double pw1, pw2;      // beta1^step, beta2^step
@@ -242,20 +241,17 @@ __device__ __forceinline__ void write_record(int i, int n, bool visible, float s
   rec[2 * n + i] = r2;
 }
 
-__device__ __forceinline__ void project_one(int i, int n, const gs2d_clip& cl, int tile_shift,
+// The record of Gaussian i; returns its rectangle.
+__device__ __forceinline__ int4 project_one(int i, int n, const gs2d_clip& cl, int tile_shift,
                                             float sigma_cut, float alpha_min, float det_eps,
                                             const float* __restrict__ params,
-                                            float4* __restrict__ rec, int4* __restrict__ rect,
-                                            int* __restrict__ count) {
+                                            float4* __restrict__ rec) {
   int tx0 = 0, ty0 = 0, tx1 = 0, ty1 = 0;
   const bool vis = gaussian_tiles(i, n, cl, tile_shift, sigma_cut, alpha_min, det_eps, params,
                                   0.0f, tx0, ty0, tx1, ty1);
-  const int4 rc = vis ? make_int4(cl.tile_off + ty0 * cl.tiles_x + tx0, cl.tiles_x, tx1 - tx0,
-                                  ty1 - ty0)
-                      : make_int4(0, 0, 0, 0);
-  rect[i] = rc;
-  count[i] = rc.z * rc.w;
   write_record(i, n, vis, sigma_cut, alpha_min, params, rec);
+  return vis ? make_int4(cl.tile_off + ty0 * cl.tiles_x + tx0, cl.tiles_x, tx1 - tx0, ty1 - ty0)
+             : make_int4(0, 0, 0, 0);
 }
 
 __host__ __device__ inline int tile_shift_of(int tile) {
@@ -280,8 +276,8 @@ struct RenderArgs {
   const int2* ranges;
   const uint32_t* list;
   const float4* rec;
-  const int4* rect;
-  const int* offs;
+  const int4* lrect;     // the rectangles the lists are built from
+  const int* offs;       // first backward slot of each Gaussian (of its listed rectangle)
   const int* order;
   WsHeader* hdr;
   float* img;            // fwd, l2 (optional)
@@ -309,9 +305,7 @@ cudaError_t launch_render_t32(int stage, int launch, RenderMode mode, const Rend
 cudaError_t prime_render_t8(int stage, int launch);
 cudaError_t prime_render_t16(int stage, int launch);
 cudaError_t prime_render_t32(int stage, int launch);
-// One-time per-device setup of the binning launches (shared-memory opt-in).
-cudaError_t prime_binning();
-// prime_binning + the render occupancy query of the plan's fit loop.
+// The render occupancy query of the plan's fit loop.
 cudaError_t prime_fit_launches(const gs2d_plan& p);
 
 // Opt-in to `bytes` of dynamic shared memory for `kernel` on the current

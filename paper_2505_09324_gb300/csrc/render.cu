@@ -35,22 +35,49 @@ __device__ __forceinline__ void chain_grads(const float* __restrict__ params, in
   gr[8] = fmaf(cr, a[0], fmaf(cg, a[1], cb * a[2]));
 }
 
-// kRL lanes share one Gaussian: lane `sub` sums slots s0 + sub, s0 + sub + kRL,
-// ..., then the group adds its kRL partial sums (a fixed order: deterministic).
+// kRL lanes share one Gaussian: lane `sub` sums the records of its tiles sub,
+// sub + kRL, ... in the raster order of its tight rectangle, then the group
+// adds its kRL partial sums (a fixed order: deterministic).  The records lie
+// at the slots of the listed rectangle, which holds the tight one (the fit
+// loop lists widened rectangles).
 constexpr int kRL = 4;
 
-__device__ __forceinline__ bool gather_partials(const float4* __restrict__ partial,
-                                                const int* __restrict__ offs, int i, bool valid,
-                                                int sub, float a[kPartials]) {
-  int s0 = 0, s1 = 0;
+struct SlotArgs {
+  const float4* partial;
+  const int* offs;
+  const int4* rect;
+  const int4* lrect;
+};
+
+__device__ __forceinline__ bool gather_partials(const SlotArgs& g, int i, bool valid, int sub,
+                                                float a[kPartials]) {
+  int4 rc = make_int4(0, 0, 0, 0);
+  int first = 0, lw = 0;
   if (valid) {
-    s0 = offs[i];
-    s1 = offs[i + 1];
+    rc = g.rect[i];
+    const int4 lr = g.lrect[i];
+    lw = lr.z;
+    if (rc.z > 0) {
+      // column and row of the tight one inside the listed one; outside it (a
+      // projection that was not binned) there are no records
+      const int rel = rc.x - lr.x;
+      const int dy = rel / rc.y, dx = rel - dy * rc.y;
+      if (rel >= 0 && dx + rc.z <= lw && dy + rc.w <= lr.w)
+        first = g.offs[i] + dy * lw + dx;
+      else
+        rc.z = 0;
+    }
   }
 #pragma unroll
   for (int k = 0; k < kPartials; k++) a[k] = 0.0f;
-  for (int sl = s0 + sub; sl < s1; sl += kRL) {
-    const float4 p = partial[2 * sl], q = partial[2 * sl + 1];
+  int dx = sub, dy = 0;
+  for (int j = sub; j < rc.z * rc.w; j += kRL, dx += kRL) {
+    while (dx >= rc.z) {
+      dx -= rc.z;
+      dy++;
+    }
+    const int sl = first + dy * lw + dx;
+    const float4 p = g.partial[2 * sl], q = g.partial[2 * sl + 1];
     a[0] += p.x;
     a[1] += p.y;
     a[2] += p.z;
@@ -64,14 +91,14 @@ __device__ __forceinline__ bool gather_partials(const float4* __restrict__ parti
   for (int o = 1; o < kRL; o <<= 1)
 #pragma unroll
     for (int k = 0; k < kPartials; k++) a[k] += __shfl_xor_sync(0xffffffffu, a[k], o);
-  return s1 > s0;
+  return rc.z > 0;
 }
 
 // GS2D_REDUCE_ATOMIC: the render added the Gaussian's sums up itself; every
 // lane of the group reads them, then lane 0 clears them for the next pass.
 // `any`: the Gaussian had a (tile, Gaussian) pair.  Every lane of the warp
 // must take part.
-__device__ __forceinline__ bool gather_acc(float* __restrict__ acc, const int* __restrict__ offs,
+__device__ __forceinline__ bool gather_acc(float* __restrict__ acc, const int4* __restrict__ rect,
                                            int i, bool valid, int sub, float a[kPartials]) {
   bool any = false;
 #pragma unroll
@@ -87,7 +114,7 @@ __device__ __forceinline__ bool gather_acc(float* __restrict__ acc, const int* _
     a[5] = y.y;
     a[6] = y.z;
     a[7] = y.w;
-    any = offs[i + 1] > offs[i];
+    any = rect[i].z > 0;
   }
   __syncwarp();  // every lane of the group has read the sums
   if (valid && sub == 0) q[0] = q[1] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -95,16 +122,16 @@ __device__ __forceinline__ bool gather_acc(float* __restrict__ acc, const int* _
 }
 
 __global__ void __launch_bounds__(256)
-k_reduce_chain(int n, const float* __restrict__ params, const int* __restrict__ offs,
-               const float4* __restrict__ partial, const WsHeader* __restrict__ hdr,
-               float* __restrict__ grads, float* __restrict__ acc) {
+k_reduce_chain(int n, const float* __restrict__ params, SlotArgs slots,
+               const WsHeader* __restrict__ hdr, float* __restrict__ grads,
+               float* __restrict__ acc) {
   pdl_begin();
   const int gt = blockIdx.x * blockDim.x + threadIdx.x;
   const int i = gt / kRL, sub = gt % kRL;
   const bool valid = i < n && hdr->entries_raw == (int64_t)hdr->n_entries;
   float a[kPartials], gr[9];
-  const bool any = acc ? gather_acc(acc, offs, i, valid, sub, a)
-                       : gather_partials(partial, offs, i, valid, sub, a);
+  const bool any = acc ? gather_acc(acc, slots.rect, i, valid, sub, a)
+                       : gather_partials(slots, i, valid, sub, a);
   if (i >= n) return;
   if (any) chain_grads(params, n, i, a, gr);
 #pragma unroll
@@ -116,8 +143,8 @@ k_reduce_chain(int n, const float* __restrict__ params, const int* __restrict__ 
 // view of pinned host memory, or NULL): every Gaussian's parameters after
 // the step are also stored there, so that no separate download is needed.
 __global__ void __launch_bounds__(256)
-k_reduce_chain_adam(int n, float* __restrict__ params, const int* __restrict__ offs,
-                    const float4* __restrict__ partial, const WsHeader* __restrict__ hdr,
+k_reduce_chain_adam(int n, float* __restrict__ params, SlotArgs slots,
+                    const WsHeader* __restrict__ hdr,
                     float* __restrict__ m, float* __restrict__ v, float4 lr_rows, float b1,
                     float b2, float eps, const uint8_t* __restrict__ select,
                     const float* __restrict__ params_eval, WsHeader* hdr_w,
@@ -133,8 +160,8 @@ k_reduce_chain_adam(int n, float* __restrict__ params, const int* __restrict__ o
   float a[kPartials], gr[9];
   // (atomic sums are read and cleared for every Gaussian: an unselected one
   // of a rendered tile has sums too)
-  const bool any = acc ? gather_acc(acc, offs, i, i < n && ok, sub, a) && on
-                       : gather_partials(partial, offs, i, on && ok, sub, a);
+  const bool any = acc ? gather_acc(acc, slots.rect, i, i < n && ok, sub, a) && on
+                       : gather_partials(slots, i, on && ok, sub, a);
   // (ok is the same for every thread of the grid)
   const bool act = on && ok;
   // the chain rule at the parameters that were rendered (the fake-quantised
@@ -294,7 +321,7 @@ static RenderArgs render_args(const gs2d_plan& p, void* ws) {
   a.ranges = ws_ptr<int2>(ws, p, kOffRanges);
   a.list = ws_ptr<uint32_t>(ws, p, kOffList);
   a.rec = ws_ptr<float4>(ws, p, kOffRec);
-  a.rect = ws_ptr<int4>(ws, p, kOffRect);
+  a.lrect = ws_ptr<int4>(ws, p, kOffLRect);
   a.offs = ws_ptr<int>(ws, p, kOffCount);
   a.order = ws_ptr<int>(ws, p, kOffOrder);
   a.hdr = ws_ptr<WsHeader>(ws, p, kOffHeader);
@@ -312,6 +339,12 @@ static RenderArgs render_args(const gs2d_plan& p, void* ws) {
   return a;
 }
 
+static SlotArgs slot_args(const gs2d_plan& p, void* ws) {
+  return SlotArgs{reinterpret_cast<const float4*>(ws_ptr<float>(ws, p, kOffPartial)),
+                  ws_ptr<int>(ws, p, kOffCount), ws_ptr<int4>(ws, p, kOffRect),
+                  ws_ptr<int4>(ws, p, kOffLRect)};
+}
+
 static cudaError_t launch_render(const gs2d_plan& p, RenderMode mode, const RenderArgs& a,
                                  cudaStream_t s) {
   switch (p.tile) {
@@ -326,8 +359,7 @@ static cudaError_t launch_reduce(const gs2d_plan& p, void* ws, const float* para
                                  cudaStream_t s) {
   if (p.n == 0) return cudaSuccess;
   return launch_pdl(k_reduce_chain, (p.n * kRL + 255) / 256, 256, 0, s, p.n, params,
-                    ws_ptr<int>(ws, p, kOffCount),
-                    reinterpret_cast<const float4*>(ws_ptr<float>(ws, p, kOffPartial)),
+                    slot_args(p, ws),
                     ws_ptr<WsHeader>(ws, p, kOffHeader), grads, atomic_sums(p, ws));
 }
 
@@ -386,8 +418,7 @@ cudaError_t launch_fit_step(const gs2d_plan& p, void* ws, const float* target, f
   if (e != cudaSuccess || p.n == 0) return e;
   WsHeader* hdr = ws_ptr<WsHeader>(ws, p, kOffHeader);
   return launch_pdl(k_reduce_chain_adam, (p.n * kRL + 255) / 256, 256, 0, s, p.n, params,
-                    ws_ptr<int>(ws, p, kOffCount),
-                    reinterpret_cast<const float4*>(ws_ptr<float>(ws, p, kOffPartial)),
+                    slot_args(p, ws),
                     (const WsHeader*)hdr, m, v, lr_rows(p.cfg), p.cfg.beta1, p.cfg.beta2,
                     p.cfg.eps, (const uint8_t*)nullptr, params_eval,
                     fit_lists_retained(p.cfg) ? hdr : (WsHeader*)nullptr, atomic_sums(p, ws),
@@ -479,19 +510,16 @@ cudaError_t launch_pframe_step(const gs2d_plan& p, void* ws, const float* target
   e = launch_render(p, kModeL2, a, s);
   if (e != cudaSuccess) return e;
   return launch_pdl(k_reduce_chain_adam, (p.n * kRL + 255) / 256, 256, 0, s, p.n, params,
-                    ws_ptr<int>(ws, p, kOffCount),
-                    reinterpret_cast<const float4*>(ws_ptr<float>(ws, p, kOffPartial)),
+                    slot_args(p, ws),
                     ws_ptr<WsHeader>(ws, p, kOffHeader), m, v, lr_rows(p.cfg), p.cfg.beta1,
                     p.cfg.beta2, p.cfg.eps, select, (const float*)nullptr, (WsHeader*)nullptr,
                     atomic_sums(p, ws), (float*)nullptr);
 }
 
-// Runs the one-time per-device queries of the fit loop's launches (occupancy
-// of the persistent render, shared-memory opt-in of the long-list sort) so that
-// a following stream capture records launches only.
+// Runs the one-time per-device query of the fit loop's launches (occupancy of
+// the persistent render) so that a following stream capture records launches
+// only.
 cudaError_t prime_fit_launches(const gs2d_plan& p) {
-  cudaError_t e = prime_binning();
-  if (e != cudaSuccess) return e;
   switch (p.tile) {
     case 8: return prime_render_t8(p.stage, p.cfg.launch);
     case 16: return prime_render_t16(p.stage, p.cfg.launch);

@@ -116,7 +116,7 @@ __device__ __forceinline__ void stage_batch(TileSmem<S>& sm, const RenderArgs& a
   for (int k = threadIdx.x; k < cnt; k += G::NT) {
     const int g = (int)a.list[b + k];
     const float4 r0 = a.rec[g], r1 = a.rec[a.n + g], r2 = a.rec[2 * a.n + g];
-    const int4 rc = a.rect[g];
+    const int4 rc = a.lrect[g];
     const int off = a.offs[g];
     const float ox = (float)f.ox, oy = (float)f.oy;
     // pixel lx contributes only if |ox + lx + 0.5 - mu_x| <= hx
@@ -126,20 +126,9 @@ __device__ __forceinline__ void stage_batch(TileSmem<S>& sm, const RenderArgs& a
     fy0 = fmaxf(fy0, 0.0f);
     fx1 = fminf(fx1, fminf((float)(T - 1), (float)(f.W - 1) - ox));
     fy1 = fminf(fy1, fminf((float)(T - 1), (float)(f.H - 1) - oy));
-    // slot: position of this tile inside the Gaussian's (tight) rectangle.
-    // Lists kept across fit iterations may hold Gaussians whose rectangle no
-    // longer covers the tile: such a pair is empty and has no slot (-1).
-    int dx = -1, dy = -1;
-    if (rc.z > 0) {
-      const int first = rc.x - (f.tile - f.ty * rc.y - f.tx);  // y0 * stride + x0 in the clip
-      const int y0 = first / rc.y;
-      dx = f.tx - (first - y0 * rc.y);
-      dy = f.ty - y0;
-    }
-    const bool covered = (unsigned)dx < (unsigned)rc.z && (unsigned)dy < (unsigned)rc.w;
     int4 bb = make_int4(1, 0, 1, 0);
     uint32_t wm = 0;
-    if (covered && fx0 <= fx1 && fy0 <= fy1) {
+    if (fx0 <= fx1 && fy0 <= fy1) {
       bb = make_int4((int)fx0, (int)fx1, (int)fy0, (int)fy1);
       const int w0 = bb.z / G::RW, w1 = bb.w / G::RW;
       wm = ((2u << w1) - 1u) & ~((1u << w0) - 1u);
@@ -149,7 +138,9 @@ __device__ __forceinline__ void stage_batch(TileSmem<S>& sm, const RenderArgs& a
     sm.my[k] = r0.y - oy;
     sm.bb[k] = bb;
     sm.wmask[k] = wm;
-    sm.slot[k] = covered ? off + dy * rc.z + dx : -1;
+    // position of this tile inside the Gaussian's listed rectangle
+    const int rel = f.tile - rc.x, row = rel / rc.y;
+    sm.slot[k] = off + row * rc.z + (rel - row * rc.y);
   }
 }
 
@@ -243,7 +234,7 @@ __device__ __forceinline__ void bwd_batch(TileSmem<S>& sm, const float4* __restr
     // Gaussians whose box misses the tile: a zero record, no reduction
     const bool empty = gi >= cnt || sm.bb[gi].x > sm.bb[gi].y;
     if (__all_sync(0xffffffffu, empty)) {
-      if (!a.acc && gi < cnt && j < 8 && sm.slot[gi] >= 0) partial[8 * sm.slot[gi] + j] = 0.0f;
+      if (!a.acc && gi < cnt && j < 8) partial[8 * sm.slot[gi] + j] = 0.0f;
       continue;
     }
     float v[8];
@@ -296,7 +287,7 @@ __device__ __forceinline__ void bwd_batch(TileSmem<S>& sm, const float4* __restr
       }
     }
     const float tot = group_transpose_sum<T>(v, j);
-    if (gi < cnt && (j % G::Q) == 0 && sm.slot[gi] >= 0) {
+    if (gi < cnt && (j % G::Q) == 0) {
       if (!a.acc)
         partial[8 * sm.slot[gi] + j / G::Q] = tot;
       else if (sm.bb[gi].x <= sm.bb[gi].y)

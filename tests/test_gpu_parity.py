@@ -408,3 +408,59 @@ def test_device_driven_loop_equals_host_driven_loop(gs, mode, check_every):
         assert od["iters"] <= 3 * check_every and od["psnr"] >= goal
     else:
         assert od["iters"] == iters and len(od["trace"]) == -(-iters // check_every)
+
+
+def _piled(n, W, H, seed, at, share):
+    """Random Gaussians, `share` of them within a pixel of `at`."""
+    p = random_gaussians(n, W, H, seed=seed, l_range=(0.5, 2.0))
+    k = int(share * n)
+    p[0, :k], p[1, :k] = at[0] + 0.5 * (p[0, :k] / W), at[1] + 0.5 * (p[1, :k] / H)
+    p[2:5, :k] *= 0.05
+    return np.ascontiguousarray(p)
+
+
+@pytest.mark.parametrize("n,W,H,share", [
+    (513, 16, 16, 1.0), (700, 64, 48, 0.8), (8192, 64, 48, 1.0), (8193, 64, 48, 1.0),
+    (17000, 64, 48, 0.97), (32768, 64, 48, 1.0), (3000, 640, 360, 0.9),
+    (400, 512, 1024, 0.0), (400, 512, 1025, 0.0), (131073, 300, 200, 0.0),
+    (524353, 300, 200, 0.0), (63, 40, 40, 0.0), (65, 40, 40, 0.0)])
+def test_bins_bit_exact_at_the_edges_of_the_sort(gs, oracle, n, W, H, share):
+    """Lists just over a warp's 512 keys, at and over the 8192 keys of a
+    shared-memory run, of several runs and at the longest; many long lists in
+    one block; tile counts and Gaussian counts on both sides of the one-block
+    scan; groups of 64 Gaussians nearly full and just over."""
+    p = _piled(n, W, H, n, (W / 2 - 3.3, H / 2 - 3.3), share)
+    r = check_bins(gs, oracle, p, W, H, max_entries=1 << 24)
+    assert r.status() == 0
+    check_bins(gs, oracle, p, W, H, max_entries=1 << 24, separate=True)
+    # binning the same workspace again, and other Gaussians after them
+    q = random_gaussians(n, W, H, seed=n + 1, l_range=(0.5, 2.0))
+    first = r.read_bins()["values"].copy()
+    r.prepare(to_dev(q))
+    r.prepare(to_dev(p))
+    np.testing.assert_array_equal(r.read_bins()["values"], first)
+
+
+def test_fit_on_large_plans_equals_per_iteration_binning(gs):
+    """Retained lists against per-iteration binning beyond the one-block scan
+    (many tiles), where the scan has a launch of its own."""
+    from paper_2505_09324_gb300 import _native as nat
+    W, H, n = 640, 600, 1500
+    p0 = random_gaussians(n, W, H, seed=3)
+    t = to_dev(smooth_noise_target(W, H, seed=4))
+    s = int(torch.cuda.current_stream().cuda_stream)
+    outs = []
+    for margin in (-1.0, 4.0):
+        r = gs.GaussianRasterizer(W, H, n, config=gs.RasterConfig.fast_fit(tile=8,
+                                                                           bin_margin=margin))
+        assert r.plan.num_tiles > 2048
+        p = to_dev(p0)
+        m, v = torch.empty_like(p), torch.empty_like(p)
+        nat.fit_reset(r.plan, r.ws_ptr, m.data_ptr(), v.data_ptr(), s)
+        for _ in range(6):
+            nat.fit_step(r.plan, r.ws_ptr, t.data_ptr(), p.data_ptr(), m.data_ptr(), v.data_ptr(),
+                         s)
+        assert r.status() == 0
+        outs.append((p, m, v))
+    for a, b in zip(*outs):
+        assert torch.equal(a, b)
