@@ -699,6 +699,20 @@ gs2d_status gs2d_col2im(const float* dcol, int32_t ldk, int32_t B, int32_t Hi, i
                         int32_t C, int32_t ks, int32_t stride, int32_t pad, const void* act,
                         void* dx, void* stream);
 
+/* Input gradient of a 3 x 3 convolution with stride 2 and padding 1, in one
+ * pass: dx[b][iy][ix][ci] = (act > 0) * the sum over the taps (ky, kx) that
+ * read (iy, ix) and over n < N of dz[b][oy][ox][n] * Wt[(3 ky + kx) C + ci][n]
+ * (FP32 accumulation, one BF16 rounding): gs2d_col2im of the FP32 product of
+ * dz and Wt without that product in memory.  dz: device BF16
+ * [B][Ho][Wo][N], Ho = (Hi + 1) / 2, Wo = (Wi + 1) / 2; Wt: device BF16
+ * [>= 9 C][N] (gs2d_cast_weights' transpose); act: device BF16 [B][Hi][Wi][C]
+ * (the ReLU output the convolution read) or NULL; dx: device BF16, shape of
+ * act.  C and N multiples of 8, all 16-byte aligned.  status as
+ * gs2d_gemm_bf16. */
+gs2d_status gs2d_conv_dgrad_bf16(const void* dz, int32_t B, int32_t Hi, int32_t Wi, int32_t C,
+                                 const void* Wt, int32_t N, const void* act, void* dx,
+                                 int32_t* status, void* stream);
+
 /* out[c][r] = in[r][c] for a BF16 R x C matrix (device; leading dimensions
  * ld_in >= C, ld_out >= R). */
 gs2d_status gs2d_transpose_bf16(const void* in, int32_t R, int32_t C, int32_t ld_in, void* out,

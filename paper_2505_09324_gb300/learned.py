@@ -15,8 +15,9 @@ reads its operands straight from the activations (gs2d_conv_bf16,
 gs2d_conv_frame_bf16; the same sums in the same order as gs2d_gemm_bf16 on
 the operand); training also writes the operand out for the backward pass.  The backward pass is one
 weight-gradient GEMM (dZ^T . col, both read as they lie, split over pixels;
-gs2d_gemm_tn_bf16) and one input-gradient
-GEMM (dZ . W) + col2im with the ReLU mask per layer.  The optimiser is the
+gs2d_gemm_tn_bf16) and one input gradient with the ReLU mask per layer: one
+implicit GEMM over shifted dZ boxes where rows are wide
+(gs2d_conv_dgrad_bf16), else a GEMM (dZ . W) + col2im.  The optimiser is the
 library's Adam on the FP32 master weights.  Training minimises the L2 render
 loss of the decoded Gaussians through the rasterizer (the colour and shape
 signal the paper's regressor lacked) plus lambda times the Chamfer distance
@@ -107,7 +108,8 @@ class LearnedInitializer:
             P = B * h * w
             self.col.append(torch.empty((P, ldk), dtype=bf, device=dev))
             self.dz.append(torch.empty((P, co), dtype=bf, device=dev))
-            self.dcol.append(torch.empty((P, ldk), device=dev) if li > 0 else None)
+            self.dcol.append(torch.empty((P, ldk), device=dev)
+                             if li > 0 and not self._implicit_dgrad(li) else None)
             if li < self.L:
                 self.x.append(torch.empty((P, co), dtype=bf, device=dev))
         self.out = torch.empty((B * self.gh * self.gw, self.ldo), device=dev)
@@ -121,6 +123,12 @@ class LearnedInitializer:
             most = max(most, nat.load().gs2d_gemm_tn_partial_bytes(co, ldk, ldk, P,
                                                                     self._splits(P)))
         self.partial = torch.empty(max(most // 4, 1), device=dev)
+
+    def _implicit_dgrad(self, li: int) -> bool:
+        """Whether layer li's input gradient runs as gs2d_conv_dgrad_bf16: the
+        3 x 3 layers whose output rows fill at least half of its 128-pixel
+        tiles; below that the GEMM and the gather after it are faster."""
+        return self.layers[li][2] == 3 and self.sizes[li + 1][1] >= 64
 
     def _splits(self, pixels: int) -> int:
         return max(1, min(512, pixels // self.cfg.wgrad_split_pixels))
@@ -241,11 +249,16 @@ class LearnedInitializer:
                      self.partial.data_ptr(), st, s)
             if li == 0:
                 break
-            # input gradient: dcol[p][k] = sum_co dZ[p][co] W[co][k], then the
-            # taps back onto the input, times the ReLU mask of that input
+            hi, wi = self.sizes[li] if li < self.L else self.sizes[-1]
+            # input gradient, times the ReLU mask of that input
+            if self._implicit_dgrad(li):
+                nat.call("gs2d_conv_dgrad_bf16", self.dz[li].data_ptr(), B, hi, wi, ci,
+                         self.wt[li].data_ptr(), co, self.x[li].data_ptr(),
+                         self.dz[li - 1].data_ptr(), st, s)
+                continue
+            # dcol[p][k] = sum_co dZ[p][co] W[co][k], then the taps back onto the input
             nat.gemm_bf16(self.dz[li].data_ptr(), co, self.wt[li].data_ptr(), co, P, ldk, co, 0,
                           False, self.dcol[li].data_ptr(), 0, ldk, 1, 0, st, s)
-            hi, wi = self.sizes[li] if li < self.L else self.sizes[-1]
             stride, pad = (2, 1) if ks == 3 else (1, 0)
             nat.call("gs2d_col2im", self.dcol[li].data_ptr(), ldk, B, hi, wi, ci, ks, stride,
                      pad, self.x[li].data_ptr(), self.dz[li - 1].data_ptr(), s)

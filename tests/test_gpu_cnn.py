@@ -552,3 +552,32 @@ def test_chamfer_nearest_neighbours(nat, name):
     assert not got[2:].any()
     if np.isfinite(loss):
         assert abs(float(dl[0]) - loss) <= 1e-5 * loss
+
+
+@pytest.mark.parametrize("B,H,W,C,N", [
+    (2, 6, 20, 32, 64), (1, 7, 21, 64, 128), (1, 5, 515, 32, 64), (1, 3, 256, 64, 40),
+    (1, 9, 300, 128, 192), (1, 4, 30, 200, 72), (3, 1, 1, 8, 8), (1, 2, 258, 24, 256),
+    (40, 9, 140, 32, 64)])
+def test_conv_input_gradient_by_definition(nat, B, H, W, C, N):
+    """gs2d_conv_dgrad_bf16 (3 x 3, stride 2, pad 1): odd and even sizes, one
+    and several column segments, partial channel blocks and chunks, resident
+    and streamed weights, several blocks of channels, more tiles than CTAs;
+    with and without the ReLU mask.  FP32 sums (the GEMM bar), one BF16
+    rounding."""
+    g = np.random.Generator(np.random.PCG64(H * W + C + N))
+    Ho, Wo, ldk = (H + 1) // 2, (W + 1) // 2, -(-(9 * C + 1) // 8) * 8
+    dz = cnn.bf16_round(g.normal(size=(B * Ho * Wo, N)))
+    w = cnn.bf16_round(g.normal(size=(N, ldk)) * 0.1)
+    act = cnn.bf16_round(g.normal(size=(B, H, W, C)))
+    d_dz, d_wt, d_act = bf16_dev(dz), bf16_dev(np.ascontiguousarray(w.T)), bf16_dev(act)
+    want = cnn.col2im(dz @ w, act.shape, 3, 2, 1)
+    scale = cnn.col2im(np.abs(dz) @ np.abs(w), act.shape, 3, 2, 1)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    for mask in (False, True):
+        out = torch.full(act.shape, 7.0, dtype=torch.bfloat16, device="cuda")
+        nat.call("gs2d_conv_dgrad_bf16", d_dz.data_ptr(), B, H, W, C, d_wt.data_ptr(), N,
+                 d_act.data_ptr() if mask else 0, out.data_ptr(), status.data_ptr(), 0)
+        ref = want * (act > 0) if mask else want
+        tol = REL * scale + np.abs(ref) * 2.0 ** -8
+        assert np.all(np.abs(to_np_bf16(out) - ref) <= tol + 1e-30)
+        assert int(status.item()) == 0
