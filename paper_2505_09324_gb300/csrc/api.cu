@@ -337,9 +337,11 @@ gs2d_status gs2d_roi_init_trace(const float* frame, const uint8_t* mask, int32_t
 }
 
 static cudaError_t fit_iteration(const gs2d_plan& p, void* ws, const float* target, float* params,
-                                 float* m, float* v, cudaStream_t s) {
+                                 float* m, float* v, cudaStream_t s,
+                                 const LoopArgs* loop = nullptr) {
   cudaError_t e = launch_prepare_fit(p, ws, params, s);
-  if (e == cudaSuccess) e = launch_fit_step(p, ws, target, params, m, v, s);
+  if (e == cudaSuccess)
+    e = launch_fit_step(p, ws, target, params, m, v, s, nullptr, nullptr, loop);
   return e;
 }
 
@@ -539,64 +541,10 @@ gs2d_status gs2d_fit_rebins(const gs2d_plan* plan, const void* ws, int64_t* rebi
   return ok();
 }
 
-// Device-driven fit loop: the body of a conditional WHILE graph node is one
-// fit iteration followed by this kernel.  It counts the iteration; every
-// check_every iterations (and at the last) it sums the render's per-tile loss
-// partials, writes the PSNR of the clamped image to the trace and clears the
-// loop condition once the target is met, the cap is reached or a kernel has
-// recorded an error.  The host reads the header and the trace once, at the
-// end.
-struct LoopArgs {
-  int num_tiles, iters, check_every;
-  float target_psnr;
-  const float2* loss_part;
-  WsHeader* hdr;
-  float* trace;  // device, one float per check
-  cudaGraphConditionalHandle handle;
-};
-
-__global__ void __launch_bounds__(1024) k_loop_control(LoopArgs a) {
-  pdl_begin();
-  __shared__ int s_it;
-  __shared__ double s_a[32], s_b[32];
-  if (threadIdx.x == 0) s_it = ++a.hdr->loop_iter;
-  __syncthreads();
-  const int it = s_it;
-  if (it % a.check_every != 0 && it < a.iters) return;
-  double x = 0.0, y = 0.0;
-  for (int t = threadIdx.x; t < a.num_tiles; t += blockDim.x) {
-    x += a.loss_part[t].x;
-    y += a.loss_part[t].y;
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    x += __shfl_xor_sync(0xffffffffu, x, o);
-    y += __shfl_xor_sync(0xffffffffu, y, o);
-  }
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (lane == 0) {
-    s_a[wid] = x;
-    s_b[wid] = y;
-  }
-  __syncthreads();
-  if (threadIdx.x != 0) return;
-  double sa = 0.0, sb = 0.0;
-  for (int w = 0; w < (int)(blockDim.x >> 5); w++) {
-    sa += s_a[w];
-    sb += s_b[w];
-  }
-  a.hdr->loss[0] = (float)sa;
-  a.hdr->loss[1] = (float)sb;
-  const double mse = (double)a.hdr->loss[1];
-  const float psnr = mse > 0.0 ? (float)(10.0 * log10(1.0 / mse)) : INFINITY;
-  a.trace[a.hdr->loop_checks++] = psnr;
-  const bool stop = it >= a.iters || a.hdr->status != 0 ||
-                    (a.target_psnr > 0.0f && psnr >= a.target_psnr);
-  if (stop) cudaGraphSetConditional(a.handle, 0u);
-}
-
 // The whole fit loop as one executable graph: a WHILE node whose body is one
-// fit iteration and k_loop_control; NULL when the stream cannot be captured,
+// fit iteration, whose last kernel also controls the loop (LoopArgs): it
+// counts the iteration, takes the PSNR checks and ends the loop, and the host
+// reads the header and the trace once, at the end.  NULL when the stream cannot be captured,
 // the trace does not fit the gradient scratch or the driver declines the
 // graph (the caller then drives the loop from the host).
 static cudaGraphExec_t capture_fit_loop(const gs2d_plan& p, void* ws, const float* target,
@@ -628,19 +576,16 @@ static cudaGraphExec_t capture_fit_loop(const gs2d_plan& p, void* ws, const floa
     e = cudaStreamBeginCaptureToGraph(s, body, nullptr, nullptr, 0,
                                       cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-      cudaError_t ce = fit_iteration(p, ws, target, params, m, v, s);
-      if (ce == cudaSuccess) {
-        LoopArgs la;
-        la.num_tiles = p.num_tiles;
-        la.iters = iters;
-        la.check_every = check_every;
-        la.target_psnr = target_psnr;
-        la.loss_part = ws_ptr<float2>(ws, p, kOffLossPart);
-        la.hdr = ws_ptr<WsHeader>(ws, p, kOffHeader);
-        la.trace = ws_ptr<float>(ws, p, kOffGrad);
-        la.handle = handle;
-        ce = launch_pdl(k_loop_control, 1, 1024, 0, s, la);
-      }
+      LoopArgs la;
+      la.num_tiles = p.num_tiles;
+      la.iters = iters;
+      la.check_every = check_every;
+      la.target_psnr = target_psnr;
+      la.loss_part = ws_ptr<float2>(ws, p, kOffLossPart);
+      la.hdr = ws_ptr<WsHeader>(ws, p, kOffHeader);
+      la.trace = ws_ptr<float>(ws, p, kOffGrad);
+      la.handle = handle;
+      const cudaError_t ce = fit_iteration(p, ws, target, params, m, v, s, &la);
       cudaGraph_t captured = nullptr;
       const cudaError_t ee = cudaStreamEndCapture(s, &captured);
       e = ce != cudaSuccess ? ce : ee;

@@ -4,6 +4,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 
 #include "../../include/gs2d.h"
@@ -161,6 +162,102 @@ inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_
 
 __device__ __forceinline__ void set_status(WsHeader* h, int code) {
   atomicCAS(&h->status, 0, code);
+}
+
+// Sum of float values as an unevaluated pair hi + lo (Knuth's two-sum: the
+// rounding error of every addition is kept, about 48 bits in all).  The loss
+// sums run over every tile in one or a few blocks, where double additions
+// (1/64 of the FP32 rate) were the whole time.
+struct FloatPair {
+  float hi = 0.0f, lo = 0.0f;
+  __device__ __forceinline__ void add(float x) {
+    const float s = __fadd_rn(hi, x), v = __fsub_rn(s, hi);
+    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, v)), __fsub_rn(x, v)));
+    hi = s;
+  }
+  __device__ __forceinline__ double value() const {
+    return isfinite(hi) ? (double)hi + (double)lo : (double)hi;  // (lo is NaN past an infinity)
+  }
+};
+
+// Sums of the loss partials of `count` tiles by one block, in the order of
+// 1024 threads (thread t: tiles t, t + 1024, ...; each warp's lanes; the 32
+// warps) whatever the block's size is: every caller gets the same bits.  Valid
+// in thread 0.  s_sum: 32 pairs.
+template <int THREADS>
+__device__ __forceinline__ double2 loss_sums(const float2* __restrict__ part, int count,
+                                             double2* s_sum) {
+  static_assert(1024 % THREADS == 0 && THREADS % 32 == 0, "whole warps of the 1024");
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll 1
+  for (int k = 0; k < 1024 / THREADS; k++) {
+    FloatPair a, b;
+    int t = k * THREADS + threadIdx.x;
+    for (; t + 3 * 1024 < count; t += 4 * 1024) {
+      float2 v[4];
+#pragma unroll
+      for (int u = 0; u < 4; u++) v[u] = part[t + u * 1024];
+#pragma unroll
+      for (int u = 0; u < 4; u++) {
+        a.add(v[u].x);
+        b.add(v[u].y);
+      }
+    }
+    for (; t < count; t += 1024) {
+      const float2 v = part[t];
+      a.add(v.x);
+      b.add(v.y);
+    }
+    double x = a.value(), y = b.value();
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      x += __shfl_xor_sync(0xffffffffu, x, o);
+      y += __shfl_xor_sync(0xffffffffu, y, o);
+    }
+    if (lane == 0) s_sum[k * (THREADS / 32) + wid] = make_double2(x, y);
+  }
+  __syncthreads();
+  double2 s = make_double2(0.0, 0.0);
+  if (threadIdx.x == 0)
+    for (int w = 0; w < 32; w++) {
+      s.x += s_sum[w].x;
+      s.y += s_sum[w].y;
+    }
+  return s;
+}
+
+// Control of the device-driven fit loop (gs2d_encode_frame), run by a block of
+// its own beside the iteration's last kernel: it counts the iteration; every
+// check_every iterations (and at the last) it sums the render's per-tile loss
+// partials, writes the PSNR of the clamped image to the trace and clears the
+// loop condition once the target is met, the cap is reached or a kernel has
+// recorded an error.
+struct LoopArgs {
+  int num_tiles, iters, check_every;
+  float target_psnr;
+  const float2* loss_part;
+  WsHeader* hdr;  // NULL: no loop
+  float* trace;   // device, one float per check
+  cudaGraphConditionalHandle handle;
+};
+
+template <int THREADS>
+__device__ __forceinline__ void loop_control(const LoopArgs& a, double2* s_sum) {
+  __shared__ int s_it;
+  if (threadIdx.x == 0) s_it = ++a.hdr->loop_iter;
+  __syncthreads();
+  const int it = s_it;
+  if (it % a.check_every != 0 && it < a.iters) return;
+  const double2 s = loss_sums<THREADS>(a.loss_part, a.num_tiles, s_sum);
+  if (threadIdx.x != 0) return;
+  a.hdr->loss[0] = (float)s.x;
+  a.hdr->loss[1] = (float)s.y;
+  const double mse = (double)a.hdr->loss[1];
+  const float psnr = mse > 0.0 ? (float)(10.0 * log10(1.0 / mse)) : INFINITY;
+  a.trace[a.hdr->loop_checks++] = psnr;
+  const bool stop = it >= a.iters || a.hdr->status != 0 ||
+                    (a.target_psnr > 0.0f && psnr >= a.target_psnr);
+  if (stop) cudaGraphSetConditional(a.handle, 0u);
 }
 
 // Projection of Gaussian i (Sec. 3.1 parameters -> screen-space record, tile
@@ -327,10 +424,12 @@ cudaError_t launch_render_l2(const gs2d_plan& p, void* ws, const float* params,
 // Follows launch_prepare_fit (it marks retained lists valid).  params_eval:
 // the values the render used, when they differ from params (the chain rule is
 // taken there; Adam updates params).  host_out: a device view of pinned host
-// memory that receives the parameters after the step, or NULL.
+// memory that receives the parameters after the step, or NULL.  loop: the
+// fit loop this iteration belongs to (n > 0), or NULL.
 cudaError_t launch_fit_step(const gs2d_plan& p, void* ws, const float* target, float* params,
                             float* m, float* v, cudaStream_t s,
-                            const float* params_eval = nullptr, float* host_out = nullptr);
+                            const float* params_eval = nullptr, float* host_out = nullptr,
+                            const LoopArgs* loop = nullptr);
 cudaError_t launch_adam(float* params, const float* grads, float* m, float* v, int64_t count,
                         int32_t step, const uint8_t* mask, const gs2d_config& cfg,
                         cudaStream_t s);

@@ -142,14 +142,21 @@ k_reduce_chain(int n, const float* __restrict__ params, SlotArgs slots,
 // `sub` of the group updates rows sub, sub + kRL, ...).  host_out (device
 // view of pinned host memory, or NULL): every Gaussian's parameters after
 // the step are also stored there, so that no separate download is needed.
+// loop: the last block of the grid controls the fit loop instead (it reads
+// only what earlier kernels wrote, so it runs beside the others).
 __global__ void __launch_bounds__(256)
 k_reduce_chain_adam(int n, float* __restrict__ params, SlotArgs slots,
                     const WsHeader* __restrict__ hdr,
                     float* __restrict__ m, float* __restrict__ v, float4 lr_rows, float b1,
                     float b2, float eps, const uint8_t* __restrict__ select,
                     const float* __restrict__ params_eval, WsHeader* hdr_w,
-                    float* __restrict__ acc, float* __restrict__ host_out) {
+                    float* __restrict__ acc, float* __restrict__ host_out, LoopArgs loop) {
   pdl_begin();
+  if (loop.hdr && blockIdx.x == gridDim.x - 1) {
+    __shared__ double2 s_sum[32];
+    loop_control<256>(loop, s_sum);
+    return;
+  }
   const int gt = blockIdx.x * blockDim.x + threadIdx.x;
   const int i = gt / kRL, sub = gt % kRL;
   const bool ok = hdr->entries_raw == (int64_t)hdr->n_entries;  // else over capacity
@@ -199,31 +206,11 @@ __global__ void __launch_bounds__(1024)
 k_loss_reduce(int num_tiles, const float2* __restrict__ loss_part, WsHeader* __restrict__ hdr,
               float* __restrict__ out) {
   pdl_begin();
-  __shared__ double s_a[32], s_b[32];
-  double a = 0.0, b = 0.0;
-  for (int t = threadIdx.x; t < num_tiles; t += blockDim.x) {
-    a += loss_part[t].x;
-    b += loss_part[t].y;
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    a += __shfl_xor_sync(0xffffffffu, a, o);
-    b += __shfl_xor_sync(0xffffffffu, b, o);
-  }
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (lane == 0) {
-    s_a[wid] = a;
-    s_b[wid] = b;
-  }
-  __syncthreads();
+  __shared__ double2 s_sum[32];
+  const double2 s = loss_sums<1024>(loss_part, num_tiles, s_sum);
   if (threadIdx.x == 0) {
-    double sa = 0.0, sb = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); w++) {
-      sa += s_a[w];
-      sb += s_b[w];
-    }
-    hdr->loss[0] = (float)sa;
-    hdr->loss[1] = (float)sb;
+    hdr->loss[0] = (float)s.x;
+    hdr->loss[1] = (float)s.y;
     if (out) {
       out[0] = hdr->loss[0];
       out[1] = hdr->loss[1];
@@ -237,32 +224,9 @@ k_clip_loss(ClipSet cs, const float2* __restrict__ loss_part, float2* __restrict
   pdl_begin();
   const int c = blockIdx.x;
   const gs2d_clip cl = cs.count == 1 ? cs.one : cs.table[c];
-  __shared__ double s_a[32], s_b[32];
-  double a = 0.0, b = 0.0;
-  const int t0 = cl.tile_off, nt = cl.tiles_x * cl.tiles_y;
-  for (int t = t0 + threadIdx.x; t < t0 + nt; t += blockDim.x) {
-    a += loss_part[t].x;
-    b += loss_part[t].y;
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    a += __shfl_xor_sync(0xffffffffu, a, o);
-    b += __shfl_xor_sync(0xffffffffu, b, o);
-  }
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (lane == 0) {
-    s_a[wid] = a;
-    s_b[wid] = b;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double sa = 0.0, sb = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); w++) {
-      sa += s_a[w];
-      sb += s_b[w];
-    }
-    clip_loss[c] = make_float2((float)sa, (float)sb);
-  }
+  __shared__ double2 s_sum[32];
+  const double2 s = loss_sums<1024>(loss_part + cl.tile_off, cl.tiles_x * cl.tiles_y, s_sum);
+  if (threadIdx.x == 0) clip_loss[c] = make_float2((float)s.x, (float)s.y);
 }
 
 // ---------------------------------------------------------------------------
@@ -411,18 +375,18 @@ cudaError_t launch_count_pairs(const gs2d_plan& p, void* ws, cudaStream_t s) {
 // step counter): fused render + loss + backward, then reduction + chain + Adam.
 cudaError_t launch_fit_step(const gs2d_plan& p, void* ws, const float* target, float* params,
                             float* m, float* v, cudaStream_t s, const float* params_eval,
-                            float* host_out) {
+                            float* host_out, const LoopArgs* loop) {
   RenderArgs a = render_args(p, ws);
   a.target = target;
   cudaError_t e = launch_render(p, kModeL2, a, s);
   if (e != cudaSuccess || p.n == 0) return e;
   WsHeader* hdr = ws_ptr<WsHeader>(ws, p, kOffHeader);
-  return launch_pdl(k_reduce_chain_adam, (p.n * kRL + 255) / 256, 256, 0, s, p.n, params,
-                    slot_args(p, ws),
-                    (const WsHeader*)hdr, m, v, lr_rows(p.cfg), p.cfg.beta1, p.cfg.beta2,
+  // (one block more for the loop's control)
+  return launch_pdl(k_reduce_chain_adam, (p.n * kRL + 255) / 256 + (loop ? 1 : 0), 256, 0, s, p.n,
+                    params, slot_args(p, ws), (const WsHeader*)hdr, m, v, lr_rows(p.cfg), p.cfg.beta1, p.cfg.beta2,
                     p.cfg.eps, (const uint8_t*)nullptr, params_eval,
                     fit_lists_retained(p.cfg) ? hdr : (WsHeader*)nullptr, atomic_sums(p, ws),
-                    host_out);
+                    host_out, loop ? *loop : LoopArgs{});
 }
 
 // ---------------------------------------------------------------------------
@@ -513,7 +477,7 @@ cudaError_t launch_pframe_step(const gs2d_plan& p, void* ws, const float* target
                     slot_args(p, ws),
                     ws_ptr<WsHeader>(ws, p, kOffHeader), m, v, lr_rows(p.cfg), p.cfg.beta1,
                     p.cfg.beta2, p.cfg.eps, select, (const float*)nullptr, (WsHeader*)nullptr,
-                    atomic_sums(p, ws), (float*)nullptr);
+                    atomic_sums(p, ws), (float*)nullptr, LoopArgs{});
 }
 
 // Runs the one-time per-device query of the fit loop's launches (occupancy of
