@@ -1,6 +1,6 @@
 // Implicit-GEMM convolution fed by TMA tap loads: the learned initialiser's
 // wide 3 x 3 stride-2 layers (paper section 3.2 B) as a persistent tcgen05
-// kernel, one CTA per SM.  At 1080p it runs layer 4 (C = 128); the 3 x 3,
+// kernel, one CTA per SM.  At 1080p it runs layers 4 and 5 (C = 128, 256); the 3 x 3,
 // stride-2, pad-1 layers with C = 32 or 64 and an even width go to the
 // row-box kernel of csrc/conv_rows.cu (fewer, larger TMA boxes), and this
 // kernel keeps every other supported shape.
@@ -8,7 +8,12 @@
 //   Z[p][n] = sum_k col(X)[p][k] W[n][k],   k = (ky ks + kx) C + ci,
 //   a column of ones at k = ks^2 C carrying the bias, zeros beyond.
 //
-// A tile is 128 consecutive output pixels of one output row.  For a fixed
+// A tile is 128 consecutive output pixels of one output row, or 64 pixels of
+// two rows where rows are 49 to 63 pixels long (one box all the same, with a
+// traversal stride along H too): layer 5 at 1080p, batch 8, 60 pixels, took
+// 81 us as im2col + GEMM and takes about 40 here (0.457 -> 0.414 ms for the
+// network).  More than 256 output channels are split into blocks, which are
+// the tiles' innermost index.  For a fixed
 // tap (ky, kx) and a chunk of cw channels, the tile's im2col rows are the
 // input pixels x0 + kx, x0 + kx + stride, ... of input row y0 + ky: one TMA
 // box of the NHWC input with traversal stride `stride` along W (out-of-image
@@ -64,6 +69,8 @@ struct TapArgs {
   int Ho, Wo, ks, stride, pad;
   int N, ldc, relu;
   int segs, tiles, nk;
+  int rows, hp;                     // output rows per tile (1, or 2 of 64 pixels), tiles down an image
+  int nblk;                         // blocks of BN output channels
   int cw, cpt, blocks_real, kbias;  // channels per block, blocks per tap, tap blocks, bias k
   int stages, resident_b;
   int per;                          // output tiles per weight load (2 when streamed)
@@ -170,12 +177,14 @@ k_conv_tap(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUten
       for (int t0 = blockIdx.x; t0 < tiles && ok && !failed(&s_fail); t0 += PER * gridDim.x) {
         const int nt = PER == 2 && t0 + (int)gridDim.x < tiles ? 2 : 1;
         int ub[2], ux0[2], uy0[2];
+        // (the grid is a multiple of nblk: a unit's tiles share their block)
+        const int nb = t0 % g.nblk;
         for (int k = 0; k < nt; k++) {
-          const int t = t0 + k * (int)gridDim.x;
+          const int t = (t0 + k * (int)gridDim.x) / g.nblk;
           const int row = t / g.segs, seg = t - row * g.segs;
-          ub[k] = row / g.Ho;
+          ub[k] = row / g.hp;
           ux0[k] = seg * kBM * g.stride - g.pad;
-          uy0[k] = (row - ub[k] * g.Ho) * g.stride - g.pad;
+          uy0[k] = (row - ub[k] * g.hp) * g.rows * g.stride - g.pad;
         }
         int qc = 0, qx = 0, qy = 0;  // chunk and tap (ky, kx) of the k-tile's first block
         for (int i = 0; i < nk; i++) {
@@ -205,7 +214,7 @@ k_conv_tap(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUten
                 }
               }
             }
-            if (!resident) tma_load_2d(st + g.b_off, &tb, &full[s], i * kBK, 0);
+            if (!resident) tma_load_2d(st + g.b_off, &tb, &full[s], i * kBK, nb * BN);
           }
           for (int j = 0; j < nl; j++) {
             if (++qc == cpt) {
@@ -321,13 +330,16 @@ k_conv_tap(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUten
           break;
         }
         tc_fence_after();
-        const int row = t / g.segs, seg = t - row * g.segs;
-        const int ox = seg * kBM + r;
-        const bool valid = ox < g.Wo;
-        const size_t o = ((size_t)row * g.Wo + ox) * g.ldc;
+        const int nb = t % g.nblk, u = t / g.nblk;
+        const int row = u / g.segs, seg = u - row * g.segs, b = row / g.hp;
+        const bool two = g.rows == 2;
+        const int oy = (row - b * g.hp) * g.rows + (two ? r >> 6 : 0);
+        const int ox = seg * kBM + (two ? r & 63 : r);
+        const bool valid = ox < g.Wo && oy < g.Ho;
+        const size_t o = (((size_t)b * g.Ho + oy) * g.Wo + ox) * g.ldc + nb * BN;
         const uint32_t taddr =
             tmem + (uint32_t)(a * Sh::kAccStride) + ((uint32_t)(quarter * 32) << 16);
-        store_acc_row<BN>(taddr, valid, o, g.N, g.relu, vec_ok, g.out_f32, g.out_bf16);
+        store_acc_row<BN>(taddr, valid, o, g.N - nb * BN, g.relu, vec_ok, g.out_f32, g.out_bf16);
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&acc_empty[a]);
@@ -346,17 +358,19 @@ k_conv_tap(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUten
 
 // 4D bf16 tensor map of an NHWC activation [B][Hi][Wi][C] for the tap loads:
 // box cw channels x 128 pixels, traversal stride `stride` along W (so the
-// box spans 128 stride pixels), one row, one image; the swizzle matches the
-// block's row width; zeros out of range.
+// box spans 128 stride pixels), one row, one image, or 64 pixels of two rows
+// `stride` apart; the swizzle matches the block's row width; zeros out of
+// range.
 bool make_tap_map(CUtensorMap* map, const void* x, int B, int Hi, int Wi, int C, int cw,
-                  int stride) {
+                  int stride, int rows) {
   EncodeTiled fn = tensor_map_encoder();
   if (!fn) return false;
   const cuuint64_t dims[4] = {(cuuint64_t)C, (cuuint64_t)Wi, (cuuint64_t)Hi, (cuuint64_t)B};
   const cuuint64_t strides[3] = {(cuuint64_t)C * 2, (cuuint64_t)Wi * C * 2,
                                  (cuuint64_t)Hi * Wi * C * 2};
-  const cuuint32_t box[4] = {(cuuint32_t)cw, (cuuint32_t)(kBM * stride), 1, 1};
-  const cuuint32_t estr[4] = {1, (cuuint32_t)stride, 1, 1};
+  const cuuint32_t box[4] = {(cuuint32_t)cw, (cuuint32_t)(kBM / rows * stride),
+                             (cuuint32_t)(rows == 2 ? 2 * stride : 1), 1};
+  const cuuint32_t estr[4] = {1, (cuuint32_t)stride, (cuuint32_t)(rows == 2 ? stride : 1), 1};
   const CUtensorMapSwizzle swz = cw == 16   ? CU_TENSOR_MAP_SWIZZLE_32B
                                  : cw == 32 ? CU_TENSOR_MAP_SWIZZLE_64B
                                             : CU_TENSOR_MAP_SWIZZLE_128B;
@@ -379,7 +393,7 @@ int sm_count() {
 // Returns the dynamic shared-memory bytes, 0 when even two stages do not fit.
 int tap_plan(int bn, int nk, TapArgs* g) {
   const int kb = bn * kBK * 2;
-  g->resident_b = nk * kb <= 64 * 1024 ? 1 : 0;
+  g->resident_b = g->nblk == 1 && nk * kb <= 64 * 1024 ? 1 : 0;
   g->per = g->resident_b ? 1 : 2;  // streamed weights: each box serves two tiles
   g->b_off = g->per * kABytes;
   g->stage_bytes = g->b_off + (g->resident_b ? 0 : kb);
@@ -399,7 +413,7 @@ cudaError_t launch_tap_per(const CUtensorMap& ta, const CUtensorMap& tb, const T
   const cudaError_t attr = opt_in_smem((const void*)k_conv_tap<BN, PER>, smem);
   if (attr != cudaSuccess) return attr;
   const int sms = sm_count();
-  const int grid = std::max(1, std::min(g.tiles, sms > 0 ? sms : 1));
+  const int grid = std::max(1, std::min(g.tiles, sms > 0 ? sms : 1) / g.nblk) * g.nblk;
   k_conv_tap<BN, PER><<<grid, kTapThreads, smem, s>>>(ta, tb, g);
   return cudaGetLastError();
 }
@@ -416,8 +430,9 @@ cudaError_t launch_tap(const CUtensorMap& ta, const CUtensorMap& tb, const TapAr
 bool tap_conv_supported(const TcConvProblem& pr) {
   const int Wo = (pr.Wi + 2 * pr.pad - pr.ks) / pr.stride + 1;
   const bool cw_ok = pr.C == 16 || pr.C == 32 || pr.C % 64 == 0;
-  return cw_ok && (pr.stride == 1 || pr.stride == 2) && pr.N >= 1 && pr.N <= 256 &&
-         Wo >= 64 && pr.pad < pr.ks;
+  // (rows of 49 to 63 pixels go two to a tile, at least three quarters full)
+  return cw_ok && (pr.stride == 1 || pr.stride == 2) && pr.N >= 1 && pr.N <= 512 &&
+         Wo >= 49 && pr.pad < pr.ks;
 }
 
 cudaError_t tap_conv(const TcConvProblem& pr, cudaStream_t s) {
@@ -435,8 +450,11 @@ cudaError_t tap_conv(const TcConvProblem& pr, cudaStream_t s) {
   g.N = pr.N;
   g.ldc = pr.ldc;
   g.relu = pr.relu;
+  g.rows = Wo < 64 ? 2 : 1;
+  g.hp = (Ho + g.rows - 1) / g.rows;
   g.segs = (Wo + kBM - 1) / kBM;
-  g.tiles = pr.B * Ho * g.segs;
+  g.nblk = (pr.N + bn - 1) / bn;
+  g.tiles = pr.B * g.hp * g.segs * g.nblk;
   g.nk = (pr.ldk + kBK - 1) / kBK;
   g.cw = pr.C < 64 ? pr.C : 64;
   g.cpt = pr.C / g.cw;
@@ -450,7 +468,7 @@ cudaError_t tap_conv(const TcConvProblem& pr, cudaStream_t s) {
   const int smem = tap_plan(bn, g.nk, &g);
   if (smem <= 0) return cudaErrorInvalidValue;
   CUtensorMap ta, tb;
-  if (!make_tap_map(&ta, pr.x, pr.B, pr.Hi, pr.Wi, pr.C, g.cw, pr.stride) ||
+  if (!make_tap_map(&ta, pr.x, pr.B, pr.Hi, pr.Wi, pr.C, g.cw, pr.stride, g.rows) ||
       !make_map(&tb, pr.W, pr.N, pr.ldk, pr.ldk, bn))
     return cudaErrorInvalidValue;
   switch (bn) {

@@ -77,7 +77,7 @@ struct TcFrameConvProblem {
 cudaError_t tc_gemm(const TcGemmProblem& pr, cudaStream_t s);
 cudaError_t tc_conv(const TcConvProblem& pr, cudaStream_t s);
 // The persistent TMA-tap convolution (csrc/conv_tap.cu): C of 16, 32 or a
-// multiple of 64, stride 1 or 2, N <= 256, output rows of 64 pixels or more.
+// multiple of 64, stride 1 or 2, N <= 512, output rows of 49 pixels or more.
 bool tap_conv_supported(const TcConvProblem& pr);
 cudaError_t tap_conv(const TcConvProblem& pr, cudaStream_t s);
 // The persistent row-box convolution (csrc/conv_rows.cu): 3 x 3, stride 2,

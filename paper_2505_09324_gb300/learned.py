@@ -182,12 +182,14 @@ class LearnedInitializer:
             last = li == self.L
             out32 = self.out.data_ptr() if last else 0
             out16 = 0 if last else self.x[li + 1].data_ptr()
-            # implicit GEMM unless K is very deep (the last 3 x 3 layer: 37
-            # k-tiles over 32 tiles, where the TMA-fed GEMM over an im2col
-            # operand is faster); the results are identical either way, so
-            # training too only writes the operand (for backward) and does
-            # not read it back here
-            implicit = (ldk + 63) // 64 <= 32
+            # implicit GEMM unless K is very deep and the output rows short
+            # (37 k-tiles over few tiles of gathered operands: the TMA-fed GEMM
+            # over an im2col operand is faster there; from 49 pixels the TMA
+            # taps serve two rows a tile); the results are identical either
+            # way, so training too only writes the operand (for backward) and
+            # does not read it back here
+            wo = self.sizes[li + 1][1] if li < self.L else wi
+            implicit = (ldk + 63) // 64 <= 32 or wo >= 49
             if keep_col or not implicit:
                 nat.call("gs2d_im2col", src.data_ptr(), B, hi, wi, ci, ks, stride, pad,
                          self.col[li].data_ptr(), ldk, s)

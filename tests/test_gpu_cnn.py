@@ -581,3 +581,36 @@ def test_conv_input_gradient_by_definition(nat, B, H, W, C, N):
         tol = REL * scale + np.abs(ref) * 2.0 ** -8
         assert np.all(np.abs(to_np_bf16(out) - ref) <= tol + 1e-30)
         assert int(status.item()) == 0
+
+
+@pytest.mark.parametrize("B,H,W,ci,co,ks,st,pad,out", [
+    (2, 17, 120, 64, 384, 3, 2, 1, "bf16"),    # two rows a tile, odd rows, two blocks of N
+    (1, 6, 98, 128, 40, 3, 2, 1, "f32"),       # 49 pixels
+    (3, 5, 63, 32, 300, 3, 1, 1, "bf16"),      # stride 1, 63 pixels, ragged N blocks
+    (1, 7, 130, 16, 512, 3, 2, 1, "f32"),      # one row a tile, two blocks of N
+    (8, 68, 120, 256, 384, 3, 2, 1, "bf16")])  # the network's last 3 x 3 layer at 1080p
+def test_tap_conv_short_rows_and_wide_outputs(nat, B, H, W, ci, co, ks, st, pad, out):
+    """The TMA-tap kernel with two output rows per tile and with several blocks
+    of output channels equals im2col + GEMM bit for bit."""
+    g = torch.Generator(device="cuda").manual_seed(co + W)
+    ldk = -(-(ks * ks * ci + 1) // 8) * 8
+    x = torch.randn((B, H, W, ci), generator=g, device="cuda").bfloat16()
+    w = torch.zeros((co, ldk), device="cuda")
+    w[:, :ks * ks * ci + 1] = torch.randn((co, ks * ks * ci + 1), generator=g,
+                                          device="cuda") / (ks * ks * ci) ** 0.5
+    w = w.bfloat16()
+    Ho, Wo = cnn.out_size(H, ks, st, pad), cnn.out_size(W, ks, st, pad)
+    P = B * Ho * Wo
+    dt = torch.bfloat16 if out == "bf16" else torch.float32
+    col = torch.empty((P, ldk), dtype=torch.bfloat16, device="cuda")
+    zs = [torch.full((P, co), 7.0, dtype=dt, device="cuda") for _ in range(2)]
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    ptrs = [(z.data_ptr(), 0) if out == "f32" else (0, z.data_ptr()) for z in zs]
+    nat.call("gs2d_im2col", x.data_ptr(), B, H, W, ci, ks, st, pad, col.data_ptr(), ldk, 0)
+    nat.gemm_bf16(col.data_ptr(), ldk, w.data_ptr(), ldk, P, co, ldk, 0, True, *ptrs[0], co, 1, 0,
+                  status.data_ptr(), 0)
+    nat.call("gs2d_conv_bf16", x.data_ptr(), B, H, W, ci, ks, st, pad, w.data_ptr(), ldk, co, 1,
+             *ptrs[1], co, status.data_ptr(), 0)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    assert torch.equal(zs[0], zs[1])
