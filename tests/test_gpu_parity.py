@@ -464,3 +464,35 @@ def test_fit_on_large_plans_equals_per_iteration_binning(gs):
         outs.append((p, m, v))
     for a, b in zip(*outs):
         assert torch.equal(a, b)
+
+
+def _sheared(n, W, H, seed):
+    """Thin and fat, strongly sheared Gaussians of both orientations, many of
+    them cut by several tiles, with negative factors and weights among them."""
+    g = np.random.Generator(np.random.PCG64(seed))
+    p = np.empty((9, n))
+    p[0], p[1] = g.uniform(-20, W + 20, n), g.uniform(-20, H + 20, n)
+    p[2], p[4] = np.exp(g.uniform(np.log(0.3), np.log(40), (2, n)))
+    p[3] = g.normal(0, 1, n) * np.exp(g.uniform(np.log(0.1), np.log(60), n))
+    p[2:5] *= np.where(g.random((3, n)) < 0.2, -1, 1)
+    p[5:8], p[8] = g.uniform(0, 1, (3, n)), g.uniform(0.02, 1, n) * np.where(g.random(n) < 0.2, -1, 1)
+    return p.astype(np.float32)
+
+
+@pytest.mark.parametrize("tile", [8, 16, 32])
+@pytest.mark.parametrize("W,H,n", [(203, 150, 250), (1100, 900, 400)])
+def test_tile_cuts_of_sheared_ellipses(gs, oracle, tile, W, H, n):
+    """The staged boxes are cut to the part of the ellipse a tile can reach: no
+    contributing pixel may be lost, whatever the shear, in the image and in
+    every gradient (usual kernels and those for few tiles)."""
+    p = _sheared(n, W, H, seed=tile + W)
+    target = smooth_noise_target(W, H, seed=7)
+    r = gs.GaussianRasterizer(W, H, n, config=gs.RasterConfig(tile=tile), max_entries=1 << 24)
+    tp, tt = to_dev(p), to_dev(target)
+    r.prepare(tp)
+    grads, loss, img = r.render_l2(tp, tt, want_image=True)
+    ref = oracle.loss_and_grad(p, target, fast=True)
+    check_image(img, ref["img"], ref["amb_lo"], ref["amb_hi"])
+    check_image(r.render_fwd(), ref["img"], ref["amb_lo"], ref["amb_hi"])
+    check_grads(grads, ref["grad"], ref["grad_unc"])
+    assert r.status() == 0
