@@ -7,26 +7,32 @@
 // A pixel is read by one, two or four taps, by the parity of its row and
 // column: with iy = 2 a + py, ix = 2 c + px the four classes (py, px) sum over
 // dZ at (a, c), (a, c + 1), (a + 1, c) and (a + 1, c + 1) only.  So a tile is
-// 128 columns c of one row a, i.e. 2 x 256 input pixels: four accumulators
-// (one per class) of C columns, and per 64 output channels four dZ boxes, each
-// shifted by a row or a column (one TMA box; zeros past the edge), with the
-// nine taps' weights:
+// 128 columns c of one row a, i.e. 2 x 256 input pixels, of 32 input channels;
+// per 64 output channels it takes four dZ boxes, each shifted by a row or a
+// column (one TMA box; zeros past the edge), and the nine taps' weights:
 //   (a, c):     taps 11, 12, 21, 22 -> classes 00, 01, 10, 11
 //   (a, c + 1): taps 10, 20 -> 01, 11     (a + 1, c): taps 01, 02 -> 10, 11
 //   (a + 1, c + 1): tap 00 -> 11
+// Each tap has its own accumulator, and the epilogue adds a pixel's taps in
+// their order: bit for bit the FP32 sums of the GEMM to an im2col gradient
+// with the gather after it (gs2d_gemm_bf16, gs2d_col2im).  One accumulator per
+// class differed from them in the last FP32 bit, which the BF16 rounding of
+// every layer below turned into relative differences of up to 6e-5 in the
+// weight gradients of small frames.
 // What bounds it is the traffic of dZ, act and dx (0.66 GB for the widest
-// layer at 1080p, batch 8).  The GEMM to an FP32 im2col gradient and the
-// gather after it moved 4.6 GB more per training step: 1.65 ms for the three
-// widest layers, 0.51 ms here (266, 140 and 101 us).
+// layer at 1080p, batch 8).  The GEMM and the gather moved 4.6 GB more per
+// training step: 1.65 ms for the three widest layers, 0.47 ms here (0.54 with
+// one accumulator per class and an epilogue that read the mask after its wait).
 //
-// A persistent CTA per SM: warp 0, one lane, brings the boxes into a ring;
-// the weights stay in shared memory when they fit, else each stage has room
-// for the (up to four) weight boxes of its dZ box.  Warp 1, one lane, issues
-// the MMAs; warps 2-9 (two per accumulator quarter, one per row parity) apply
-// the mask, convert and store 16-byte vectors, overlapping the next tile where
-// tensor memory holds more than one set of accumulators (C <= 64).  Every wait
-// is bounded as in csrc/conv_tap.cu; the producer also waits (bounded) for its
-// last copies before the CTA may leave.
+// A persistent CTA per SM, of one block of 32 channels: warp 0, one lane,
+// brings the boxes into a ring; the weights stay in shared memory when they
+// fit (up to 256 output channels), else each stage has room for the (up to
+// four) weight boxes of its dZ box.  Warp 1, one lane, issues the MMAs; warps
+// 2-9 (two per accumulator quarter, one per row parity) add the taps, mask,
+// convert and store.  The mask of a tile is read before its accumulators are
+// waited for, and they are given back before the stores, so both overlap the
+// MMAs of the next tile.  Every wait is bounded as in csrc/conv_tap.cu; the
+// producer also waits (bounded) for its last copies before the CTA may leave.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <stdio.h>
@@ -47,60 +53,56 @@ constexpr int kDgBudget = 226 * 1024;
 
 struct DgArgs {
   int Hi, Wi, C, Ho, Wo;
-  int segs, nblk, tiles, chunks;  // column segments, blocks of channels, tiles, 64-channel chunks
+  int segs, nblk, tiles, chunks;  // column segments, blocks of 32 channels, tiles of a block,
+                                  // 64-channel chunks
   int stages, resident, stage_bytes, bres_off;
   const __nv_bfloat16* act;
   __nv_bfloat16* dx;
   int* status;
 };
 
-template <int CI>
-struct DgShape {
-  static constexpr int kAcc = 128 / CI;      // sets of four accumulators: 4, 2, 1
-  static constexpr int kSet = 4 * CI;        // TMEM columns of a set
-  static constexpr int kBBytes = CI * 128;   // one tap's weights: CI rows of 64 channels
-};
+constexpr int kCI = 32;              // input channels of a tile
+constexpr int kDgB = kCI * kBK * 2;  // one tap's weights: 32 rows of 64 channels, 4 KB
 
-// The taps of dZ box v (0: (a, c), 1: (a, c + 1), 2: (a + 1, c), 3: both) and
-// the classes they add to.
+// The taps of dZ box v (0: (a, c), 1: (a, c + 1), 2: (a + 1, c), 3: both);
+// taps 3, 4 and 5 are those of even rows.
 __device__ __forceinline__ int dg_taps(int v) { return v == 0 ? 4 : v == 3 ? 1 : 2; }
 __device__ __forceinline__ int dg_tap(int v, int k) {
   constexpr uint32_t kTap[4] = {0x8754u, 0x63u, 0x21u, 0x0u};
   return (int)((kTap[v] >> (4 * k)) & 15u);
 }
-__device__ __forceinline__ int dg_class(int v, int k) {
-  constexpr uint32_t kClass[4] = {0x3210u, 0x31u, 0x32u, 0x3u};
-  return (int)((kClass[v] >> (4 * k)) & 15u);
-}
+// The first column of a tap's accumulator.
+__device__ __forceinline__ uint32_t dg_col(int tap) { return (uint32_t)(tap * kCI); }
 
 __device__ __forceinline__ bool dg_failed(const int* flag) {
   return *reinterpret_cast<const volatile int*>(flag) != 0;
 }
 
-template <int CI>
 __global__ void __launch_bounds__(kDgThreads, 1)
 k_conv_dgrad(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb,
              DgArgs g) {
-  using Sh = DgShape<CI>;
   pdl_begin();
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t full[kDgStages], empty[kDgStages];
-  __shared__ __align__(8) uint64_t acc_full[Sh::kAcc], acc_empty[Sh::kAcc], bres_full;
+  __shared__ __align__(8) uint64_t acc_full[2], acc_empty[2], bres_full;
   __shared__ uint32_t s_tmem;
   __shared__ int s_fail;
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~uintptr_t(1023));
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int ST = g.stages;
+  // this CTA's block of channels and its tiles of that block
+  const int nb = (int)blockIdx.x % g.nblk, first = (int)blockIdx.x / g.nblk;
+  const int step = (int)gridDim.x / g.nblk;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < ST; s++) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
     }
-    for (int a = 0; a < Sh::kAcc; a++) {
-      mbar_init(&acc_full[a], 1);
-      mbar_init(&acc_empty[a], 8);  // one arrival per epilogue warp
+    for (int py = 0; py < 2; py++) {  // the accumulators of even and of odd rows
+      mbar_init(&acc_full[py], 1);
+      mbar_init(&acc_empty[py], 4);  // one arrival per epilogue warp
     }
     mbar_init(&bres_full, 1);
     s_fail = 0;
@@ -122,18 +124,17 @@ k_conv_dgrad(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
       const int C = g.C, chunks = g.chunks, tiles = g.tiles, stage_bytes = g.stage_bytes;
       const bool resident = g.resident != 0;
       if (resident) {
-        mbar_expect_tx(&bres_full, (uint32_t)(9 * chunks * Sh::kBBytes));
+        mbar_expect_tx(&bres_full, (uint32_t)(9 * chunks * kDgB));
         for (int q = 0; q < chunks; q++)
           for (int tap = 0; tap < 9; tap++)
-            tma_load_2d(smem + g.bres_off + (9 * q + tap) * Sh::kBBytes, &tb, &bres_full, q * kBK,
-                        tap * C);
+            tma_load_2d(smem + g.bres_off + (9 * q + tap) * kDgB, &tb, &bres_full, q * kBK,
+                        tap * C + nb * kCI);
       }
       int s = 0, issued = 0;
       uint32_t ph = 0;
       bool ok = true;
-      for (int t = blockIdx.x; t < tiles && ok && !dg_failed(&s_fail); t += gridDim.x) {
-        const int nb = t % g.nblk, u = t / g.nblk;
-        const int row = u / g.segs, c0 = (u - row * g.segs) * kBM;
+      for (int t = first; t < tiles && ok && !dg_failed(&s_fail); t += step) {
+        const int row = t / g.segs, c0 = (t - row * g.segs) * kBM;
         const int b = row / g.Ho, a = row - b * g.Ho;
         for (int i = 0; i < 4 * chunks; i++) {
           const int q = i >> 2, v = i & 3;
@@ -143,11 +144,11 @@ k_conv_dgrad(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
           }
           uint8_t* st = smem + s * stage_bytes;
           const int nt = resident ? 0 : dg_taps(v);
-          mbar_expect_tx(&full[s], (uint32_t)(kDgA + nt * Sh::kBBytes));
+          mbar_expect_tx(&full[s], (uint32_t)(kDgA + nt * kDgB));
           tma_load_4d(st, &ta, &full[s], q * kBK, c0 + (v & 1), a + (v >> 1), b);
           for (int k = 0; k < nt; k++)
-            tma_load_2d(st + kDgA + k * Sh::kBBytes, &tb, &full[s], q * kBK,
-                        dg_tap(v, k) * C + nb * CI);
+            tma_load_2d(st + kDgA + k * kDgB, &tb, &full[s], q * kBK,
+                        dg_tap(v, k) * C + nb * kCI);
           issued++;
           if (++s == ST) {
             s = 0;
@@ -165,24 +166,21 @@ k_conv_dgrad(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
     }
   } else if (warp == 1) {
     if (lane == 0) {
-      constexpr uint32_t idesc = idesc_bf16(kBM, CI);
+      constexpr uint32_t idesc = idesc_bf16(kBM, kCI);
       const int chunks = g.chunks, tiles = g.tiles;
       const bool resident = g.resident != 0;
       bool ok = !resident || mbar_wait(&bres_full, 0);
       const uint64_t a0 = sw128_desc(smem_u32(smem));
       const uint64_t b0 = resident ? sw128_desc(smem_u32(smem + g.bres_off)) : a0 + (kDgA >> 4);
       const uint64_t stage_d = (uint64_t)(g.stage_bytes >> 4);
-      constexpr uint64_t tap_d = Sh::kBBytes >> 4;
+      constexpr uint64_t tap_d = kDgB >> 4;
       int s = 0;
       uint32_t ph = 0, at = 0;
-      for (int t = blockIdx.x; t < tiles && ok && !dg_failed(&s_fail); t += gridDim.x, at++) {
-        const int acc = (int)(at % (uint32_t)Sh::kAcc);
-        if (!mbar_wait(&acc_empty[acc], ((at / (uint32_t)Sh::kAcc) & 1u) ^ 1u)) {
-          ok = false;
-          break;
-        }
+      for (int t = first; t < tiles && ok && !dg_failed(&s_fail); t += step, at++) {
+        // (a fresh barrier passes the wait for the parity before its first)
+        ok = mbar_wait(&acc_empty[0], (at & 1u) ^ 1u) && mbar_wait(&acc_empty[1], (at & 1u) ^ 1u);
+        if (!ok) break;
         tc_fence_after();
-        const uint32_t d = tmem + (uint32_t)(acc * Sh::kSet);
         for (int q = 0; q < chunks && ok; q++) {
 #pragma unroll
           for (int v = 0; v < 4; v++) {
@@ -192,19 +190,19 @@ k_conv_dgrad(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
             }
             tc_fence_after();
             const uint64_t ad = a0 + (uint64_t)s * stage_d;
-            // the first box of a tile touches every class first
-            const uint32_t keep = q > 0 || v > 0;
 #pragma unroll
             for (int k = 0; k < dg_taps(v); k++) {
-              const uint64_t bd = resident
-                                      ? b0 + (uint64_t)(9 * q + dg_tap(v, k)) * tap_d
-                                      : b0 + (uint64_t)s * stage_d + (uint64_t)k * tap_d;
+              const int tap = dg_tap(v, k);
+              const uint64_t bd = resident ? b0 + (uint64_t)(9 * q + tap) * tap_d
+                                           : b0 + (uint64_t)s * stage_d + (uint64_t)k * tap_d;
 #pragma unroll
               for (int kk = 0; kk < kBK / 16; kk++)
-                mma_bf16(d + (uint32_t)(dg_class(v, k) * CI), ad + 2 * kk, bd + 2 * kk, idesc,
-                         kk > 0 ? 1u : keep);
+                mma_bf16(tmem + dg_col(tap), ad + 2 * kk, bd + 2 * kk, idesc,
+                         q > 0 || kk > 0 ? 1u : 0u);
             }
             mma_commit(&empty[s]);
+            // the even rows' taps end with box 1 of the last chunk
+            if (v == 1 && q == chunks - 1) mma_commit(&acc_full[0]);
             if (++s == ST) {
               s = 0;
               ph ^= 1u;
@@ -212,61 +210,114 @@ k_conv_dgrad(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
           }
         }
         if (!ok) break;
-        mma_commit(&acc_full[acc]);
+        mma_commit(&acc_full[1]);
       }
       if (!ok) s_fail = 1;
     }
   } else {
     // epilogue: TMEM lanes 32 (warp % 4) ..., row parity by the warp's group
     const int quarter = warp & 3, py = (warp - 2) >> 2, r = quarter * 32 + lane;
+    const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16);
+    const int cols = min(kCI, g.C - nb * kCI) / 8;  // 16-byte vectors of a pixel
     uint32_t at = 0;
-    for (int t = blockIdx.x; t < g.tiles; t += gridDim.x, at++) {
-      const int acc = (int)(at % (uint32_t)Sh::kAcc);
-      // (tcgen05.ld is warp-collective: the warp goes on only if every lane
-      // saw the accumulators complete)
-      if (!__all_sync(0xffffffffu, mbar_wait(&acc_full[acc], (at / (uint32_t)Sh::kAcc) & 1u))) {
-        s_fail = 1;
-        break;
-      }
-      tc_fence_after();
-      const int nb = t % g.nblk, u = t / g.nblk;
-      const int row = u / g.segs, c = (u - row * g.segs) * kBM + r;
+    for (int t = first; t < g.tiles; t += step, at++) {
+      const int row = t / g.segs, c = (t - row * g.segs) * kBM + r;
       const int b = row / g.Ho, iy = 2 * (row - b * g.Ho) + py;
-      const uint32_t taddr = tmem + (uint32_t)(acc * Sh::kSet + 2 * py * CI) +
-                             ((uint32_t)(quarter * 32) << 16);
-      if (iy < g.Hi) {
-#pragma unroll 1
+      const bool in = iy < g.Hi;  // (the last odd row may be missing)
+      const size_t o = (((size_t)b * g.Hi + iy) * g.Wi + 2 * c) * g.C + nb * kCI;
+      // the mask of this lane's two pixels, a bit per channel
+      uint32_t mask[2] = {0xffffffffu, 0xffffffffu};
+      if (g.act) {
+#pragma unroll
         for (int px = 0; px < 2; px++) {
-          const int ix = 2 * c + px;
-          const bool valid = ix < g.Wi;
-          const size_t o = (((size_t)b * g.Hi + iy) * g.Wi + ix) * g.C + nb * CI;
-#pragma unroll 1
-          for (int c0 = 0; c0 < CI; c0 += 32) {
-            float w[32];
-            tmem_ld32(taddr + (uint32_t)(px * CI + c0), w);
-            if (!valid) continue;
+          uint4 av[4];
 #pragma unroll
-            for (int k = 0; k < 32; k += 8) {
-              if (nb * CI + c0 + k >= g.C) break;
-              if (g.act) {
-                const uint4 av = *reinterpret_cast<const uint4*>(g.act + o + c0 + k);
-                const __nv_bfloat16* ab = reinterpret_cast<const __nv_bfloat16*>(&av);
+          for (int k = 0; k < 4; k++)
+            av[k] = in && 2 * c + px < g.Wi && k < cols
+                        ? *reinterpret_cast<const uint4*>(g.act + o + px * g.C + 8 * k)
+                        : make_uint4(0, 0, 0, 0);
+          mask[px] = 0;
 #pragma unroll
-                for (int j = 0; j < 8; j++)
-                  if (!(__bfloat162float(ab[j]) > 0.0f)) w[k + j] = 0.0f;
-              }
-              __align__(16) __nv_bfloat162 h[4];
+          for (int k = 0; k < 4; k++) {
+            const uint32_t w[4] = {av[k].x, av[k].y, av[k].z, av[k].w};
 #pragma unroll
-              for (int j = 0; j < 4; j++)
-                h[j] = __floats2bfloat162_rn(w[k + 2 * j], w[k + 2 * j + 1]);
-              *reinterpret_cast<uint4*>(g.dx + o + c0 + k) = *reinterpret_cast<const uint4*>(h);
+            for (int i = 0; i < 4; i++) {
+              const float lo = __uint_as_float(w[i] << 16);
+              const float hi = __uint_as_float(w[i] & 0xffff0000u);
+              mask[px] |= (lo > 0.0f ? 1u : 0u) << (8 * k + 2 * i);
+              mask[px] |= (hi > 0.0f ? 2u : 0u) << (8 * k + 2 * i);
             }
           }
         }
       }
+      // (tcgen05.ld is warp-collective: the warp goes on only if every lane
+      // saw the accumulators complete)
+      if (!__all_sync(0xffffffffu, mbar_wait(&acc_full[py], at & 1u))) {
+        s_fail = 1;
+        break;
+      }
+      tc_fence_after();
+      // column parity px: taps ky x kx in their order, ky = 1 (even rows) or
+      // 0, 2 (odd), kx = 1 (even columns) or 0, 2 (odd)
+      uint32_t h[2][16];
+#pragma unroll
+      for (int px = 0; px < 2; px++) {
+        float w[32], x[32];
+        tmem_ld32(taddr + dg_col((py ? 0 : 3) + (px ? 0 : 1)), w);
+        if (px) {
+          tmem_ld32(taddr + dg_col((py ? 0 : 3) + 2), x);
+#pragma unroll
+          for (int i = 0; i < 32; i++) w[i] += x[i];
+        }
+        if (py) {
+          tmem_ld32(taddr + dg_col(6 + (px ? 0 : 1)), x);
+#pragma unroll
+          for (int i = 0; i < 32; i++) w[i] += x[i];
+          if (px) {
+            tmem_ld32(taddr + dg_col(8), x);
+#pragma unroll
+            for (int i = 0; i < 32; i++) w[i] += x[i];
+          }
+        }
+#pragma unroll
+        for (int i = 0; i < 16; i++) {
+          const float lo = mask[px] >> (2 * i) & 1u ? w[2 * i] : 0.0f;
+          const float hi = mask[px] >> (2 * i + 1) & 1u ? w[2 * i + 1] : 0.0f;
+          const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+          h[px][i] = *reinterpret_cast<const uint32_t*>(&v);
+        }
+      }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&acc_empty[acc]);
+      if (lane == 0) mbar_arrive(&acc_empty[py]);
+      if (!in) continue;
+      // pairs of lanes exchange vectors, so that the two write a 32-byte
+      // sector at a time: first the even lane's pixel, then the odd lane's
+      const bool odd = lane & 1;
+      const size_t oe = o - (odd ? 2 * (size_t)g.C : 0);
+#pragma unroll
+      for (int px = 0; px < 2; px++) {
+        const int ix = 2 * (c - (odd ? 1 : 0)) + px;  // of the even lane
+        __nv_bfloat16* const dst = g.dx + oe + (size_t)px * g.C;
+#pragma unroll
+        for (int k = 0; k < 4; k += 2) {
+          uint32_t own[4], got[4];
+#pragma unroll
+          for (int i = 0; i < 4; i++) {
+            own[i] = odd ? h[px][4 * (k + 1) + i] : h[px][4 * k + i];
+            got[i] = __shfl_xor_sync(0xffffffffu, odd ? h[px][4 * k + i] : h[px][4 * (k + 1) + i],
+                                     1);
+          }
+          const int kv = k + (odd ? 1 : 0);  // the vector this lane writes
+          if (kv < cols) {
+            const uint4 mine = make_uint4(own[0], own[1], own[2], own[3]);
+            const uint4 other = make_uint4(got[0], got[1], got[2], got[3]);
+            if (ix < g.Wi) *reinterpret_cast<uint4*>(dst + 8 * kv) = odd ? other : mine;
+            if (ix + 2 < g.Wi)
+              *reinterpret_cast<uint4*>(dst + 2 * (size_t)g.C + 8 * kv) = odd ? mine : other;
+          }
+        }
+      }
     }
   }
   __syncwarp();
@@ -292,23 +343,24 @@ bool dg_map(CUtensorMap* map, const void* x, int B, int H, int W, int C) {
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int CI>
 cudaError_t launch_dgrad(const CUtensorMap& ta, const CUtensorMap& tb, DgArgs g, cudaStream_t s) {
-  const int bres = 9 * g.chunks * DgShape<CI>::kBBytes;
+  const int bres = 9 * g.chunks * kDgB;
   // resident weights leave room for at least four dZ boxes
-  g.resident = g.nblk == 1 && bres + 4 * kDgA + 1024 <= kDgBudget;
-  g.stage_bytes = kDgA + (g.resident ? 0 : 4 * DgShape<CI>::kBBytes);
+  g.resident = bres + 4 * kDgA + 1024 <= kDgBudget;
+  g.stage_bytes = kDgA + (g.resident ? 0 : 4 * kDgB);
   const int fixed = (g.resident ? bres : 0) + 1024;  // + alignment slack
   g.stages = std::min(kDgStages, (kDgBudget - fixed) / g.stage_bytes);
   g.bres_off = g.stages * g.stage_bytes;
   const int smem = g.bres_off + fixed;
-  cudaError_t e = opt_in_smem((const void*)k_conv_dgrad<CI>, smem);
+  cudaError_t e = opt_in_smem((const void*)k_conv_dgrad, smem);
   if (e != cudaSuccess) return e;
   int dev = 0, sms = 0;
   e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  return launch_pdl(k_conv_dgrad<CI>, std::min(g.tiles, sms), kDgThreads, smem, s, ta, tb, g);
+  // a whole number of CTAs for each block of channels
+  const int per = std::max(1, std::min(g.tiles, sms / g.nblk));
+  return launch_pdl(k_conv_dgrad, per * g.nblk, kDgThreads, smem, s, ta, tb, g);
 }
 
 }  // namespace
@@ -331,11 +383,10 @@ extern "C" gs2d_status gs2d_conv_dgrad_bf16(const void* dz, int32_t B, int32_t H
   g.C = C;
   g.Ho = (Hi + 1) / 2;
   g.Wo = (Wi + 1) / 2;
-  const int ci = C <= 32 ? 32 : C <= 64 ? 64 : 128;
   g.segs = (g.Wo + kBM - 1) / kBM;
-  g.nblk = (C + ci - 1) / ci;
+  g.nblk = (C + kCI - 1) / kCI;
   g.chunks = (N + kBK - 1) / kBK;
-  const int64_t tiles = (int64_t)B * g.Ho * g.segs * g.nblk;
+  const int64_t tiles = (int64_t)B * g.Ho * g.segs;
   if (tiles > INT32_MAX - 65536 || (int64_t)9 * C > INT32_MAX)
     return set_error(GS2D_ERR_INVALID_ARG, "gs2d_conv_dgrad_bf16: sizes");
   g.tiles = (int)tiles;
@@ -343,12 +394,10 @@ extern "C" gs2d_status gs2d_conv_dgrad_bf16(const void* dz, int32_t B, int32_t H
   g.dx = static_cast<__nv_bfloat16*>(dx);
   g.status = status;
   CUtensorMap ta, tb;
-  if (!dg_map(&ta, dz, B, g.Ho, g.Wo, N) || !make_map(&tb, Wt, 9 * C, N, N, ci))
+  if (!dg_map(&ta, dz, B, g.Ho, g.Wo, N) || !make_map(&tb, Wt, 9 * C, N, N, kCI))
     return set_error(GS2D_ERR_CUDA, "gs2d_conv_dgrad_bf16: tensor map");
   cudaStream_t s = (cudaStream_t)stream;
-  const cudaError_t e = ci == 32   ? launch_dgrad<32>(ta, tb, g, s)
-                        : ci == 64 ? launch_dgrad<64>(ta, tb, g, s)
-                                   : launch_dgrad<128>(ta, tb, g, s);
+  const cudaError_t e = launch_dgrad(ta, tb, g, s);
   if (e != cudaSuccess) {
     char msg[200];
     snprintf(msg, sizeof(msg), "gs2d_conv_dgrad_bf16: %s", cudaGetErrorString(e));

@@ -583,6 +583,31 @@ def test_conv_input_gradient_by_definition(nat, B, H, W, C, N):
         assert int(status.item()) == 0
 
 
+@pytest.mark.parametrize("B,H,W,C,N", [(2, 9, 130, 32, 64), (1, 6, 259, 72, 136),
+                                       (1, 5, 200, 64, 384), (1, 1, 1, 8, 8)])
+def test_conv_input_gradient_equals_the_gathered_gemm(nat, B, H, W, C, N):
+    """gs2d_conv_dgrad_bf16 equals the GEMM to an FP32 im2col gradient with
+    the gather after it (gs2d_gemm_bf16, gs2d_col2im) bit for bit: a tap's
+    sum over the output channels first, then the taps in their order."""
+    g = torch.Generator(device="cuda").manual_seed(W + C)
+    P, ldk = B * ((H + 1) // 2) * ((W + 1) // 2), 9 * C + 8
+    dz = torch.randn((P, N), generator=g, device="cuda").bfloat16()
+    wt = torch.randn((ldk, N), generator=g, device="cuda").bfloat16()
+    act = torch.randn((B, H, W, C), generator=g, device="cuda").bfloat16()
+    dcol = torch.empty((P, ldk), device="cuda")
+    dx = [torch.full((B, H, W, C), 7.0, dtype=torch.bfloat16, device="cuda") for _ in range(2)]
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    nat.gemm_bf16(dz.data_ptr(), N, wt.data_ptr(), N, P, ldk, N, 0, False, dcol.data_ptr(), 0,
+                  ldk, 1, 0, status.data_ptr(), 0)
+    nat.call("gs2d_col2im", dcol.data_ptr(), ldk, B, H, W, C, 3, 2, 1, act.data_ptr(),
+             dx[0].data_ptr(), 0)
+    nat.call("gs2d_conv_dgrad_bf16", dz.data_ptr(), B, H, W, C, wt.data_ptr(), N, act.data_ptr(),
+             dx[1].data_ptr(), status.data_ptr(), 0)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    assert torch.equal(dx[0], dx[1])
+
+
 @pytest.mark.parametrize("B,H,W,ci,co,ks,st,pad,out", [
     (2, 17, 120, 64, 384, 3, 2, 1, "bf16"),    # two rows a tile, odd rows, two blocks of N
     (1, 6, 98, 128, 40, 3, 2, 1, "f32"),       # 49 pixels
