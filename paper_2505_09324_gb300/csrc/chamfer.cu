@@ -79,6 +79,7 @@ __global__ void __launch_bounds__(kNnThreads) k_nn_build(NnArgs a) {
   const float* py = px + set.ld;
   float lo_x = INFINITY, hi_x = -INFINITY, lo_y = INFINITY, hi_y = -INFINITY;
   float sx = 0.f, sxx = 0.f, sy = 0.f, syy = 0.f, cnt = 0.f;
+#pragma unroll 8
   for (int i = t; i < n; i += kNnThreads) {
     const float x = px[i], y = py[i];
     if (!isfinite(x) || !isfinite(y)) continue;
@@ -147,6 +148,7 @@ __global__ void __launch_bounds__(kNnThreads) k_nn_build(NnArgs a) {
     if (!isfinite(x) || !isfinite(y)) return cells;
     return nn_axis(y, g.lo_y, g.inv, g.gy) * g.gx + nn_axis(x, g.lo_x, g.inv, g.gx);
   };
+#pragma unroll 8
   for (int i = t; i < n; i += kNnThreads) atomicAdd(&s_cnt[cell_of(px[i], py[i])], 1);
   __syncthreads();
   // exclusive scan of the counts (the cells, then the non-finite points)
@@ -181,6 +183,7 @@ __global__ void __launch_bounds__(kNnThreads) k_nn_build(NnArgs a) {
   }
   if (t == 0) start[kNnCells + 1] = n;
   __syncthreads();
+#pragma unroll 8
   for (int i = t; i < n; i += kNnThreads) {
     const float x = px[i], y = py[i];
     const size_t o = (size_t)b * n + atomicAdd(&s_cnt[cell_of(x, y)], 1);

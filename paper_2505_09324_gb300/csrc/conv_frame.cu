@@ -134,6 +134,7 @@ k_conv_frame(const __grid_constant__ CUtensorMap tf256, const __grid_constant__ 
   // planes and mask alike); 128 otherwise
   constexpr int kTW = PAR ? 120 : kBM;
   using Sm = FrameSmem<PAR>;
+  pdl_begin();
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t raw_full[kRawStages], raw_empty[kRawStages];
   __shared__ __align__(8) uint64_t a_empty[kAStages];
@@ -480,9 +481,8 @@ cudaError_t launch_frame(const CUtensorMap (&maps)[5], const FrameArgs& g, int s
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     sms = 1;
   const int grid = std::max(1, std::min(g.tiles, sms));
-  k_conv_frame<BN, PAR><<<grid, kFrThreads, smem, s>>>(maps[0], maps[1], maps[2], maps[3],
-                                                        maps[4], g);
-  return cudaGetLastError();
+  return launch_pdl(k_conv_frame<BN, PAR>, grid, kFrThreads, smem, s, maps[0], maps[1], maps[2],
+                    maps[3], maps[4], g);
 }
 
 }  // namespace

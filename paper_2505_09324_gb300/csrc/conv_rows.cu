@@ -101,6 +101,7 @@ k_conv_rows(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUte
   using Sh = RowsShape<BN>;
   constexpr bool kRes = PER == 1;                 // weights resident
   constexpr int kBoxes = C == 32 ? 1 : C / 32;    // boxes per A slot
+  pdl_begin();
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t a_full[kMaxA], a_empty[kMaxA], b_full[kMaxB], b_empty[kMaxB];
   __shared__ __align__(8) uint64_t acc_full[Sh::kAcc], acc_empty[Sh::kAcc], bres_full;
@@ -445,8 +446,7 @@ cudaError_t launch_rows_per(const CUtensorMap& ta, const CUtensorMap& tb, const 
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     sms = 1;
   const int grid = std::max(1, std::min(g.tiles, sms));
-  k_conv_rows<BN, PER, C><<<grid, kThreads, smem, s>>>(ta, tb, g);
-  return cudaGetLastError();
+  return launch_pdl(k_conv_rows<BN, PER, C>, grid, kThreads, smem, s, ta, tb, g);
 }
 
 // Whether the weights of a C-channel layer with BN-column tiles stay

@@ -69,7 +69,7 @@ struct TapArgs {
   int Ho, Wo, ks, stride, pad;
   int N, ldc, relu;
   int segs, tiles, nk;
-  int rows, hp;                     // output rows per tile (1, or 2 of 64 pixels), tiles down an image
+  int rows, hp;                     // output rows per tile (1, or 2 of 64 pixels), tiles down
   int nblk;                         // blocks of BN output channels
   int cw, cpt, blocks_real, kbias;  // channels per block, blocks per tap, tap blocks, bias k
   int stages, resident_b;
@@ -113,6 +113,7 @@ __global__ void __launch_bounds__(kTapThreads, 1)
 k_conv_tap(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb,
            TapArgs g) {
   using Sh = TapShape<BN>;
+  pdl_begin();
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t full[kMaxStages], empty[kMaxStages];
   __shared__ __align__(8) uint64_t acc_full[Sh::kAcc], acc_empty[Sh::kAcc], bres_full;
@@ -414,8 +415,7 @@ cudaError_t launch_tap_per(const CUtensorMap& ta, const CUtensorMap& tb, const T
   if (attr != cudaSuccess) return attr;
   const int sms = sm_count();
   const int grid = std::max(1, std::min(g.tiles, sms > 0 ? sms : 1) / g.nblk) * g.nblk;
-  k_conv_tap<BN, PER><<<grid, kTapThreads, smem, s>>>(ta, tb, g);
-  return cudaGetLastError();
+  return launch_pdl(k_conv_tap<BN, PER>, grid, kTapThreads, smem, s, ta, tb, g);
 }
 
 template <int BN>

@@ -104,6 +104,7 @@ template <int BN, int ST>
 __global__ void __launch_bounds__(128, 1)
 k_gemm_bf16(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb,
             TcGemmArgs g) {
+  pdl_begin();
   constexpr int kStages = ST;
   using Sh = GemmShape<BN, ST>;
   extern __shared__ uint8_t smem_raw[];
@@ -206,6 +207,7 @@ struct ConvGeom {
 template <int BN, int ST>
 __global__ void __launch_bounds__(160, 1)
 k_conv_bf16(const __grid_constant__ CUtensorMap tb, ConvGeom cg, TcGemmArgs g) {
+  pdl_begin();
   constexpr int kStages = ST;
   using Sh = GemmShape<BN, ST>;
   extern __shared__ uint8_t smem_raw[];
@@ -347,6 +349,7 @@ k_conv_bf16(const __grid_constant__ CUtensorMap tb, ConvGeom cg, TcGemmArgs g) {
 // Sum of the split-K partials in split order, then bias, ReLU and the store.
 __global__ void __launch_bounds__(256)
 k_splitk_reduce(TcGemmArgs g, int splits, const float* __restrict__ partial) {
+  pdl_begin();
   const size_t total = (size_t)g.M * g.N;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total;
        i += (size_t)gridDim.x * blockDim.x) {
@@ -368,8 +371,7 @@ cudaError_t launch_bn_st(const CUtensorMap& ta, const CUtensorMap& tb, const TcG
                          dim3 grid, cudaStream_t s) {
   const cudaError_t attr = opt_in_smem((const void*)k_gemm_bf16<BN, ST>, GemmShape<BN, ST>::kSmem);
   if (attr != cudaSuccess) return attr;
-  k_gemm_bf16<BN, ST><<<grid, 128, GemmShape<BN, ST>::kSmem, s>>>(ta, tb, g);
-  return cudaGetLastError();
+  return launch_pdl(k_gemm_bf16<BN, ST>, grid, 128, GemmShape<BN, ST>::kSmem, s, ta, tb, g);
 }
 
 template <int BN, int ST>
@@ -377,8 +379,7 @@ cudaError_t launch_conv_st(const CUtensorMap& tb, const ConvGeom& cg, const TcGe
                            dim3 grid, cudaStream_t s) {
   const cudaError_t attr = opt_in_smem((const void*)k_conv_bf16<BN, ST>, GemmShape<BN, ST>::kSmem);
   if (attr != cudaSuccess) return attr;
-  k_conv_bf16<BN, ST><<<grid, 160, GemmShape<BN, ST>::kSmem, s>>>(tb, cg, g);
-  return cudaGetLastError();
+  return launch_pdl(k_conv_bf16<BN, ST>, grid, 160, GemmShape<BN, ST>::kSmem, s, tb, cg, g);
 }
 
 // Two stages up to 16 k-tiles, three beyond: shared memory for more CTAs per
@@ -500,8 +501,7 @@ cudaError_t tc_gemm(const TcGemmProblem& pr, cudaStream_t s) {
   r.relu = pr.relu;
   const size_t total = (size_t)pr.M * pr.N;
   const int blocks = (int)std::min<size_t>((total + 255) / 256, 152 * 16);
-  k_splitk_reduce<<<blocks, 256, 0, s>>>(r, splits, pr.partial);
-  return cudaGetLastError();
+  return launch_pdl(k_splitk_reduce, blocks, 256, 0, s, r, splits, (const float*)pr.partial);
 }
 
 cudaError_t tc_conv(const TcConvProblem& pr, cudaStream_t s) {

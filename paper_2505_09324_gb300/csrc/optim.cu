@@ -17,6 +17,7 @@ __global__ void __launch_bounds__(256)
 k_adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
        float* __restrict__ v, int64_t count, int64_t per_row, const uint8_t* __restrict__ mask,
        float lr, float b1, float b2, float eps, float ibc1, float ibc2) {
+  pdl_begin();
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < count;
        k += (int64_t)gridDim.x * blockDim.x) {
     if (mask && !mask[k % per_row]) continue;
@@ -32,6 +33,7 @@ __global__ void __launch_bounds__(256)
 k_adam4(float4* __restrict__ p, const float4* __restrict__ g, float4* __restrict__ m,
         float4* __restrict__ v, int64_t count4, float lr, float b1, float b2, float eps,
         float ibc1, float ibc2) {
+  pdl_begin();
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < count4;
        k += (int64_t)gridDim.x * blockDim.x) {
     float4 pp = p[k], mm = m[k], vv = v[k];
@@ -58,9 +60,9 @@ cudaError_t launch_adam(float* params, const float* grads, float* m, float* v, i
     const int64_t c4 = count / 4;
     int64_t blocks = (c4 + 255) / 256;
     if (blocks > 152 * 16) blocks = 152 * 16;
-    k_adam4<<<(int)blocks, 256, 0, s>>>((float4*)params, (const float4*)grads, (float4*)m,
-                                        (float4*)v, c4, cfg.lr, cfg.beta1, cfg.beta2, cfg.eps,
-                                        ibc1, ibc2);
+    return launch_pdl(k_adam4, (int)blocks, 256, 0, s, (float4*)params, (const float4*)grads,
+                      (float4*)m, (float4*)v, c4, cfg.lr, cfg.beta1, cfg.beta2, cfg.eps, ibc1,
+                      ibc2);
   } else {
     int64_t blocks = (count + 255) / 256;
     if (blocks > 152 * 16) blocks = 152 * 16;
