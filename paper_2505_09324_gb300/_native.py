@@ -34,7 +34,9 @@ EXPORTS = (
     "gs2d_encode_batch",
     "gs2d_autotune_ws_bytes", "gs2d_autotune",
     "gs2d_gemm_bf16", "gs2d_gemm_partial_bytes", "gs2d_cnn_input", "gs2d_conv_frame_bf16",
-    "gs2d_conv_wait_check", "gs2d_gemm_tn_bf16", "gs2d_gemm_tn_partial_bytes", "gs2d_conv_dgrad_bf16", "gs2d_im2col", "gs2d_col2im",
+    "gs2d_conv_wait_check", "gs2d_gemm_tn_bf16", "gs2d_gemm_tn_partial_bytes",
+    "gs2d_conv_dgrad_bf16", "gs2d_conv_wgrad_supported", "gs2d_conv_wgrad_partial_bytes",
+    "gs2d_conv_wgrad_bf16", "gs2d_im2col", "gs2d_col2im",
     "gs2d_transpose_bf16", "gs2d_relu_bwd", "gs2d_cast_weights", "gs2d_head_decode",
     "gs2d_head_smem_bytes", "gs2d_head_decode_bwd", "gs2d_chamfer", "gs2d_chamfer_scratch_bytes",
     "gs2d_read_bins", "gs2d_count_pairs", "gs2d_ws_status",
@@ -203,6 +205,9 @@ def load(build_if_missing: bool = False):
             "gs2d_gemm_tn_bf16": (i32, [P, i32, P, i32, i32, i32, i32, P, i32, i32, P, P, P]),
             "gs2d_gemm_tn_partial_bytes": (ctypes.c_uint64, [i32, i32, i32, i32, i32]),
             "gs2d_conv_dgrad_bf16": (i32, [P, i32, i32, i32, i32, P, i32, P, P, P, P]),
+            "gs2d_conv_wgrad_supported": (i32, [i32, i32, i32, i32, i32]),
+            "gs2d_conv_wgrad_partial_bytes": (ctypes.c_uint64, [i32] * 7),
+            "gs2d_conv_wgrad_bf16": (i32, [P, i32, P, i32, i32, i32, i32, P, i32, i32, P, P, P]),
             "gs2d_im2col": (i32, [P, i32, i32, i32, i32, i32, i32, i32, P, i32, P]),
             "gs2d_col2im": (i32, [P, i32, i32, i32, i32, i32, i32, i32, i32, P, P, P]),
             "gs2d_transpose_bf16": (i32, [P, i32, i32, i32, P, i32, P]),

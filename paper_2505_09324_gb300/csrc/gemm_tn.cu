@@ -1,5 +1,6 @@
 // BF16 tensor-core GEMM over the rows of both operands (tcgen05), the weight
-// gradient of the learned initialiser's layers:
+// gradient of the learned initialiser's head and of the layers that
+// csrc/conv_wgrad.cu has no form for:
 //
 //   C[M][N] = sum_p A[p][m] B[p][n]     A [K][lda], B [K][ldb] bf16, FP32 accumulation
 //
@@ -28,6 +29,7 @@
 #include <stdio.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "gs2d_internal.cuh"
 #include "tc_gemm.cuh"
@@ -55,20 +57,6 @@ struct TnArgs {
   float* out;  // partials, or the result when there is one split
   int* status;
 };
-
-// MN-major operand in the 128-byte swizzle layout: 64 contiguous elements (one
-// 128-byte row) per k, 8-row groups 1024 bytes apart along k (the stride
-// offset), the next 64 elements of m or n `chunk` bytes on (the leading
-// offset); descriptor version 1.
-__device__ __forceinline__ uint64_t mn_major_desc(uint32_t addr, uint32_t chunk) {
-  return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)((chunk >> 4) & 0x3FFFu) << 16) |
-         ((uint64_t)(1024 >> 4) << 32) | ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
-}
-
-// Both operands MN-major: the transpose bits 15 and 16.
-__host__ __device__ constexpr uint32_t idesc_bf16_mn(int m, int n) {
-  return idesc_bf16(m, n) | (1u << 15) | (1u << 16);
-}
 
 template <int NA, int NB>
 __global__ void __launch_bounds__(128, 1)
@@ -141,8 +129,8 @@ k_gemm_tn(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtens
       tc_fence_after();
       const uint32_t a_s = smem_u32(smem + s * Sh::kStageBytes), b_s = a_s + NA * kTnBox;
       // one A box: rows 64 ... 127 of the tile read the same columns again
-      const uint64_t ad = mn_major_desc(a_s, NA > 1 ? kTnBox : 0);
-      const uint64_t bd = mn_major_desc(b_s, kTnBox), bd2 = bd + 4 * (kTnBox >> 4);
+      const uint64_t ad = mn_major_desc(a_s, NA > 1 ? kTnBox : 0, 128);
+      const uint64_t bd = mn_major_desc(b_s, kTnBox, 128), bd2 = bd + 4 * (kTnBox >> 4);
 #pragma unroll
       for (int kk = 0; kk < kTnRows / 16; kk++) {  // 16 rows of 128 bytes: 128 units
         const uint32_t acc = (i > 0 || kk > 0) ? 1u : 0u;
@@ -175,28 +163,69 @@ k_gemm_tn(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtens
   if (threadIdx.x == 0 && s_fail && g.status) atomicCAS(g.status, 0, (int)GS2D_ERR_TIMEOUT);
 }
 
-// Sum of the partial tiles: 32 outputs x 8 slices of the splits per block, the
-// slices' sums added in a fixed order (deterministic).
+// Sum of the partial tiles: a block takes 256 / SL vectors of V outputs, in SL
+// slices of the splits whose sums are added in a fixed order (deterministic),
+// with up to eight loads in flight per thread.  SL is chosen so that a thread
+// sums at most about 20 splits: one scheme of 8 slices left the many-split
+// layers waiting on a few loads (75 splits a thread, 80 blocks) and gave the
+// few-split layers a barrier and a division for every one or two of them.  The
+// training step's six reductions at 1080p, batch 8: 294 -> 206 us, each with
+// its wait for the kernel before it.
+template <int SL, int V>
 __global__ void __launch_bounds__(256)
-k_tn_reduce(int M, int N, int ldc, int splits, size_t stride, const float* __restrict__ partial,
-            float* __restrict__ out) {
+k_tn_reduce(uint32_t M, uint32_t nv, uint32_t ldv, int splits, size_t stride,
+            const float* __restrict__ partial, float* __restrict__ out) {
+  using Vec = std::conditional_t<V == 4, float4, float>;
+  constexpr int kOut = 256 / SL;
   pdl_begin();
-  __shared__ float s_sum[8][33];
-  const int lane = threadIdx.x & 31, slice = threadIdx.x >> 5;
-  const size_t i = (size_t)blockIdx.x * 32 + lane, total = (size_t)M * N;
-  const size_t o = i < total ? (i / N) * ldc + i % N : 0;
-  float x = 0.0f;
-  if (i < total) {
-#pragma unroll 4
-    for (int z = slice; z < splits; z += 8) x += partial[(size_t)z * stride + o];
-  }
-  s_sum[slice][lane] = x;
-  __syncthreads();
-  if (slice == 0 && i < total) {
+  __shared__ float s_sum[SL > 1 ? SL - 1 : 1][kOut * V];
+  const uint32_t k = threadIdx.x % kOut, slice = threadIdx.x / kOut;
+  const size_t i = (size_t)blockIdx.x * kOut + k;
+  const bool in = i < (size_t)M * nv;
+  size_t o = i;
+  if (nv != ldv) o = in ? (i / nv) * ldv + i % nv : 0;
+  const Vec* src = reinterpret_cast<const Vec*>(partial) + o;
+  const size_t step = stride / V;
+  float x[V];
 #pragma unroll
-    for (int k = 1; k < 8; k++) x += s_sum[k][lane];
-    out[o] = x;
+  for (int j = 0; j < V; j++) x[j] = 0.0f;
+  if (in) {
+#pragma unroll 8
+    for (int z = (int)slice; z < splits; z += SL) {
+      const Vec v = src[(size_t)z * step];
+      const float* f = reinterpret_cast<const float*>(&v);
+#pragma unroll
+      for (int j = 0; j < V; j++) x[j] += f[j];
+    }
   }
+  if constexpr (SL > 1) {
+    if (slice > 0)
+#pragma unroll
+      for (int j = 0; j < V; j++) s_sum[slice - 1][k * V + j] = x[j];
+    __syncthreads();
+    if (slice > 0) return;
+#pragma unroll
+    for (int z = 0; z < SL - 1; z++)
+#pragma unroll
+      for (int j = 0; j < V; j++) x[j] += s_sum[z][k * V + j];
+  }
+  if (in) {
+    Vec v;
+#pragma unroll
+    for (int j = 0; j < V; j++) reinterpret_cast<float*>(&v)[j] = x[j];
+    reinterpret_cast<Vec*>(out)[o] = v;
+  }
+}
+
+template <int SL>
+cudaError_t launch_reduce(int M, int N, int ldc, int splits, size_t stride, const float* partial,
+                          float* out, cudaStream_t s) {
+  const bool vec = N % 4 == 0 && ldc % 4 == 0 && stride % 4 == 0 &&
+                   (((uintptr_t)partial | (uintptr_t)out) & 15) == 0;
+  const int v = vec ? 4 : 1;
+  const unsigned blocks = (unsigned)(((size_t)M * (N / v) + 256 / SL - 1) / (256 / SL));
+  return launch_pdl(vec ? k_tn_reduce<SL, 4> : k_tn_reduce<SL, 1>, blocks, 256, 0, s, (uint32_t)M,
+                    (uint32_t)(N / v), (uint32_t)(ldc / v), splits, stride, partial, out);
 }
 
 // 2D map of a rows x cols matrix (cols contiguous): 64 x 128 boxes, 128-byte
@@ -215,30 +244,21 @@ bool tn_map(CUtensorMap* map, const void* base, int rows, int cols, int ld) {
 }
 
 // Tile width and split of one product.  NB: as wide as shared memory allows (B
-// read fewest times), in even tiles.  splits: at least min_splits (the FP32
-// sums in tensor memory lose precision with their length, so the caller says
-// how short they are to be), and more where that completes the last wave of
-// 152 CTAs, one k-tile each at most.
+// read fewest times), in even tiles.
 struct TnPlan {
-  int na, nb, mt, nt, num_kt, per, splits;
+  int na, nb, mt, nt;
+  TnSplit sp;
 };
 
 TnPlan tn_plan(int M, int N, int K, int min_splits) {
   TnPlan p;
   p.na = M <= 64 ? 1 : 2;
   p.mt = (M + 64 * p.na - 1) / (64 * p.na);
-  p.num_kt = (K + kTnRows - 1) / kTnRows;
   const int chunks = (N + 63) / 64, widest = p.na == 1 ? 5 : 4;
   p.nt = (chunks + widest - 1) / widest;
   p.nb = (chunks + p.nt - 1) / p.nt;
   p.nt = (chunks + p.nb - 1) / p.nb;
-  const int64_t tiles = (int64_t)p.mt * p.nt;
-  const int64_t need = std::max<int64_t>(1, std::min<int64_t>(min_splits, p.num_kt));
-  const int64_t waves = (need * tiles + 151) / 152;
-  const int64_t most = std::min<int64_t>(p.num_kt, 65535);  // gridDim.z
-  p.splits = (int)std::min(most, std::max(need, waves * 152 / tiles));
-  p.per = (p.num_kt + p.splits - 1) / p.splits;
-  p.splits = (p.num_kt + p.per - 1) / p.per;
+  p.sp = tn_split((int64_t)p.mt * p.nt, (K + kTnRows - 1) / kTnRows, min_splits);
   return p;
 }
 
@@ -264,6 +284,27 @@ cudaError_t launch_tn_na(int nb, const CUtensorMap& ta, const CUtensorMap& tb, c
 }
 
 }  // namespace
+
+TnSplit tn_split(int64_t tiles, int num_kt, int min_splits) {
+  TnSplit p;
+  p.num_kt = num_kt;
+  const int64_t need = std::max<int64_t>(1, std::min<int64_t>(min_splits, num_kt));
+  const int64_t waves = (need * tiles + 151) / 152;
+  const int64_t most = std::min<int64_t>(num_kt, 65535);  // gridDim.z
+  p.splits = (int)std::min(most, std::max(need, waves * 152 / tiles));
+  p.per = (num_kt + p.splits - 1) / p.splits;
+  p.splits = (num_kt + p.per - 1) / p.per;
+  return p;
+}
+
+cudaError_t launch_tn_reduce(int M, int N, int ldc, int splits, size_t stride,
+                             const float* partial, float* out, cudaStream_t s) {
+  if (splits <= 20) return launch_reduce<1>(M, N, ldc, splits, stride, partial, out, s);
+  if (splits <= 80) return launch_reduce<4>(M, N, ldc, splits, stride, partial, out, s);
+  if (splits <= 240) return launch_reduce<8>(M, N, ldc, splits, stride, partial, out, s);
+  return launch_reduce<32>(M, N, ldc, splits, stride, partial, out, s);
+}
+
 }  // namespace gs2d
 
 using namespace gs2d;
@@ -272,7 +313,7 @@ extern "C" uint64_t gs2d_gemm_tn_partial_bytes(int32_t M, int32_t N, int32_t ldc
                                                int32_t min_splits) {
   if (M < 1 || N < 1 || K < 1 || ldc < N) return 0;
   const TnPlan p = tn_plan(M, N, K, min_splits);
-  return p.splits > 1 ? (uint64_t)p.splits * M * ldc * sizeof(float) : 0;
+  return p.sp.splits > 1 ? (uint64_t)p.sp.splits * M * ldc * sizeof(float) : 0;
 }
 
 extern "C" gs2d_status gs2d_gemm_tn_bf16(const void* A, int32_t lda, const void* B, int32_t ldb,
@@ -290,7 +331,7 @@ extern "C" gs2d_status gs2d_gemm_tn_bf16(const void* A, int32_t lda, const void*
     e = cudaMemset2DAsync(out, (size_t)ldc * 4, 0, (size_t)N * 4, M, s);
   } else {
     const TnPlan p = tn_plan(M, N, K, min_splits);
-    if (p.splits > 1 && !partial)
+    if (p.sp.splits > 1 && !partial)
       return set_error(GS2D_ERR_INVALID_ARG, "gs2d_gemm_tn_bf16: the split needs partial");
     CUtensorMap ta, tb;
     if (!tn_map(&ta, A, K, M, lda) || !tn_map(&tb, B, K, N, ldb))
@@ -298,18 +339,17 @@ extern "C" gs2d_status gs2d_gemm_tn_bf16(const void* A, int32_t lda, const void*
     TnArgs g;
     g.M = M;
     g.N = N;
-    g.num_kt = p.num_kt;
-    g.kt_per_split = p.per;
+    g.num_kt = p.sp.num_kt;
+    g.kt_per_split = p.sp.per;
     g.ldc = ldc;
-    g.split_stride = p.splits > 1 ? (size_t)M * ldc : 0;
-    g.out = p.splits > 1 ? partial : out;
+    g.split_stride = p.sp.splits > 1 ? (size_t)M * ldc : 0;
+    g.out = p.sp.splits > 1 ? partial : out;
     g.status = status;
-    const dim3 grid(p.mt, p.nt, p.splits);
+    const dim3 grid(p.mt, p.nt, p.sp.splits);
     e = p.na == 1 ? launch_tn_na<1>(p.nb, ta, tb, g, grid, s)
                   : launch_tn_na<2>(p.nb, ta, tb, g, grid, s);
-    if (e == cudaSuccess && p.splits > 1)
-      e = launch_pdl(k_tn_reduce, (unsigned)(((size_t)M * N + 31) / 32), 256, 0, s, (int)M, (int)N,
-                     (int)ldc, p.splits, g.split_stride, (const float*)partial, out);
+    if (e == cudaSuccess && p.sp.splits > 1)
+      e = launch_tn_reduce(M, N, ldc, p.sp.splits, g.split_stride, partial, out, s);
   }
   if (e != cudaSuccess) {
     char msg[200];

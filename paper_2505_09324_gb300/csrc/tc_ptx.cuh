@@ -1,8 +1,8 @@
 // Inline-PTX building blocks of the tcgen05 kernels (csrc/gemm_tc.cu,
-// csrc/conv_tap.cu, csrc/conv_rows.cu, csrc/conv_frame.cu): mbarriers with
-// time-bounded waits, TMA tensor loads, shared-memory matrix descriptors,
-// tcgen05.mma / commit / ld and the
-// tcgen05 thread-sync fences.
+// csrc/conv_tap.cu, csrc/conv_rows.cu, csrc/conv_frame.cu, csrc/conv_dgrad.cu,
+// csrc/gemm_tn.cu, csrc/conv_wgrad.cu): mbarriers with time-bounded waits, TMA
+// tensor loads, shared-memory matrix descriptors, tcgen05.mma / commit / ld and
+// the tcgen05 thread-sync fences.
 #pragma once
 
 #include <cuda.h>
@@ -125,6 +125,19 @@ __device__ __forceinline__ uint64_t sw128_desc(uint32_t addr) {
 __host__ __device__ constexpr uint32_t idesc_bf16(int m, int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) |
          ((uint32_t)(m >> 4) << 24);
+}
+
+// MN-major operand in a swizzled layout of `row` (128, 64 or 32) bytes: row / 2
+// contiguous elements of m or n per k, 8-row groups 8 rows apart along k (the
+// stride offset), the next row / 2 elements of m or n `chunk` bytes on (the
+// leading offset); descriptor version 1.
+__device__ __forceinline__ uint64_t mn_major_desc(uint32_t addr, uint32_t chunk, uint32_t row) {
+  return kmajor_desc(addr, chunk, 8 * row, row == 128 ? 2 : row == 64 ? 4 : 6);
+}
+
+// Both operands MN-major: the transpose bits 15 and 16.
+__host__ __device__ constexpr uint32_t idesc_bf16_mn(int m, int n) {
+  return idesc_bf16(m, n) | (1u << 15) | (1u << 16);
 }
 
 __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc,

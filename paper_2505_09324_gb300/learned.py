@@ -13,11 +13,11 @@ Every convolution is a BF16 tensor-core GEMM over its im2col operand (the
 bias a weight column against a column of ones), run as an implicit GEMM that
 reads its operands straight from the activations (gs2d_conv_bf16,
 gs2d_conv_frame_bf16; the same sums in the same order as gs2d_gemm_bf16 on
-the operand); training also writes the operand out for the backward pass.  The backward pass is one
-weight-gradient GEMM (dZ^T . col, both read as they lie, split over pixels;
-gs2d_gemm_tn_bf16) and one input gradient with the ReLU mask per layer: one
-implicit GEMM over shifted dZ boxes where rows are wide
-(gs2d_conv_dgrad_bf16), else a GEMM (dZ . W) + col2im.  The optimiser is the
+the operand).  The backward pass is one weight gradient (dZ^T . col, split over
+pixels: straight from the activations by gs2d_conv_wgrad_bf16, else from the
+operand, which the forward pass then writes, by gs2d_gemm_tn_bf16) and one
+input gradient with the ReLU mask per layer: one implicit GEMM over shifted dZ
+boxes where rows are wide (gs2d_conv_dgrad_bf16), else a GEMM (dZ . W) + col2im.  The optimiser is the
 library's Adam on the FP32 master weights.  Training minimises the L2 render
 loss of the decoded Gaussians through the rasterizer (the colour and shape
 signal the paper's regressor lacked) plus lambda times the Chamfer distance
@@ -52,6 +52,31 @@ class NetConfig:
     lr: float = 1e-3
     chamfer_lambda: float = 1e-5
     wgrad_split_pixels: int = 4096  # pixels per split of the weight-gradient GEMMs
+
+
+class _Columns:
+    """The layers' im2col operands of the last forward, [pixels, ldk] each:
+    those that a kernel reads are written by forward(), the others when asked
+    for."""
+
+    def __init__(self, net: "LearnedInitializer"):
+        self._net = net
+
+    def __len__(self):
+        return len(self._net.layers)
+
+    def __getitem__(self, li: int) -> torch.Tensor:
+        li = range(len(self))[li]
+        net = self._net
+        if net._col[li] is not None and not net._implicit_wgrad(li):
+            return net._col[li]
+        ci, co, ks, ldk = net.layers[li]
+        hi, wi = net.sizes[li] if li < net.L else net.sizes[-1]
+        col = torch.empty((net.dz[li].shape[0], ldk), dtype=torch.bfloat16, device=net.dev)
+        stride, pad = (2, 1) if ks == 3 else (1, 0)
+        nat.call("gs2d_im2col", net.x[li].data_ptr(), net.B, hi, wi, ci, ks, stride, pad,
+                 col.data_ptr(), ldk, net._s())
+        return col
 
 
 class LearnedInitializer:
@@ -102,11 +127,14 @@ class LearnedInitializer:
     def _alloc(self):
         B, dev, bf = self.B, self.dev, torch.bfloat16
         self.x = [torch.empty((B * self.H * self.W, 8), dtype=bf, device=dev)]
-        self.col, self.dz, self.dcol = [], [], []
+        self.col = _Columns(self)
+        self._col, self.dz, self.dcol = [], [], []
         for li, (ci, co, ks, ldk) in enumerate(self.layers):
             h, w = self.sizes[li + 1] if li < self.L else self.sizes[-1]
             P = B * h * w
-            self.col.append(torch.empty((P, ldk), dtype=bf, device=dev))
+            # (the operand only where some kernel reads it)
+            needed = not self._implicit_wgrad(li) or not self._implicit_conv(li)
+            self._col.append(torch.empty((P, ldk), dtype=bf, device=dev) if needed else None)
             self.dz.append(torch.empty((P, co), dtype=bf, device=dev))
             self.dcol.append(torch.empty((P, ldk), device=dev)
                              if li > 0 and not self._implicit_dgrad(li) else None)
@@ -120,9 +148,28 @@ class LearnedInitializer:
         for li, (ci, co, ks, ldk) in enumerate(self.layers):
             h, w = self.sizes[li + 1] if li < self.L else self.sizes[-1]
             P = B * h * w
-            most = max(most, nat.load().gs2d_gemm_tn_partial_bytes(co, ldk, ldk, P,
-                                                                    self._splits(P)))
+            if self._implicit_wgrad(li):
+                need = nat.load().gs2d_conv_wgrad_partial_bytes(B, *self.sizes[li], ci, co, ldk,
+                                                                self._splits(P))
+            else:
+                need = nat.load().gs2d_gemm_tn_partial_bytes(co, ldk, ldk, P, self._splits(P))
+            most = max(most, need)
         self.partial = torch.empty(max(most // 4, 1), device=dev)
+
+    def _implicit_conv(self, li: int) -> bool:
+        """Whether layer li's forward runs as an implicit GEMM: unless K is very
+        deep and the output rows short (37 k-tiles over few tiles of gathered
+        operands: the TMA-fed GEMM over an im2col operand is faster there; from
+        49 pixels the TMA taps serve two rows a tile)."""
+        wo = self.sizes[li + 1][1] if li < self.L else self.sizes[-1][1]
+        return (self.layers[li][3] + 63) // 64 <= 32 or wo >= 49
+
+    def _implicit_wgrad(self, li: int) -> bool:
+        """Whether layer li's weight gradient reads the activations themselves
+        (gs2d_conv_wgrad_bf16, wherever it has a form for the layer)."""
+        ci, co, ks, ldk = self.layers[li]
+        return ks == 3 and bool(nat.load().gs2d_conv_wgrad_supported(self.B, *self.sizes[li], ci,
+                                                                     co))
 
     def _implicit_dgrad(self, li: int) -> bool:
         """Whether layer li's input gradient runs as gs2d_conv_dgrad_bf16: the
@@ -156,7 +203,8 @@ class LearnedInitializer:
         (gs2d_conv_bf16; the first one, gs2d_conv_frame_bf16, straight from
         the frames when W is a multiple of 16; the same result bit for bit)
         and keeps neither the im2col operands nor the 8-channel input, which
-        backward() needs."""
+        backward() reads (the operands of layers without an implicit weight
+        gradient only)."""
         B, s = self.B, self._s()
         if tuple(frames.shape) != (B, 3, self.H, self.W) or frames.dtype != torch.float32:
             raise ValueError("frames must be [B, 3, H, W] float32")
@@ -182,17 +230,11 @@ class LearnedInitializer:
             last = li == self.L
             out32 = self.out.data_ptr() if last else 0
             out16 = 0 if last else self.x[li + 1].data_ptr()
-            # implicit GEMM unless K is very deep and the output rows short
-            # (37 k-tiles over few tiles of gathered operands: the TMA-fed GEMM
-            # over an im2col operand is faster there; from 49 pixels the TMA
-            # taps serve two rows a tile); the results are identical either
-            # way, so training too only writes the operand (for backward) and
-            # does not read it back here
-            wo = self.sizes[li + 1][1] if li < self.L else wi
-            implicit = (ldk + 63) // 64 <= 32 or wo >= 49
-            if keep_col or not implicit:
+            # (the results are identical either way)
+            implicit = self._implicit_conv(li)
+            if not implicit or (keep_col and not self._implicit_wgrad(li)):
                 nat.call("gs2d_im2col", src.data_ptr(), B, hi, wi, ci, ks, stride, pad,
-                         self.col[li].data_ptr(), ldk, s)
+                         self._col[li].data_ptr(), ldk, s)
             if li == 0 and from_frames:
                 nat.call("gs2d_conv_frame_bf16", frames.data_ptr(), mptr, B, self.H, self.W, 3, 2,
                          1, self.wb[0].data_ptr(), ldk, co, 1, 0, out16, co, st, s)
@@ -201,9 +243,9 @@ class LearnedInitializer:
                          self.wb[li].data_ptr(), ldk, co, 0 if last else 1, out32, out16, co, st,
                          s)
             else:
-                nat.gemm_bf16(self.col[li].data_ptr(), ldk, self.wb[li].data_ptr(), ldk,
-                              self.col[li].shape[0], co, ldk, 0, not last, out32, out16, co, 1, 0,
-                              st, s)
+                nat.gemm_bf16(self._col[li].data_ptr(), ldk, self.wb[li].data_ptr(), ldk,
+                              self._col[li].shape[0], co, ldk, 0, not last, out32, out16, co, 1,
+                              0, st, s)
         c = self.cfg
         nat.call("gs2d_head_decode", self.out.data_ptr(), self.ldo, B, self.gh, self.gw, c.slots,
                  self.cell, c.scale, self.n, self.params.data_ptr(), B * self.n,
@@ -244,14 +286,19 @@ class LearnedInitializer:
                  dparams.contiguous().data_ptr(), B * self.n, self.dz[self.L].data_ptr(), s)
         for li in range(self.L, -1, -1):
             ci, co, ks, ldk = self.layers[li]
-            P = self.col[li].shape[0]
+            P = self.dz[li].shape[0]
+            hi, wi = self.sizes[li] if li < self.L else self.sizes[-1]
             # weight gradient: dW[co][k] = sum_p dZ[p][co] col[p][k]
-            nat.call("gs2d_gemm_tn_bf16", self.dz[li].data_ptr(), co, self.col[li].data_ptr(),
-                     ldk, co, ldk, P, self.dw[li].data_ptr(), ldk, self._splits(P),
-                     self.partial.data_ptr(), st, s)
+            if self._implicit_wgrad(li):
+                nat.call("gs2d_conv_wgrad_bf16", self.dz[li].data_ptr(), co,
+                         self.x[li].data_ptr(), B, hi, wi, ci, self.dw[li].data_ptr(), ldk,
+                         self._splits(P), self.partial.data_ptr(), st, s)
+            else:
+                nat.call("gs2d_gemm_tn_bf16", self.dz[li].data_ptr(), co,
+                         self._col[li].data_ptr(), ldk, co, ldk, P, self.dw[li].data_ptr(), ldk,
+                         self._splits(P), self.partial.data_ptr(), st, s)
             if li == 0:
                 break
-            hi, wi = self.sizes[li] if li < self.L else self.sizes[-1]
             # input gradient, times the ReLU mask of that input
             if self._implicit_dgrad(li):
                 nat.call("gs2d_conv_dgrad_bf16", self.dz[li].data_ptr(), B, hi, wi, ci,

@@ -476,6 +476,36 @@ def test_gemm_over_rows_matches_oracle(nat, M, N, K, splits):
         assert np.all(np.isnan(got[:, N:]))
 
 
+@pytest.mark.parametrize("B,H,W,C,N,splits", [
+    (1, 7, 258, 64, 40, 3),      # pairs, two steps a row, odd rows
+    (2, 9, 129, 64, 200, 1),     # odd width: traversal stride; two blocks of M, ragged
+    (3, 21, 34, 128, 64, 2),     # 17 pixels: four rows a step, ragged rows
+    (1, 50, 9, 192, 128, 40),    # eight rows a step, more splits than steps
+    (2, 6, 300, 32, 64, 5), (1, 11, 64, 32, 136, 1),     # pairs of 32 channels
+    (2, 6, 514, 8, 32, 7), (1, 33, 62, 8, 64, 1), (1, 1, 2, 8, 8, 1)])  # pairs of 8
+def test_conv_weight_gradient_matches_oracle(nat, B, H, W, C, N, splits):
+    """gs2d_conv_wgrad_bf16 (3 x 3, stride 2, pad 1) against dZ^T im2col(x), the
+    bias column and the zeros beyond it, within the GEMM bar, for each of its
+    forms."""
+    g = np.random.Generator(np.random.PCG64(H * W + C + N))
+    Ho, Wo, ldc = (H + 1) // 2, (W + 1) // 2, 9 * C + 8
+    dz = cnn.bf16_round(g.normal(size=(B * Ho * Wo, N)))
+    x = cnn.bf16_round(g.normal(size=(B, H, W, C)))
+    col = cnn.im2col(x, 3, 2, 1, ldc)
+    lib = nat.load()
+    assert lib.gs2d_conv_wgrad_supported(B, H, W, C, N) == 1
+    part = torch.empty(max(lib.gs2d_conv_wgrad_partial_bytes(B, H, W, C, N, ldc, splits) // 4, 1),
+                       device="cuda")
+    out = torch.full((N, ldc), float("nan"), device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    d_dz, d_x = bf16_dev(dz), bf16_dev(x)
+    nat.call("gs2d_conv_wgrad_bf16", d_dz.data_ptr(), N, d_x.data_ptr(), B, H, W, C,
+             out.data_ptr(), ldc, splits, part.data_ptr(), status.data_ptr(), 0)
+    got = out.cpu().numpy().astype(np.float64)
+    assert int(status.item()) == 0
+    assert np.all(np.abs(got - cnn.gemm(dz.T, col.T)) <= REL * cnn.gemm_abs(dz.T, col.T) + 1e-30)
+
+
 @pytest.mark.parametrize("C,ks,st,pad,H,W", [(8, 3, 2, 1, 5, 301), (24, 3, 2, 1, 3, 40),
                                              (16, 5, 3, 2, 11, 9), (256, 3, 2, 1, 4, 7)])
 def test_im2col_and_col2im_by_definition(nat, C, ks, st, pad, H, W):
