@@ -322,8 +322,8 @@ gs2d_status gs2d_pframe_step(const gs2d_plan* plan, void* ws, const float* targe
                              float* adam_m, float* adam_v, const uint8_t* selected,
                              void* stream);
 
-/* Fits a P-frame: `iters` gs2d_pframe_step iterations replayed as a captured
- * CUDA graph (moments zeroed first), then final_psnr (host, may be NULL) = the
+/* Fits a P-frame: `iters` gs2d_pframe_step iterations (moments zeroed first;
+ * more than 64 on a non-default stream replayed as a captured CUDA graph), then final_psnr (host, may be NULL) = the
  * full-frame PSNR of the result.  Synchronises the stream. */
 gs2d_status gs2d_encode_pframe(const gs2d_plan* plan, void* ws, const float* target,
                                float* params, float* adam_m, float* adam_v,
@@ -521,14 +521,15 @@ gs2d_status gs2d_roi_init_trace(const float* frame, const uint8_t* mask, int32_t
  * iterations (>= 1, and after the last) the PSNR of the clamped render is
  * taken; the loop stops once it reaches target_psnr (<= 0 disables the test)
  * or a kernel records an error.  On a non-default stream the device drives
- * the loop: the whole fit is one CUDA graph whose WHILE node repeats one
- * iteration and a control kernel that counts iterations, takes the PSNR
- * checks and ends the loop, with one host read at the end (the trace is kept
- * in the workspace's gradient scratch, so it needs iters / check_every + 1
- * <= 9n).  Otherwise (the legacy default stream, a longer trace, or a driver
- * that declines the graph) the host replays one captured iteration, or
- * launches it plainly on the legacy stream, and reads the PSNR back at each
- * check.  Both give the same results bit for bit.
+ * the loop of a longer fit: the whole fit is one CUDA graph whose WHILE node
+ * repeats a few iterations (a divisor of check_every and iters) with a control
+ * block that counts iterations, takes the PSNR checks and ends the loop, with
+ * one host read at the end (the trace is kept in the workspace's gradient
+ * scratch, so it needs iters / check_every + 1 <= 9n).  Otherwise (up to 64
+ * iterations with at most 8 checks, the legacy default stream, a longer trace,
+ * or a driver that declines the graph) the host launches the iterations, or
+ * replays one captured iteration, and reads the PSNR back at each check.  Both
+ * give the same results bit for bit.
  * target: device [3][H][W].  params: device 9n floats, in: start, out: fitted.
  * adam_m, adam_v: device 9n floats each, zeroed by this call (the optimiser
  * state restarts per frame).  psnr_trace: host, NULL or room for
@@ -549,7 +550,8 @@ gs2d_status gs2d_clip_losses(const gs2d_plan* plan, void* ws, float* out, void* 
 
 /* Fits every clip of a batch plan for `iters` iterations (Sec. 3.2 A applied
  * to many independent frames at once: one launch per step of the path covers
- * all clips), replayed as one captured CUDA graph.  Each clip's Gaussians get
+ * all clips; more than 64 iterations on a non-default stream are replayed as a
+ * captured CUDA graph).  Each clip's Gaussians get
  * exactly the updates a gs2d_encode_frame of that clip alone would give them.
  * targets: device, the batch image layout.  params, adam_m, adam_v: device
  * 9 n_total floats each (moments zeroed by this call).  clip_psnr: host,

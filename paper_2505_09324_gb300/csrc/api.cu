@@ -6,6 +6,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <numeric>
 #include <vector>
 
 #include "gs2d_internal.cuh"
@@ -357,18 +358,41 @@ static cudaError_t reset_fit(const gs2d_plan& p, void* ws, float* m, float* v, c
   return e;
 }
 
-// One fit iteration captured as a CUDA graph (non-default streams), or NULL:
-// the caller then launches the iterations directly.
-static cudaGraphExec_t capture_fit(const gs2d_plan& p, void* ws, const float* target,
-                                   float* params, float* m, float* v, int iters, cudaStream_t s) {
+// Fits of at most this many iterations are launched kernel by kernel.  Making a
+// graph costs 100 to 250 us with the device idle, and dependent launches in a
+// stream overlap across iterations, where a graph's end breaks the chain.
+// Direct launches against one graph per iteration: 586 against 655 us (8
+// iterations of a 256 x 256 P-frame fit), 998 / 1059 (1080p), 1523 / 1612 (32
+// iterations), 4114 / 4292 (100); 12 clips in a batch, 4 iterations: 2624 /
+// 2683.  Longer fits keep the graph, which leaves the host thread free.
+constexpr int kDirectIters = 64;
+
+// Iterations per graph of a longer fit of `iters`: a divisor of g, so that the
+// graph ends where the loop may end.  An iteration's nodes cost about 16 us to
+// instantiate and an iteration at a graph's end about 4 us, hence near
+// sqrt(iters) / 2 (480 iterations at 256 x 256, 1, 4, 8, 16 or 32 a graph:
+// 14.2, 12.7, 12.5, 12.5, 12.8 ms; at 1080p 46.7, 45.6, 45.4, 45.4, 45.6).
+static int graph_unroll(int iters, int g) {
+  int best = 1;
+  for (int u = 2; u <= 16 && 4 * u * u <= iters; u++)
+    if (g % u == 0) best = u;
+  return best;
+}
+
+extern "C++" {  // (templates within the C entry points' block)
+// `unroll` iterations of a fit (launched by `iteration`) captured as a CUDA
+// graph (non-default streams, longer fits), or NULL: the caller then launches
+// the iterations directly.
+template <typename F>
+static cudaGraphExec_t capture_fit(const gs2d_plan& p, int iters, int unroll, cudaStream_t s,
+                                   const F& iteration) {
   cudaGraphExec_t exec = nullptr;
-  if (s == nullptr || iters <= 0 || prime_fit_launches(p) != cudaSuccess) {
-    cudaGetLastError();
-    return nullptr;
-  }
+  if (s == nullptr || iters <= kDirectIters) return nullptr;
   cudaGraph_t graph = nullptr;
-  if (cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
-    cudaError_t ce = fit_iteration(p, ws, target, params, m, v, s);
+  if (prime_fit_launches(p) == cudaSuccess &&
+      cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
+    cudaError_t ce = cudaSuccess;
+    for (int k = 0; k < unroll && ce == cudaSuccess; k++) ce = iteration();
     cudaError_t ee = cudaStreamEndCapture(s, &graph);
     if (ce == cudaSuccess && ee == cudaSuccess && graph) {
       if (cudaGraphInstantiate(&exec, graph, 0) != cudaSuccess) exec = nullptr;
@@ -378,6 +402,19 @@ static cudaGraphExec_t capture_fit(const gs2d_plan& p, void* ws, const float* ta
   cudaGetLastError();  // a failed capture falls back to plain launches
   return exec;
 }
+
+// All iterations of a fit without checks.
+template <typename F>
+static cudaError_t run_fit(const gs2d_plan& p, int iters, cudaStream_t s, const F& iteration) {
+  const int unroll = graph_unroll(iters, iters);
+  cudaGraphExec_t exec = capture_fit(p, iters, unroll, s, iteration);
+  cudaError_t e = cudaSuccess;
+  for (int it = 0; it < iters && e == cudaSuccess; it += exec ? unroll : 1)
+    e = exec ? cudaGraphLaunch(exec, s) : iteration();
+  if (exec) cudaGraphExecDestroy(exec);
+  return e;
+}
+}  // extern "C++"
 
 gs2d_status gs2d_fit_step(const gs2d_plan* plan, void* ws, const float* target, float* params,
                           float* adam_m, float* adam_v, void* stream) {
@@ -541,17 +578,21 @@ gs2d_status gs2d_fit_rebins(const gs2d_plan* plan, const void* ws, int64_t* rebi
   return ok();
 }
 
-// The whole fit loop as one executable graph: a WHILE node whose body is one
-// fit iteration, whose last kernel also controls the loop (LoopArgs): it
-// counts the iteration, takes the PSNR checks and ends the loop, and the host
-// reads the header and the trace once, at the end.  NULL when the stream cannot be captured,
-// the trace does not fit the gradient scratch or the driver declines the
-// graph (the caller then drives the loop from the host).
+// The whole fit loop as one executable graph: a WHILE node whose body is a few
+// fit iterations (graph_unroll), the last kernel of each of which also controls
+// the loop (LoopArgs): it counts the iteration, takes the PSNR checks and ends
+// the loop, and the host reads the header and the trace once, at the end.  NULL
+// for short fits with few checks (a check from the host costs about 25 us, the
+// graph 200 to 250: 8 iterations at 256 x 256 435 us by the graph, 312 from the
+// host; 32 iterations, 4 checks, 1051 and 976), when the stream cannot be
+// captured, the trace does not fit the gradient scratch or the driver declines
+// the graph (the caller then drives the loop from the host).
 static cudaGraphExec_t capture_fit_loop(const gs2d_plan& p, void* ws, const float* target,
                                         float* params, float* m, float* v, int iters,
                                         int check_every, float target_psnr, cudaStream_t s) {
   const int checks = iters / check_every + 1;
-  if (s == nullptr || iters <= 0 || (size_t)checks > (size_t)9 * p.n ||
+  if (s == nullptr || (iters <= kDirectIters && checks <= 9) ||
+      (size_t)checks > (size_t)9 * p.n ||
       prime_fit_launches(p) != cudaSuccess) {
     cudaGetLastError();
     return nullptr;
@@ -585,7 +626,12 @@ static cudaGraphExec_t capture_fit_loop(const gs2d_plan& p, void* ws, const floa
       la.hdr = ws_ptr<WsHeader>(ws, p, kOffHeader);
       la.trace = ws_ptr<float>(ws, p, kOffGrad);
       la.handle = handle;
-      const cudaError_t ce = fit_iteration(p, ws, target, params, m, v, s, &la);
+      // (the loop ends at a check or after the last iteration only)
+      const int unroll =
+          graph_unroll(iters, check_every < iters ? std::gcd(iters, check_every) : iters);
+      cudaError_t ce = cudaSuccess;
+      for (int k = 0; k < unroll && ce == cudaSuccess; k++)
+        ce = fit_iteration(p, ws, target, params, m, v, s, &la);
       cudaGraph_t captured = nullptr;
       const cudaError_t ee = cudaStreamEndCapture(s, &captured);
       e = ce != cudaSuccess ? ce : ee;
@@ -642,8 +688,10 @@ gs2d_status gs2d_encode_frame(const gs2d_plan* plan, void* ws, const float* targ
                   h.loop_iter);
     return ok();
   }
-  // ... or, where that graph is unavailable, the host polls every check_every
-  cudaGraphExec_t exec = capture_fit(p, ws, target, params, adam_m, adam_v, iters, s);
+  // ... or, for short fits and where that graph is unavailable, the host polls
+  // every check_every
+  const auto iteration = [&] { return fit_iteration(p, ws, target, params, adam_m, adam_v, s); };
+  cudaGraphExec_t exec = capture_fit(p, iters, 1, s, iteration);
 
   int done = 0, checks = 0;
   float psnr = 0.0f;
@@ -651,7 +699,7 @@ gs2d_status gs2d_encode_frame(const gs2d_plan* plan, void* ws, const float* targ
   while (done < iters) {
     const int k = std::min(check_every, iters - done);
     for (int it = 0; it < k && e == cudaSuccess; it++)
-      e = exec ? cudaGraphLaunch(exec, s) : fit_iteration(p, ws, target, params, adam_m, adam_v, s);
+      e = exec ? cudaGraphLaunch(exec, s) : iteration();
     if (e != cudaSuccess) break;
     done += k;
     e = launch_loss_reduce(p, ws, nullptr, s);
@@ -732,23 +780,10 @@ gs2d_status gs2d_encode_pframe(const gs2d_plan* plan, void* ws, const float* tar
   const gs2d_plan& p = *plan;
   cudaStream_t s = (cudaStream_t)stream;
   cudaError_t e = reset_fit(p, ws, adam_m, adam_v, s);
-  cudaGraphExec_t exec = nullptr;
-  if (e == cudaSuccess && s != nullptr && iters > 0 && prime_fit_launches(p) == cudaSuccess) {
-    cudaGraph_t graph = nullptr;
-    if (cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
-      cudaError_t ce = pframe_iteration(p, ws, target, params, adam_m, adam_v, selected, s);
-      cudaError_t ee = cudaStreamEndCapture(s, &graph);
-      if (ce == cudaSuccess && ee == cudaSuccess && graph &&
-          cudaGraphInstantiate(&exec, graph, 0) != cudaSuccess)
-        exec = nullptr;
-      if (graph) cudaGraphDestroy(graph);
-    }
-  }
-  cudaGetLastError();  // a failed capture falls back to plain launches
-  for (int it = 0; it < iters && e == cudaSuccess; it++)
-    e = exec ? cudaGraphLaunch(exec, s)
-             : pframe_iteration(p, ws, target, params, adam_m, adam_v, selected, s);
-  if (exec) cudaGraphExecDestroy(exec);
+  if (e == cudaSuccess)
+    e = run_fit(p, iters, s, [&] {
+      return pframe_iteration(p, ws, target, params, adam_m, adam_v, selected, s);
+    });
   // full-frame PSNR of the result
   if (e == cudaSuccess) e = launch_prepare(p, ws, params, false, s);
   if (e == cudaSuccess)
@@ -794,13 +829,9 @@ gs2d_status gs2d_encode_batch(const gs2d_plan* plan, void* ws, const float* targ
   const gs2d_plan& p = *plan;
   cudaStream_t s = (cudaStream_t)stream;
   cudaError_t e = reset_fit(p, ws, adam_m, adam_v, s);
-  cudaGraphExec_t exec = e == cudaSuccess ? capture_fit(p, ws, targets, params, adam_m, adam_v,
-                                                        iters, s)
-                                          : nullptr;
-  for (int it = 0; it < iters && e == cudaSuccess; it++)
-    e = exec ? cudaGraphLaunch(exec, s)
-             : fit_iteration(p, ws, targets, params, adam_m, adam_v, s);
-  if (exec) cudaGraphExecDestroy(exec);
+  if (e == cudaSuccess)
+    e = run_fit(p, iters, s,
+                [&] { return fit_iteration(p, ws, targets, params, adam_m, adam_v, s); });
   // evaluate the fitted Gaussians (gradients into the scratch section)
   if (e == cudaSuccess) e = launch_prepare(p, ws, params, false, s);
   if (e == cudaSuccess)

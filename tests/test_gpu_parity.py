@@ -410,6 +410,40 @@ def test_device_driven_loop_equals_host_driven_loop(gs, mode, check_every):
         assert od["iters"] == iters and len(od["trace"]) == -(-iters // check_every)
 
 
+@pytest.mark.parametrize("iters,check_every,stop", [(64, 8, None), (65, 8, None), (100, 10, 3),
+                                                    (96, 200, None), (72, 24, 2)])
+def test_graphs_of_several_iterations_equal_direct_launches(gs, iters, check_every, stop):
+    """Longer fits run as graphs of several iterations (WHILE body, replayed
+    graph and their remainders): the same Gaussians bit for bit as launched one
+    by one on the legacy default stream, for encode_frame (cap, early stop),
+    encode_pframe and encode_batch."""
+    W, H, n = 72, 56, 90
+    p0 = to_dev(random_gaussians(n, W, H, seed=41, l_range=(2.0, 6.0)))
+    target = to_dev(smooth_noise_target(W, H, seed=42))
+    sel = (torch.arange(n, device="cuda") % 3 == 0).to(torch.uint8)
+
+    def run(s, goal):
+        out = []
+        with torch.cuda.stream(s):
+            r, b = gs.GaussianRasterizer(W, H, n), gs.BatchRasterizer([(W, H, n)] * 2)
+            p, q = p0.clone(), p0.clone()
+            o = r.encode_frame(target, p, iters, target_psnr=goal, check_every=check_every,
+                               stream=s)
+            f = r.encode_pframe(target, q, sel, iters, stream=s)
+            pb = torch.cat([p0, p0], 1).contiguous()
+            c = b.encode_batch(b.pack_images([target, target]), pb, iters, stream=s)
+            s.synchronize()
+        return (p, q, pb), (o["iters"], o["trace"], o["psnr"], f, list(c))
+
+    goal = 0.0
+    if stop:
+        goal = run(torch.cuda.default_stream(), 0.0)[1][1][stop - 1]
+    (ta, a), (tb, b) = run(torch.cuda.default_stream(), goal), run(torch.cuda.Stream(), goal)
+    assert a == b and (not stop or a[0] <= stop * check_every)
+    for x, y in zip(ta, tb):
+        assert torch.equal(x, y)
+
+
 def _piled(n, W, H, seed, at, share):
     """Random Gaussians, `share` of them within a pixel of `at`."""
     p = random_gaussians(n, W, H, seed=seed, l_range=(0.5, 2.0))
