@@ -81,8 +81,8 @@ PAPER_ENCODE = {"reduction": 1.0 - 1.5 / 13.1, "superpixel_s": 1.5, "random_init
 # DRAM bytes (read + write) of one fused render launch (k_render, tile 32,
 # stage 128, grid) from an ncu capture of this workload, valid for the render
 # source with this sha256 (else null)
-NCU_TRAFFIC = {"bytes": 26836224, "schedule": (32, 128, 1),
-               "render_sha256": "4e5b099f6bca4bcae99dff9622978e0c215a19696df27bb96fad98d84882224a"}
+NCU_TRAFFIC = {"bytes": 26825472, "schedule": (32, 128, 1),
+               "render_sha256": "1d4062adeb042c4d7a9ccfe84e7962242f419a5b03778825d937d5740a3029d9"}
 
 
 def hbm_peak_gbs() -> float:
@@ -812,11 +812,12 @@ def run_ours(args):
         nat.fit_step(plan, ws, frame.data_ptr(), p_t.data_ptr(), m.data_ptr(), v.data_ptr(), sp)
 
     # our kernels per step: projection (+ containment test of the retained
-    # lists), list rebuild counts, scans, scatter, short-list sort, long-list
-    # sort (the last four return at once while the lists hold), fused render,
-    # reduction + Adam; per-iteration binning fuses the first two
+    # lists), list rebuild counts with their scan (a launch of its own above
+    # 2048 tiles or Gaussian groups), scatter, sort (these return at once while
+    # the lists hold), fused render, reduction + Adam; per-iteration binning
+    # fuses the first two
     retained = tuned["config"].bin_margin >= 0
-    launches_per_step = (6 if retained else 5) + 1 + 1
+    launches_per_step = (4 if retained else 3) + (int(plan.num_tiles) > 2048) + 1 + 1
 
     for _ in range(args.warmup):
         fit_step(params)
