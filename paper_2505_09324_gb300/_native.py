@@ -119,6 +119,8 @@ def library_path() -> str:
 def load(build_if_missing: bool = False):
     """Loads libgs2d.so (building it first only if asked)."""
     global _lib
+    if _lib is not None:  # (set once, when complete)
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -328,7 +330,9 @@ def autotune(sizes, params: int, targets: int, ws: int, ws_bytes: int, tiles, st
 
 
 def _p(x):
-    return None if x is None or x == 0 else ctypes.c_void_p(x)
+    """A device address as an argument declared c_void_p: ctypes converts the
+    integer itself (a c_void_p object per argument doubled a call's cost)."""
+    return x or None
 
 
 def project(plan: Plan, ws: int, params: int, stream: int):

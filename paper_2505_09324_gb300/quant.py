@@ -28,6 +28,7 @@ import numpy as np
 import torch
 
 from . import _native as nat
+from .raster import _stream
 
 HALF = -16
 ROWS = ("mu_x", "mu_y", "l1", "l2", "l3", "c_r", "c_g", "c_b", "w")
@@ -101,9 +102,8 @@ class Quantizer:
         c = torch.empty((9, n), dtype=torch.uint16, device=params.device) if codes else None
         v = torch.empty_like(params) if values else None
         ranges = torch.empty((2, 9), dtype=torch.float32, device=params.device)
-        s = torch.cuda.current_stream() if stream is None else stream
         nat.quantize(params.data_ptr(), n, self.c, 0 if c is None else c.data_ptr(),
-                     0 if v is None else v.data_ptr(), ranges.data_ptr(), int(s.cuda_stream))
+                     0 if v is None else v.data_ptr(), ranges.data_ptr(), _stream(stream))
         return c, v, ranges
 
 

@@ -71,8 +71,15 @@ FAST_FIT = {"lr_mu": 50.0, "lr_shape": 30.0, "lr_color": 10.0, "lr_weight": 3.0,
             "lr_decay": 0.995}
 
 
+# The current stream's handle without a Stream object around it (the object
+# costs as much as a kernel launch): (device index) -> int.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream) -> int:
     if stream is None:
+        if _raw_stream is not None:
+            return _raw_stream(torch.cuda.current_device())
         stream = torch.cuda.current_stream()
     return int(stream.cuda_stream)
 
@@ -86,7 +93,7 @@ def _check(t: torch.Tensor, name: str, shape=None, dtype=torch.float32):
         raise ValueError(f"{name} must be {dtype}, got {t.dtype}")
     if not t.is_contiguous():
         raise ValueError(f"{name} must be contiguous")
-    if shape is not None and tuple(t.shape) != tuple(shape):
+    if shape is not None and t.shape != tuple(shape):
         raise ValueError(f"{name} must have shape {tuple(shape)}, got {tuple(t.shape)}")
     return t.data_ptr()
 
