@@ -22,6 +22,7 @@
 #include <math.h>
 #include <stdio.h>
 
+#include <algorithm>
 
 #include "gs2d_internal.cuh"
 
@@ -64,6 +65,7 @@ struct SpArgs {
 // window is (2 S)^2 pixels per centre, 4 A in all whatever S is, so only the
 // number of warps falls with S: at 32 a warp has 128 steps of 32 pixels.
 constexpr float kGatherS = 32.0f;
+constexpr int kWave = 152;  // blocks of one wave
 
 // The pixel's colour on the 2^-20 grid: a power-of-two scaling, exact in
 // float, then one rounding to the nearest integer.
@@ -206,15 +208,16 @@ __device__ __forceinline__ long long lanes_sum64(unsigned mask, long long v) {
   return (long long)hi * (1ll << 24) + (long long)lo;
 }
 
-// The nine exact sums of centre c's segment, by half a warp (a lane per
-// column): every pixel that can have joined it lies within S of it.  The
+// The nine exact sums of one of `parts` bands of rows of centre c's segment, by
+// half a warp (a lane per column): every pixel that can have joined it lies within S of it.  The
 // labels of kRows rows are loaded together and then the colours of those that
 // match, so a window of 14 x 14 pixels (S of 7) costs a few load latencies
 // rather than one per row.
 constexpr int kRows = 7;
 
-__device__ __forceinline__ void gather_segment(const SpArgs& a, const SpGeom& g, int c, int hl,
-                                               unsigned mask, long long out[kSums]) {
+__device__ __forceinline__ void gather_segment(const SpArgs& a, const SpGeom& g, int c, int part,
+                                               int parts, int hl, unsigned mask,
+                                               long long out[kSums]) {
   const int M = a.n;
   const size_t HW = (size_t)a.W * a.H;
   const float cx = a.cen[3 * M + c], cy = a.cen[4 * M + c];
@@ -222,8 +225,11 @@ __device__ __forceinline__ void gather_segment(const SpArgs& a, const SpGeom& g,
   // |x + 1/2 - cx| <= S, with room for FP32 rounding (2^-7 at 65536)
   const int xa = max(0, (int)ceilf(cx - g.S32 - 0.52f));
   const int xb = min(a.W - 1, (int)floorf(cx + g.S32 - 0.48f));
-  const int ya = max(0, (int)ceilf(cy - g.S32 - 0.52f));
-  const int yb = min(a.H - 1, (int)floorf(cy + g.S32 - 0.48f));
+  int ya = max(0, (int)ceilf(cy - g.S32 - 0.52f));
+  int yb = min(a.H - 1, (int)floorf(cy + g.S32 - 0.48f));
+  const int band = (yb - ya + parts) / parts;
+  ya += part * band;
+  yb = min(yb, ya + band - 1);
   // per lane at most (2 S + 2)^2 / 16 pixels: moments stay below 2^31, the
   // colours need 64 bits
   int s[6] = {0, 0, 0, 0, 0, 0};
@@ -335,30 +341,42 @@ __device__ __forceinline__ void segment_gaussian(const SpArgs& a, const SpGeom& 
 // sums, 2 centres each, then one warp does the double-precision arithmetic of
 // all 32 at once (FP64 costs per warp instruction, however few lanes it has):
 // 20 us at 14 000 centres.  With the assignment, the whole initialisation of a
-// 1920 x 1080 frame went from 842 to 372 us.  Large segments: the sums come from the assignment's atomics and are cleared
-// for the next one.
+// 1920 x 1080 frame went from 842 to 372 us.  Few centres have longer windows
+// and would leave most SMs idle: up to a wave of blocks of 16 or 8 centres,
+// blocks take that many, with 2 or 4 half-warps to each centre's window (340
+// centres of a 565 x 315 frame: 31 -> 18 us, its wait for the assignment
+// included).  Large segments: the sums come from the assignment's atomics and
+// are cleared for the next one.
 template <bool FINAL>
 __global__ void __launch_bounds__(256) k_sp_update(SpArgs a, float* __restrict__ params) {
   pdl_begin();
   __shared__ long long s_sum[kSums][32];
   const SpGeom g = *a.geo;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, c0 = blockIdx.x * 32;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int per = g.M <= kWave * 8 ? 8 : g.M <= kWave * 16 ? 16 : 32;  // centres of a block
+  const int c0 = blockIdx.x * per;
   if (c0 >= g.M) return;
+  const bool mine = lane < per && c0 + lane < g.M;
   if (g.S32 <= kGatherS) {
     const int half = threadIdx.x >> 4, hl = threadIdx.x & 15;
     const unsigned mask = 0xffffu << (lane & 16);
+    for (int k = threadIdx.x; k < kSums * 32; k += 256) (&s_sum[0][0])[k] = 0;
+    __syncthreads();
 #pragma unroll 1
-    for (int k = half; k < 32 && c0 + k < g.M; k += 16) {
+    for (int k = half; k < 32; k += 16) {
+      const int c = k % per;
+      if (c0 + c >= g.M) continue;
       long long sum[kSums];
-      gather_segment(a, g, c0 + k, hl, mask, sum);
+      gather_segment(a, g, c0 + c, k / per, 32 / per, hl, mask, sum);
       if (hl < kSums) {
         long long v = sum[0];
 #pragma unroll
         for (int q = 1; q < kSums; q++) v = hl == q ? sum[q] : v;
-        s_sum[hl][k] = v;
+        // (exact integers: any order)
+        atomicAdd(reinterpret_cast<unsigned long long*>(&s_sum[hl][c]), (unsigned long long)v);
       }
     }
-  } else if (wid == 0 && c0 + lane < g.M) {
+  } else if (wid == 0 && mine) {
 #pragma unroll
     for (int q = 0; q < kSums; q++) {
       unsigned long long* p = &a.acc[(size_t)q * a.n + c0 + lane];
@@ -367,7 +385,7 @@ __global__ void __launch_bounds__(256) k_sp_update(SpArgs a, float* __restrict__
     }
   }
   __syncthreads();
-  if (wid != 0 || c0 + lane >= g.M) return;
+  if (wid != 0 || !mine) return;
   long long acc[kSums];
 #pragma unroll
   for (int q = 0; q < kSums; q++) acc[q] = s_sum[q][lane];
@@ -623,7 +641,7 @@ gs2d_status roi_init(const float* frame, const uint8_t* mask, int W, int H, int 
   a.blk = reinterpret_cast<int*>(take(kSeedBlocks * 4));
   // everything on the device; the region count comes back at the end
   const dim3 tiles((W + kTileW - 1) / kTileW, (H + kTileH - 1) / kTileH);
-  const int cb = (n + 31) / 32;
+  const int cb = std::max((n + 31) / 32, std::min((n + 7) / 8, kWave));  // k_sp_update's
   cudaError_t e = cudaMemsetAsync(a.area, 0, 8, s);
   if (e == cudaSuccess) e = launch_pdl(k_sp_area, 152 * 8, 256, 0, s, a);
   if (e == cudaSuccess) e = launch_pdl(k_sp_seed_count, kSeedBlocks, 256, 0, s, a);

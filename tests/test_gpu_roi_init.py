@@ -187,3 +187,10 @@ def test_tile_edges_and_both_sum_paths(gs, w, h, n, frac):
     if w == 97:
         mask[:, ::3] = False
     check_step_by_step(gs, frame, mask, n, frac, seed=5)
+
+
+@pytest.mark.parametrize("n", [1100, 1300, 2300, 2560])
+def test_blocks_of_8_16_and_32_centres(gs, n):
+    """Centre counts on both sides of the update's two lines (152 blocks of 8
+    and of 16 centres), against the oracle."""
+    test_tile_edges_and_both_sum_paths(gs, 64, 40, n, 1.0)
