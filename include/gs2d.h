@@ -460,7 +460,8 @@ gs2d_status gs2d_fit_step_rgb8(const gs2d_plan* plan, void* ws, const uint8_t* r
                                float* params, float* adam_m, float* adam_v, float* params_out_host,
                                void* stream);
 
-/* Number of times the fit loop has rebuilt its tile lists in this workspace
+/* Number of times a fit loop (or gs2d_encode_pframe's, until its last, full
+ * evaluation) has rebuilt its tile lists in this workspace
  * (see gs2d_config.bin_margin) since it was zero-filled or gs2d_fit_reset;
  * synchronises the stream. */
 gs2d_status gs2d_fit_rebins(const gs2d_plan* plan, const void* ws, int64_t* rebins,

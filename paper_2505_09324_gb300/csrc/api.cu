@@ -748,11 +748,17 @@ gs2d_status gs2d_select_changed(const gs2d_plan* plan, void* ws, const float* re
   return cuda_check(e, "gs2d_select_changed");
 }
 
+// loop: one of many iterations, with the fit loop's retained lists (binning
+// every iteration took 26 of some 85 us at 1080p, 20 000 Gaussians, tile 16: a
+// P-frame of 8 iterations 969 us so, 864 with retained lists).
 static cudaError_t pframe_iteration(const gs2d_plan& p, void* ws, const float* target,
                                     float* params, float* m, float* v, const uint8_t* select,
-                                    cudaStream_t s) {
-  cudaError_t e = launch_prepare(p, ws, params, true, s);
-  if (e == cudaSuccess) e = launch_pframe_step(p, ws, target, params, m, v, select, s);
+                                    bool loop, cudaStream_t s) {
+  cudaError_t e = loop ? launch_prepare_fit(p, ws, params, s)
+                       : launch_prepare(p, ws, params, true, s);
+  if (e == cudaSuccess)
+    e = launch_pframe_step(p, ws, target, params, m, v, select, loop && fit_lists_retained(p.cfg),
+                           s);
   return e;
 }
 
@@ -763,7 +769,7 @@ gs2d_status gs2d_pframe_step(const gs2d_plan* plan, void* ws, const float* targe
   if (st) return st;
   if (!target || (plan->n > 0 && (!params || !adam_m || !adam_v || !selected)))
     return fail(GS2D_ERR_INVALID_ARG, "gs2d_pframe_step: NULL pointer");
-  return cuda_check(pframe_iteration(*plan, ws, target, params, adam_m, adam_v, selected,
+  return cuda_check(pframe_iteration(*plan, ws, target, params, adam_m, adam_v, selected, false,
                                      (cudaStream_t)stream),
                     "gs2d_pframe_step");
 }
@@ -782,7 +788,7 @@ gs2d_status gs2d_encode_pframe(const gs2d_plan* plan, void* ws, const float* tar
   cudaError_t e = reset_fit(p, ws, adam_m, adam_v, s);
   if (e == cudaSuccess)
     e = run_fit(p, iters, s, [&] {
-      return pframe_iteration(p, ws, target, params, adam_m, adam_v, selected, s);
+      return pframe_iteration(p, ws, target, params, adam_m, adam_v, selected, true, s);
     });
   // full-frame PSNR of the result
   if (e == cudaSuccess) e = launch_prepare(p, ws, params, false, s);

@@ -443,9 +443,10 @@ cudaError_t launch_count_flags(int n, const uint8_t* flags, int* out, cudaStream
 // Quantisation (quant.cu): codes, dequantised values and ranges of params.
 cudaError_t launch_quantize(const float* params, int n, const gs2d_quant& q, uint16_t* codes,
                             float* dequant, float* ranges, cudaStream_t s);
+// retained: after launch_prepare_fit with retained lists (it marks them valid).
 cudaError_t launch_pframe_step(const gs2d_plan& p, void* ws, const float* target,
                                float* params, float* m, float* v, const uint8_t* select,
-                               cudaStream_t s);
+                               bool retained, cudaStream_t s);
 // project + bin_sort; with adam_tick the fit loop's Adam step counter and bias
 // corrections advance in the same launch.
 cudaError_t launch_prepare(const gs2d_plan& p, void* ws, const float* params, bool adam_tick,

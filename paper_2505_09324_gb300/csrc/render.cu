@@ -490,7 +490,7 @@ cudaError_t launch_select_changed(const gs2d_plan& p, void* ws, const float* ref
 // render over them, reduction + Adam of the selected Gaussians.
 cudaError_t launch_pframe_step(const gs2d_plan& p, void* ws, const float* target,
                                float* params, float* m, float* v, const uint8_t* select,
-                               cudaStream_t s) {
+                               bool retained, cudaStream_t s) {
   if (p.n == 0) return cudaSuccess;
   uint8_t* active = ws_ptr<uint8_t>(ws, p, kOffActive);
   int* act_order = ws_ptr<int>(ws, p, kOffActOrder);
@@ -507,11 +507,12 @@ cudaError_t launch_pframe_step(const gs2d_plan& p, void* ws, const float* target
   a.active = act_count;
   e = launch_render(p, kModeL2, a, s);
   if (e != cudaSuccess) return e;
+  WsHeader* hdr = ws_ptr<WsHeader>(ws, p, kOffHeader);
   return launch_pdl(k_reduce_chain_adam, (p.n * kRL + 255) / 256, 256, 0, s, p.n, params,
-                    slot_args(p, ws),
-                    ws_ptr<WsHeader>(ws, p, kOffHeader), m, v, lr_rows(p.cfg), p.cfg.beta1,
-                    p.cfg.beta2, p.cfg.eps, select, (const float*)nullptr, (WsHeader*)nullptr,
-                    atomic_sums(p, ws), (float*)nullptr, LoopArgs{});
+                    slot_args(p, ws), (const WsHeader*)hdr, m, v, lr_rows(p.cfg), p.cfg.beta1,
+                    p.cfg.beta2, p.cfg.eps, select, (const float*)nullptr,
+                    retained ? hdr : (WsHeader*)nullptr, atomic_sums(p, ws), (float*)nullptr,
+                    LoopArgs{});
 }
 
 // Runs the one-time per-device query of the fit loop's launches (occupancy of

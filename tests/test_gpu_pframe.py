@@ -102,3 +102,35 @@ def test_selective_sequence(gs):
     for x, y in zip(a[1:], b[1:]):
         assert 0 < y["selected"] < n
         assert y["psnr"] > x["psnr"] - 1.5, (x, y)
+
+
+@pytest.mark.parametrize("tile,lr", [(8, 0.02), (16, 0.6), (32, 2.0)])
+def test_encode_pframe_equals_its_steps(gs, tile, lr):
+    """gs2d_encode_pframe keeps the tile lists across iterations, rebuilding
+    them when a selected Gaussian leaves its listed tiles; the same Gaussians
+    and moments bit for bit as gs2d_pframe_step, which bins every time."""
+    from paper_2505_09324_gb300 import _native as nat
+    W, H, n, iters = 150, 90, 300, 12
+    fr, _ = scene(W, H, n, seed=5)
+    p, _ = fitted(gs, fr, n, seed=5, iters=40)
+    t = torch.from_numpy(fr[1][0]).cuda()
+    sel = (torch.arange(n, device="cuda") % 2 == 0).to(torch.uint8)
+    cfg = gs.RasterConfig(tile=tile, lr=lr)
+    out = []
+    for whole in (True, False):
+        r = gs.GaussianRasterizer(W, H, n, config=cfg)
+        q = p.clone()
+        m, v = torch.empty_like(q), torch.empty_like(q)
+        if whole:
+            r.encode_pframe(t, q, sel, iters, adam_state=(m, v))
+        else:
+            r.fit_reset((m, v))
+            for _ in range(iters):
+                nat.pframe_step(r.plan, r.ws_ptr, t.data_ptr(), q.data_ptr(), m.data_ptr(),
+                                v.data_ptr(), sel.data_ptr(),
+                                int(torch.cuda.current_stream().cuda_stream))
+        torch.cuda.synchronize()
+        assert r.status() == 0
+        out.append((q, m, v))
+    for a, b in zip(*out):
+        assert torch.equal(a, b)
