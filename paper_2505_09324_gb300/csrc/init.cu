@@ -360,8 +360,10 @@ __global__ void __launch_bounds__(256) k_sp_update(SpArgs a, float* __restrict__
   if (g.S32 <= kGatherS) {
     const int half = threadIdx.x >> 4, hl = threadIdx.x & 15;
     const unsigned mask = 0xffffu << (lane & 16);
-    for (int k = threadIdx.x; k < kSums * 32; k += 256) (&s_sum[0][0])[k] = 0;
-    __syncthreads();
+    if (per < 32) {
+      for (int k = threadIdx.x; k < kSums * 32; k += 256) (&s_sum[0][0])[k] = 0;
+      __syncthreads();
+    }
 #pragma unroll 1
     for (int k = half; k < 32; k += 16) {
       const int c = k % per;
@@ -372,8 +374,11 @@ __global__ void __launch_bounds__(256) k_sp_update(SpArgs a, float* __restrict__
         long long v = sum[0];
 #pragma unroll
         for (int q = 1; q < kSums; q++) v = hl == q ? sum[q] : v;
-        // (exact integers: any order)
-        atomicAdd(reinterpret_cast<unsigned long long*>(&s_sum[hl][c]), (unsigned long long)v);
+        // (exact integers: the parts in any order)
+        if (per == 32)
+          s_sum[hl][c] = v;
+        else
+          atomicAdd(reinterpret_cast<unsigned long long*>(&s_sum[hl][c]), (unsigned long long)v);
       }
     }
   } else if (wid == 0 && mine) {
