@@ -526,11 +526,12 @@ gs2d_status gs2d_roi_init_trace(const float* frame, const uint8_t* mask, int32_t
  * repeats a few iterations (a divisor of check_every and iters) with a control
  * block that counts iterations, takes the PSNR checks and ends the loop, with
  * one host read at the end (the trace is kept in the workspace's gradient
- * scratch, so it needs iters / check_every + 1 <= 9n).  Otherwise (up to 64
- * iterations with at most 8 checks, the legacy default stream, a longer trace,
- * or a driver that declines the graph) the host launches the iterations, or
- * replays one captured iteration, and reads the PSNR back at each check.  Both
- * give the same results bit for bit.
+ * scratch, so it needs iters / check_every + 1 <= 9n).  Up to 64 iterations
+ * without a target are launched at once, with the device taking the checks.
+ * Otherwise (up to 64 iterations with at most 8 checks, the legacy default
+ * stream, a longer trace, or a driver that declines the graph) the host
+ * launches the iterations, or replays one captured iteration, and reads the
+ * PSNR back at each check.  All give the same results bit for bit.
  * target: device [3][H][W].  params: device 9n floats, in: start, out: fitted.
  * adam_m, adam_v: device 9n floats each, zeroed by this call (the optimiser
  * state restarts per frame).  psnr_trace: host, NULL or room for

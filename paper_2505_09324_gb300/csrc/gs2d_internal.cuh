@@ -69,7 +69,8 @@ struct WsHeader {
   int32_t lists_tight;  // the last rebuild listed tight rectangles (widened ones overflowed)
   int32_t loop_iter;    // device-driven fit loop: iterations run
   int32_t loop_checks;  // device-driven fit loop: PSNR checks made
-  int32_t pad[36];
+  int32_t loop_end;     // device-driven fit loop: it has ended
+  int32_t pad[35];
 };
 static_assert(sizeof(WsHeader) == 256, "header is one 256-byte block");
 
@@ -229,24 +230,28 @@ __device__ __forceinline__ double2 loss_sums(const float2* __restrict__ part, in
 // Control of the device-driven fit loop (gs2d_encode_frame), run by a block of
 // its own beside the iteration's last kernel: it counts the iteration; every
 // check_every iterations (and at the last) it sums the render's per-tile loss
-// partials, writes the PSNR of the clamped image to the trace and clears the
-// loop condition once the target is met, the cap is reached or a kernel has
-// recorded an error.
+// partials, writes the PSNR of the clamped image to the trace and ends the loop
+// once the target is met, the cap is reached or a kernel has recorded an error:
+// it clears the condition of the graph's WHILE node, and counts and checks no
+// further iteration (one launched without a graph; after an error it changes
+// nothing).
 struct LoopArgs {
   int num_tiles, iters, check_every;
   float target_psnr;
   const float2* loss_part;
   WsHeader* hdr;  // NULL: no loop
   float* trace;   // device, one float per check
+  int graph;      // whether there is a WHILE node
   cudaGraphConditionalHandle handle;
 };
 
 template <int THREADS>
 __device__ __forceinline__ void loop_control(const LoopArgs& a, double2* s_sum) {
   __shared__ int s_it;
-  if (threadIdx.x == 0) s_it = ++a.hdr->loop_iter;
+  if (threadIdx.x == 0) s_it = a.hdr->loop_end ? 0 : ++a.hdr->loop_iter;
   __syncthreads();
   const int it = s_it;
+  if (it == 0) return;
   if (it % a.check_every != 0 && it < a.iters) return;
   const double2 s = loss_sums<THREADS>(a.loss_part, a.num_tiles, s_sum);
   if (threadIdx.x != 0) return;
@@ -257,7 +262,10 @@ __device__ __forceinline__ void loop_control(const LoopArgs& a, double2* s_sum) 
   a.trace[a.hdr->loop_checks++] = psnr;
   const bool stop = it >= a.iters || a.hdr->status != 0 ||
                     (a.target_psnr > 0.0f && psnr >= a.target_psnr);
-  if (stop) cudaGraphSetConditional(a.handle, 0u);
+  if (stop) {
+    a.hdr->loop_end = 1;
+    if (a.graph) cudaGraphSetConditional(a.handle, 0u);
+  }
 }
 
 // Projection of Gaussian i (Sec. 3.1 parameters -> screen-space record, tile

@@ -444,6 +444,28 @@ def test_graphs_of_several_iterations_equal_direct_launches(gs, iters, check_eve
         assert torch.equal(x, y)
 
 
+@pytest.mark.parametrize("check_every,entries", [(7, 0), (64, 0), (1, 0), (5, 400)])
+def test_short_fit_without_a_target_equals_a_polled_one(gs, check_every, entries):
+    """Up to 64 iterations without a target are launched at once, the device
+    taking the checks; with a target that is never met the host polls.  The same
+    Gaussians, trace and counts, also where the entry capacity is exceeded (the
+    fit ends at its first check)."""
+    W, H, n, iters = 96, 80, 120, 64
+    p0 = to_dev(random_gaussians(n, W, H, seed=29, l_range=(2.0, 6.0)))
+    target = to_dev(smooth_noise_target(W, H, seed=30))
+    out = []
+    for goal in (0.0, 99.0):
+        r = gs.GaussianRasterizer(W, H, n, max_entries=entries)
+        p = p0.clone()
+        m, v = torch.empty_like(p), torch.empty_like(p)
+        o = r.encode_frame(target, p, iters, target_psnr=goal, check_every=check_every,
+                           adam_state=(m, v))
+        out.append((p, m, v, o))
+    (pa, ma, va, a), (pb, mb, vb, b) = out
+    assert a == b and a["iters"] == (check_every if entries else iters)
+    assert torch.equal(pa, pb) and torch.equal(ma, mb) and torch.equal(va, vb)
+
+
 def _piled(n, W, H, seed, at, share):
     """Random Gaussians, `share` of them within a pixel of `at`."""
     p = random_gaussians(n, W, H, seed=seed, l_range=(0.5, 2.0))
