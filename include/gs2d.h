@@ -612,15 +612,16 @@ uint64_t gs2d_gemm_partial_bytes(int32_t M, int32_t N, int32_t ldc, int32_t K, i
  * B (device, row-major [K][lda] and [K][ldb], leading dimensions in elements,
  * multiples of 8; 16-byte aligned), FP32 accumulation and FP32 output (device
  * [M][ldc]): the weight gradient of a convolution from dZ and the im2col
- * operand, without transposing either.  K is split over at least min_splits
+ * operand, without transposing either; bit for bit what gs2d_gemm_bf16 gives of
+ * the transposed operands with the same `splits`.  K is split over that many
  * groups of thread blocks, as far as it goes (FP32 sums lose precision with
  * their length); partial (device, gs2d_gemm_tn_partial_bytes bytes) then holds
  * FP32 partial sums that a second kernel adds in a fixed order (deterministic).  status as gs2d_gemm_bf16. */
 gs2d_status gs2d_gemm_tn_bf16(const void* A, int32_t lda, const void* B, int32_t ldb, int32_t M,
-                              int32_t N, int32_t K, float* out, int32_t ldc, int32_t min_splits,
+                              int32_t N, int32_t K, float* out, int32_t ldc, int32_t splits,
                               float* partial, int32_t* status, void* stream);
 uint64_t gs2d_gemm_tn_partial_bytes(int32_t M, int32_t N, int32_t ldc, int32_t K,
-                                    int32_t min_splits);
+                                    int32_t splits);
 
 /* Failure-detection check of the GEMM's bounded waits (not part of the
  * paper's method).  Launches the gs2d_gemm_bf16 kernel on one 128 x 32 x 64
@@ -720,18 +721,18 @@ gs2d_status gs2d_conv_dgrad_bf16(const void* dz, int32_t B, int32_t Hi, int32_t 
 /* Weight gradient of a 3 x 3 convolution with stride 2 and padding 1 from its
  * input x (device BF16 [B][Hi][Wi][C]) and dz (device BF16 [B][Ho][Wo][N], Ho =
  * (Hi + 1) / 2, Wo = (Wi + 1) / 2): what gs2d_gemm_tn_bf16 gives of dz and
- * gs2d_im2col's operand, without that operand.  out: device float32 [N][ldc],
+ * gs2d_im2col's operand, bit for bit, without that operand.  out: device float32 [N][ldc],
  * ldc >= 9 C + 1: column (3 ky + kx) C + ci, the bias in column 9 C, zeros
- * beyond.  C a multiple of 64 (any Wi), or 32, or 8 with N <= 64 (both with an
- * even Wi); N a multiple of 8; dz and x 16-byte aligned;
- * gs2d_conv_wgrad_supported is 1 for these.  min_splits, partial (device,
+ * beyond.  Wo at least 64 and a multiple of 16; C a multiple of 64 (any Wi), or
+ * 32, or 8 with N <= 64 (both with an even Wi); N a multiple of 8; dz and x
+ * 16-byte aligned; gs2d_conv_wgrad_supported is 1 for these.  splits, partial (device,
  * gs2d_conv_wgrad_partial_bytes bytes) and status as gs2d_gemm_tn_bf16. */
 int32_t gs2d_conv_wgrad_supported(int32_t B, int32_t Hi, int32_t Wi, int32_t C, int32_t N);
 uint64_t gs2d_conv_wgrad_partial_bytes(int32_t B, int32_t Hi, int32_t Wi, int32_t C, int32_t N,
-                                       int32_t ldc, int32_t min_splits);
+                                       int32_t ldc, int32_t splits);
 gs2d_status gs2d_conv_wgrad_bf16(const void* dz, int32_t N, const void* x, int32_t B, int32_t Hi,
                                  int32_t Wi, int32_t C, float* out, int32_t ldc,
-                                 int32_t min_splits, float* partial, int32_t* status,
+                                 int32_t splits, float* partial, int32_t* status,
                                  void* stream);
 
 /* out[c][r] = in[r][c] for a BF16 R x C matrix (device; leading dimensions

@@ -6,17 +6,16 @@
 //   dW[co][9 C]                = sum over p of dZ[p][co]  (the bias), zeros beyond
 //
 // i.e. gs2d_gemm_tn_bf16 of dZ and the im2col operand, which is neither
-// written nor read: at 1080p, batch 8, that operand is 1.8 GB for the five
-// layers, 0.79 ms of gs2d_im2col per training step.
+// written nor read: at 1080p, batch 8, that operand is 1.6 GB for the first
+// three layers, most of 0.79 ms of gs2d_im2col per training step.
 //
 // Both operands are MN-major as in csrc/gemm_tn.cu: a row is a pixel, its
-// channels lie contiguously.  A k-step is 128 output pixels: pw of each of
-// 128 / pw output rows (pw the power of two from 16 to 128 that the row needs),
-// zero rows past the edges of dZ.  For a fixed tap their inputs are every
-// second pixel of every second input row, so one TMA box brings a tap's
-// channels.  With an even width, X is read as pairs of pixels [2 ox, 2 ox + 1]
-// of 2 C channels: taps kx = 1 and 2 are the two halves of pair ox, kx = 0 the
-// second half of pair ox - 1, and no box steps along W.  Three forms:
+// channels lie contiguously.  A k-step is up to 128 output pixels of one row.
+// For a fixed tap their inputs are every second pixel of an input row, so one
+// TMA box brings a tap's channels.  With an even width, X is read as pairs of
+// pixels [2 ox, 2 ox + 1] of 2 C channels: taps kx = 1 and 2 are the two halves
+// of pair ox, kx = 0 the second half of pair ox - 1, and no box steps along W.
+// Three forms:
 //   C = 64 j:  boxes of 64 channels of a tap, three of them a tile's columns
 //              (odd widths: a traversal stride of 2 along W instead of pairs);
 //   C = 32:    all taps in a tile: per ky the pair (64 columns) and the second
@@ -26,11 +25,14 @@
 // The bias column comes from a constant block of ones.
 //
 // What bounds it is the staging of dZ and the taps (each input pixel is read
-// 2.25 times, but from DRAM once).  Against im2col and gs2d_gemm_tn_bf16 the
-// training step went from 2.84 to 2.27 ms at 1080p, batch 8: the operands'
-// 0.79 ms became 0.04 (the head's remains), the products took 0.52 and take 0.45.
+// 2.25 times, but from DRAM once).  Against im2col and gs2d_gemm_tn_bf16 in every
+// layer the training step went from 2.84 to 2.46 ms at 1080p, batch 8, where the
+// first three layers run here and the last two (120 and 60 pixels a row) there.
 //
-// Splits, ring, waits and epilogue as in csrc/gemm_tn.cu.
+// Splits, ring, waits and epilogue as in csrc/gemm_tn.cu.  Output rows are
+// multiples of 16 pixels (of at least 64), so that the tensor core adds the same
+// 16 pixels at a time, in the same order, as over the operand: the result is
+// that of the GEMM bit for bit (why that matters: csrc/gemm_tn.cu).
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <stdio.h>
@@ -49,8 +51,7 @@ constexpr int kWgOnes = 2048;  // 16 rows of 64 columns, column 0 all ones
 
 struct WgArgs {
   int M, C, ldc;               // output channels, input channels, dW's leading dimension
-  int segs, hp, pw, rows;      // k-steps along a row and down an image; pixels x rows of a step
-  int num_kt, kt_per_split;
+  int Ho, Wo, pixels, per;     // dZ's rows and columns, all pixels, 64-pixel tiles of a split
   int pairs, cpt;              // X as pixel pairs; 64-channel chunks per tap (C = 64 j)
   size_t split_stride;
   float* out;  // partials, or the result when there is one split
@@ -87,8 +88,9 @@ k_conv_wgrad(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
   uint8_t* ones = smem + ST * Sh::kStageBytes;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int m0 = blockIdx.x * AC * NA, nt = blockIdx.y;
-  const int kt0 = blockIdx.z * g.kt_per_split;
-  const int nk = min(g.num_kt, kt0 + g.kt_per_split) - kt0;  // >= 1 (host)
+  const int64_t first = (int64_t)blockIdx.z * g.per * 64;
+  const int px = (int)min((int64_t)g.pixels - first, (int64_t)g.per * 64);  // >= 16 (host)
+  const int row0 = (int)first / g.Wo, ox0 = (int)first - row0 * g.Wo;
   const bool bias = nt == 0;  // this tile brings the columns from 9 C on
 
   if (threadIdx.x == 0) {
@@ -138,17 +140,15 @@ k_conv_wgrad(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
         h0[k] = k - 1;
       }
     }
-    int b = kt0 / (g.segs * g.hp), r = kt0 - b * g.segs * g.hp;
-    int hy = r / g.segs, seg = r - hy * g.segs;
+    int b = row0 / g.Ho, oy = row0 - b * g.Ho, ox = ox0;
     int issued = 0;
-    for (; issued < nk; issued++) {
+    for (int left = px; left > 0; issued++) {
       const int s = issued % ST;
       if (!mbar_wait(&empty[s], ((uint32_t)(issued / ST) & 1u) ^ 1u)) {
         s_fail = 1;
         break;
       }
       uint8_t* st = smem + s * Sh::kStageBytes;
-      const int ox = seg * g.pw, oy = hy * g.rows;
       mbar_expect_tx(&full[s], (uint32_t)Sh::kStageBytes);
 #pragma unroll
       for (int k = 0; k < NA; k++)
@@ -165,10 +165,13 @@ k_conv_wgrad(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
           tma_load_4d(st + k * Sh::kShiftBox, &ts, &full[s], CM == 32 ? 32 : 0, ox - 1,
                       2 * oy + h0[k], b);
       }
-      if (++seg == g.segs) {
-        seg = 0;
-        if (++hy == g.hp) {
-          hy = 0;
+      const int n = min(min(kWgRows, left), g.Wo - ox);
+      left -= n;
+      ox += n;
+      if (ox == g.Wo) {
+        ox = 0;
+        if (++oy == g.Ho) {
+          oy = 0;
           b++;
         }
       }
@@ -178,20 +181,24 @@ k_conv_wgrad(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
       if (!mbar_wait(&full[i % ST], (uint32_t)(i / ST) & 1u)) s_fail = 1;
   } else if (warp == 1 && lane == 0) {
     const uint64_t od = mn_major_desc(smem_u32(ones), 0, 128);
-    for (int i = 0; i < nk; i++) {
+    int ox = ox0;
+    for (int i = 0, left = px; left > 0; i++) {
       const int s = i % ST;
       if (!mbar_wait(&full[s], (uint32_t)(i / ST) & 1u)) {
         s_fail = 1;
         break;
       }
       tc_fence_after();
+      const int n = min(min(kWgRows, left), g.Wo - ox);  // a multiple of 16
+      left -= n;
+      ox = ox + n == g.Wo ? 0 : ox + n;
       const uint32_t a_s = smem_u32(smem + s * Sh::kStageBytes), b_s = a_s + NA * Sh::kABox;
       // one A box: the other rows of the tile read the same columns again
       const uint64_t ad = mn_major_desc(a_s, NA > 1 ? Sh::kABox : 0, 2 * AC);
       const uint64_t bd = mn_major_desc(b_s, Sh::kPairBox, CM == 8 ? 32 : 128);
       const uint64_t sd = mn_major_desc(b_s + 3 * Sh::kPairBox, Sh::kShiftBox, 64);
-#pragma unroll
-      for (int kk = 0; kk < kWgRows / 16; kk++) {  // 16 rows, in units of 16 bytes
+#pragma unroll 2
+      for (int kk = 0; kk < n / 16; kk++) {  // 16 rows, in units of 16 bytes
         const uint32_t acc = (i > 0 || kk > 0) ? 1u : 0u;
         const uint64_t a = ad + 2 * AC * kk;
         if constexpr (CM == 8) {  // six boxes of 16 columns
@@ -275,17 +282,17 @@ k_conv_wgrad(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
   if (threadIdx.x == 0 && s_fail && g.status) atomicCAS(g.status, 0, (int)GS2D_ERR_TIMEOUT);
 }
 
-// 4D map of an NHWC tensor [B][H][W][C]: boxes of `cols` channels x px pixels x
-// rows rows, stepping sw along W and sh along H; zeros out of range.
+// 4D map of an NHWC tensor [B][H][W][C]: boxes of `cols` channels x 128 pixels
+// of a row, stepping sw along it; zeros out of range.
 bool wg_map(CUtensorMap* map, const void* x, int B, int H, int W, int C, int64_t row_bytes,
-            int cols, int px, int rows, int sw, int sh) {
+            int cols, int sw) {
   EncodeTiled fn = tensor_map_encoder();
   if (!fn) return false;
   const cuuint64_t dims[4] = {(cuuint64_t)C, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)B};
   const cuuint64_t strides[3] = {(cuuint64_t)C * 2, (cuuint64_t)row_bytes,
                                  (cuuint64_t)row_bytes * H};
-  const cuuint32_t box[4] = {(cuuint32_t)cols, (cuuint32_t)(px * sw), (cuuint32_t)(rows * sh), 1};
-  const cuuint32_t estr[4] = {1, (cuuint32_t)sw, (cuuint32_t)sh, 1};
+  const cuuint32_t box[4] = {(cuuint32_t)cols, (cuuint32_t)(kWgRows * sw), 1, 1};
+  const cuuint32_t estr[4] = {1, (cuuint32_t)sw, 1, 1};
   const CUtensorMapSwizzle swz = cols == 16   ? CU_TENSOR_MAP_SWIZZLE_32B
                                  : cols == 32 ? CU_TENSOR_MAP_SWIZZLE_64B
                                               : CU_TENSOR_MAP_SWIZZLE_128B;
@@ -296,30 +303,26 @@ bool wg_map(CUtensorMap* map, const void* x, int B, int H, int W, int C, int64_t
 
 // The form of one product: 64, 32, 8, or 0 when there is none for it.
 int wg_form(int Wi, int C, int N) {
+  const int Wo = (Wi + 1) / 2;
+  if (Wo < 64 || Wo % 16) return 0;
   if (C % 64 == 0) return 64;
   if (Wi % 2) return 0;
   return C == 32 ? 32 : C == 8 && N <= 64 ? 8 : 0;
 }
 
 struct WgPlan {
-  int form, na, ac, mt, nt, pw, rows, segs, hp;
+  int form, na, ac, mt, nt;
   TnSplit sp;
 };
 
-WgPlan wg_plan(int B, int Hi, int Wi, int C, int N, int min_splits) {
+WgPlan wg_plan(int B, int Hi, int Wi, int C, int N, int splits) {
   WgPlan p;
   p.form = wg_form(Wi, C, N);
   p.ac = p.form == 8 && N <= 32 ? 32 : 64;
   p.na = N <= 64 ? 1 : 2;
   p.mt = (N + p.ac * p.na - 1) / (p.ac * p.na);
   p.nt = p.form == 64 ? 9 * (C / 64) / 3 : 1;
-  const int Ho = (Hi + 1) / 2, Wo = (Wi + 1) / 2;
-  p.pw = 16;
-  while (p.pw < Wo && p.pw < kWgRows) p.pw *= 2;
-  p.rows = kWgRows / p.pw;
-  p.segs = (Wo + p.pw - 1) / p.pw;
-  p.hp = (Ho + p.rows - 1) / p.rows;
-  p.sp = tn_split((int64_t)p.mt * p.nt, B * p.segs * p.hp, min_splits);
+  p.sp = tn_split((int64_t)B * ((Hi + 1) / 2) * ((Wi + 1) / 2), splits);
   return p;
 }
 
@@ -351,34 +354,32 @@ extern "C" int32_t gs2d_conv_wgrad_supported(int32_t B, int32_t Hi, int32_t Wi, 
 }
 
 extern "C" uint64_t gs2d_conv_wgrad_partial_bytes(int32_t B, int32_t Hi, int32_t Wi, int32_t C,
-                                                  int32_t N, int32_t ldc, int32_t min_splits) {
+                                                  int32_t N, int32_t ldc, int32_t splits) {
   if (!wg_sizes(B, Hi, Wi, C, N, ldc)) return 0;
-  const WgPlan p = wg_plan(B, Hi, Wi, C, N, min_splits);
+  const WgPlan p = wg_plan(B, Hi, Wi, C, N, splits);
   return p.sp.splits > 1 ? (uint64_t)p.sp.splits * N * ldc * sizeof(float) : 0;
 }
 
 extern "C" gs2d_status gs2d_conv_wgrad_bf16(const void* dz, int32_t N, const void* x, int32_t B,
                                             int32_t Hi, int32_t Wi, int32_t C, float* out,
-                                            int32_t ldc, int32_t min_splits, float* partial,
+                                            int32_t ldc, int32_t splits, float* partial,
                                             int32_t* status, void* stream) {
   if (!wg_sizes(B, Hi, Wi, C, N, ldc))
     return set_error(GS2D_ERR_INVALID_ARG, "gs2d_conv_wgrad_bf16: sizes");
   if (!dz || !x || !out || ((uintptr_t)dz & 15) || ((uintptr_t)x & 15))
     return set_error(GS2D_ERR_INVALID_ARG, "gs2d_conv_wgrad_bf16: NULL or misaligned operand");
-  const WgPlan p = wg_plan(B, Hi, Wi, C, N, min_splits);
+  const WgPlan p = wg_plan(B, Hi, Wi, C, N, splits);
   if (p.sp.splits > 1 && !partial)
     return set_error(GS2D_ERR_INVALID_ARG, "gs2d_conv_wgrad_bf16: the split needs partial");
-  const int Ho = (Hi + 1) / 2, Wo = (Wi + 1) / 2, sh = p.rows > 1 ? 2 : 1;
+  const int Ho = (Hi + 1) / 2, Wo = (Wi + 1) / 2;
   WgArgs g;
   g.M = N;
   g.C = C;
   g.ldc = ldc;
-  g.segs = p.segs;
-  g.hp = p.hp;
-  g.pw = p.pw;
-  g.rows = p.rows;
-  g.num_kt = p.sp.num_kt;
-  g.kt_per_split = p.sp.per;
+  g.Ho = Ho;
+  g.Wo = Wo;
+  g.pixels = B * Ho * Wo;
+  g.per = p.sp.per;
   g.pairs = Wi % 2 == 0;
   g.cpt = p.form == 64 ? C / 64 : 1;
   g.split_stride = p.sp.splits > 1 ? (size_t)N * ldc : 0;
@@ -387,11 +388,10 @@ extern "C" gs2d_status gs2d_conv_wgrad_bf16(const void* dz, int32_t N, const voi
   CUtensorMap ta, tb, ts;
   const int64_t row = (int64_t)Wi * C * 2;
   const int pc = g.pairs ? 2 * C : C, pwd = g.pairs ? Wi / 2 : Wi, sw = g.pairs ? 1 : 2;
-  bool ok = wg_map(&ta, dz, B, Ho, Wo, N, (int64_t)Wo * N * 2, p.ac, p.pw, p.rows, 1, 1) &&
-            wg_map(&tb, x, B, Hi, pwd, pc, row, p.form == 64 ? 64 : 2 * p.form, p.pw, p.rows, sw,
-                   sh);
+  bool ok = wg_map(&ta, dz, B, Ho, Wo, N, (int64_t)Wo * N * 2, p.ac, 1) &&
+            wg_map(&tb, x, B, Hi, pwd, pc, row, p.form == 64 ? 64 : 2 * p.form, sw);
   ts = tb;
-  if (ok && p.form == 32) ok = wg_map(&ts, x, B, Hi, pwd, pc, row, 32, p.pw, p.rows, 1, sh);
+  if (ok && p.form == 32) ok = wg_map(&ts, x, B, Hi, pwd, pc, row, 32, 1);
   if (!ok) return set_error(GS2D_ERR_CUDA, "gs2d_conv_wgrad_bf16: tensor map");
   const dim3 grid(p.mt, p.nt, p.sp.splits);
   cudaStream_t s = (cudaStream_t)stream;

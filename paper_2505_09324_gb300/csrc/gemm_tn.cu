@@ -18,8 +18,12 @@
 //  * a tile is 64 NA rows (m) x 64 NB columns (n), as wide as two stages of
 //    shared memory allow: NB up to 5 for NA = 1 (two MMAs, of 256 and 64 columns,
 //    into 320 TMEM columns), up to 4 for NA = 2;
-//  * K is split over whole waves of one CTA per SM, each writing an FP32
-//    partial tile; k_tn_reduce sums the splits in a fixed order.
+//  * K is split as gs2d_gemm_bf16 splits it, each split writing an FP32
+//    partial tile; k_tn_reduce sums them in order.  The sums are the K-major
+//    GEMM's bit for bit: an Adam step turns the sign of a gradient that is zero
+//    but for rounding into a step of the whole rate, so other splits (over whole
+//    waves: 0.2 ms less of a training step) moved the gradients of the next step
+//    by up to 3e-4 now and then.
 // Warp 0, one lane, issues the TMA boxes into a ring of ST stages; warp 1, one
 // lane, the MMAs (eight K = 16 steps per stage); warps 0-3 the epilogue.
 // Waits are bounded as in csrc/gemm_tc.cu; the producer also waits (bounded)
@@ -52,7 +56,7 @@ struct TnShape {
 };
 
 struct TnArgs {
-  int M, N, num_kt, kt_per_split, ldc;
+  int M, N, K, per, ldc;  // per: 64-row tiles of a split
   size_t split_stride;
   float* out;  // partials, or the result when there is one split
   int* status;
@@ -73,8 +77,11 @@ k_gemm_tn(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtens
                                              ~uintptr_t(1023));
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int m0 = blockIdx.x * 64 * NA, n0 = blockIdx.y * Sh::kBN;
-  const int kt0 = blockIdx.z * g.kt_per_split;
-  const int nk = min(g.num_kt, kt0 + g.kt_per_split) - kt0;  // >= 1 (host)
+  // this split's rows, a multiple of 64 (or to the end): stages of 128, the
+  // last of which may be half used
+  const int64_t row0 = (int64_t)blockIdx.z * g.per * 64;
+  const int rows = (int)min((int64_t)g.K - row0, (int64_t)g.per * 64);  // >= 1 (host)
+  const int nk = (rows + kTnRows - 1) / kTnRows;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < ST; s++) {
@@ -105,7 +112,7 @@ k_gemm_tn(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtens
         break;
       }
       uint8_t* st = smem + s * Sh::kStageBytes;
-      const int row = (kt0 + issued) * kTnRows;
+      const int row = (int)row0 + issued * kTnRows;
       mbar_expect_tx(&full[s], (uint32_t)Sh::kStageBytes);
 #pragma unroll
       for (int c = 0; c < NA; c++) tma_load_2d(st + c * kTnBox, &ta, &full[s], m0 + 64 * c, row);
@@ -131,8 +138,9 @@ k_gemm_tn(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtens
       // one A box: rows 64 ... 127 of the tile read the same columns again
       const uint64_t ad = mn_major_desc(a_s, NA > 1 ? kTnBox : 0, 128);
       const uint64_t bd = mn_major_desc(b_s, kTnBox, 128), bd2 = bd + 4 * (kTnBox >> 4);
-#pragma unroll
-      for (int kk = 0; kk < kTnRows / 16; kk++) {  // 16 rows of 128 bytes: 128 units
+      const int used = min(kTnRows / 64, (rows - i * kTnRows + 63) / 64) * 4;
+#pragma unroll 4
+      for (int kk = 0; kk < used; kk++) {  // 16 rows of 128 bytes: 128 units
         const uint32_t acc = (i > 0 || kk > 0) ? 1u : 0u;
         mma_bf16(tmem, ad + 128 * kk, bd + 128 * kk, id1, acc);
         if (kN2) mma_bf16(tmem + 256, ad + 128 * kk, bd2 + 128 * kk, id2, acc);
@@ -163,69 +171,49 @@ k_gemm_tn(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtens
   if (threadIdx.x == 0 && s_fail && g.status) atomicCAS(g.status, 0, (int)GS2D_ERR_TIMEOUT);
 }
 
-// Sum of the partial tiles: a block takes 256 / SL vectors of V outputs, in SL
-// slices of the splits whose sums are added in a fixed order (deterministic),
-// with up to eight loads in flight per thread.  SL is chosen so that a thread
-// sums at most about 20 splits: one scheme of 8 slices left the many-split
-// layers waiting on a few loads (75 splits a thread, 80 blocks) and gave the
-// few-split layers a barrier and a division for every one or two of them.  The
-// training step's six reductions at 1080p, batch 8: 294 -> 206 us, each with
-// its wait for the kernel before it.
-template <int SL, int V>
-__global__ void __launch_bounds__(256)
+// Sum of the partial tiles, split after split (deterministic, the order of
+// csrc/gemm_tc.cu), V outputs a thread with kFlight loads in flight.
+template <int V, int kFlight>
+__global__ void __launch_bounds__(128)
 k_tn_reduce(uint32_t M, uint32_t nv, uint32_t ldv, int splits, size_t stride,
             const float* __restrict__ partial, float* __restrict__ out) {
   using Vec = std::conditional_t<V == 4, float4, float>;
-  constexpr int kOut = 256 / SL;
   pdl_begin();
-  __shared__ float s_sum[SL > 1 ? SL - 1 : 1][kOut * V];
-  const uint32_t k = threadIdx.x % kOut, slice = threadIdx.x / kOut;
-  const size_t i = (size_t)blockIdx.x * kOut + k;
-  const bool in = i < (size_t)M * nv;
+  const size_t i = (size_t)blockIdx.x * 128 + threadIdx.x;
+  if (i >= (size_t)M * nv) return;
   size_t o = i;
-  if (nv != ldv) o = in ? (i / nv) * ldv + i % nv : 0;
+  if (nv != ldv) o = (i / nv) * ldv + i % nv;
   const Vec* src = reinterpret_cast<const Vec*>(partial) + o;
   const size_t step = stride / V;
   float x[V];
 #pragma unroll
   for (int j = 0; j < V; j++) x[j] = 0.0f;
-  if (in) {
-#pragma unroll 8
-    for (int z = (int)slice; z < splits; z += SL) {
-      const Vec v = src[(size_t)z * step];
-      const float* f = reinterpret_cast<const float*>(&v);
+  const auto add = [&](const Vec& v) {
+    const float* f = reinterpret_cast<const float*>(&v);
 #pragma unroll
-      for (int j = 0; j < V; j++) x[j] += f[j];
-    }
+    for (int j = 0; j < V; j++) x[j] += f[j];
+  };
+  int z = 0;
+  for (; z + kFlight <= splits; z += kFlight) {
+    Vec v[kFlight];
+#pragma unroll
+    for (int u = 0; u < kFlight; u++) v[u] = src[(size_t)(z + u) * step];
+#pragma unroll
+    for (int u = 0; u < kFlight; u++) add(v[u]);
   }
-  if constexpr (SL > 1) {
-    if (slice > 0)
+  for (; z < splits; z++) add(src[(size_t)z * step]);
+  Vec v;
 #pragma unroll
-      for (int j = 0; j < V; j++) s_sum[slice - 1][k * V + j] = x[j];
-    __syncthreads();
-    if (slice > 0) return;
-#pragma unroll
-    for (int z = 0; z < SL - 1; z++)
-#pragma unroll
-      for (int j = 0; j < V; j++) x[j] += s_sum[z][k * V + j];
-  }
-  if (in) {
-    Vec v;
-#pragma unroll
-    for (int j = 0; j < V; j++) reinterpret_cast<float*>(&v)[j] = x[j];
-    reinterpret_cast<Vec*>(out)[o] = v;
-  }
+  for (int j = 0; j < V; j++) reinterpret_cast<float*>(&v)[j] = x[j];
+  reinterpret_cast<Vec*>(out)[o] = v;
 }
 
-template <int SL>
+template <int V, int kFlight>
 cudaError_t launch_reduce(int M, int N, int ldc, int splits, size_t stride, const float* partial,
                           float* out, cudaStream_t s) {
-  const bool vec = N % 4 == 0 && ldc % 4 == 0 && stride % 4 == 0 &&
-                   (((uintptr_t)partial | (uintptr_t)out) & 15) == 0;
-  const int v = vec ? 4 : 1;
-  const unsigned blocks = (unsigned)(((size_t)M * (N / v) + 256 / SL - 1) / (256 / SL));
-  return launch_pdl(vec ? k_tn_reduce<SL, 4> : k_tn_reduce<SL, 1>, blocks, 256, 0, s, (uint32_t)M,
-                    (uint32_t)(N / v), (uint32_t)(ldc / v), splits, stride, partial, out);
+  return launch_pdl(k_tn_reduce<V, kFlight>, (unsigned)(((size_t)M * (N / V) + 127) / 128), 128, 0,
+                    s, (uint32_t)M, (uint32_t)(N / V), (uint32_t)(ldc / V), splits, stride,
+                    partial, out);
 }
 
 // 2D map of a rows x cols matrix (cols contiguous): 64 x 128 boxes, 128-byte
@@ -250,7 +238,7 @@ struct TnPlan {
   TnSplit sp;
 };
 
-TnPlan tn_plan(int M, int N, int K, int min_splits) {
+TnPlan tn_plan(int M, int N, int K, int splits) {
   TnPlan p;
   p.na = M <= 64 ? 1 : 2;
   p.mt = (M + 64 * p.na - 1) / (64 * p.na);
@@ -258,7 +246,7 @@ TnPlan tn_plan(int M, int N, int K, int min_splits) {
   p.nt = (chunks + widest - 1) / widest;
   p.nb = (chunks + p.nt - 1) / p.nt;
   p.nt = (chunks + p.nb - 1) / p.nb;
-  p.sp = tn_split((int64_t)p.mt * p.nt, (K + kTnRows - 1) / kTnRows, min_splits);
+  p.sp = tn_split(K, splits);
   return p;
 }
 
@@ -285,13 +273,10 @@ cudaError_t launch_tn_na(int nb, const CUtensorMap& ta, const CUtensorMap& tb, c
 
 }  // namespace
 
-TnSplit tn_split(int64_t tiles, int num_kt, int min_splits) {
+TnSplit tn_split(int64_t pixels, int splits) {
   TnSplit p;
-  p.num_kt = num_kt;
-  const int64_t need = std::max<int64_t>(1, std::min<int64_t>(min_splits, num_kt));
-  const int64_t waves = (need * tiles + 151) / 152;
-  const int64_t most = std::min<int64_t>(num_kt, 65535);  // gridDim.z
-  p.splits = (int)std::min(most, std::max(need, waves * 152 / tiles));
+  const int num_kt = (int)((pixels + 63) / 64);
+  p.splits = std::max(1, std::min(std::min(splits, num_kt), 65535));  // gridDim.z
   p.per = (num_kt + p.splits - 1) / p.splits;
   p.splits = (num_kt + p.per - 1) / p.per;
   return p;
@@ -299,10 +284,12 @@ TnSplit tn_split(int64_t tiles, int num_kt, int min_splits) {
 
 cudaError_t launch_tn_reduce(int M, int N, int ldc, int splits, size_t stride,
                              const float* partial, float* out, cudaStream_t s) {
-  if (splits <= 20) return launch_reduce<1>(M, N, ldc, splits, stride, partial, out, s);
-  if (splits <= 80) return launch_reduce<4>(M, N, ldc, splits, stride, partial, out, s);
-  if (splits <= 240) return launch_reduce<8>(M, N, ldc, splits, stride, partial, out, s);
-  return launch_reduce<32>(M, N, ldc, splits, stride, partial, out, s);
+  // one output a thread while that leaves SMs without work otherwise
+  const bool vec = N % 4 == 0 && ldc % 4 == 0 && stride % 4 == 0 &&
+                   (((uintptr_t)partial | (uintptr_t)out) & 15) == 0;
+  if (vec && (size_t)M * N >= 152 * 1024)
+    return launch_reduce<4, 8>(M, N, ldc, splits, stride, partial, out, s);
+  return launch_reduce<1, 16>(M, N, ldc, splits, stride, partial, out, s);
 }
 
 }  // namespace gs2d
@@ -310,15 +297,15 @@ cudaError_t launch_tn_reduce(int M, int N, int ldc, int splits, size_t stride,
 using namespace gs2d;
 
 extern "C" uint64_t gs2d_gemm_tn_partial_bytes(int32_t M, int32_t N, int32_t ldc, int32_t K,
-                                               int32_t min_splits) {
+                                               int32_t splits) {
   if (M < 1 || N < 1 || K < 1 || ldc < N) return 0;
-  const TnPlan p = tn_plan(M, N, K, min_splits);
+  const TnPlan p = tn_plan(M, N, K, splits);
   return p.sp.splits > 1 ? (uint64_t)p.sp.splits * M * ldc * sizeof(float) : 0;
 }
 
 extern "C" gs2d_status gs2d_gemm_tn_bf16(const void* A, int32_t lda, const void* B, int32_t ldb,
                                          int32_t M, int32_t N, int32_t K, float* out, int32_t ldc,
-                                         int32_t min_splits, float* partial, int32_t* status,
+                                         int32_t splits, float* partial, int32_t* status,
                                          void* stream) {
   if (M < 0 || N < 0 || K < 0 || lda < M || ldb < N || ldc < N || (lda % 8) || (ldb % 8))
     return set_error(GS2D_ERR_INVALID_ARG, "gs2d_gemm_tn_bf16: sizes / leading dimensions");
@@ -330,7 +317,7 @@ extern "C" gs2d_status gs2d_gemm_tn_bf16(const void* A, int32_t lda, const void*
   if (K == 0) {
     e = cudaMemset2DAsync(out, (size_t)ldc * 4, 0, (size_t)N * 4, M, s);
   } else {
-    const TnPlan p = tn_plan(M, N, K, min_splits);
+    const TnPlan p = tn_plan(M, N, K, splits);
     if (p.sp.splits > 1 && !partial)
       return set_error(GS2D_ERR_INVALID_ARG, "gs2d_gemm_tn_bf16: the split needs partial");
     CUtensorMap ta, tb;
@@ -339,8 +326,8 @@ extern "C" gs2d_status gs2d_gemm_tn_bf16(const void* A, int32_t lda, const void*
     TnArgs g;
     g.M = M;
     g.N = N;
-    g.num_kt = p.sp.num_kt;
-    g.kt_per_split = p.sp.per;
+    g.K = K;
+    g.per = p.sp.per;
     g.ldc = ldc;
     g.split_stride = p.sp.splits > 1 ? (size_t)M * ldc : 0;
     g.out = p.sp.splits > 1 ? partial : out;

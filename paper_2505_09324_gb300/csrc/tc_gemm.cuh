@@ -92,15 +92,12 @@ cudaError_t tc_conv_frame(const TcFrameConvProblem& pr, cudaStream_t s);
 int tc_gemm_bn(int n);
 size_t tc_gemm_partial_floats(int M, int N, int ldc, int K, int splits);
 
-// Split of a weight gradient's pixels (csrc/gemm_tn.cu): num_kt steps of 128
-// pixels, `per` of them to each of `splits` CTAs of a tile.  At least min_splits
-// (the FP32 sums in tensor memory lose precision with their length, so the
-// caller says how short they are to be), and more where that completes the last
-// wave of 152 CTAs, one step each at most.
+// Split of a weight gradient's pixels (csrc/gemm_tn.cu), that of gs2d_gemm_bf16:
+// `per` tiles of 64 pixels to each of `splits` splits.
 struct TnSplit {
-  int num_kt, per, splits;
+  int per, splits;
 };
-TnSplit tn_split(int64_t tiles, int num_kt, int min_splits);
+TnSplit tn_split(int64_t pixels, int splits);
 
 // out[M][ldc] = sum of the splits' partial tiles, `stride` floats apart.
 cudaError_t launch_tn_reduce(int M, int N, int ldc, int splits, size_t stride,

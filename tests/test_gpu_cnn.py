@@ -477,12 +477,12 @@ def test_gemm_over_rows_matches_oracle(nat, M, N, K, splits):
 
 
 @pytest.mark.parametrize("B,H,W,C,N,splits", [
-    (1, 7, 258, 64, 40, 3),      # pairs, two steps a row, odd rows
-    (2, 9, 129, 64, 200, 1),     # odd width: traversal stride; two blocks of M, ragged
-    (3, 21, 34, 128, 64, 2),     # 17 pixels: four rows a step, ragged rows
-    (1, 50, 9, 192, 128, 40),    # eight rows a step, more splits than steps
-    (2, 6, 300, 32, 64, 5), (1, 11, 64, 32, 136, 1),     # pairs of 32 channels
-    (2, 6, 514, 8, 32, 7), (1, 33, 62, 8, 64, 1), (1, 1, 2, 8, 8, 1)])  # pairs of 8
+    (1, 7, 256, 64, 40, 3),      # pairs, odd rows
+    (2, 9, 127, 64, 200, 1),     # odd width: traversal stride; two blocks of M, ragged
+    (3, 5, 160, 128, 64, 2),     # 80 pixels a row: splits within rows
+    (1, 4, 288, 192, 128, 40),   # two steps a row, more splits than tiles of 64 pixels
+    (2, 6, 320, 32, 64, 5), (1, 11, 128, 32, 136, 1),     # pairs of 32 channels
+    (2, 6, 512, 8, 32, 7), (1, 33, 160, 8, 64, 2), (1, 1, 128, 8, 8, 1)])  # pairs of 8
 def test_conv_weight_gradient_matches_oracle(nat, B, H, W, C, N, splits):
     """gs2d_conv_wgrad_bf16 (3 x 3, stride 2, pad 1) against dZ^T im2col(x), the
     bias column and the zeros beyond it, within the GEMM bar, for each of its
@@ -504,6 +504,25 @@ def test_conv_weight_gradient_matches_oracle(nat, B, H, W, C, N, splits):
     got = out.cpu().numpy().astype(np.float64)
     assert int(status.item()) == 0
     assert np.all(np.abs(got - cnn.gemm(dz.T, col.T)) <= REL * cnn.gemm_abs(dz.T, col.T) + 1e-30)
+    # bit for bit the GEMM over the operand, read as it lies and transposed
+    P, Pl = dz.shape[0], -(-dz.shape[0] // 8) * 8
+    d_col, others = bf16_dev(col), []
+    for tn in (True, False):
+        o = torch.full((N, ldc), float("nan"), device="cuda")
+        part = torch.empty((splits + 1) * N * ldc, device="cuda")
+        if tn:
+            nat.call("gs2d_gemm_tn_bf16", d_dz.data_ptr(), N, d_col.data_ptr(), ldc, N, ldc, P,
+                     o.data_ptr(), ldc, splits, part.data_ptr(), status.data_ptr(), 0)
+        else:
+            T = [torch.zeros((t.shape[1], Pl), dtype=torch.bfloat16, device="cuda")
+                 for t in (d_dz, d_col)]
+            for t, u in zip(T, (d_dz, d_col)):
+                t[:, :P] = u.reshape(P, -1).T
+            nat.gemm_bf16(T[0].data_ptr(), Pl, T[1].data_ptr(), Pl, N, ldc, P, 0, False,
+                          o.data_ptr(), 0, ldc, splits, part.data_ptr(), status.data_ptr(), 0)
+        others.append(o)
+    assert int(status.item()) == 0
+    assert torch.equal(out, others[0]) and torch.equal(out, others[1])
 
 
 @pytest.mark.parametrize("C,ks,st,pad,H,W", [(8, 3, 2, 1, 5, 301), (24, 3, 2, 1, 3, 40),
