@@ -279,7 +279,7 @@ k_chamfer_grad(const float* __restrict__ P, int np, int ldp, const float* __rest
 // per thread, doubles only across threads and one division per mean: FP64 issues
 // at 1/64 of the FP32 rate, and double sums and divisions in every thread took
 // 33 us for 20 000 points a side, 23 so with its wait (training step 2.264 ->
-// 2.253 ms).
+// 2.253 ms then).
 __global__ void __launch_bounds__(1024)
 k_chamfer_loss(const float* __restrict__ d1, int np, const float* __restrict__ d2, int nq,
                float* __restrict__ loss) {

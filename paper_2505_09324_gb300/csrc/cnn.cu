@@ -272,10 +272,11 @@ constexpr int kColChunks = 2048;
 
 // A block writes the col rows of `run` consecutive output pixels of one output
 // row, consecutive threads consecutive 16-byte chunks.  Memory-bound by what
-// it writes (1.8 GB per training step at 1080p, batch 8), provided the index
-// work stays small: the tap of a chunk is looked up in a table that the block
-// builds once, and the row is the block's, so a chunk costs one division by a
-// multiplication: 461 us a step (599 with three or four divisions each).
+// it writes (1.8 GB per training step at 1080p, batch 8, when every layer wrote
+// it), provided the index work stays small: the tap of a chunk is looked up in a
+// table that the block builds once, and the row is the block's, so a chunk costs
+// one division by a multiplication: 461 us for those (599 with three or four
+// divisions each).
 __global__ void __launch_bounds__(256)
 k_im2col(int Hi, int Wi, int C, int Ho, int Wo, int ks, int stride, int pad, int ldk, int run,
          int segs, const bf16* __restrict__ x, bf16* __restrict__ col) {
@@ -348,9 +349,9 @@ __global__ void k_im2col_any(int B, int Hi, int Wi, int C, int Ho, int Wo, int k
 // read it, FP32 sums in the order of the taps, 16-byte loads and one 16-byte
 // store.  KS and ST fixed at compile time for the network's 3 x 3 stride-2
 // layers (0: runtime), where a pixel is read by one, two or four taps.
-// Memory-bound by dcol (2.3 GB per training step at 1080p, batch 8); with a
-// thread per channel the index arithmetic bounded it at a tenth of that rate
-// (3.74 ms a step, 0.69 now).
+// Memory-bound by dcol (2.3 GB per training step at 1080p, batch 8, when every
+// layer went through it); with a thread per channel the index arithmetic bounded
+// it at a tenth of that rate (3.74 ms for those, 0.69 so).
 template <int KS, int ST>
 __global__ void __launch_bounds__(256)
 k_col2im8(const float* __restrict__ dcol, int ldk, unsigned total, int Hi, int Wi, int C8, int Ho,
