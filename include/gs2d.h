@@ -323,8 +323,9 @@ gs2d_status gs2d_pframe_step(const gs2d_plan* plan, void* ws, const float* targe
                              void* stream);
 
 /* Fits a P-frame: `iters` gs2d_pframe_step iterations (moments zeroed first;
- * more than 64 on a non-default stream replayed as a captured CUDA graph), then final_psnr (host, may be NULL) = the
- * full-frame PSNR of the result.  Synchronises the stream. */
+ * more than 64 on a non-default stream replayed as a captured CUDA graph), then
+ * final_psnr (host, may be NULL) = the full-frame PSNR of the result.
+ * Synchronises the stream. */
 gs2d_status gs2d_encode_pframe(const gs2d_plan* plan, void* ws, const float* target,
                                float* params, float* adam_m, float* adam_v,
                                const uint8_t* selected, int32_t iters, float* final_psnr,
@@ -616,7 +617,8 @@ uint64_t gs2d_gemm_partial_bytes(int32_t M, int32_t N, int32_t ldc, int32_t K, i
  * the transposed operands with the same `splits`.  K is split over that many
  * groups of thread blocks, as far as it goes (FP32 sums lose precision with
  * their length); partial (device, gs2d_gemm_tn_partial_bytes bytes) then holds
- * FP32 partial sums that a second kernel adds in a fixed order (deterministic).  status as gs2d_gemm_bf16. */
+ * FP32 partial sums that a second kernel adds in a fixed order (deterministic).
+ * status as gs2d_gemm_bf16. */
 gs2d_status gs2d_gemm_tn_bf16(const void* A, int32_t lda, const void* B, int32_t ldb, int32_t M,
                               int32_t N, int32_t K, float* out, int32_t ldc, int32_t splits,
                               float* partial, int32_t* status, void* stream);

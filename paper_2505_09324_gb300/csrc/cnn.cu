@@ -882,8 +882,8 @@ extern "C" gs2d_status gs2d_head_decode(const float* out, int32_t ldo, int32_t B
              (int)gh, (int)gw, (int)slots, (int)n, sel);
   const size_t total = (size_t)B * n;
   const size_t want = (total + 255) / 256;
-  launch_pdl(k_head_decode, (int)(want < 152 * 8 ? want : 152 * 8), 256, 0, s, out, (int)ldo, (int)B,
-             (int)gh, (int)gw, (int)slots, (int)cell_px, scale, (int)n, params, (int)ldp,
+  launch_pdl(k_head_decode, (int)(want < 152 * 8 ? want : 152 * 8), 256, 0, s, out, (int)ldo,
+             (int)B, (int)gh, (int)gw, (int)slots, (int)cell_px, scale, (int)n, params, (int)ldp,
              (const int*)sel);
   return launched("gs2d_head_decode");
 }

@@ -327,8 +327,8 @@ WgPlan wg_plan(int B, int Hi, int Wi, int C, int N, int splits) {
 }
 
 bool wg_sizes(int B, int Hi, int Wi, int C, int N, int ldc) {
-  return B >= 1 && Hi >= 1 && Wi >= 1 && C >= 8 && C <= 1 << 20 && C % 8 == 0 && N >= 8 && N % 8 == 0 &&
-         ldc >= 9 * (int64_t)C + 1 && wg_form(Wi, C, N) != 0 &&
+  return B >= 1 && Hi >= 1 && Wi >= 1 && C >= 8 && C <= 1 << 20 && C % 8 == 0 && N >= 8 &&
+         N % 8 == 0 && ldc >= 9 * (int64_t)C + 1 && wg_form(Wi, C, N) != 0 &&
          (int64_t)B * ((Hi + 1) / 2) * ((Wi + 1) / 2 + kWgRows) <= INT32_MAX &&
          (int64_t)N * ldc <= INT32_MAX;
 }

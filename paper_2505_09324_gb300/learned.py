@@ -17,8 +17,8 @@ the operand).  The backward pass is one weight gradient (dZ^T . col, split over
 pixels: straight from the activations by gs2d_conv_wgrad_bf16, else from the
 operand, which the forward pass then writes, by gs2d_gemm_tn_bf16) and one
 input gradient with the ReLU mask per layer: one implicit GEMM over shifted dZ
-boxes where rows are wide (gs2d_conv_dgrad_bf16), else a GEMM (dZ . W) + col2im.  The optimiser is the
-library's Adam on the FP32 master weights.  Training minimises the L2 render
+boxes where rows are wide (gs2d_conv_dgrad_bf16), else a GEMM (dZ . W) + col2im.
+The optimiser is the library's Adam on the FP32 master weights.  Training minimises the L2 render
 loss of the decoded Gaussians through the rasterizer (the colour and shape
 signal the paper's regressor lacked) plus lambda times the Chamfer distance
 between the predicted means and those of Gaussians the encoder fitted to the
