@@ -169,7 +169,7 @@ gs2d_status gs2d_plan_init_batch(gs2d_plan* plan, gs2d_clip* clips, int32_t num_
   sz[kOffClips] = (uint64_t)num_clips * sizeof(gs2d_clip);
   sz[kOffRec] = 3 * nn * sizeof(float4);
   sz[kOffRect] = nn * sizeof(int4);
-  sz[kOffCount] = (nn + 1) * sizeof(int);
+  sz[kOffCount] = nn * sizeof(int);
   // up to three sums per group of at least 64 Gaussians
   sz[kOffBlockSum] = 3 * (nn / 64 + 1) * sizeof(long long);
   sz[kOffTileCnt] = nt * sizeof(int);

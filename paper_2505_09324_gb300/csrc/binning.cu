@@ -56,7 +56,7 @@ struct BinArgs {
   float4* rec;
   int4* rect;              // tight rectangles
   int4* lrect;             // the rectangles the lists are built from
-  int* offs;               // [n + 1] first backward slot of each Gaussian
+  int* offs;               // [n] first backward slot of each Gaussian
   int* tile_cnt;           // zero between calls
   int* tile_cnt2;          // the same for the tight rectangles of a rebuild
   long long* sums;         // [2][groups] entries per group, then exclusive offsets
@@ -485,7 +485,6 @@ k_bin_scatter(const __grid_constant__ BinArgs a, const long long* __restrict__ f
   long long ex;
   const long long total = group_entries(gs, rc, a.group, &ex);
   if (mine) a.offs[i] = over ? 0 : (int)(base + ex);
-  if (i == a.n - 1) a.offs[a.n] = over ? 0 : (int)(base + total);
   if (over) return;
   for (int e0 = t; e0 < (int)total; e0 += kThreads * kInFlight) {
     int pos[kInFlight], gi[kInFlight];

@@ -25,7 +25,7 @@ enum WsSection {
   kOffClips,        // gs2d_clip[num_clips] (batch plans)
   kOffRec,          // float4[3][n]  render records (SoA of float4 rows)
   kOffRect,         // int4[n]       tile rectangle (first tile, row stride, w, h)
-  kOffCount,        // int32[n + 1]  first backward slot of each Gaussian (listed rectangles)
+  kOffCount,        // int32[n]  first backward slot of each Gaussian (listed rectangles)
   kOffBlockSum,     // int64[3][n / 64 + 1]  entries per group of Gaussians, their offsets
   kOffTileCnt,      // int32[num_tiles]  entries per tile (zero between calls)
   kOffCursor,       // int32[num_tiles]  next free slot of each tile's list

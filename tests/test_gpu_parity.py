@@ -497,6 +497,24 @@ def test_bins_bit_exact_at_the_edges_of_the_sort(gs, oracle, n, W, H, share):
     np.testing.assert_array_equal(r.read_bins()["values"], first)
 
 
+@pytest.mark.parametrize("n", [1, 63, 65, 130, 300])
+def test_scatter_stores_one_slot_per_gaussian(gs, n):
+    """The blocks of the scatter have more threads than Gaussians: the first
+    slots are those of the n Gaussians, in their order, and the word behind
+    them (padding of the section) is not theirs to write."""
+    W, H = 90, 70
+    r = gs.GaussianRasterizer(W, H, n)
+    first = int(r.plan.off[4])  # header, clips, records, rectangles, first slots
+    words = r.ws[first:first + 4 * (n + 1)].view(torch.int32)
+    words[n] = -12345
+    r.prepare(to_dev(random_gaussians(n, W, H, seed=n)))
+    bins = r.read_bins()
+    counts = np.asarray(bins["counts"])
+    got = words.cpu().numpy()
+    np.testing.assert_array_equal(got[:n], np.cumsum(counts) - counts)
+    assert got[n] == -12345 and r.status() == 0
+
+
 def test_fit_on_large_plans_equals_per_iteration_binning(gs):
     """Retained lists against per-iteration binning beyond the one-block scan
     (many tiles), where the scan has a launch of its own."""
