@@ -86,8 +86,8 @@ typedef struct {
    * has left its listed tiles (checked on the device every iteration).  The
    * results are the same as binning every iteration (tiles a Gaussian does
    * not reach contribute nothing; a rebuild whose widened lists would not
-   * fit max_entries lists the tight boxes instead).  Negative: bin every
-   * iteration.  Default 4. */
+   * fit max_entries, or one of them the longest list that is sorted, lists
+   * the tight boxes instead).  Negative: bin every iteration.  Default 4. */
   float bin_margin;
   /* Backward reduction to per-Gaussian sums: GS2D_REDUCE_SLOTS (default: one
    * record per (tile, Gaussian) pair, summed per Gaussian in a fixed order,

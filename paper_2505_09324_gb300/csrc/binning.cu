@@ -221,10 +221,26 @@ __device__ __forceinline__ long long scan_sums(const long long* sums, long long*
   return run;
 }
 
+// Whether a rebuild lists the tight rectangles instead of the widened ones:
+// where these overflow the capacity, or one tile's list of them is too long to
+// sort, and the tight ones do neither.  Lists hold a Gaussian at most once, so
+// the tiles are looked at only beyond kLongMax Gaussians.  The same in every
+// thread of every block: the counts are complete and the totals global.
+__device__ __forceinline__ bool rebuild_tight(const BinArgs& a, long long total,
+                                              long long total2) {
+  if (total2 > a.max_entries) return false;
+  if (total > a.max_entries || a.n <= kLongMax) return total > a.max_entries;
+  bool wide = false, tight = false;
+  for (int i = threadIdx.x; i < a.num_tiles; i += kThreads) {
+    wide |= __ldcg(&a.tile_cnt[i]) > kLongMax;
+    tight |= __ldcg(&a.tile_cnt2[i]) > kLongMax;
+  }
+  return __syncthreads_or(wide) && !__syncthreads_or(tight);
+}
+
 // The whole scan by one block (k_count's last): group offsets, the capacity
 // decision, list ranges, cursors and queue ranks of the tiles; the tile counts
-// are cleared for the next binning.  LAZY: a rebuild whose widened lists
-// overflow lists the tight rectangles instead.
+// are cleared for the next binning.  LAZY: a rebuild, see rebuild_tight.
 template <bool LAZY>
 __device__ __forceinline__ void one_block_scan(const BinArgs& a, GroupSmem& gs, int* s_hist) {
   const int t = threadIdx.x;
@@ -233,7 +249,7 @@ __device__ __forceinline__ void one_block_scan(const BinArgs& a, GroupSmem& gs, 
   if (LAZY) {
     const long long total2 =
         scan_sums(a.sums + a.groups, a.sums + a.groups, a.groups, gs.warp_sum);
-    tight = total > a.max_entries && total2 <= a.max_entries;
+    tight = rebuild_tight(a, total, total2);
     if (tight) total = total2;
   }
   const bool over = total > a.max_entries;
@@ -406,8 +422,7 @@ k_bin_scan(const __grid_constant__ BinArgs a, long long* __restrict__ first) {
   }
   block_scan(tot, warp_sum, &total);
   if (LAZY) block_scan(tot2, warp_sum, &total2);
-  // the same decision in every block: the totals are global
-  const bool tight = LAZY && total > a.max_entries && total2 <= a.max_entries;
+  const bool tight = LAZY && rebuild_tight(a, total, total2);
   if (tight) total = total2;
   const bool over = total > a.max_entries;
   if (tb < 0) {

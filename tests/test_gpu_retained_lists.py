@@ -249,3 +249,54 @@ def test_empty_gaussian_sets(gs):
     gs.GaussianRasterizer(w2, h2, n2, config=cfg).encode_frame(t2, alone, iters,
                                                                 check_every=iters)
     assert torch.equal(pp, alone)
+
+
+def _two_piles(n, near, tile, grid, size, seed):
+    """n Gaussians of a frame of `grid` tiles: `near` of them well inside the
+    first tile, the others in the second one, within the widening of their
+    common edge: the first tile's widened list holds all n."""
+    g = np.random.Generator(np.random.PCG64(seed))
+    p = np.empty((9, n))
+    p[0, :near] = g.uniform(4, tile - 4, near)
+    p[0, near:] = g.uniform(tile + 1.5, tile + 2.5, n - near)
+    p[1] = g.uniform(4, tile - 4, n)
+    p[2:5] = size
+    p[3] = 0.0
+    p[5:8], p[8] = g.uniform(0, 1e-4, (3, n)), 1.0
+    return p, tile * grid[0], tile * grid[1]
+
+
+@pytest.mark.parametrize("n,near,tile,grid,size", [
+    (32769, 20000, 16, (2, 2), 0.1), (33500, 32768, 32, (3, 2), 0.1),
+    (33000, 16400, 8, (64, 40), 0.1),  # (no Gaussian reaches a pixel's centre)
+    (33000, 16400, 8, (64, 40), 0.3)])
+def test_widened_list_past_the_longest_falls_back_to_tight(gs, n, near, tile, grid, size):
+    """A tile whose widened list is too long to sort while its tight one is
+    not: the rebuild lists the tight rectangles, as it does when the widened
+    ones exceed the capacity, for a fit and for a P-frame (scan in the counting
+    launch's last block and in a launch of its own).  The same Gaussians as with
+    lists rebuilt every iteration."""
+    from paper_2505_09324_gb300 import _native as nat
+    p0, W, H = _two_piles(n, near, tile, grid, size, seed=n)
+    t = to_dev(smooth_noise_target(W, H, seed=3))
+    sel = (torch.arange(n, device="cuda") % 3 > 0).to(torch.uint8)
+    s = int(torch.cuda.current_stream().cuda_stream)
+    fit, pframe = [], []
+    for margin in (-1.0, 4.0):
+        cfg = gs.RasterConfig(tile=tile, bin_margin=margin, lr=1e-3)
+        r = gs.GaussianRasterizer(W, H, n, config=cfg)
+        assert (r.plan.num_tiles > 2048) == (grid[0] * grid[1] > 2048)
+        for out, step in ((fit, 0), (pframe, 1)):
+            p = to_dev(p0)
+            m, v = torch.empty_like(p), torch.empty_like(p)
+            if step:
+                r.encode_pframe(t, p, sel, 3, adam_state=(m, v))
+            else:
+                r.fit_reset((m, v))
+                for _ in range(3):
+                    r.fit_step(t, p, (m, v))
+            assert r.status() == 0
+            assert size == 0.1 and tile == 8 or not torch.equal(p, to_dev(p0))
+            out.append((p, m, v))
+    for a, b in zip(fit[0] + pframe[0], fit[1] + pframe[1]):
+        assert torch.equal(a, b)
