@@ -129,16 +129,19 @@ __device__ __forceinline__ bool gather_partials(const SlotArgs& g, int i, bool v
 }
 
 // GS2D_REDUCE_ATOMIC: the render added the Gaussian's sums up itself; every
-// lane of the group reads them, then lane 0 clears them for the next pass.
-// `any`: the Gaussian had a (tile, Gaussian) pair.  Every lane of the warp
-// must take part.
+// lane of the group reads them, then lane 0 clears them for the next pass, also
+// where they do not count (`ok` false: a binning over capacity; one that only
+// rejected a list too long to sort was rendered in its other tiles).  Returns
+// whether the Gaussian had a (tile, Gaussian) pair.  Every lane of the warp must
+// take part.
 __device__ __forceinline__ bool gather_acc(float* __restrict__ acc, const int4* __restrict__ rect,
-                                           int i, bool valid, int sub, float a[kPartials]) {
+                                           int i, bool valid, bool ok, int sub,
+                                           float a[kPartials]) {
   bool any = false;
 #pragma unroll
   for (int k = 0; k < kPartials; k++) a[k] = 0.0f;
   float4* q = reinterpret_cast<float4*>(acc + (size_t)kPartials * i);
-  if (valid) {
+  if (valid && ok) {
     const float4 x = q[0], y = q[1];
     a[0] = x.x;
     a[1] = x.y;
@@ -162,10 +165,10 @@ k_reduce_chain(int n, const float* __restrict__ params, SlotArgs slots,
   pdl_begin();
   const int gt = blockIdx.x * blockDim.x + threadIdx.x;
   const int i = gt / kRL, sub = gt % kRL;
-  const bool valid = i < n && hdr->entries_raw == (int64_t)hdr->n_entries;
+  const bool ok = hdr->entries_raw == (int64_t)hdr->n_entries;  // else over capacity
   float a[kPartials], gr[9];
-  const bool any = acc ? gather_acc(acc, slots.rect, i, valid, sub, a)
-                       : gather_partials(slots, i, valid, sub, a);
+  const bool any = acc ? gather_acc(acc, slots.rect, i, i < n, ok, sub, a)
+                       : gather_partials(slots, i, i < n && ok, sub, a);
   if (i >= n) return;
   if (any) chain_grads(params, n, i, a, gr);
 #pragma unroll
@@ -201,7 +204,7 @@ k_reduce_chain_adam(int n, float* __restrict__ params, SlotArgs slots,
   float a[kPartials], gr[9];
   // (atomic sums are read and cleared for every Gaussian: an unselected one
   // of a rendered tile has sums too)
-  const bool any = acc ? gather_acc(acc, slots.rect, i, i < n && ok, sub, a) && on
+  const bool any = acc ? gather_acc(acc, slots.rect, i, i < n, ok, sub, a) && on
                        : gather_partials(slots, i, on && ok, sub, a);
   // (ok is the same for every thread of the grid)
   const bool act = on && ok;

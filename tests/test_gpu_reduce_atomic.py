@@ -105,6 +105,45 @@ def test_atomic_pframe_step_leaves_no_stale_sums(gs):
     assert float(((ga - gs_).abs() / scale).max()) < 1e-2
 
 
+@pytest.mark.parametrize("call", ["render_l2", "render_bwd", "fit_step", "pframe_step"])
+def test_atomic_sums_are_cleared_after_a_rejected_list(gs, call):
+    """A list too long to sort is reported and no gradient is reduced from that
+    binning, but the other tiles were rendered and their sums added up: the next
+    call on the workspace must not find them."""
+    from paper_2505_09324_gb300 import _native as nat
+    W, H, n = 64, 32, 33000
+    good = random_gaussians(n, W, H, seed=41, l_range=(0.3, 0.6))
+    bad = good.copy()
+    bad[0, 200:], bad[1, 200:] = 8.0, 8.0   # all but 200 in one tile
+    good, bad = to_dev(good), to_dev(bad)
+    t = to_dev(smooth_noise_target(W, H, seed=42))
+    s = int(torch.cuda.current_stream().cuda_stream)
+    sel = torch.ones(n, dtype=torch.uint8, device="cuda")
+    out = []
+    for broken_first in (True, False):
+        r = gs.GaussianRasterizer(W, H, n, config=atomic(gs, tile=16))
+        m, v = torch.zeros_like(bad), torch.zeros_like(bad)
+        if broken_first:
+            q = bad.clone()
+            r.fit_reset((m, v))
+            if call == "fit_step":
+                r.fit_step(t, q, (m, v))
+            elif call == "pframe_step":
+                nat.pframe_step(r.plan, r.ws_ptr, t.data_ptr(), q.data_ptr(), m.data_ptr(),
+                                v.data_ptr(), sel.data_ptr(), s)
+            else:
+                r.prepare(q)
+                g = r.render_l2(q, t)[0] if call == "render_l2" else r.render_bwd(q, t)
+                assert not g.any()
+            assert torch.equal(q, bad) and r.status(reset=True) == nat.GS2D_ERR_CAPACITY
+        r.prepare(good)
+        out.append(r.render_l2(good, t)[0])
+        assert r.status() == 0
+    scale = out[1].abs().amax(dim=1, keepdim=True)
+    # float atomics: sums of up to a few dozen terms in any order
+    assert float(((out[0] - out[1]).abs() / scale).max()) < 1e-5
+
+
 def test_stage_256_renders_like_stage_64(gs, oracle):
     """Lists longer than 256 Gaussians in one tile: several 256-wide batches.
     The batch size changes neither a pixel's accumulation order nor any
