@@ -165,26 +165,13 @@ __device__ __forceinline__ void set_status(WsHeader* h, int code) {
   atomicCAS(&h->status, 0, code);
 }
 
-// Sum of float values as an unevaluated pair hi + lo (Knuth's two-sum: the
-// rounding error of every addition is kept, about 48 bits in all).  The loss
-// sums run over every tile in one or a few blocks, where double additions
-// (1/64 of the FP32 rate) were the whole time.
-struct FloatPair {
-  float hi = 0.0f, lo = 0.0f;
-  __device__ __forceinline__ void add(float x) {
-    const float s = __fadd_rn(hi, x), v = __fsub_rn(s, hi);
-    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, v)), __fsub_rn(x, v)));
-    hi = s;
-  }
-  __device__ __forceinline__ double value() const {
-    return isfinite(hi) ? (double)hi + (double)lo : (double)hi;  // (lo is NaN past an infinity)
-  }
-};
-
-// Sums of the loss partials of `count` tiles by one block, in the order of
-// 1024 threads (thread t: tiles t, t + 1024, ...; each warp's lanes; the 32
-// warps) whatever the block's size is: every caller gets the same bits.  Valid
-// in thread 0.  s_sum: 32 pairs.
+// Sums of the loss partials of `count` tiles by one block, in double, in the
+// order of 1024 threads (thread t: tiles t, t + 1024, ...; each warp's lanes;
+// the 32 warps) whatever the block's size is: every caller gets the same bits.
+// Valid in thread 0.  s_sum: 32 pairs.  What bounds it is the SM's FP64 pipe
+// (1/64 of the FP32 rate: some 8 us for the 8160 tiles of a 1080p frame at tile
+// 16); float pairs were faster and kept about 48 bits, too few for a sum that
+// decides when a fit stops.
 template <int THREADS>
 __device__ __forceinline__ double2 loss_sums(const float2* __restrict__ part, int count,
                                              double2* s_sum) {
@@ -192,7 +179,7 @@ __device__ __forceinline__ double2 loss_sums(const float2* __restrict__ part, in
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll 1
   for (int k = 0; k < 1024 / THREADS; k++) {
-    FloatPair a, b;
+    double x = 0.0, y = 0.0;
     int t = k * THREADS + threadIdx.x;
     for (; t + 3 * 1024 < count; t += 4 * 1024) {
       float2 v[4];
@@ -200,16 +187,15 @@ __device__ __forceinline__ double2 loss_sums(const float2* __restrict__ part, in
       for (int u = 0; u < 4; u++) v[u] = part[t + u * 1024];
 #pragma unroll
       for (int u = 0; u < 4; u++) {
-        a.add(v[u].x);
-        b.add(v[u].y);
+        x += v[u].x;
+        y += v[u].y;
       }
     }
     for (; t < count; t += 1024) {
       const float2 v = part[t];
-      a.add(v.x);
-      b.add(v.y);
+      x += v.x;
+      y += v.y;
     }
-    double x = a.value(), y = b.value();
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       x += __shfl_xor_sync(0xffffffffu, x, o);

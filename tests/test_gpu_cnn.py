@@ -603,6 +603,23 @@ def test_chamfer_nearest_neighbours(nat, name):
         assert abs(float(dl[0]) - loss) <= 1e-5 * loss
 
 
+def test_chamfer_loss_adds_in_double(nat):
+    """Squared distances of 1, 2^-24 and 2^-50 in one thread's share: the last
+    one decides the rounding of the FP32 result, and only a sum of 51 bits or
+    more holds it."""
+    n = 4096
+    P, Q = np.zeros((9, n)), np.zeros((9, 1))
+    P[0, [0, 1024, 2048]] = 1.0, 2.0 ** -12, 2.0 ** -25
+    want = np.float32((1 + 2.0 ** -24 + 2.0 ** -50) / n)
+    assert want > np.float32(1.0 / n)
+    dP, dQ, dl = dev_f32(P), dev_f32(Q), torch.zeros(1, device="cuda")
+    scratch = torch.empty(nat.load().gs2d_chamfer_scratch_bytes(n, 1, 1), dtype=torch.uint8,
+                          device="cuda")
+    nat.call("gs2d_chamfer", dP.data_ptr(), n, n, dQ.data_ptr(), 1, 1, 1, 1.0, 0, dl.data_ptr(),
+             scratch.data_ptr(), 0)
+    assert dl.cpu().numpy()[0] == want
+
+
 @pytest.mark.parametrize("B,H,W,C,N", [
     (2, 6, 20, 32, 64), (1, 7, 21, 64, 128), (1, 5, 515, 32, 64), (1, 3, 256, 64, 40),
     (1, 9, 300, 128, 192), (1, 4, 30, 200, 72), (3, 1, 1, 8, 8), (1, 2, 258, 24, 256),

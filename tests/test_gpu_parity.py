@@ -466,6 +466,34 @@ def test_short_fit_without_a_target_equals_a_polled_one(gs, check_every, entries
     assert torch.equal(pa, pb) and torch.equal(ma, mb) and torch.equal(va, vb)
 
 
+@pytest.mark.parametrize("clips", [False, True])
+def test_losses_add_in_double(gs, clips):
+    """Tile losses in the ratio 1 : 2^-24 : 2^-50 in one thread's share: the
+    last one decides the rounding of the FP32 result, and only a sum of 51 bits
+    or more holds it."""
+    W = H = 512
+    t = np.zeros((3, H, W))
+    for tile, v in ((0, 1.0), (1024, 2.0 ** -12), (2048, 2.0 ** -25)):
+        t[:, 8 * (tile // 64), 8 * (tile % 64)] = v
+    p = np.ones((9, 1))
+    p[:2] = -1e4  # (an empty frame)
+    p, t = to_dev(p), to_dev(t)
+    cfg = gs.RasterConfig(tile=8)
+    want = np.float32((1 + 2.0 ** -24 + 2.0 ** -50) / (W * H))
+    assert want > np.float32(1.0 / (W * H))
+    if clips:
+        r = gs.BatchRasterizer([(W, H, 1), (W, H, 1)], config=cfg)
+        pp = r.pack_params([p, p])
+        r.prepare(pp)
+        r.render_l2(pp, r.pack_images([t, t]))
+        got = np.asarray(r.clip_losses(), np.float32)
+    else:
+        r = gs.GaussianRasterizer(W, H, 1, config=cfg)
+        r.prepare(p)
+        got = r.render_l2(p, t)[1].cpu().numpy()
+    np.testing.assert_array_equal(got, np.full(got.shape, want))
+
+
 def _piled(n, W, H, seed, at, share):
     """Random Gaussians, `share` of them within a pixel of `at`."""
     p = random_gaussians(n, W, H, seed=seed, l_range=(0.5, 2.0))
