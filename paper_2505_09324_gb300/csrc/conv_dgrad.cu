@@ -222,7 +222,7 @@ k_conv_dgrad(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
     uint32_t at = 0;
     for (int t = first; t < g.tiles; t += step, at++) {
       const int row = t / g.segs, c = (t - row * g.segs) * kBM + r;
-      const int b = row / g.Ho, iy = 2 * (row - b * g.Ho) + py;
+      const int b = row / g.Ho, oy = row - b * g.Ho, iy = 2 * oy + py;
       const bool in = iy < g.Hi;  // (the last odd row may be missing)
       const size_t o = (((size_t)b * g.Hi + iy) * g.Wi + 2 * c) * g.C + nb * kCI;
       // the mask of this lane's two pixels, a bit per channel
@@ -258,26 +258,29 @@ k_conv_dgrad(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
       }
       tc_fence_after();
       // column parity px: taps ky x kx in their order, ky = 1 (even rows) or
-      // 0, 2 (odd), kx = 1 (even columns) or 0, 2 (odd)
+      // 0, 2 (odd), kx = 1 (even columns) or 0, 2 (odd).  Taps past dZ's edge
+      // (ky = 0 in the last row, kx = 0 in the last column) are left out, as by
+      // the gather: their accumulators hold zeros times weights, which a
+      // non-finite weight makes NaN
+      const bool below = oy + 1 < g.Ho, right = c + 1 < g.Wo;
       uint32_t h[2][16];
 #pragma unroll
       for (int px = 0; px < 2; px++) {
         float w[32], x[32];
+        const auto add = [&](int tap, bool has) {
+          tmem_ld32(taddr + dg_col(tap), x);
+#pragma unroll
+          for (int i = 0; i < 32; i++) w[i] = has ? w[i] + x[i] : w[i];
+        };
         tmem_ld32(taddr + dg_col((py ? 0 : 3) + (px ? 0 : 1)), w);
-        if (px) {
-          tmem_ld32(taddr + dg_col((py ? 0 : 3) + 2), x);
+        if (!((py == 0 || below) && (px == 0 || right))) {
 #pragma unroll
-          for (int i = 0; i < 32; i++) w[i] += x[i];
+          for (int i = 0; i < 32; i++) w[i] = 0.0f;
         }
+        if (px) add((py ? 0 : 3) + 2, py == 0 || below);
         if (py) {
-          tmem_ld32(taddr + dg_col(6 + (px ? 0 : 1)), x);
-#pragma unroll
-          for (int i = 0; i < 32; i++) w[i] += x[i];
-          if (px) {
-            tmem_ld32(taddr + dg_col(8), x);
-#pragma unroll
-            for (int i = 0; i < 32; i++) w[i] += x[i];
-          }
+          add(6 + (px ? 0 : 1), px == 0 || right);
+          if (px) add(8, true);
         }
 #pragma unroll
         for (int i = 0; i < 16; i++) {

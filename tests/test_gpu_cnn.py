@@ -674,6 +674,30 @@ def test_conv_input_gradient_equals_the_gathered_gemm(nat, B, H, W, C, N):
     assert torch.equal(dx[0], dx[1])
 
 
+@pytest.mark.parametrize("B,H,W,C,N", [(2, 9, 130, 32, 64), (1, 6, 131, 8, 8),
+                                       (1, 5, 200, 64, 384), (1, 1, 256, 8, 8),
+                                       (2, 2, 2, 40, 16)])
+def test_conv_input_gradient_of_non_finite_weights(nat, B, H, W, C, N):
+    """Infinite and NaN weights of one tap at a time reach the pixels that the
+    tap is gathered to, and not those whose tap lies past dZ's edge."""
+    g = torch.Generator(device="cuda").manual_seed(W + C)
+    P, ldk = B * ((H + 1) // 2) * ((W + 1) // 2), 9 * C + 8
+    dz = torch.randn((P, N), generator=g, device="cuda").bfloat16()
+    for tap in range(9):
+        wt = torch.randn((ldk, N), generator=g, device="cuda").bfloat16()
+        wt[tap * C:(tap + 1) * C:2, 3] = float("inf") if tap % 2 else float("nan")
+        dcol = torch.empty((P, ldk), device="cuda")
+        dx = [torch.full((B, H, W, C), 7.0, dtype=torch.bfloat16, device="cuda") for _ in range(2)]
+        status = torch.zeros(1, dtype=torch.int32, device="cuda")
+        nat.gemm_bf16(dz.data_ptr(), N, wt.data_ptr(), N, P, ldk, N, 0, False, dcol.data_ptr(), 0,
+                      ldk, 1, 0, status.data_ptr(), 0)
+        nat.call("gs2d_col2im", dcol.data_ptr(), ldk, B, H, W, C, 3, 2, 1, 0, dx[0].data_ptr(), 0)
+        nat.call("gs2d_conv_dgrad_bf16", dz.data_ptr(), B, H, W, C, wt.data_ptr(), N, 0,
+                 dx[1].data_ptr(), status.data_ptr(), 0)
+        a, b = (x.float().cpu().numpy() for x in dx)
+        np.testing.assert_array_equal(a, b)  # (NaN equals NaN)
+
+
 @pytest.mark.parametrize("B,H,W,ci,co,ks,st,pad,out", [
     (2, 17, 120, 64, 384, 3, 2, 1, "bf16"),    # two rows a tile, odd rows, two blocks of N
     (1, 6, 98, 128, 40, 3, 2, 1, "f32"),       # 49 pixels
