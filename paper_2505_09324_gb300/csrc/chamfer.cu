@@ -275,28 +275,45 @@ k_chamfer_grad(const float* __restrict__ P, int np, int ldp, const float* __rest
   }
 }
 
-// Mean squared distances of both directions of frame b, one block.  Sums and
-// means in double (FP64 issues at 1/64 of the FP32 rate: 33 us for 20 000 points
-// a side; float pairs took 23 and kept about 48 bits).
+// Mean squared distances of both directions of frame b, one block.  Float sums
+// per thread (FloatSum: no less accurate than double additions), doubles only
+// across threads and one division per mean: FP64 issues at 1/64 of the FP32
+// rate, and double sums and divisions in every thread took 33 us for 20 000
+// points a side, 24 so.
 __global__ void __launch_bounds__(1024)
 k_chamfer_loss(const float* __restrict__ d1, int np, const float* __restrict__ d2, int nq,
                float* __restrict__ loss) {
   pdl_begin();
-  __shared__ double s[32];
+  __shared__ double2 s[32];
   const int b = blockIdx.x;
-  double a = 0.0, c = 0.0;
+  FloatSum a, c;
 #pragma unroll 4
-  for (int i = threadIdx.x; i < np; i += blockDim.x) a += d1[(size_t)b * np + i];
+  for (int i = threadIdx.x; i < np; i += blockDim.x) a.add(d1[(size_t)b * np + i]);
 #pragma unroll 4
-  for (int i = threadIdx.x; i < nq; i += blockDim.x) c += d2[(size_t)b * nq + i];
-  double v = a / np + c / nq;
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = v;
+  for (int i = threadIdx.x; i < nq; i += blockDim.x) c.add(d2[(size_t)b * nq + i]);
+  double x = a.value(), y = c.value();
+  // (sums past FP32's range, whose mean may still lie within it)
+  if (!isfinite(x)) {
+    x = 0.0;
+    for (int i = threadIdx.x; i < np; i += blockDim.x) x += d1[(size_t)b * np + i];
+  }
+  if (!isfinite(y)) {
+    y = 0.0;
+    for (int i = threadIdx.x; i < nq; i += blockDim.x) y += d2[(size_t)b * nq + i];
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    x += __shfl_xor_sync(0xffffffffu, x, o);
+    y += __shfl_xor_sync(0xffffffffu, y, o);
+  }
+  if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = make_double2(x, y);
   __syncthreads();
   if (threadIdx.x == 0) {
-    double tot = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); w++) tot += s[w];
-    loss[b] = (float)tot;
+    x = y = 0.0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); w++) {
+      x += s[w].x;
+      y += s[w].y;
+    }
+    loss[b] = (float)(x / np + y / nq);
   }
 }
 

@@ -165,13 +165,35 @@ __device__ __forceinline__ void set_status(WsHeader* h, int code) {
   atomicCAS(&h->status, 0, code);
 }
 
-// Sums of the loss partials of `count` tiles by one block, in double, in the
-// order of 1024 threads (thread t: tiles t, t + 1024, ...; each warp's lanes;
-// the 32 warps) whatever the block's size is: every caller gets the same bits.
-// Valid in thread 0.  s_sum: 32 pairs.  What bounds it is the SM's FP64 pipe
-// (1/64 of the FP32 rate: some 8 us for the 8160 tiles of a 1080p frame at tile
-// 16); float pairs were faster and kept about 48 bits, too few for a sum that
-// decides when a fit stops.
+// Sum of float values as an unevaluated sum hi + mid + lo of three floats: the
+// rounding error of every addition (Knuth's two-sum) is added to mid, the error
+// of that to lo.  What is lost is the rounding of lo, of the order of n^2 2^-72
+// of the sum after n additions, so value() is the sum rounded to double once,
+// where n double additions round n - 1 times.  The loss sums run over every tile
+// in one or a few blocks, where double additions (1/64 of the FP32 rate) were
+// the whole time: 65 us for the 65 280 tiles of eight 1080p frames.
+struct FloatSum {
+  float hi = 0.0f, mid = 0.0f, lo = 0.0f;
+  __device__ __forceinline__ static float two_sum(float& a, float x) {
+    const float s = __fadd_rn(a, x), v = __fsub_rn(s, a);
+    const float e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, v)), __fsub_rn(x, v));
+    a = s;
+    return e;
+  }
+  __device__ __forceinline__ void add(float x) {
+    x = two_sum(hi, x);
+    lo = __fadd_rn(lo, two_sum(mid, x));
+  }
+  __device__ __forceinline__ double value() const {
+    // (the others are NaN past an infinity)
+    return isfinite(hi) ? (double)hi + ((double)mid + (double)lo) : (double)hi;
+  }
+};
+
+// Sums of the loss partials of `count` tiles by one block, in the order of
+// 1024 threads (thread t: tiles t, t + 1024, ...; each warp's lanes; the 32
+// warps) whatever the block's size is: every caller gets the same bits.  Valid
+// in thread 0.  s_sum: 32 pairs.
 template <int THREADS>
 __device__ __forceinline__ double2 loss_sums(const float2* __restrict__ part, int count,
                                              double2* s_sum) {
@@ -179,7 +201,7 @@ __device__ __forceinline__ double2 loss_sums(const float2* __restrict__ part, in
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll 1
   for (int k = 0; k < 1024 / THREADS; k++) {
-    double x = 0.0, y = 0.0;
+    FloatSum a, b;
     int t = k * THREADS + threadIdx.x;
     for (; t + 3 * 1024 < count; t += 4 * 1024) {
       float2 v[4];
@@ -187,15 +209,16 @@ __device__ __forceinline__ double2 loss_sums(const float2* __restrict__ part, in
       for (int u = 0; u < 4; u++) v[u] = part[t + u * 1024];
 #pragma unroll
       for (int u = 0; u < 4; u++) {
-        x += v[u].x;
-        y += v[u].y;
+        a.add(v[u].x);
+        b.add(v[u].y);
       }
     }
     for (; t < count; t += 1024) {
       const float2 v = part[t];
-      x += v.x;
-      y += v.y;
+      a.add(v.x);
+      b.add(v.y);
     }
+    double x = a.value(), y = b.value();
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       x += __shfl_xor_sync(0xffffffffu, x, o);
