@@ -5,10 +5,10 @@
 // The nearest neighbours are exact (smallest FP32 squared distance, ties to the
 // lowest index: what a scan of all pairs gives), found through a uniform grid
 // over each set: a query looks at its own cell and at rings of cells around it
-// until no further ring can hold a closer point.  The scan of all pairs was
-// 2 x 0.94 ms at 20 000 points and batch 8 (6.4 10^9 distances, bound by
-// instruction issue); a query now evaluates a few dozen points, and build and
-// query together take 0.16 ms.
+// until no further ring can hold a closer point, or so many have been looked at
+// that a scan of the set is faster.  The scan of all pairs was 2 x 0.94 ms at
+// 20 000 points and batch 8 (6.4 10^9 distances, bound by instruction issue); a
+// query of spread points evaluates a few dozen.
 #include <math.h>
 
 #include <algorithm>
@@ -37,6 +37,8 @@ struct NnSet {
   int* index;        // [B][n] their index in the frame
   int* start;        // [B][kNnCells + 2] first position of each cell; then the others
   NnGrid* grid;      // [B]
+  int* hard;         // [B][n] points left to k_nn_scan, by index in the frame
+  int* hards;        // [B] how many
   int* nn;           // [B][n] out: nearest of the other set, by index in the frame
   float* dist;       // [B][n] out: its squared distance
 };
@@ -139,6 +141,7 @@ __global__ void __launch_bounds__(kNnThreads) k_nn_build(NnArgs a) {
     }
     s_grid = g;
     set.grid[b] = g;
+    set.hards[b] = 0;
   }
   for (int i = t; i <= kNnCells; i += kNnThreads) s_cnt[i] = 0;
   __syncthreads();
@@ -195,7 +198,15 @@ __global__ void __launch_bounds__(kNnThreads) k_nn_build(NnArgs a) {
 
 // A thread per point, in its own set's cell order (neighbouring threads search
 // neighbouring cells).  A point of ring k (its cell k columns or rows away) is
-// at least (k - 1) h away, whichever of the two lies outside the grid.
+// (k - 1) h farther than the nearest edge of the own cell that has cells behind
+// it, whichever of the two points lies outside the grid.  A point whose search
+// grows past a share of the set (a cell with most of the points, as with a far
+// outlier or tight clusters; a query far outside the grid) goes to k_nn_scan,
+// which takes a quarter of the time for a point: so no set takes longer than the
+// scan of all pairs did.  A run of cells counts like kHardCell points (its two
+// look-ups).
+constexpr int kHardShare = 8, kHardMin = 64, kHardCell = 8;
+
 __global__ void __launch_bounds__(128) k_nn_query(NnArgs a) {
   pdl_begin();
   const int b = blockIdx.y;
@@ -211,10 +222,12 @@ __global__ void __launch_bounds__(128) k_nn_query(NnArgs a) {
   const float* __restrict__ qy = to.y + (size_t)b * to.n;
   const int* __restrict__ qi = to.index + (size_t)b * to.n;
   float best = INFINITY;
-  int arg = 0;
+  int arg = 0, left = to.n / kHardShare + kHardMin;  // points it may still look at
   const auto scan = [&](int c0, int c1) {  // cells c0 ... c1 of one row
-    const int e = start[c1 + 1];
-    for (int j = start[c0]; j < e; j++) {
+    const int s = start[c0], e = start[c1 + 1];
+    left -= e - s + kHardCell;
+    if (left < 0) return;
+    for (int j = s; j < e; j++) {
       const float dx = px - qx[j], dy = py - qy[j];
       const float d = fmaf(dx, dx, dy * dy);
       if (d <= best) {
@@ -229,12 +242,16 @@ __global__ void __launch_bounds__(128) k_nn_query(NnArgs a) {
   if (isfinite(px) && isfinite(py)) {
     const int cx = nn_axis(px, g.lo_x, g.inv, g.gx), cy = nn_axis(py, g.lo_y, g.inv, g.gy);
     const int rings = max(max(cx, g.gx - 1 - cx), max(cy, g.gy - 1 - cy));
-    for (int k = 0; k <= rings; k++) {
+    // distance to the nearest edge of the cell with cells behind it
+    const float ux = px - fmaf((float)cx, g.h, g.lo_x), uy = py - fmaf((float)cy, g.h, g.lo_y);
+    const float edge = fminf(fminf(cx > 0 ? ux : INFINITY, cx + 1 < g.gx ? g.h - ux : INFINITY),
+                             fminf(cy > 0 ? uy : INFINITY, cy + 1 < g.gy ? g.h - uy : INFINITY));
+    for (int k = 0; k <= rings && left >= 0; k++) {
       // strictly farther than the best, FP32 rounding of the distances included
-      const float away = (float)(k - 1) * g.h * 0.99999f - g.err;
+      const float away = k > 0 ? fmaf((float)(k - 1), g.h, edge) * 0.99999f - g.err : 0.f;
       if (away > 0.f && away * away * 0.99999f > best) break;
       const int x0 = max(cx - k, 0), x1 = min(cx + k, g.gx - 1);
-      for (int y = max(cy - k, 0); y <= min(cy + k, g.gy - 1); y++) {
+      for (int y = max(cy - k, 0); y <= min(cy + k, g.gy - 1) && left >= 0; y++) {
         const int row = y * g.gx;
         if (y == cy - k || y == cy + k) {
           scan(row + x0, row + x1);
@@ -245,8 +262,131 @@ __global__ void __launch_bounds__(128) k_nn_query(NnArgs a) {
       }
     }
   }
-  from.nn[fo + from.index[o]] = arg;
-  from.dist[fo + from.index[o]] = best;
+  const int index = from.index[o];
+  if (left < 0) {
+    from.hard[fo + atomicAdd(&from.hards[b], 1)] = index;
+    return;
+  }
+  from.nn[fo + index] = arg;
+  from.dist[fo + index] = best;
+}
+
+// Two FP32 operations an instruction, each rounded like the single one.
+__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
+  return (uint64_t)__float_as_uint(hi) << 32 | __float_as_uint(lo);
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ float lo2(uint64_t v) { return __uint_as_float((uint32_t)v); }
+__device__ __forceinline__ float hi2(uint64_t v) { return __uint_as_float((uint32_t)(v >> 32)); }
+
+// The points that k_nn_query left, against all of the other set.  A block takes
+// 128 of them, four a lane and the same for every warp, and brings the other set
+// through shared memory in tiles, of which each warp looks at its share, four
+// points at a time: a load serves 16 distances, and the smallest of four is
+// compared and kept at once (with the first of its four points; which one it was
+// is looked up at the end).  Bound by the FP32 pipe (four operations a pair): 8 x
+// 20 000 points a side, all of them, take 1.05 ms, where a thread per point over
+// tiles in shared memory took 1.9, and 1.9 too a block per 8 points whose threads
+// read the other set from L2.
+constexpr int kScanLane = 4, kScanQ = 32 * kScanLane;
+constexpr int kScanThreads = 512, kScanWarps = kScanThreads / 32;
+constexpr int kScanTile = kScanWarps * kScanQ;  // points of a tile
+constexpr int kScanShare = kScanTile / kScanWarps;
+
+__global__ void __launch_bounds__(kScanThreads, 2) k_nn_scan(NnArgs a) {
+  pdl_begin();
+  __shared__ __align__(16) float s_x[kScanTile], s_y[kScanTile];  // negated
+  const int b = blockIdx.y, t = threadIdx.x, lane = t & 31, wid = t >> 5;
+  const NnSet& from = a.set[blockIdx.z];
+  const NnSet& to = a.set[1 - blockIdx.z];
+  const size_t fo = (size_t)b * from.n;
+  const float* __restrict__ qx = to.pts + (size_t)b * to.n;
+  const float* __restrict__ qy = qx + to.ld;
+  const int count = from.hards[b], n = to.n;
+  for (int h0 = blockIdx.x * kScanQ; h0 < count; h0 += gridDim.x * kScanQ) {
+    float px[kScanLane], py[kScanLane], best[kScanLane];
+    int arg[kScanLane];
+#pragma unroll
+    for (int q = 0; q < kScanLane; q++) {
+      const int i = from.hard[fo + min(h0 + 32 * q + lane, count - 1)];
+      px[q] = from.pts[fo + i];
+      py[q] = from.pts[fo + from.ld + i];
+      best[q] = INFINITY;
+      arg[q] = 0;
+    }
+    for (int j0 = 0; j0 < n; j0 += kScanTile) {
+      __syncthreads();
+      for (int k = t; k < kScanTile; k += kScanThreads) {
+        s_x[k] = j0 + k < n ? -qx[j0 + k] : INFINITY;
+        s_y[k] = j0 + k < n ? -qy[j0 + k] : INFINITY;
+      }
+      __syncthreads();
+      const int k0 = wid * kScanShare, k1 = min(k0 + kScanShare, n - j0);
+#pragma unroll 2
+      for (int k = k0; k < k1; k += 4) {
+        const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(s_x + k);
+        const ulonglong2 y = *reinterpret_cast<const ulonglong2*>(s_y + k);
+#pragma unroll
+        for (int q = 0; q < kScanLane; q++) {
+          const uint64_t ax = pack2(px[q], px[q]), ay = pack2(py[q], py[q]);
+          const uint64_t dx0 = add2(ax, x.x), dy0 = add2(ay, y.x);
+          const uint64_t dx1 = add2(ax, x.y), dy1 = add2(ay, y.y);
+          const uint64_t d0 = fma2(dx0, dx0, mul2(dy0, dy0));
+          const uint64_t d1 = fma2(dx1, dx1, mul2(dy1, dy1));
+          // (fminf passes over a NaN, as a comparison does)
+          const float d = fminf(fminf(lo2(d0), hi2(d0)), fminf(lo2(d1), hi2(d1)));
+          if (d < best[q]) {
+            best[q] = d;
+            arg[q] = j0 + k;
+          }
+        }
+      }
+    }
+    // each warp's smallest, at the first point that has it; then the block's, of
+    // equal ones the lowest index
+    __syncthreads();
+    int* s_j = reinterpret_cast<int*>(s_y);
+#pragma unroll
+    for (int q = 0; q < kScanLane; q++) {
+      int j = arg[q];
+      for (const int end = min(n, j + 4) - 1; best[q] < INFINITY && j < end; j++) {
+        const float dx = px[q] - qx[j], dy = py[q] - qy[j];
+        if (fmaf(dx, dx, dy * dy) == best[q]) break;
+      }
+      s_x[wid * kScanQ + 32 * q + lane] = best[q];
+      s_j[wid * kScanQ + 32 * q + lane] = j;
+    }
+    __syncthreads();
+    if (t < kScanQ && h0 + t < count) {
+      float d = s_x[t];
+      int j = s_j[t];
+      for (int w = 1; w < kScanWarps; w++) {
+        const float dw = s_x[w * kScanQ + t];
+        const int jw = s_j[w * kScanQ + t];
+        if (dw < d || (dw == d && jw < j)) {
+          d = dw;
+          j = jw;
+        }
+      }
+      const int i = from.hard[fo + h0 + t];
+      from.nn[fo + i] = j;
+      from.dist[fo + i] = d;
+    }
+  }
 }
 
 // Gradient of the Chamfer term with respect to the predicted means: each
@@ -322,12 +462,13 @@ k_chamfer_loss(const float* __restrict__ d1, int np, const float* __restrict__ d
 
 using namespace gs2d;
 
-// Four-byte words of scratch: nearest neighbours, distances and the three
-// sorted arrays of every point, cell starts and grid of every set.
+// Four-byte words of scratch: nearest neighbours, distances, the three sorted
+// arrays and the list of the points to scan for of every point, cell starts,
+// grid and that list's length of every set.
 extern "C" uint64_t gs2d_chamfer_scratch_bytes(int32_t n, int32_t m, int32_t B) {
   const uint64_t points = (uint64_t)B * ((uint64_t)n + m);
   const uint64_t sets = 2 * (uint64_t)B;
-  return points * 5 * 4 + sets * (kNnCells + 2) * 4 + sets * sizeof(NnGrid) + 64;
+  return points * 6 * 4 + sets * (kNnCells + 3) * 4 + sets * sizeof(NnGrid) + 64;
 }
 
 extern "C" gs2d_status gs2d_chamfer(const float* params, int32_t n, int32_t ldp,
@@ -358,6 +499,8 @@ extern "C" gs2d_status gs2d_chamfer(const float* params, int32_t n, int32_t ldp,
     set.x = reinterpret_cast<float*>(take(all));
     set.y = reinterpret_cast<float*>(take(all));
     set.index = take(all);
+    set.hard = take(all);
+    set.hards = take(B);
     set.start = take((size_t)B * (kNnCells + 2));
     set.grid = reinterpret_cast<NnGrid*>(take((size_t)B * sizeof(NnGrid) / 4));
   }
@@ -365,6 +508,11 @@ extern "C" gs2d_status gs2d_chamfer(const float* params, int32_t n, int32_t ldp,
   cudaError_t e = launch_pdl(k_nn_build, dim3(B, 2), kNnThreads, 0, s, a);
   if (e == cudaSuccess)
     e = launch_pdl(k_nn_query, dim3((std::max(n, m) + 127) / 128, B, 2), 128, 0, s, a);
+  // (most often nothing is left: at most a wave of blocks to find that out)
+  if (e == cudaSuccess)
+    e = launch_pdl(k_nn_scan,
+                   dim3(std::max(1, std::min((std::max(n, m) + kScanQ - 1) / kScanQ,
+                                             152 * 2 / (2 * B))), B, 2), kScanThreads, 0, s, a);
   if (e == cudaSuccess && dparams)
     e = launch_pdl(k_chamfer_grad, dim3((std::max(n, m) + 255) / 256, B), 256, 0, s, params, (int)n,
                    (int)ldp, targets, (int)m, (int)ldq, (const int*)p.nn, (const int*)q.nn, lambda,

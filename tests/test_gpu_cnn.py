@@ -603,6 +603,58 @@ def test_chamfer_nearest_neighbours(nat, name):
         assert abs(float(dl[0]) - loss) <= 1e-5 * loss
 
 
+@pytest.mark.parametrize("n,m,kinds", [
+    (3001, 2503, ("dense", "dense")), (1000, 4000, ("spread", "away")), (2000, 9, ("away", "dense")),
+    (257, 5000, ("same", "spread")), (4096, 4095, ("two", "away"))])
+def test_chamfer_of_dense_and_distant_sets(nat, n, m, kinds):
+    """Sets whose points the grid does not separate (one cell with most of them
+    next to far outliers, tight clusters, a set far from the other, equal points)
+    go to the scan of the other set, in a batch beside frames that do not.  Whole
+    coordinates, so that the FP32 distances and their many ties are exact: the
+    nearest neighbours, of equal ones the first, show in the gradient and loss."""
+    g = np.random.Generator(np.random.PCG64(n + m))
+
+    def points(kind, k, second):
+        if kind == "same":
+            return np.full((2, k), 7.0)
+        if kind == "two":
+            return g.integers(0, 4, (2, k)) + 1500.0 * g.integers(0, 2, (1, k))
+        p = g.integers(0, 1500 if kind == "spread" else 40, (2, k)).astype(np.float64)
+        if kind == "dense":
+            p[:, :2] = [[1.0e6, -3.0e5], [-1.0e6, 2.0e4]]
+        return p + (3000.0 if kind == "away" and second else 0.0)
+
+    B = len(kinds)
+    P = np.concatenate([points(k, n, False) for k in kinds], 1).astype(np.float32)
+    Q = np.concatenate([points(k, m, True) for k in kinds], 1).astype(np.float32)
+    want, loss = np.zeros((2, B * n)), []
+    for b in range(B):
+        p, q = P[:, b * n:(b + 1) * n], Q[:, b * m:(b + 1) * m]
+        d = [(p[r][:, None] - q[r][None]).astype(np.float32) for r in (0, 1)]
+        # fma(dx, dx, dy * dy) in FP32
+        D = (d[0].astype(np.float64) ** 2 + (d[1] * d[1]).astype(np.float64)).astype(np.float32)
+        j1, j2 = D.argmin(1), D.argmin(0)
+        for r in (0, 1):
+            w = want[r, b * n:(b + 1) * n]
+            w += 2.0 * (p[r] - q[r][j1]) / n
+            np.add.at(w, j2, 2.0 * (p[r][j2] - q[r]).astype(np.float64) / m)
+        loss.append(D.min(1).astype(np.float64).mean() + D.min(0).astype(np.float64).mean())
+    dP, dQ = (dev_f32(np.concatenate([x, np.zeros((7, x.shape[1]))])) for x in (P, Q))
+    dg, dl = torch.zeros((9, B * n), device="cuda"), torch.zeros(B, device="cuda")
+    scratch = torch.empty(nat.load().gs2d_chamfer_scratch_bytes(n, m, B), dtype=torch.uint8,
+                          device="cuda")
+    for _ in range(2):  # (again in the same scratch)
+        dg.zero_()
+        nat.call("gs2d_chamfer", dP.data_ptr(), n, B * n, dQ.data_ptr(), m, B * m, B, 1.0,
+                 dg.data_ptr(), dl.data_ptr(), scratch.data_ptr(), 0)
+        got = dg.cpu().numpy().astype(np.float64)
+        # FP32 sums of up to m + 1 terms of one sign or another, in any order
+        size = np.abs(want).max(1, keepdims=True) + 1e-3
+        assert np.all(np.abs(got[:2] - want) <= 1e-4 * size)
+        assert not got[2:].any()
+        np.testing.assert_allclose(dl.cpu().numpy(), loss, rtol=1e-6)
+
+
 def test_chamfer_loss_adds_in_double(nat):
     """Squared distances of 1, 2^-24 and 2^-50 in one thread's share: the last
     one decides the rounding of the FP32 result, and only a sum of 51 bits or
