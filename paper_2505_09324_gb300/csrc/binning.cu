@@ -12,8 +12,8 @@
 //      ranges, capacity);
 //   2. k_bin_scatter: every entry claims the next slot of its tile's list;
 //   3. k_sort: each tile's list is sorted by Gaussian index (a warp bitonic
-//      network in registers for lists of up to 512, the block's shared memory
-//      for longer ones), restoring exactly the order a stable sort of the
+//      network in registers for lists of up to 512, by the block through a
+//      bitmap in shared memory for longer ones), restoring exactly the order a stable sort of the
 //      index-ordered entries would give.
 // Each is a chain of a few dependent memory latencies, so the number of
 // launches and of warps in flight is what counts: a group is 64 Gaussians
@@ -33,11 +33,14 @@
 namespace gs2d {
 
 constexpr int kLongMax = 1 << 15;   // longest list that is sorted
-constexpr int kSmemKeys = 1 << 13;  // keys of one shared-memory sort (32 KB)
+constexpr int kSmemKeys = 1 << 13;  // words of shared memory of a sort (32 KB)
 constexpr int kThreads = 256;
 constexpr int kGroup = 64;          // Gaussians per block
 constexpr int kGroupLarge = 256;    // the same beyond kManyGroups groups
-constexpr int kManyGroups = 1 << 13;
+// (what one block scans in two steps, and some two waves of blocks: 300 000
+// Gaussians, most of them off a 64 x 48 frame, 40 us in groups of 64, 29 in groups
+// of 256; 500 000 at 1080p 68 / 62)
+constexpr int kManyGroups = 1 << 11;
 // Up to two steps of the one-block scan (1024 tiles or groups each, 2.3 us a
 // step: a chain of loads, scans and class counts) it is faster than another
 // launch: k_count with its scan takes 10 us at 256 tiles against 8.5 + 4.5,
@@ -612,7 +615,7 @@ __device__ __forceinline__ int lower_count(const uint32_t* seg, int len, uint32_
 // Sort of a list of up to kLongMax keys by the block: runs of kSmemKeys in
 // shared memory, then each key's place among the other runs by binary search
 // (the keys are distinct), through `spare`.
-__device__ __forceinline__ void block_sort_long(uint32_t* seg, int len, uint32_t* spare,
+__device__ __noinline__ void block_sort_long(uint32_t* seg, int len, uint32_t* spare,
                                                 uint32_t* s_keys) {
   for (int r = 0; r < len; r += kSmemKeys)
     block_sort(seg + r, min(kSmemKeys, len - r), s_keys);
@@ -629,6 +632,66 @@ __device__ __forceinline__ void block_sort_long(uint32_t* seg, int len, uint32_t
   __syncthreads();
 }
 
+// Sort of a list of any length by the block through a bitmap of the keys, which
+// are distinct and lie in [first, first + n), the tile's clip: 2^18 of them at a
+// time, each pass one reading of the list and its set bits in order.  What
+// bounds it is the latency of these loads and stores, where the bitonic network
+// is a chain of shared-memory exchanges: binning 600 / 8192 / 32 768 Gaussians of
+// one tile takes 12.7 / 28.5 / 83 us so, 19 / 98 / 743 by networks of 256 threads,
+// and took 24 / 86 / 362 by networks of 1024 threads with the whole list in shared
+// memory, in a launch of their own.
+constexpr int kBitKeys = 32 * kSmemKeys;
+
+__device__ __noinline__ void block_sort_bits(uint32_t* seg, int len, uint32_t first, int n,
+                                                uint32_t* spare, uint32_t* s_bits) {
+  __shared__ int s_warp[kThreads / 32];
+  const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+  uint32_t* out = n <= kBitKeys ? seg : spare;  // (one pass: read before it is written)
+  int done = 0;
+  for (int k0 = 0; k0 < n; k0 += kBitKeys) {
+    // rows of 32 words, shared out to the warps in order
+    const int rows = (min(kBitKeys, n - k0) + 1023) / 1024;
+    const int r0 = rows * wid / (kThreads / 32), r1 = rows * (wid + 1) / (kThreads / 32);
+    __syncthreads();
+    for (int i = t; i < 32 * rows; i += kThreads) s_bits[i] = 0u;
+    __syncthreads();
+#pragma unroll 4
+    for (int i = t; i < len; i += kThreads) {
+      const uint32_t k = seg[i] - first - (uint32_t)k0;
+      if (k < (uint32_t)kBitKeys) atomicOr(&s_bits[k >> 5], 1u << (k & 31u));
+    }
+    __syncthreads();
+    int mine = 0;
+    for (int r = r0; r < r1; r++) mine += __popc(s_bits[32 * r + lane]);
+    mine = __reduce_add_sync(0xffffffffu, mine);
+    if (lane == 0) s_warp[wid] = mine;
+    __syncthreads();
+    int at = done;
+    for (int w = 0; w < kThreads / 32; w++) {
+      at += w < wid ? s_warp[w] : 0;
+      done += s_warp[w];
+    }
+    for (int r = r0; r < r1; r++) {
+      uint32_t bits = s_bits[32 * r + lane];
+      const int c = __popc(bits);
+      int inc = c;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += y;
+      }
+      const uint32_t key = first + (uint32_t)k0 + 32u * (uint32_t)(32 * r + lane);
+      for (int p = at + inc - c; bits; bits &= bits - 1)
+        out[p++] = key + (uint32_t)(__ffs(bits) - 1);
+      at += __shfl_sync(0xffffffffu, inc, 31);
+    }
+  }
+  __syncthreads();
+  if (out != seg)
+    for (int i = t; i < len; i += kThreads) seg[i] = spare[i];
+  __syncthreads();
+}
+
 // Segment sort: one warp per tile for lists of up to 512 (bitonic network in
 // registers), the block for its longer ones, one after another; TPB tiles per
 // block (8, or 1 with few tiles, whose lists may all be long), a grid apart:
@@ -641,7 +704,7 @@ __device__ __forceinline__ void block_sort_long(uint32_t* seg, int len, uint32_t
 template <bool LAZY, int TPB>
 __global__ void __launch_bounds__(kThreads) k_sort(const __grid_constant__ BinArgs a) {
   pdl_begin();
-  __shared__ uint32_t s_keys[kSmemKeys];
+  extern __shared__ uint32_t s_keys[];  // kSmemKeys
   __shared__ int s_len[TPB];
   if (LAZY && a.hdr->lists_valid) return;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -699,7 +762,14 @@ __global__ void __launch_bounds__(kThreads) k_sort(const __grid_constant__ BinAr
       }
       continue;
     }
-    block_sort_long(a.list + x, len, a.spare + x, s_keys);
+    // one pass is always the faster way; each further one costs about what
+    // 1024 keys cost the networks (8 M Gaussians, 31 passes: 32 768 keys 742 us
+    // against 857, 20 000 keys 595 against 555)
+    const gs2d_clip cl = clip_of_tile(a.cs, tl);
+    if ((cl.n - 1) / kBitKeys <= len / 1024)
+      block_sort_bits(a.list + x, len, (uint32_t)cl.g_off, cl.n, a.spare + x, s_keys);
+    else
+      block_sort_long(a.list + x, len, a.spare + x, s_keys);
   }
 }
 
@@ -767,9 +837,23 @@ static cudaError_t launch_bin(const BinArgs& a, AdamTick tick, cudaStream_t s) {
   if (e == cudaSuccess && a.n > 0)
     e = launch_pdl(k_bin_scatter<kLazy>, blocks, kThreads, 0, s, a, (const long long*)first);
   if (e != cudaSuccess) return e;
-  // few tiles: a block each (eight per block would leave most SMs idle)
-  if (a.num_tiles <= 152 * 4) return launch_pdl(k_sort<kLazy, 1>, a.num_tiles, kThreads, 0, s, a);
-  return launch_pdl(k_sort<kLazy, 8>, (a.num_tiles + 7) / 8, kThreads, 0, s, a);
+  // a block for each tile where there are few (eight per block would leave most
+  // SMs idle), or where most lists are too long for a warp: 300 000 Gaussians in
+  // 920 tiles, lists of about 700: 217 us in eights, 124 so
+  if (a.num_tiles <= 152 * 4 || a.n / 256 >= a.num_tiles)
+    return launch_pdl(k_sort<kLazy, 1>, a.num_tiles, kThreads, kSmemKeys * 4, s, a);
+  // The blocks are launched while the scatter drains, and an SM must drain first
+  // to give them its shared memory: the first SMs to do so take all they can hold.
+  // With lists of some length each block asks for its SM's share instead (140 000
+  // Gaussians in 920 tiles, lists of about 325: 115 blocks on some 23 SMs took 23
+  // us, 7.5 so); waiting for more SMs to drain costs 1.5 us, which short lists do
+  // not bring back (4000 Gaussians there).
+  const int grid = (a.num_tiles + 7) / 8, per_sm = (grid + 151) / 152;
+  const int smem = per_sm >= 6 || a.n / 32 < a.num_tiles ? kSmemKeys * 4
+                                                         : (226 * 1024) / per_sm - 2048;
+  e = opt_in_smem((const void*)k_sort<kLazy, 8>, smem);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(k_sort<kLazy, 8>, grid, kThreads, smem, s, a);
 }
 
 cudaError_t launch_bin_sort(const gs2d_plan& p, void* ws, cudaStream_t s) {

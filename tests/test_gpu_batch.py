@@ -150,6 +150,29 @@ def batch_inputs(sizes_seeds):
     return ps, ts
 
 
+@pytest.mark.parametrize("counts", [(300, 900), (300, 1300), (270000, 3000, 10000)])
+def test_batch_long_lists_are_those_of_the_clips(gs, counts):
+    """Lists beyond a warp's, of clips behind others: a clip's lists are its own
+    plan's with its first Gaussian's index added."""
+    W, H = 32, 16
+    ps = []
+    for k, n in enumerate(counts):
+        p = random_gaussians(n, W, H, seed=k, l_range=(0.2, 0.4))
+        p[0, 5000:] = -1e4
+        ps.append(to_dev(p))
+    b = gs.BatchRasterizer([(W, H, n) for n in counts])
+    b.prepare(b.pack_params(ps))
+    got = b.read_bins()
+    want = []
+    for c, p in enumerate(ps):
+        r = gs.GaussianRasterizer(W, H, counts[c])
+        r.prepare(p)
+        want.append(r.read_bins()["values"].astype(np.int64) + b.clips[c].g_off)
+    assert max(y - x for x, y in got["ranges"]) > (512 if max(counts) > 1000 else 450)
+    np.testing.assert_array_equal(got["values"].astype(np.int64), np.concatenate(want))
+    assert b.status() == 0
+
+
 @pytest.mark.parametrize("tile,stage", [(16, 64), (8, 32), (32, 128)])
 def test_batch_bins_bit_exact(gs, oracle, tile, stage):
     ps, ts = batch_inputs(BATCH)

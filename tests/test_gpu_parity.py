@@ -503,6 +503,28 @@ def _piled(n, W, H, seed, at, share):
     return np.ascontiguousarray(p)
 
 
+@pytest.mark.parametrize("n,piles", [
+    (262144, (600, 9000)), (262145, (600, 9000)), (300000, (513, 32768)),
+    (800000, (600, 2000, 20000)), (800000, (3071, 3072, 8193))])
+def test_bins_bit_exact_where_long_lists_meet_many_gaussians(gs, oracle, n, piles):
+    """The bitmap of a long list's keys in one and in several passes, and the
+    networks where the passes would be too many for the list's length: piles of
+    Gaussians in tiles of their own, their indices spread over all n."""
+    W, H = 16 * len(piles), 16
+    g = np.random.Generator(np.random.PCG64(n))
+    p = random_gaussians(n, W, H, seed=n, l_range=(0.2, 0.4))
+    p[0] = -1e4  # (the others off the frame)
+    at = 0
+    order = g.permutation(n)
+    for k, count in enumerate(piles):
+        p[0, order[at:at + count]] = g.uniform(16 * k + 5, 16 * k + 11, count)
+        p[1, order[at:at + count]] = g.uniform(5, 11, count)
+        at += count
+    r = check_bins(gs, oracle, p, W, H)
+    assert r.status() == 0
+    assert [b - a for a, b in r.read_bins()["ranges"]] == list(piles)
+
+
 @pytest.mark.parametrize("n,W,H,share", [
     (513, 16, 16, 1.0), (700, 64, 48, 0.8), (8192, 64, 48, 1.0), (8193, 64, 48, 1.0),
     (17000, 64, 48, 0.97), (32768, 64, 48, 1.0), (3000, 640, 360, 0.9),
