@@ -156,13 +156,18 @@ class LearnedInitializer:
             most = max(most, need)
         self.partial = torch.empty(max(most // 4, 1), device=dev)
 
-    def _implicit_conv(self, li: int) -> bool:
-        """Whether layer li's forward runs as an implicit GEMM: unless K is very
-        deep and the output rows short (37 k-tiles over few tiles of gathered
-        operands: the TMA-fed GEMM over an im2col operand is faster there; from
-        49 pixels the TMA taps serve two rows a tile)."""
+    def _implicit_conv(self, li: int, written: bool = False) -> bool:
+        """Whether layer li's forward runs as an implicit GEMM: where TMA brings
+        the taps (rows of at least 49 pixels, channels in whole boxes, at most
+        512 outputs); else gathered, unless K is very deep (37 k-tiles over few
+        tiles: im2col and the TMA-fed GEMM are faster) or the operand is
+        `written` anyway (a training step at 320 x 180: 418 us
+        gathered, 384 so)."""
+        ci, co, _, ldk = self.layers[li]
         wo = self.sizes[li + 1][1] if li < self.L else self.sizes[-1][1]
-        return (self.layers[li][3] + 63) // 64 <= 32 or wo >= 49
+        if wo >= 49 and co <= 512 and (ci in (16, 32) or ci % 64 == 0):
+            return True
+        return not written and (ldk + 63) // 64 <= 32
 
     def _implicit_wgrad(self, li: int) -> bool:
         """Whether layer li's weight gradient reads the activations themselves
@@ -231,8 +236,9 @@ class LearnedInitializer:
             out32 = self.out.data_ptr() if last else 0
             out16 = 0 if last else self.x[li + 1].data_ptr()
             # (the results are identical either way)
-            implicit = self._implicit_conv(li)
-            if not implicit or (keep_col and not self._implicit_wgrad(li)):
+            written = keep_col and not self._implicit_wgrad(li)
+            implicit = self._implicit_conv(li, written)
+            if not implicit or written:
                 nat.call("gs2d_im2col", src.data_ptr(), B, hi, wi, ci, ks, stride, pad,
                          self._col[li].data_ptr(), ldk, s)
             if li == 0 and from_frames:
