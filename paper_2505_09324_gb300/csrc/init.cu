@@ -67,6 +67,13 @@ struct SpArgs {
 constexpr float kGatherS = 32.0f;
 constexpr int kWave = 152;  // blocks of one wave
 
+// Whether the update gathers: with at most a wave of centres half the step (the
+// whole initialisation of a 256 x 256 frame with 70 centres 31 pixels apart: 286 us
+// gathered, 226 by atomics).
+__device__ __forceinline__ bool gathered(const SpGeom& g) {
+  return g.S32 <= (g.M > kWave ? kGatherS : 0.5f * kGatherS);
+}
+
 // The pixel's colour on the 2^-20 grid: a power-of-two scaling, exact in
 // float, then one rounding to the nearest integer.
 __device__ __forceinline__ int colour_int(float c) {
@@ -133,7 +140,7 @@ __global__ void __launch_bounds__(256) k_sp_assign(SpArgs a, int first) {
   }
   __syncthreads();
   const size_t HW = (size_t)a.W * a.H;
-  const bool gather = g.S32 <= kGatherS;
+  const bool gather = gathered(g);
 #pragma unroll
   for (int k = 0; k < 2; k++) {
     const int y = yt + 8 * k;
@@ -345,19 +352,26 @@ __device__ __forceinline__ void segment_gaussian(const SpArgs& a, const SpGeom& 
 // and would leave most SMs idle: up to a wave of blocks of 16 or 8 centres,
 // blocks take that many, with 2 or 4 half-warps to each centre's window (340
 // centres of a 565 x 315 frame: 31 -> 18 us, its wait for the assignment
-// included).  Large segments: the sums come from the assignment's atomics and
-// are cleared for the next one.
-template <bool FINAL>
+// included).  FEW, launched for at most kFewCentres wanted: gathered blocks of
+// 4, 2 or 1 too, with up to 32 bands (280 centres 29 pixels apart, the whole
+// initialisation: 540 us with 4, 344 so); a kernel of its own, whose registers
+// the usual one would feel.  Large segments: the sums come from the assignment's
+// atomics and are cleared for the next one.
+constexpr int kFewCentres = kWave * 4;
+
+template <bool FINAL, bool FEW>
 __global__ void __launch_bounds__(256) k_sp_update(SpArgs a, float* __restrict__ params) {
   pdl_begin();
   __shared__ long long s_sum[kSums][32];
   const SpGeom g = *a.geo;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int per = g.M <= kWave * 8 ? 8 : g.M <= kWave * 16 ? 16 : 32;  // centres of a block
+  int per = g.M <= kWave * 8 ? 8 : g.M <= kWave * 16 ? 16 : 32;  // centres of a block
+  if (FEW && gathered(g))
+    per = g.M <= kWave ? 1 : g.M <= kWave * 2 ? 2 : g.M <= kWave * 4 ? 4 : per;
   const int c0 = blockIdx.x * per;
   if (c0 >= g.M) return;
   const bool mine = lane < per && c0 + lane < g.M;
-  if (g.S32 <= kGatherS) {
+  if (gathered(g)) {
     const int half = threadIdx.x >> 4, hl = threadIdx.x & 15;
     const unsigned mask = 0xffffu << (lane & 16);
     if (per < 32) {
@@ -646,7 +660,8 @@ gs2d_status roi_init(const float* frame, const uint8_t* mask, int W, int H, int 
   a.blk = reinterpret_cast<int*>(take(kSeedBlocks * 4));
   // everything on the device; the region count comes back at the end
   const dim3 tiles((W + kTileW - 1) / kTileW, (H + kTileH - 1) / kTileH);
-  const int cb = std::max((n + 31) / 32, std::min((n + 7) / 8, kWave));  // k_sp_update's
+  const bool few = a.k_target <= kFewCentres;
+  const int cb = std::max((n + 31) / 32, std::min(n, kWave));  // k_sp_update's
   cudaError_t e = cudaMemsetAsync(a.area, 0, 8, s);
   if (e == cudaSuccess) e = launch_pdl(k_sp_area, 152 * 8, 256, 0, s, a);
   if (e == cudaSuccess) e = launch_pdl(k_sp_seed_count, kSeedBlocks, 256, 0, s, a);
@@ -664,8 +679,11 @@ gs2d_status roi_init(const float* frame, const uint8_t* mask, int W, int H, int 
         e = cudaMemcpyAsync(label_trace + (size_t)it * hw, a.label, hw * sizeof(int32_t),
                             cudaMemcpyDeviceToDevice, s);
       if (e == cudaSuccess)
-        e = it + 1 < kIterations ? launch_pdl(k_sp_update<false>, cb, 256, 0, s, a, params)
-                                 : launch_pdl(k_sp_update<true>, cb, 256, 0, s, a, params);
+        e = it + 1 < kIterations
+                ? launch_pdl(few ? k_sp_update<false, true> : k_sp_update<false, false>, cb, 256,
+                             0, s, a, params)
+                : launch_pdl(few ? k_sp_update<true, true> : k_sp_update<true, false>, cb, 256,
+                             0, s, a, params);
     }
   }
   SpGeom g;

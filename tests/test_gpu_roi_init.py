@@ -194,3 +194,10 @@ def test_blocks_of_8_16_and_32_centres(gs, n):
     """Centre counts on both sides of the update's two lines (152 blocks of 8
     and of 16 centres), against the oracle."""
     test_tile_edges_and_both_sum_paths(gs, 64, 40, n, 1.0)
+
+
+@pytest.mark.parametrize("n", [3, 7, 148, 160, 300, 320, 600, 640])
+def test_blocks_of_one_to_eight_centres(gs, n):
+    """Few centres: the lines between blocks of 1, 2, 4 and 8 (152 blocks
+    each), windows shorter than their number of bands, against the oracle."""
+    test_tile_edges_and_both_sum_paths(gs, 64, 40, n, 1.0)
