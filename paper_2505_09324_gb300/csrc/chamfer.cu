@@ -415,46 +415,53 @@ k_chamfer_grad(const float* __restrict__ P, int np, int ldp, const float* __rest
   }
 }
 
-// Mean squared distances of both directions of frame b, one block.  Float sums
-// per thread (FloatSum: no less accurate than double additions), doubles only
-// across threads and one division per mean: FP64 issues at 1/64 of the FP32
-// rate, and double sums and divisions in every thread took 33 us for 20 000
-// points a side, 24 so.
+// Mean squared distances of both directions of frame b, one block.  Sums of three
+// floats (FloatSum: no less accurate than double), one division per mean: with
+// double sums and divisions in every thread 33 us for 20 000 points a side, 17 so.
 __global__ void __launch_bounds__(1024)
 k_chamfer_loss(const float* __restrict__ d1, int np, const float* __restrict__ d2, int nq,
                float* __restrict__ loss) {
   pdl_begin();
-  __shared__ double2 s[32];
-  const int b = blockIdx.x;
+  __shared__ WarpSums s_sum[2];
+  __shared__ double s_d[32];
+  __shared__ int s_past;
+  const int b = blockIdx.x, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  d1 += (size_t)b * np;
+  d2 += (size_t)b * nq;
   FloatSum a, c;
 #pragma unroll 4
-  for (int i = threadIdx.x; i < np; i += blockDim.x) a.add(d1[(size_t)b * np + i]);
+  for (int i = threadIdx.x; i < np; i += blockDim.x) a.add(d1[i]);
 #pragma unroll 4
-  for (int i = threadIdx.x; i < nq; i += blockDim.x) c.add(d2[(size_t)b * nq + i]);
-  double x = a.value(), y = c.value();
-  // (sums past FP32's range, whose mean may still lie within it)
-  if (!isfinite(x)) {
-    x = 0.0;
-    for (int i = threadIdx.x; i < np; i += blockDim.x) x += d1[(size_t)b * np + i];
+  for (int i = threadIdx.x; i < nq; i += blockDim.x) c.add(d2[i]);
+  a.warp_sum();
+  c.warp_sum();
+  if (lane == 0) {
+    s_sum[0].put(wid, a);
+    s_sum[1].put(wid, c);
   }
-  if (!isfinite(y)) {
-    y = 0.0;
-    for (int i = threadIdx.x; i < nq; i += blockDim.x) y += d2[(size_t)b * nq + i];
-  }
-  for (int o = 16; o > 0; o >>= 1) {
-    x += __shfl_xor_sync(0xffffffffu, x, o);
-    y += __shfl_xor_sync(0xffffffffu, y, o);
-  }
-  if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = make_double2(x, y);
   __syncthreads();
-  if (threadIdx.x == 0) {
-    x = y = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); w++) {
-      x += s[w].x;
-      y += s[w].y;
+  if (wid == 0) {
+    a = s_sum[0].sum(lane);
+    c = s_sum[1].sum(lane);
+    if (lane == 0) {
+      s_past = !isfinite(a.hi) || !isfinite(c.hi);
+      loss[b] = (float)(a.value() / np + c.value() / nq);
     }
-    loss[b] = (float)(x / np + y / nq);
   }
+  __syncthreads();
+  if (!s_past) return;
+  // a sum past FP32's range, whose mean may still lie within it
+  double x = 0.0, y = 0.0;
+  for (int i = threadIdx.x; i < np; i += blockDim.x) x += d1[i];
+  for (int i = threadIdx.x; i < nq; i += blockDim.x) y += d2[i];
+  double v = x / np + y / nq;
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if (lane == 0) s_d[wid] = v;
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  v = 0.0;
+  for (int w = 0; w < (int)(blockDim.x >> 5); w++) v += s_d[w];
+  loss[b] = (float)v;
 }
 
 }  // namespace

@@ -170,8 +170,10 @@ __device__ __forceinline__ void set_status(WsHeader* h, int code) {
 // of that to lo.  What is lost is the rounding of lo, of the order of n^2 2^-72
 // of the sum after n additions, so value() is the sum rounded to double once,
 // where n double additions round n - 1 times.  The loss sums run over every tile
-// in one or a few blocks, where double additions (1/64 of the FP32 rate) were
-// the whole time: 65 us for the 65 280 tiles of eight 1080p frames.
+// in one or a few blocks, where FP64 (1/64 of the FP32 rate, and a warp
+// instruction costs the same however few lanes it has) was the whole time: 65 us
+// for the additions of the 65 280 tiles of eight 1080p frames, 2.5 us for the warps'
+// shuffle tree of any frame.
 struct FloatSum {
   float hi = 0.0f, mid = 0.0f, lo = 0.0f;
   __device__ __forceinline__ static float two_sum(float& a, float x) {
@@ -184,19 +186,53 @@ struct FloatSum {
     x = two_sum(hi, x);
     lo = __fadd_rn(lo, two_sum(mid, x));
   }
+  __device__ __forceinline__ void add(const FloatSum& o) {
+    const float e = two_sum(hi, o.hi);
+    const float f = two_sum(mid, o.mid), g = two_sum(mid, e);
+    lo = __fadd_rn(__fadd_rn(lo, o.lo), __fadd_rn(f, g));
+  }
+  // the sum over the warp, in lane 0
+  __device__ __forceinline__ void warp_sum() {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      FloatSum x;
+      x.hi = __shfl_down_sync(0xffffffffu, hi, o);
+      x.mid = __shfl_down_sync(0xffffffffu, mid, o);
+      x.lo = __shfl_down_sync(0xffffffffu, lo, o);
+      add(x);
+    }
+  }
   __device__ __forceinline__ double value() const {
     // (the others are NaN past an infinity)
     return isfinite(hi) ? (double)hi + ((double)mid + (double)lo) : (double)hi;
   }
 };
 
+// The sums of 32 warps (a column each), summed by one warp.
+struct WarpSums {
+  float hi[32], mid[32], lo[32];
+  __device__ __forceinline__ void put(int w, const FloatSum& x) {
+    hi[w] = x.hi;
+    mid[w] = x.mid;
+    lo[w] = x.lo;
+  }
+  __device__ __forceinline__ FloatSum sum(int lane) const {  // in lane 0
+    FloatSum x;
+    x.hi = hi[lane];
+    x.mid = mid[lane];
+    x.lo = lo[lane];
+    x.warp_sum();
+    return x;
+  }
+};
+
 // Sums of the loss partials of `count` tiles by one block, in the order of
 // 1024 threads (thread t: tiles t, t + 1024, ...; each warp's lanes; the 32
 // warps) whatever the block's size is: every caller gets the same bits.  Valid
-// in thread 0.  s_sum: 32 pairs.
+// in thread 0.
 template <int THREADS>
 __device__ __forceinline__ double2 loss_sums(const float2* __restrict__ part, int count,
-                                             double2* s_sum) {
+                                             WarpSums (&s_sum)[2]) {
   static_assert(1024 % THREADS == 0 && THREADS % 32 == 0, "whole warps of the 1024");
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll 1
@@ -218,21 +254,19 @@ __device__ __forceinline__ double2 loss_sums(const float2* __restrict__ part, in
       a.add(v.x);
       b.add(v.y);
     }
-    double x = a.value(), y = b.value();
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      x += __shfl_xor_sync(0xffffffffu, x, o);
-      y += __shfl_xor_sync(0xffffffffu, y, o);
+    a.warp_sum();
+    b.warp_sum();
+    if (lane == 0) {
+      s_sum[0].put(k * (THREADS / 32) + wid, a);
+      s_sum[1].put(k * (THREADS / 32) + wid, b);
     }
-    if (lane == 0) s_sum[k * (THREADS / 32) + wid] = make_double2(x, y);
   }
   __syncthreads();
   double2 s = make_double2(0.0, 0.0);
-  if (threadIdx.x == 0)
-    for (int w = 0; w < 32; w++) {
-      s.x += s_sum[w].x;
-      s.y += s_sum[w].y;
-    }
+  if (wid == 0) {
+    const FloatSum a = s_sum[0].sum(lane), b = s_sum[1].sum(lane);
+    if (lane == 0) s = make_double2(a.value(), b.value());
+  }
   return s;
 }
 
@@ -255,7 +289,7 @@ struct LoopArgs {
 };
 
 template <int THREADS>
-__device__ __forceinline__ void loop_control(const LoopArgs& a, double2* s_sum) {
+__device__ __forceinline__ void loop_control(const LoopArgs& a, WarpSums (&s_sum)[2]) {
   __shared__ int s_it;
   if (threadIdx.x == 0) s_it = a.hdr->loop_end ? 0 : ++a.hdr->loop_iter;
   __syncthreads();

@@ -190,7 +190,7 @@ k_reduce_chain_adam(int n, float* __restrict__ params, SlotArgs slots,
                     float* __restrict__ acc, float* __restrict__ host_out, LoopArgs loop) {
   pdl_begin();
   if (loop.hdr && blockIdx.x == gridDim.x - 1) {
-    __shared__ double2 s_sum[32];
+    __shared__ WarpSums s_sum[2];
     loop_control<256>(loop, s_sum);
     return;
   }
@@ -243,7 +243,7 @@ __global__ void __launch_bounds__(1024)
 k_loss_reduce(int num_tiles, const float2* __restrict__ loss_part, WsHeader* __restrict__ hdr,
               float* __restrict__ out) {
   pdl_begin();
-  __shared__ double2 s_sum[32];
+  __shared__ WarpSums s_sum[2];
   const double2 s = loss_sums<1024>(loss_part, num_tiles, s_sum);
   if (threadIdx.x == 0) {
     hdr->loss[0] = (float)s.x;
@@ -261,7 +261,7 @@ k_clip_loss(ClipSet cs, const float2* __restrict__ loss_part, float2* __restrict
   pdl_begin();
   const int c = blockIdx.x;
   const gs2d_clip cl = cs.count == 1 ? cs.one : cs.table[c];
-  __shared__ double2 s_sum[32];
+  __shared__ WarpSums s_sum[2];
   const double2 s = loss_sums<1024>(loss_part + cl.tile_off, cl.tiles_x * cl.tiles_y, s_sum);
   if (threadIdx.x == 0) clip_loss[c] = make_float2((float)s.x, (float)s.y);
 }
