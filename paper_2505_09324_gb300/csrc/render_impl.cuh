@@ -705,23 +705,32 @@ k_render(RenderArgs a) {
   }
 }
 
-// Warps of the usual kernels (kRows<T> rows per thread) up to which a launch
-// takes the kernels with one row per thread (four times the warps).  With few
-// tiles the usual ones leave the chip's 608 schedulers a warp or two each, and
-// both passes are chains of dependent instructions.  The backward gains, since
-// the warps share a tile's Gaussians; the forward does not (a pixel's chain
-// is as long as before and a warp's setup per Gaussian serves a quarter of
-// the pixels: 4.5 -> 5.3 us at 256 x 256), so it never does alone and the
-// fused call does only while the backward's gain is the larger.  Measured with
-// 104 pixels per Gaussian, usual kernels against these, us: fused, tile 16:
-// 22.3 / 15.3 at 256 x 256 (512 warps), 27.4 / 25.9 at 640 x 360 (1840), 36.2 /
-// 39.7 at 960 x 540 (4080); tile 32: 20.2 / 19.5 (512 warps), 24.5 / 31.5
-// (1920); backward alone, tile 16: 18.2 / 11.3, 38.4 / 36.5 at 1280 x 720
-// (7200); tile 32: 17.7 / 16.5 (1920), 19.1 / 21.3 (3000).
+// Whether a launch of num_tiles tiles with n Gaussians takes the kernels with one
+// row per thread (four times the warps).  With few tiles the usual ones leave the
+// chip's 608 schedulers a warp or two each, and both passes are chains of dependent
+// instructions.  The backward gains, since the warps share a tile's Gaussians; the
+// forward does not (a pixel's chain is as long as before and a warp's setup per
+// Gaussian serves a quarter of the pixels: 4.5 -> 5.3 us at 256 x 256), so it never
+// does alone and the fused call does only while the backward's gain is the larger.
+// Lines in warps of the usual kernels: up to kAny, up to kDense with at most 48
+// pixels per Gaussian.  Usual kernels / these, us, at 10, 104 and 1000 pixels per
+// Gaussian (warps):
+//   fused, tile 16: 33.4 / 22.8, 20.1 / 16.0, 18.7 / 16.6 (512); 42.1 / 40.9, 23.7 /
+//     25.1, 25.0 / 25.9 (1840); 62.5 / 66.6, 32.7 / 37.8, 30.4 / 36.6 (4080)
+//   fused, tile 32: 35.3 / 30.7, 19.5 / 20.6, 16.3 / 18.5 (512); 36.0 / 31.8, 19.1 /
+//     20.5, 16.8 / 19.2 (1080)
+//   backward, tile 16: 47.7 / 38.3, 23.7 / 21.4, 20.5 / 21.2 (4080); 64.8 / 60.8,
+//     32.1 / 32.1, 26.7 / 29.6 (7200)
+//   backward, tile 32: 24.9 / 16.3, 12.7 / 10.3, 11.4 / 10.4 (1080); 27.9 / 26.9,
+//     13.3 / 14.8, 13.6 / 13.8 (1920)
 template <int T, int MODE>
-constexpr int kFewWarps = MODE == kModeL2    ? (T == 16 ? 2400 : 1200)
-                          : MODE == kModeBwd ? (T == 16 ? 7200 : 1920)
-                                             : 0;
+bool few_tiles(int num_tiles, int n) {
+  constexpr int kAny = MODE == kModeL2 ? (T == 16 ? 1400 : 0) : T == 16 ? 4800 : 1400;
+  constexpr int kDense = MODE == kModeL2 ? (T == 16 ? 2400 : 1200) : T == 16 ? 7200 : 1920;
+  constexpr int kWarps = TileGeom<T, kRows<T>>::NW;  // of a tile
+  return num_tiles <= kAny / kWarps ||
+         (num_tiles <= kDense / kWarps && n >= num_tiles * (T * T / 48));
+}
 
 template <int T, int S, int MODE, int LAUNCH, int R>
 cudaError_t launch_rows(const RenderArgs& a, cudaStream_t s) {
@@ -736,9 +745,9 @@ cudaError_t launch_rows(const RenderArgs& a, cudaStream_t s) {
 template <int T, int S, int MODE, int LAUNCH>
 cudaError_t launch_mode(const RenderArgs& a, cudaStream_t s) {
   if (a.num_tiles <= 0) return cudaSuccess;
-  if constexpr (T > 8 && LAUNCH == GS2D_LAUNCH_GRID && kFewWarps<T, MODE> > 0) {
-    if (a.num_tiles <= kFewWarps<T, MODE> / TileGeom<T, kRows<T>>::NW)
-      return launch_rows<T, S, MODE, LAUNCH, 1>(a, s);
+  if constexpr (T > 8 && LAUNCH == GS2D_LAUNCH_GRID &&
+                (MODE == kModeL2 || MODE == kModeBwd)) {
+    if (few_tiles<T, MODE>(a.num_tiles, a.n)) return launch_rows<T, S, MODE, LAUNCH, 1>(a, s);
   }
   return launch_rows<T, S, MODE, LAUNCH, kRows<T>>(a, s);
 }
