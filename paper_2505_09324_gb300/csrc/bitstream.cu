@@ -65,6 +65,19 @@ __device__ __forceinline__ void tally_count(EntropySmem& sm, unsigned c, double&
     acc += (double)c * log2((double)c);
 }
 
+// The row's code length from the threads' sums.  Valid in thread 0.
+__device__ __forceinline__ double row_length(EntropySmem& sm, double total, double acc) {
+  constexpr int kWarps = kEntropyThreads / 32;
+  const int t = threadIdx.x;
+  for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if ((t & 31) == 0) sm.acc[t >> 5] = acc;
+  __syncthreads();
+  if (t != 0) return 0.0;
+  double sum = 0.0;
+  for (int w = 0; w < kWarps; w++) sum += sm.acc[w];
+  return total > 1.0 ? total * log2(total) - sum : 0.0;
+}
+
 // The row's code length from the tally and the threads' sums over the larger
 // counts, in a fixed order (ascending counts over the threads, then a fixed
 // reduction tree), so the result is reproducible.  Valid in thread 0.
@@ -96,13 +109,7 @@ __device__ __forceinline__ double tally_finish(EntropySmem& sm, double total, do
     const double c = (double)sm.item[j];
     acc += (double)sm.tally[sm.item[j]] * (c * log2(c));
   }
-  for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if (lane == 0) sm.acc[wid] = acc;
-  __syncthreads();
-  if (t != 0) return 0.0;
-  double sum = 0.0;
-  for (int w = 0; w < kWarps; w++) sum += sm.acc[w];
-  return total > 1.0 ? total * log2(total) - sum : 0.0;
+  return row_length(sm, total, acc);
 }
 
 // Up to 65 535 columns: block r counts row r's symbols in shared memory and
@@ -179,13 +186,19 @@ k_code_entropy(const uint32_t* __restrict__ hist, RowBits rb, double* __restrict
     if (threadIdx.x == 0) out[r] = 32.0 * total;
     return;
   }
-  tally_clear(sm);
-  __syncthreads();
   const int nb = 1 << symbol_bits(b);
-  double acc = 0.0;
-  for (int j = threadIdx.x; j < nb; j += kEntropyThreads)
-    tally_count(sm, hist[(size_t)r * kBins + j], acc);
-  const double length = tally_finish(sm, total, acc);
+  const uint32_t* counts = hist + (size_t)r * kBins;
+  double acc = 0.0, length;
+  if (nb <= 256) {  // (few symbols: the tally takes longer than it spares)
+    for (int j = threadIdx.x; j < nb; j += kEntropyThreads)
+      if (counts[j] > 1u) acc += (double)counts[j] * log2((double)counts[j]);
+    length = row_length(sm, total, acc);
+  } else {
+    tally_clear(sm);
+    __syncthreads();
+    for (int j = threadIdx.x; j < nb; j += kEntropyThreads) tally_count(sm, counts[j], acc);
+    length = tally_finish(sm, total, acc);
+  }
   if (threadIdx.x == 0) out[r] = length;
 }
 
