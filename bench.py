@@ -123,6 +123,18 @@ def render_traffic(schedule):
     return NCU_TRAFFIC["bytes"] if ok else None
 
 
+def fit_launches(num_tiles: int, n: int, retained: bool) -> int:
+    """Our kernels per fit step: projection (+ containment test of the retained
+    lists), list rebuild counts, their scan (a launch of its own above 2048 tiles
+    or groups of Gaussians: 64 to a group up to 2048 groups, else 256), scatter,
+    sort (these return at once while the lists hold), fused render, reduction +
+    Adam; per-iteration binning fuses the first two."""
+    groups = -(-n // 64)
+    if groups > 2048:
+        groups = -(-n // 256)
+    return (4 if retained else 3) + (num_tiles > 2048 or groups > 2048) + 1 + 1
+
+
 def parse():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
@@ -811,13 +823,8 @@ def run_ours(args):
     def fit_step(p_t):
         nat.fit_step(plan, ws, frame.data_ptr(), p_t.data_ptr(), m.data_ptr(), v.data_ptr(), sp)
 
-    # our kernels per step: projection (+ containment test of the retained
-    # lists), list rebuild counts with their scan (a launch of its own above
-    # 2048 tiles or Gaussian groups), scatter, sort (these return at once while
-    # the lists hold), fused render, reduction + Adam; per-iteration binning
-    # fuses the first two
-    retained = tuned["config"].bin_margin >= 0
-    launches_per_step = (4 if retained else 3) + (int(plan.num_tiles) > 2048) + 1 + 1
+    launches_per_step = fit_launches(int(plan.num_tiles), int(plan.n),
+                                     tuned["config"].bin_margin >= 0)
 
     for _ in range(args.warmup):
         fit_step(params)

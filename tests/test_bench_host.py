@@ -88,3 +88,13 @@ def test_paper_encode_reference(bench):
     p = bench.PAPER_ENCODE
     assert p["superpixel_s"] == 1.5 and p["random_init_s"] == 13.1
     assert abs(p["reduction"] - 0.885) < 1e-3  # the paper rounds it to 88 %
+
+
+@pytest.mark.parametrize("num_tiles,n,retained,launches", [
+    (2040, 20000, True, 6), (8160, 20000, True, 7), (8160, 20000, False, 6),
+    (2048, 131072, False, 5), (920, 131073, True, 6), (920, 524288, True, 6),
+    (920, 524289, True, 7), (2049, 524289, False, 6)])
+def test_launches_per_fit_step(bench, num_tiles, n, retained, launches):
+    """The scan is a launch of its own above 2048 tiles and above 2048 groups of
+    Gaussians (of 256, where groups of 64 would be more)."""
+    assert bench.fit_launches(num_tiles, n, retained) == launches
