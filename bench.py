@@ -82,7 +82,7 @@ PAPER_ENCODE = {"reduction": 1.0 - 1.5 / 13.1, "superpixel_s": 1.5, "random_init
 # stage 128, grid) from an ncu capture of this workload, valid for the render
 # source with this sha256 (else null)
 NCU_TRAFFIC = {"bytes": 26823936, "schedule": (32, 128, 1),
-               "render_sha256": "611a9e93f9283da6da0c59246587000d7f9e12df6ba430e6c61717ac6ab78e06"}
+               "render_sha256": "0b8161a973cb76d86c3405c5f08bc7dc7797ea89a13aa008c14b27865c15998f"}
 
 
 def hbm_peak_gbs() -> float:

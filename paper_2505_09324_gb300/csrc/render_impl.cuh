@@ -714,7 +714,9 @@ k_render(RenderArgs a) {
 // does alone and the fused call does only while the backward's gain is the larger.
 // Lines in warps of the usual kernels: up to kAny, up to kDense with at most 48
 // pixels per Gaussian.  Usual kernels / these, us, at 10, 104 and 1000 pixels per
-// Gaussian (warps):
+// Gaussian that tile the frame (warps); where Gaussians of many sizes leave a few
+// tiles with long lists, as fits do, these gain more (a fit step at 640 x 360, 4000
+// Gaussians, tile 16: 42 / 37):
 //   fused, tile 16: 33.4 / 22.8, 20.1 / 16.0, 18.7 / 16.6 (512); 42.1 / 40.9, 23.7 /
 //     25.1, 25.0 / 25.9 (1840); 62.5 / 66.6, 32.7 / 37.8, 30.4 / 36.6 (4080)
 //   fused, tile 32: 35.3 / 30.7, 19.5 / 20.6, 16.3 / 18.5 (512); 36.0 / 31.8, 19.1 /
@@ -725,7 +727,7 @@ k_render(RenderArgs a) {
 //     13.3 / 14.8, 13.6 / 13.8 (1920)
 template <int T, int MODE>
 bool few_tiles(int num_tiles, int n) {
-  constexpr int kAny = MODE == kModeL2 ? (T == 16 ? 1400 : 0) : T == 16 ? 4800 : 1400;
+  constexpr int kAny = MODE == kModeL2 ? (T == 16 ? 2400 : 0) : T == 16 ? 4800 : 1400;
   constexpr int kDense = MODE == kModeL2 ? (T == 16 ? 2400 : 1200) : T == 16 ? 7200 : 1920;
   constexpr int kWarps = TileGeom<T, kRows<T>>::NW;  // of a tile
   return num_tiles <= kAny / kWarps ||

@@ -65,8 +65,10 @@ class _Columns:
     def __len__(self):
         return len(self._net.layers)
 
-    def __getitem__(self, li: int) -> torch.Tensor:
+    def __getitem__(self, li):
         li = range(len(self))[li]
+        if isinstance(li, range):  # (a slice)
+            return [self[k] for k in li]
         net = self._net
         if net._col[li] is not None and not net._implicit_wgrad(li):
             return net._col[li]
