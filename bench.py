@@ -823,8 +823,8 @@ def run_ours(args):
     def fit_step(p_t):
         nat.fit_step(plan, ws, frame.data_ptr(), p_t.data_ptr(), m.data_ptr(), v.data_ptr(), sp)
 
-    launches_per_step = fit_launches(int(plan.num_tiles), int(plan.n),
-                                     tuned["config"].bin_margin >= 0)
+    retained = tuned["config"].bin_margin >= 0
+    launches_per_step = fit_launches(int(plan.num_tiles), int(plan.n), retained)
 
     for _ in range(args.warmup):
         fit_step(params)

@@ -98,3 +98,20 @@ def test_launches_per_fit_step(bench, num_tiles, n, retained, launches):
     """The scan is a launch of its own above 2048 tiles and above 2048 groups of
     Gaussians (of 256, where groups of 64 would be more)."""
     assert bench.fit_launches(num_tiles, n, retained) == launches
+
+
+def test_bench_defines_every_name_it_uses():
+    """The benchmark's GPU parts do not run here: at least no function of it
+    names a global that the module lacks."""
+    import builtins
+    import symtable
+    with open(os.path.join(ROOT, "bench.py")) as f:
+        top = symtable.symtable(f.read(), "bench.py", "exec")
+    known = {s.get_name() for s in top.get_symbols()}
+
+    def missing(table):
+        own = [s.get_name() for s in table.get_symbols() if s.is_global()]
+        return [n for n in own if n not in known and not hasattr(builtins, n)] + [
+            n for c in table.get_children() for n in missing(c)]
+
+    assert not missing(top)
