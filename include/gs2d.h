@@ -529,8 +529,9 @@ gs2d_status gs2d_roi_init_trace(const float* frame, const uint8_t* mask, int32_t
  * one host read at the end (the trace is kept in the workspace's gradient
  * scratch, so it needs iters / check_every + 1 <= 9n).  Up to 64 iterations
  * without a target are launched at once, with the device taking the checks.
- * Otherwise (up to 64 iterations with at most 8 checks, the legacy default
- * stream, a longer trace, or a driver that declines the graph) the host
+ * Otherwise (up to 64 iterations with iters / check_every at most 8, the
+ * legacy default stream, a longer trace, or a driver that declines the graph)
+ * the host
  * launches the iterations, or replays one captured iteration, and reads the
  * PSNR back at each check.  All give the same results bit for bit.
  * target: device [3][H][W].  params: device 9n floats, in: start, out: fitted.
@@ -738,7 +739,8 @@ gs2d_status gs2d_conv_wgrad_bf16(const void* dz, int32_t N, const void* x, int32
                                  void* stream);
 
 /* out[c][r] = in[r][c] for a BF16 R x C matrix (device; leading dimensions
- * ld_in >= C, ld_out >= R). */
+ * ld_in >= C, ld_out >= R).  A utility for callers of gs2d_gemm_bf16 whose
+ * operands lie the other way round; the library itself needs none. */
 gs2d_status gs2d_transpose_bf16(const void* in, int32_t R, int32_t C, int32_t ld_in, void* out,
                                 int32_t ld_out, void* stream);
 

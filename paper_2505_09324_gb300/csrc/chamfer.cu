@@ -417,7 +417,8 @@ k_chamfer_grad(const float* __restrict__ P, int np, int ldp, const float* __rest
 
 // Mean squared distances of both directions of frame b, one block.  Sums of three
 // floats (FloatSum: no less accurate than double), one division per mean: with
-// double sums and divisions in every thread 33 us for 20 000 points a side, 17 so.
+// double sums and divisions in every thread 33 us for 20 000 points a side, 23 so
+// (cold; load latency of one block a frame).
 __global__ void __launch_bounds__(1024)
 k_chamfer_loss(const float* __restrict__ d1, int np, const float* __restrict__ d2, int nq,
                float* __restrict__ loss) {

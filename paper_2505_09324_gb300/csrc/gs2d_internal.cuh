@@ -172,8 +172,8 @@ __device__ __forceinline__ void set_status(WsHeader* h, int code) {
 // where n double additions round n - 1 times.  The loss sums run over every tile
 // in one or a few blocks, where FP64 (1/64 of the FP32 rate, and a warp
 // instruction costs the same however few lanes it has) was the whole time: 65 us
-// for the additions of the 65 280 tiles of eight 1080p frames, 2.5 us for the warps'
-// shuffle tree of any frame.
+// for the additions of the 65 280 tiles of eight 1080p frames, 5 to 6 us for the
+// warps' shuffle trees and the last sums of any frame.
 struct FloatSum {
   float hi = 0.0f, mid = 0.0f, lo = 0.0f;
   __device__ __forceinline__ static float two_sum(float& a, float x) {

@@ -16,8 +16,8 @@
 // Arithmetic: the assignment decides in single precision (explicitly rounded
 // FP32 operations, centres kept as float); every segment sum is an exact
 // integer (pixel centres as 2 x + 1 - 2 floor(seed), colours as
-// rint(c 2^20)), accumulated by warp-aggregated 64-bit atomics in any order;
-// means and covariances follow in a fixed sequence of double operations, so
+// rint(c 2^20)), gathered by the update or accumulated by warp-aggregated
+// 64-bit atomics, in any order; means and covariances follow in a fixed sequence of double operations, so
 // the result is reproducible bit for bit.
 #include <math.h>
 #include <stdio.h>
@@ -59,11 +59,11 @@ struct SpArgs {
 };
 
 // Segment sums of up to kGatherS pixels of grid step are gathered by the
-// update (one warp per centre over the pixels that can have joined it);
-// beyond that a centre's window is long and the centres are few, and the
-// assignment adds each pixel's moments with atomics instead.  The gathered
+// update (half a warp per centre, or several, over the pixels that can have
+// joined it); beyond that a centre's window is long and the centres are few, and
+// the assignment adds each pixel's moments with atomics instead.  The gathered
 // window is (2 S)^2 pixels per centre, 4 A in all whatever S is, so only the
-// number of warps falls with S: at 32 a warp has 128 steps of 32 pixels.
+// number of half-warps falls with S: at 32 each has 256 steps of 16 pixels.
 constexpr float kGatherS = 32.0f;
 constexpr int kWave = 152;  // blocks of one wave
 

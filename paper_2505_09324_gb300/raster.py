@@ -197,7 +197,7 @@ class GaussianRasterizer:
             adam_state = (torch.empty_like(params), torch.empty_like(params))
         m, v = adam_state
         shape = (9, self.n)
-        # the P-frame loop re-bins the workspace every iteration
+        # the P-frame loop re-bins the workspace (lists of other parameters)
         self.version += 1
         return nat.encode_pframe(self.plan, self.ws_ptr,
                                  _check(target, "target", self.image_shape()),
