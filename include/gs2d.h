@@ -785,7 +785,8 @@ gs2d_status gs2d_head_decode_bwd(const float* out, int32_t ldo, int32_t B, int32
  * means (rows 0, 1 of targets, [9][ldq], frame b in columns b m ...), per
  * frame: mean over predictions of the squared distance to the nearest target
  * plus mean over targets of the squared distance to the nearest prediction
- * (brute force).  loss: device float32[B] or NULL.  dparams: device, layout
+ * (exact: those a scan of all pairs in FP32 gives, of equal ones the first).
+ * loss: device float32[B] or NULL.  dparams: device, layout
  * of params, or NULL; rows 0, 1 get += lambda d(Chamfer)/d(mu) (float
  * atomics: the order of additions varies between runs).  scratch: device,
  * gs2d_chamfer_scratch_bytes(n, m, B). */

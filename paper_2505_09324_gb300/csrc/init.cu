@@ -17,8 +17,8 @@
 // FP32 operations, centres kept as float); every segment sum is an exact
 // integer (pixel centres as 2 x + 1 - 2 floor(seed), colours as
 // rint(c 2^20)), gathered by the update or accumulated by warp-aggregated
-// 64-bit atomics, in any order; means and covariances follow in a fixed sequence of double operations, so
-// the result is reproducible bit for bit.
+// 64-bit atomics, in any order; means and covariances follow in a fixed
+// sequence of double operations, so the result is reproducible bit for bit.
 #include <math.h>
 #include <stdio.h>
 

@@ -604,8 +604,8 @@ def test_chamfer_nearest_neighbours(nat, name):
 
 
 @pytest.mark.parametrize("n,m,kinds", [
-    (3001, 2503, ("dense", "dense")), (1000, 4000, ("spread", "away")), (2000, 9, ("away", "dense")),
-    (257, 5000, ("same", "spread")), (4096, 4095, ("two", "away"))])
+    (3001, 2503, ("dense", "dense")), (1000, 4000, ("spread", "away")),
+    (2000, 9, ("away", "dense")), (257, 5000, ("same", "spread")), (4096, 4095, ("two", "away"))])
 def test_chamfer_of_dense_and_distant_sets(nat, n, m, kinds):
     """Sets whose points the grid does not separate (one cell with most of them
     next to far outliers, tight clusters, a set far from the other, equal points)
